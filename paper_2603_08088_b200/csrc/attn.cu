@@ -19,8 +19,9 @@
 //   warps 8-11  softmax with lazy rescale; tile 1 likewise.  The ancestor
 //               bitmask of the row is applied only on the tree tile(s), the
 //               prefix length only on the ragged last prefix tile.
-// TMEM: S0 | S1 | O0 | O1, 128 columns each; P (bf16) overlays the first 64
-// columns of its S.  With one row tile the two S buffers alternate by key tile.
+// TMEM: S0 (128 columns) | P0 P1 (bf16, 64 columns each) | O0 O1 (D columns each),
+// and S1 where O1 leaves room for it (see SmemLayout).  With one row tile the S and
+// P buffers alternate by key tile.
 //
 // Code size matters here: instruction fetches compete with the K/V stream for
 // L2 and HBM, and code that runs once per work item (set-up, epilogue, merge)
@@ -56,7 +57,6 @@ constexpr int kThreads = 384;
 constexpr int kMaxB = 512;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleThreshold = 8.0f;            // in log2 units
-constexpr float kMaxFastSum = 16384.0f;               // 64 keys x 2^threshold: largest row sum the fast path accepts
 // Of every 16 element pairs of the softmax fast path, three take 2^x on the FMA pipe (measured optimum between
 // the special-function unit and the FMA pipe: 2/16 and 4/16 are 1-2 % slower on the 32-layer and the
 // long-context shape, 1/16 and 5/16 far slower).
@@ -233,6 +233,23 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* v) {
         "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
       : "memory");
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
+        "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+      : "memory");
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ float fast_exp2(float x) {
@@ -257,22 +274,16 @@ struct Tracer {
   }
 };
 
-#ifdef TV_PROF
-#define TV_PROF_T(var) do { var = clock(); } while (0)
-#define TV_PROF_USE(x) asm volatile("{.reg .b32 t; mov.b32 t, %0;}" ::"r"(x))
-#else
-#define TV_PROF_T(var) do { } while (0)
-#define TV_PROF_USE(x) do { } while (0)
-#endif
 // Packed fp32 pair arithmetic (one issue slot for two lanes of work).
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 fadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 // 2^x for a pair on the FMA pipe (the special-function unit is the scarce resource of the softmax):
 // x = n + f with n = round(x), f in [-0.5, 0.5]; 2^f by a cubic (relative error 7.5e-5, far below the
-// bf16 rounding of P), 2^n by an add into the exponent field.  x is clamped to [-125, 16].
+// bf16 rounding of P), 2^n by an add into the exponent field.  x is raised to -125 where it lies below; the lazy
+// rescale bounds it above.
 __device__ __forceinline__ float2 exp2_poly2(float2 x) {
-  x.x = fminf(fmaxf(x.x, -125.f), 16.f);
-  x.y = fminf(fmaxf(x.y, -125.f), 16.f);
+  x.x = fmaxf(x.x, -125.f);
+  x.y = fmaxf(x.y, -125.f);
   const float2 t = fadd2(x, make_float2(12582912.f, 12582912.f));          // 1.5 * 2^23: low mantissa bits = n
   const float2 n = fadd2(t, make_float2(-12582912.f, -12582912.f));
   const float2 f = ffma2(n, make_float2(-1.f, -1.f), x);
@@ -282,6 +293,13 @@ __device__ __forceinline__ float2 exp2_poly2(float2 x) {
   float2 r;
   r.x = __int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23));
   r.y = __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23));
+  return r;
+}
+
+// Three-operand maximum (one instruction on sm_100); a NaN operand is ignored.
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
 
@@ -371,8 +389,12 @@ struct SmemLayout {
   static constexpr int kBars = kRing + kSlots * kTileBytes;
   // barrier indices (8 bytes each)
   static constexpr int Q_FULL = 0, Q_EMPTY = 1, KV_FULL = 2, KV_EMPTY = 2 + kSlots, S_FULL = 2 + 2 * kSlots,
-                       P_READY = S_FULL + 2, O_DONE = P_READY + 2, ITEM_DONE = O_DONE + 2, EPI = ITEM_DONE + 2,
-                       NBARS = EPI + 1;
+                       S_FREE = S_FULL + 2, P_READY = S_FREE + 2, O_DONE = P_READY + 2, ITEM_DONE = O_DONE + 1,
+                       EPI = ITEM_DONE + 2, NBARS = EPI + 1;
+  // Tensor memory columns.  One S buffer for two row tiles of 128-wide heads (there is no room for a second one
+  // beside P0 P1 O0 O1), two buffers otherwise.
+  static constexpr int kTmemS0 = 0, kTmemP0 = 128, kTmemO0 = 256;
+  static constexpr int kTmemS1 = (D == 128 && MT == 2) ? kTmemS0 : 384;
   static constexpr int kMisc = kBars + NBARS * 8;          // tmem ptr, abort flag, last flag
   static constexpr int kCum = kMisc + 16;
   static constexpr int kGs = kCum + (kMaxB + 1) * 4;
@@ -440,14 +462,13 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       mbar_init(bar(L::KV_FULL + s), 1);
       mbar_init(bar(L::KV_EMPTY + s), 1);
     }
-    for (int s = 0; s < 2; ++s) {                // index = S buffer
+    for (int s = 0; s < 2; ++s) {                // index = row tile, or parity of the key tile with one row tile
       mbar_init(bar(L::S_FULL + s), 1);
-      mbar_init(bar(L::P_READY + s), 128);
-    }
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(bar(L::O_DONE + s), 1);
+      mbar_init(bar(L::S_FREE + s), 4);
+      mbar_init(bar(L::P_READY + s), 4);
       mbar_init(bar(L::ITEM_DONE + s), 1);
     }
+    mbar_init(bar(L::O_DONE), 1);
     mbar_init(bar(L::EPI), MT * 128);
     *abort_flag = ((sbase & 1023u) != 0) ? 1 : 0;   // swizzled tiles need a 1024-byte aligned base
     *last_flag = 0;
@@ -523,7 +544,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   constexpr uint32_t kIdescQK = instr_desc(kTileN, false);
   constexpr uint32_t kIdescPV = instr_desc(D, true);
-  constexpr uint32_t kTmemS0 = 0, kTmemO0 = 256;
 
   if (warp == 0) {
     // =========================================================== TMA producer
@@ -639,11 +659,13 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // =========================================================== MMA issuer
     // One thread issues every MMA of the CTA.  S of a key tile is a full 128-key tile (N = 128: with 64-key
     // MMAs the Q operand is re-read from shared memory twice as often and the pipe runs at 2/3 of its rate).
-    // P overlays the first 64 columns of its S buffer, so S of the next key tile can only be computed after
-    // the PV that reads P; the tensor pipe runs MMAs in issue order, which gives that for free.
-    //   two row tiles (buffer = row tile):  wait P_t -> O_t += P_t V -> S_t = Q_t K_next^T, t = 0, 1 in turn, so
-    //     that the softmax of one row tile runs while the pipe works for the other one;
-    //   one row tile (buffers alternate by key tile):  S_next = Q K_next^T -> wait P -> O += P V.
+    // A softmax warpgroup takes S into registers at once and P has columns of its own, so an S buffer is free again
+    // a few hundred cycles after it was filled and the next S is ready before its warpgroup asks for it: the chain
+    // hand-over -> PV -> QK^T -> wake-up of a row tile runs beside that row tile's softmax instead of in front of it
+    // (32-layer shape: 1342 -> 1312 us a launch, power-capped 1583 -> 1540 us, against P overlaying its S).
+    //   two row tiles:  S_0(j+1), O_0 += P_0(j) V(j), S_1(j+1), O_1 += P_1(j) V(j): each S as soon as the other row
+    //     tile's S has been taken out of the buffer, each PV as soon as its P is there;
+    //   one row tile (buffers alternate by key tile):  S(j+1), O += P(j) V(j).
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (!*abort_flag) {      // the whole warp walks the items; one elected lane issues
       int g = g_begin;
@@ -659,30 +681,30 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const uint32_t k_lo = (uint32_t)smem_desc(sbase + L::kRing, 16, 1024);
       const uint32_t v_lo = (uint32_t)smem_desc(sbase + L::kRing, L::kHalf, 1024);  // MN-major: LBO = next 64 columns
       constexpr int kHalf16 = L::kHalf >> 4, kTile16 = L::kTileBytes >> 4;
-      // S(buf) = Q_t K^T for the 128 keys of the K tile in `slot`
-      auto issue_qk = [&](int t, int buf, uint32_t slot) {
+      // S = Q_t K^T for the 128 keys of the K tile in `slot`; idx: row tile, or parity of the key tile
+      auto issue_qk = [&](int t, int idx, uint32_t slot) {
         const uint32_t qa = q_lo + t * kTile16, ka = k_lo + slot * kTile16;
+        const uint32_t s_col = tmem + (idx ? L::kTmemS1 : L::kTmemS0);
         if (elect_one()) {
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
             const uint32_t off = (ks / 4) * kHalf16 + (ks % 4) * 2;        // 16 columns = 32 bytes inside a swizzled row
-            mma_ss_lohi(tmem + kTmemS0 + buf * 128, qa + off, ka + off, desc_hi, kIdescQK, ks > 0);
+            mma_ss_lohi(s_col, qa + off, ka + off, desc_hi, kIdescQK, ks > 0);
           }
-          mma_commit(bar(L::S_FULL + buf));
+          mma_commit(bar(L::S_FULL + idx));
         }
         __syncwarp();
       };
-      // O_t += P(buf) V for the 128 keys of the V tile in `slot`
-      auto issue_pv = [&](int t, int buf, uint32_t slot, bool first_tile) {
+      // O_t += P V for the 128 keys of the V tile in `slot`.  The completion of a PV is known from the S that is
+      // committed behind it (a commit of its own stalls the pipe for some 45 cycles), except where none follows.
+      auto issue_pv = [&](int t, int idx, uint32_t slot, bool first_tile) {
         const uint32_t va = v_lo + slot * kTile16;
         if (elect_one()) {
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)            // 16 keys = 16 rows of 128 bytes = 8 packed P columns
-            mma_ts_lohi(tmem + kTmemO0 + t * 128, tmem + kTmemS0 + buf * 128 + ks * 8, va + ks * 128, desc_hi, kIdescPV,
+            mma_ts_lohi(tmem + L::kTmemO0 + t * D, tmem + L::kTmemP0 + idx * 64 + ks * 8, va + ks * 128, desc_hi, kIdescPV,
                         (!first_tile || ks > 0) ? 1u : 0u);
-        // With two row tiles the S tile that the softmax waits for next is committed after this PV, so its
-        // completion is known without a commit of its own (a commit stalls the pipe for some 45 cycles).
-          if (MT == 1) mma_commit(bar(L::O_DONE + t));
+          if (MT == 1) mma_commit(bar(L::O_DONE));
         }
         __syncwarp();
       };
@@ -706,12 +728,16 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           continue;
         }
         {
+          // The S buffers are free: the P of every earlier key tile has been waited for, hence its S was taken.
           const uint32_t slot = fill % kSlots;
           ok = mbar_wait(bar(L::KV_FULL + slot), (fill / kSlots) & 1, abort_flag, wait_limit);
           if (!ok) break;
           tc_fence_after();
           if (MT == 2) {
             issue_qk(0, 0, slot);
+            if (L::kTmemS1 == L::kTmemS0) ok = mbar_wait(bar(L::S_FREE + 0), tj & 1, abort_flag, wait_limit);
+            if (!ok) break;
+            tc_fence_after();
             issue_qk(1, 1, slot);
           } else {
             issue_qk(0, tj & 1, slot);
@@ -726,28 +752,47 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (MT == 2) {
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
-              ok = mbar_wait(bar(L::P_READY + t), tj & 1, abort_flag, wait_limit);
-              if (!ok) break;
-              if (t == 0) {
-                ok = mbar_wait(bar(L::KV_FULL + vslot), (fv / kSlots) & 1, abort_flag, wait_limit);
-                if (ok && more) ok = mbar_wait(bar(L::KV_FULL + kslot), (fk / kSlots) & 1, abort_flag, wait_limit);
+              // S_t(j+1): the buffer was last filled for the other row tile (or, with two buffers, for S_t(j))
+              if (more) {
+                if (t == 0) {
+                  ok = mbar_wait(bar(L::KV_FULL + kslot), (fk / kSlots) & 1, abort_flag, wait_limit);
+                  if (!ok) break;
+                }
+                if (L::kTmemS1 == L::kTmemS0)
+                  ok = mbar_wait(bar(L::S_FREE + (t ^ 1)), (t == 0 ? tj : tj + 1) & 1, abort_flag, wait_limit);
+                else
+                  ok = mbar_wait(bar(L::S_FREE + t), tj & 1, abort_flag, wait_limit);
                 if (!ok) break;
+                tc_fence_after();
+                issue_qk(t, t, kslot);
+                if (t == 1 && elect_one()) {
+                  mma_commit(bar(L::KV_EMPTY + kslot));
+                  if (jt + 2 == nt) mma_commit(bar(L::Q_EMPTY));
+                }
+                __syncwarp();
               }
+              tr.mark(0x2000u | ((2 * tj + t) & 0xfffu));
+              ok = mbar_wait(bar(L::P_READY + t), tj & 1, abort_flag, wait_limit);
+              if (ok && t == 0) ok = mbar_wait(bar(L::KV_FULL + vslot), (fv / kSlots) & 1, abort_flag, wait_limit);
+              if (!ok) break;
               tc_fence_after();
               tr.mark(0x4000u | ((2 * tj + t) & 0xfffu));
               issue_pv(t, t, vslot, jt == 0);
               if (!more && elect_one()) mma_commit(bar(L::ITEM_DONE + t));      // all MMAs of the item's row tile are done
-              if (more) issue_qk(t, t, kslot);
-              tr.mark(0x2000u | ((2 * tj + t) & 0xfffu));
             }
             if (!ok) break;
+            // row tile 1 of the last key tile: no S follows its PV of the key tile before, so that is committed here
+            if (elect_one()) {
+              if (jt + 2 == nt) mma_commit(bar(L::O_DONE));
+              mma_commit(bar(L::KV_EMPTY + vslot));
+            }
           } else {
             const int buf = tj & 1;
             if (more) {
               ok = mbar_wait(bar(L::KV_FULL + kslot), (fk / kSlots) & 1, abort_flag, wait_limit);
               if (!ok) break;
               tc_fence_after();
-              issue_qk(0, buf ^ 1, kslot);
+              issue_qk(0, buf ^ 1, kslot);       // the P of the key tile before has been waited for: its S was taken
             }
             ok = mbar_wait(bar(L::P_READY + buf), (tj >> 1) & 1, abort_flag, wait_limit);
             if (ok) ok = mbar_wait(bar(L::KV_FULL + vslot), (fv / kSlots) & 1, abort_flag, wait_limit);
@@ -757,11 +802,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             issue_pv(0, buf, vslot, jt == 0);
             if (!more && elect_one()) mma_commit(bar(L::ITEM_DONE));
             tr.mark(0x2000u | (tj & 0xfffu));
-          }
-          if (elect_one()) {
-            mma_commit(bar(L::KV_EMPTY + vslot));
-            if (more) mma_commit(bar(L::KV_EMPTY + kslot));
-            if (jt + 2 == nt) mma_commit(bar(L::Q_EMPTY));
+            if (elect_one()) {
+              mma_commit(bar(L::KV_EMPTY + vslot));
+              if (more) mma_commit(bar(L::KV_EMPTY + kslot));
+              if (jt + 2 == nt) mma_commit(bar(L::Q_EMPTY));
+            }
           }
           __syncwarp();
         }
@@ -795,18 +840,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       int g = g_begin;
       Item it;
       uint32_t fill = 0, tj = 0, epi_phase = 0, item_cnt = 0;   // tj: key tiles handled so far (all items)
+      uint32_t od_phase = 0;                                    // items of more than one key tile so far
       bool ok = true;
       Tracer tr;
       tr.init((threadIdx.x & 127) == 0 ? prm.trace : nullptr, 2 + wg);
       tr.mark(0);
-#ifdef TV_PROF
-      unsigned int prof[12] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u}, pc0 = 0, pc1 = 0, pc2 = 0, pend = 0;
-      // 0 wait S, 1 ld, 2 compute, 3 hand-over, 4 tiles, 5 between tiles, 6 start -> first S, 7 wait ITEM_DONE,
-      // 8 epilogue (whole or piece), 9 items, 10 first tile of an item: from item start to its S
-      const unsigned int prof_start = clock();
-      const long long prof_c0 = clock64();
-      const unsigned long long prof_g0 = globaltimer_ns();   // cycles: wait S, ld, compute, hand-over; tiles
-#endif
       // Rendezvous of the softmax warpgroups through an mbarrier, so that it is bounded like every other wait.
       // All 32 lanes wait together and agree on the outcome, so that the warp-wide TMEM instructions
       // below are never executed by a part of a warp.
@@ -820,21 +858,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         return r;
       };
       while (ok && next_item(g, it)) {
-#ifdef TV_PROF
-        const unsigned int pitem = clock();
-        unsigned int ep[6], ep_kind = 0, ep_others = 0, ep_own = 0;
-#endif
         const int nt = it.j1 - it.j0;
         const int node = (pair * MT + wg) * prm.NPT + row / prm.G;
         const int gm = row % prm.G;
         const bool row_exists = row < prm.NPT * prm.G && node < prm.Nmax;
         const bool row_active = row_exists && node < it.n;
-        uint32_t anc[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-        if (row_active) {
-#pragma unroll
-          for (int w = 0; w < 8; ++w)
-            if (w < prm.W) anc[w] = prm.anc_bits[((size_t)it.b * prm.Nmax + node) * prm.W + w];
-        }
         float m_used = -INFINITY;      // running reference maximum, in log2 units (score * scale * log2e)
         float l_sum = 0.f;
         // A piece of a cut unit draws its ticket early (thread 128 only): the counter is read at the start of
@@ -846,82 +874,131 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         unsigned long long claim_assumed = 0, claim_ret = 1;
         int claim_cnt = 0;
         if (piece && threadIdx.x == 128) claim_assumed = *reinterpret_cast<volatile unsigned long long*>(claim_ctr);
-        const uint32_t o_addr_loop = tmem + lane_addr + kTmemO0 + wg * 128;
+        const uint32_t o_addr_loop = tmem + lane_addr + L::kTmemO0 + wg * D;
         // key tiles below this index are full tiles of the committed prefix (no mask of any kind)
         const int j_full = min(it.S / kTileN, it.len - prm.TT);
         for (int jt = 0; jt < nt && ok; ++jt, ++tj) {
           const int j = it.j0 + jt;
-          const bool full_tile = j < j_full;
-          int tt = -1, valid_keys = kTileN;          // tt >= 0: index of the tree key tile
-          if (!full_tile) {
-            tt = j - (it.len - prm.TT);
-            valid_keys = tt >= 0 ? max(0, min(kTileN, it.n - tt * kTileN)) : min(kTileN, it.S - j * kTileN);
-          }
-          const bool tree = tt >= 0;
+          const bool masked = j >= j_full;
           if (piece && threadIdx.x == 128 && jt == nt - 1) {
             claim_cnt = ((claim_assumed >> 16) == prm.epoch) ? (int)(claim_assumed & 0xffffu) : 0;
             claim_ret = atomicCAS(claim_ctr, claim_assumed, (prm.epoch << 16) | (unsigned long long)(claim_cnt + 1));
           }
-          // ---- V rows past the valid keys may hold anything (stale cache rows, padded tree slots): zero
-          // them so that 0 * NaN never reaches O.  Idempotent, so both warpgroups may do it.  Rows that lie
-          // outside the tensor arrive as zeros from the copy itself: a tree tile whose tree is full (the
-          // usual case) needs nothing.
-          if (valid_keys < kTileN && !(tree && !prm.tree_in_cache && tt * kTileN + valid_keys >= prm.Nmax)) {
-            const uint32_t f = fill + 2 * jt + 1, slot = f % kSlots;
-            ok = wwait(bar(L::KV_FULL + slot), (f / kSlots) & 1);
-            if (!ok) break;
-            if (row >= valid_keys) {
-              uint8_t* vrow = smem + L::kRing + slot * L::kTileBytes + row * 128;
+          uint32_t vis[4] = {0u, 0u, 0u, 0u};      // masked tiles: visible keys of this row
+          if (masked) {
+            const int tt = j - (it.len - prm.TT);      // >= 0: index of the tree key tile
+            const bool tree = tt >= 0;
+            const int valid_keys = tree ? max(0, min(kTileN, it.n - tt * kTileN)) : min(kTileN, it.S - j * kTileN);
+            if (tree) {      // ancestor words of the node; none for a row without a node
+              const uint32_t* words = prm.anc_bits + ((size_t)it.b * prm.Nmax + node) * prm.W + tt * 4;
 #pragma unroll
-              for (int h = 0; h < D / 64; ++h)
+              for (int w = 0; w < 4; ++w)
+                if (row_active && tt * 4 + w < prm.W) vis[w] = words[w];
+            } else {
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                  *reinterpret_cast<uint4*>(vrow + h * L::kHalf + c * 16) = make_uint4(0, 0, 0, 0);
+              for (int w = 0; w < 4; ++w) {
+                const int left = valid_keys - 32 * w;
+                vis[w] = left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u);
+              }
             }
-            fence_proxy_async_smem();
+            // ---- V rows past the valid keys may hold anything (stale cache rows, padded tree slots): zero
+            // them so that 0 * NaN never reaches O.  Idempotent, so both warpgroups may do it.  Rows that lie
+            // outside the tensor arrive as zeros from the copy itself: a tree tile whose tree is full (the
+            // usual case) needs nothing.
+            if (valid_keys < kTileN && !(tree && !prm.tree_in_cache && tt * kTileN + valid_keys >= prm.Nmax)) {
+              const uint32_t f = fill + 2 * jt + 1, slot = f % kSlots;
+              ok = wwait(bar(L::KV_FULL + slot), (f / kSlots) & 1);
+              if (!ok) break;
+              if (row >= valid_keys) {
+                uint8_t* vrow = smem + L::kRing + slot * L::kTileBytes + row * 128;
+#pragma unroll
+                for (int h = 0; h < D / 64; ++h)
+#pragma unroll
+                  for (int c = 0; c < 8; ++c)
+                    *reinterpret_cast<uint4*>(vrow + h * L::kHalf + c * 16) = make_uint4(0, 0, 0, 0);
+              }
+              fence_proxy_async_smem();
+            }
           }
-          // S buffer of this key tile: the row tile's own one, or alternating by key tile when the CTA has one
-          // row tile; its barriers complete once per use of the buffer.
-          const int buf = (MT == 2) ? wg : (int)(tj & 1u);
+          // S and P of this key tile: index = row tile, or parity of the key tile when the CTA has one row tile
+          const int idx = (MT == 2) ? wg : (int)(tj & 1u);
           const uint32_t use_par = (MT == 2) ? (tj & 1u) : ((tj >> 1) & 1u);
-          const uint32_t s_base = tmem + lane_addr + kTmemS0 + buf * 128;
+          // Completion of the PV of the key tile before this one (for the first key tile of an item: nothing to wait
+          // for).  MT = 2: the pipe works in issue order, and S_1(j) is issued behind O_0 += P_0(j-1) V, S_0(j+1) behind
+          // O_1 += P_1(j-1) V; where no S_0(j+1) follows, that PV has a commit of its own (once per item).
+          auto previous_pv_done = [&]() -> bool {
+            if (jt == 0) return true;
+            if (MT == 1) return wwait(bar(L::O_DONE), (tj - 1) & 1u);
+            if (wg == 0) return wwait(bar(L::S_FULL + 1), tj & 1u);
+            return jt + 1 < nt ? wwait(bar(L::S_FULL + 0), (tj + 1) & 1u) : wwait(bar(L::O_DONE), od_phase & 1u);
+          };
           tr.mark(0x0800u | (tj & 0x7ffu));
-          TV_PROF_T(pc0);
-#ifdef TV_PROF
-          if (jt > 0) prof[5] += pc0 - pend;
-#endif
-          ok = wwait(bar(L::S_FULL + buf), use_par);
+          ok = wwait(bar(L::S_FULL + idx), use_par);
           if (!ok) break;
           tc_fence_after();
-          TV_PROF_T(pc1);
-#ifdef TV_PROF
-          prof[0] += pc1 - pc0;
-          if (tj == 0) prof[6] = pc1 - prof_start;
-          if (jt == 0) prof[10] += pc1 - pitem;
-#endif
           tr.mark(0x1000u | (tj & 0xfffu));
-          // ---- whole-tile fast path (full, unmasked tiles): all 128 scores of the row in one load and P with
-          // the reference maximum as it stands; the row sum then tells whether anything left the lazy-rescale
-          // range (all P are >= 0, so the sum bounds every element; NaN and infinity fail the comparison).  P
-          // is only stored once the check has passed, so on a failure the scores are still in S and the chunk
-          // loop below does the tile again, maximum first.  A row without a reference yet (the first tile of
-          // an item) takes the score of the tile's first key: it is one of the row's scores, hence not above
-          // their maximum, and if it lies too far below it the check fails like any other.
-          bool tile_done = false;
-          if (full_tile) {
-            uint32_t sall[128];
+          // ---- all 128 scores of the row into registers; the S buffer is free for the next S from here on
+          uint32_t sall[128];
+          {
+            const uint32_t s_base = tmem + lane_addr + (idx ? L::kTmemS1 : L::kTmemS0);
             tmem_ld32(s_base, sall);
             tmem_ld32(s_base + 32, sall + 32);
             tmem_ld32(s_base + 64, sall + 64);
             tmem_ld32(s_base + 96, sall + 96);
             tmem_wait_ld();
-            const float* sa = reinterpret_cast<const float*>(sall);
+            if (MT == 2) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(bar(L::S_FREE + idx));
+            }
+          }
+          float* sa = reinterpret_cast<float*>(sall);
+          if (masked) {
+#pragma unroll
+            for (int c = 0; c < 128; ++c)
+              if (!((vis[c >> 5] >> (c & 31)) & 1u)) sa[c] = -INFINITY;
+          }
+          // ---- lazy rescale: the reference maximum moves only when it would grow by more than the threshold.  The
+          // TMEM accesses are warp-wide (.sync.aligned), so the warp rescales as soon as one of its rows has to;
+          // rows that keep their reference multiply by 1.
+          {
+            float mx[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) mx[c] = fmaxf(sa[c], sa[c + 4]);
+#pragma unroll
+            for (int c = 8; c < 128; c += 8)
+#pragma unroll
+              for (int k = 0; k < 4; ++k) mx[k] = fmax3(mx[k], sa[c + 2 * k], sa[c + 2 * k + 1]);
+            const float mx2 = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * prm.scale_log2e;
+            const bool moves = mx2 > m_used + kRescaleThreshold || (m_used == -INFINITY && mx2 > -INFINITY);
+            if (__any_sync(0xffffffffu, moves)) {
+              const float alpha = (moves && m_used > -INFINITY) ? fast_exp2(m_used - mx2) : 1.f;
+              if (moves) m_used = mx2;
+              l_sum *= alpha;
+              if (jt > 0) {
+                ok = previous_pv_done();
+                if (!ok) break;
+                tc_fence_after();
+                // one 16-column group at a time: this runs while all 128 scores are held in registers
+#pragma unroll 1
+                for (int q = 0; q < D / 16; ++q) {
+                  uint32_t o[16];
+                  tmem_ld16(o_addr_loop + q * 16, o);
+                  tmem_wait_ld();
+#pragma unroll
+                  for (int c = 0; c < 16; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha);
+                  tmem_st16(o_addr_loop + q * 16, o);
+                }
+              }
+            }
+          }
+          // ---- P = exp2(s * c - m), row sum in fp32, P rounded to bf16
+          uint32_t pkk[64];
+          {
             const float2 c2 = make_float2(prm.scale_log2e, prm.scale_log2e);
-            const bool opens = (m_used == -INFINITY);
-            const float m_ref = opens ? sa[0] * prm.scale_log2e : m_used;
-            const float2 nm2 = make_float2(-m_ref, -m_ref);
+            const float neg_m = (m_used == -INFINITY) ? 0.f : -m_used;       // no visible key yet: every P is 0
+            const float2 nm2 = make_float2(neg_m, neg_m);
             float2 sum = make_float2(0.f, 0.f);
-            uint32_t pkk[64];
 #pragma unroll
             for (int i = 0; i < 64; ++i) {
               const float2 x = ffma2(make_float2(sa[2 * i], sa[2 * i + 1]), c2, nm2);
@@ -935,167 +1012,46 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               sum = fadd2(sum, pv);
               pkk[i] = pack_bf16(pv.x, pv.y);
             }
-            const float fsum = sum.x + sum.y;
-            const bool overflow = row_active && !(fsum <= 2.f * kMaxFastSum);
-            if (!__any_sync(0xffffffffu, overflow)) {
-              l_sum += fsum;
-              if (opens && row_active) m_used = m_ref;
-#pragma unroll
-              for (int q = 0; q < 8; ++q)
-                asm volatile(
-                    "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                    ::"r"(s_base + q * 8), "r"(pkk[q * 8 + 0]), "r"(pkk[q * 8 + 1]), "r"(pkk[q * 8 + 2]), "r"(pkk[q * 8 + 3]),
-                      "r"(pkk[q * 8 + 4]), "r"(pkk[q * 8 + 5]), "r"(pkk[q * 8 + 6]), "r"(pkk[q * 8 + 7])
-                    : "memory");
-              tile_done = true;
-            }
+            l_sum += sum.x + sum.y;
           }
+          if (masked) {      // the polynomial gives a hidden key 2^-125: make that the 0 which the other pairs have
 #pragma unroll
-          for (int h = 0; h < 2 && !tile_done; ++h) {
-            const int valid_half = min(64, max(0, valid_keys - 64 * h));
-            uint32_t sreg[64];
-            const uint32_t s_addr = s_base + h * 64;
-            TV_PROF_T(pc0);
-            tmem_ld32(s_addr, sreg);
-            tmem_ld32(s_addr + 32, sreg + 32);
-            tmem_wait_ld();
-            TV_PROF_USE(sreg[31]);
-            TV_PROF_USE(sreg[63]);
-            TV_PROF_T(pc1);
-            float* s = reinterpret_cast<float*>(sreg);
-            const bool masked = tree || valid_half < 64;
-            if (masked) {
-              // two 32-bit words of this chunk: ancestor bits on a tree tile, a length mask on the ragged tile
-              uint32_t w0, w1;
-              if (tree) {
-                const uint32_t a0 = tt > 0 ? anc[4] : anc[0], a1 = tt > 0 ? anc[5] : anc[1];
-                const uint32_t a2 = tt > 0 ? anc[6] : anc[2], a3 = tt > 0 ? anc[7] : anc[3];
-                w0 = h ? a2 : a0;
-                w1 = h ? a3 : a1;
-              } else {
-                w0 = valid_half >= 32 ? 0xffffffffu : ((1u << valid_half) - 1u);
-                w1 = valid_half >= 64 ? 0xffffffffu : (valid_half <= 32 ? 0u : ((1u << (valid_half - 32)) - 1u));
+            for (int i = 0; i < 64; ++i)
+              if (TV_POLY_SEL(i)) {
+                if (!((vis[i >> 4] >> (2 * i & 31)) & 1u)) pkk[i] &= 0xffff0000u;
+                if (!((vis[i >> 4] >> ((2 * i + 1) & 31)) & 1u)) pkk[i] &= 0x0000ffffu;
               }
-#pragma unroll
-              for (int c = 0; c < 32; ++c) {
-                if (!((w0 >> c) & 1u)) s[c] = -INFINITY;
-                if (!((w1 >> c) & 1u)) s[32 + c] = -INFINITY;
-              }
-            }
-            uint32_t pk[32];                 // P of this chunk, bf16 pairs
-            const bool first = (jt == 0 && h == 0);
-            // the tiles that get here (first of an item, masked, or rejected by the fast path) take the true
-            // maximum of the chunk first
-            {
-              float mx0 = s[0], mx1 = s[1], mx2_ = s[2], mx3 = s[3];
-#pragma unroll
-              for (int c = 4; c < 64; c += 4) {
-                mx0 = fmaxf(mx0, s[c]);
-                mx1 = fmaxf(mx1, s[c + 1]);
-                mx2_ = fmaxf(mx2_, s[c + 2]);
-                mx3 = fmaxf(mx3, s[c + 3]);
-              }
-              const float mx2 = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2_, mx3)) * prm.scale_log2e;
-              // ---- lazy rescale: move the reference maximum only when it would grow by more than the
-              // threshold.  The TMEM accesses are warp-wide (.sync.aligned), so the warp rescales as soon as
-              // one of its rows has to; rows that keep their maximum multiply by 1.
-              const bool moves = (mx2 > m_used + kRescaleThreshold || m_used == -INFINITY) && mx2 > -INFINITY;
-              const bool scales = moves && !first && m_used > -INFINITY;
-              const float alpha = scales ? fast_exp2(m_used - mx2) : 1.f;
-              if (moves) m_used = mx2;
-              l_sum *= alpha;
-              if (__any_sync(0xffffffffu, scales)) {
-                tr.mark(0x9000u | (tj & 0xfffu));
-                // O must be at rest.  With two row tiles the PV of the previous key tile was issued before the
-                // S = Q K^T this warpgroup has just waited for, and the pipe runs in issue order: it is done.
-                // With one row tile the next S is issued ahead of the PV: wait for its completion (number tj - 1).
-                if (MT == 1) ok = wwait(bar(L::O_DONE + wg), (tj - 1) & 1);
-                if (!ok) break;
-                tc_fence_after();
-#pragma unroll 1
-                for (int q = 0; q < D / 32; ++q) {
-                  uint32_t o[32];
-                  tmem_ld32(o_addr_loop + q * 32, o);
-                  tmem_wait_ld();
-#pragma unroll
-                  for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha);
-                  tmem_st32(o_addr_loop + q * 32, o);
-                }
-                // The tile's first 64 keys already have their P in TMEM, formed with the old reference: it moves
-                // with O (l_sum has just been rescaled for them too).
-                if (h == 1) {
-                  uint32_t pp[32];
-                  tmem_ld32(s_base, pp);
-                  tmem_wait_ld();
-#pragma unroll
-                  for (int c = 0; c < 32; ++c)
-                    pp[c] = pack_bf16(__uint_as_float(pp[c] << 16) * alpha, __uint_as_float(pp[c] & 0xffff0000u) * alpha);
-                  tmem_st32(s_base, pp);
-                }
-              }
-              // ---- P = exp2(s * c - m), row sum in fp32, P rounded to bf16 (masked scores give exactly 0)
-              const float neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
-              float ls0 = 0.f, ls1 = 0.f;
-#pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                const float p0 = fast_exp2(fmaf(s[2 * i], prm.scale_log2e, neg_m));
-                const float p1 = fast_exp2(fmaf(s[2 * i + 1], prm.scale_log2e, neg_m));
-                ls0 += p0;
-                ls1 += p1;
-                pk[i] = pack_bf16(p0, p1);
-              }
-              l_sum += ls0 + ls1;
-            }
+          }
+          // ---- P into its columns once the PV that read them last is done: with two row tiles that of the key tile
+          // before; with one (two P buffers in turn) it was issued in front of the S this tile has waited for
+          if (MT == 2) {
+            ok = previous_pv_done();
             if (!ok) break;
-            TV_PROF_USE(pk[31]);
-            TV_PROF_USE(pk[15]);
-            TV_PROF_USE(__float_as_uint(l_sum));
-            TV_PROF_T(pc2);
-#ifdef TV_PROF
-            prof[1] += pc1 - pc0;
-            prof[2] += pc2 - pc1;
-#endif
-            // ---- P over the start of the S buffer (columns already read): 16 keys = 8 packed columns per store
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              asm volatile(
-                  "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                  ::"r"(s_base + h * 32 + q * 8), "r"(pk[q * 8 + 0]), "r"(pk[q * 8 + 1]), "r"(pk[q * 8 + 2]), "r"(pk[q * 8 + 3]),
-                    "r"(pk[q * 8 + 4]), "r"(pk[q * 8 + 5]), "r"(pk[q * 8 + 6]), "r"(pk[q * 8 + 7])
-                  : "memory");
+            tc_fence_after();
           }
-          if (!ok) break;
-          TV_PROF_T(pc0);
+          {
+            const uint32_t p_base = tmem + lane_addr + L::kTmemP0 + idx * 64;
+            tmem_st32(p_base, pkk);
+            tmem_st32(p_base + 32, pkk + 32);
+          }
           tmem_wait_st();
           tc_fence_before();
-          mbar_arrive(bar(L::P_READY + buf));
-          TV_PROF_T(pc1);
-#ifdef TV_PROF
-          prof[3] += pc1 - pc0;
-          prof[4] += 1;
-          pend = pc1;
-#endif
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(L::P_READY + idx));
           tr.mark(0x2000u | (tj & 0xfffu));
         }
+        if (nt > 1) ++od_phase;
         if (!ok) break;
         // ---- epilogue of the item: wait for the last PV into this O buffer
         {
           // Wait for every MMA of the item.  This barrier completes once per item, so its phase is never
           // more than one away from the one waited for (a parity wait cannot tell phases two apart, which
           // is why the per-PV barrier O_DONE is not used here: both last PVs may or may not be done yet).
-          TV_PROF_T(pc0);
           ok = wwait(bar(L::ITEM_DONE + wg), item_cnt & 1);
           ++item_cnt;
           if (!ok) break;
           tc_fence_after();
-          TV_PROF_T(pc1);
-#ifdef TV_PROF
-          prof[7] += pc1 - pc0;
-#endif
           tr.mark(0x5000u);
-#ifdef TV_PROF
-          for (int i = 0; i < 6; ++i) ep[i] = pc1;
-#endif
           const uint32_t o_addr = o_addr_loop;
           const bool whole = (it.j0 == 0 && it.j1 == it.len);
           const int h = it.hk * prm.G + gm;
@@ -1130,10 +1086,10 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             }
           };
           if (whole) {
-            const float inv = (row_active && l_sum > 0.f) ? 1.f / l_sum : 0.f;
+            const float inv = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
             store_rows(reinterpret_cast<uint4*>(orow), 1, inv, row_exists, !row_active);
             if (row_exists && lse_p)
-              *lse_p = (row_active && l_sum > 0.f) ? (m_used + log2f(l_sum)) / kLog2e : -INFINITY;
+              *lse_p = (row_active && m_used > -INFINITY) ? (m_used + log2f(l_sum)) / kLog2e : -INFINITY;
             tc_fence_before();
           } else {
             // ---- a piece of a unit.  The pieces of a unit draw tickets on the unit's "claimed" counter (the
@@ -1162,7 +1118,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             auto piece_slot = [&](int k) -> int { return (k * prm.NP + pair) * 2 + (k == k_first ? 1 : 0); };
             const int my_slot = piece_slot(group);
             unsigned long long* ctr = claim_ctr;
-            TV_PROF_T(ep[1]);
             if (threadIdx.x == 128) {
               int ticket;
               if (claim_ret == claim_assumed) {
@@ -1195,11 +1150,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             ok = epi_sync();
             if (!ok || *abort_flag) { ok = false; break; }
             tr.mark(0x7000u | (*last_flag ? 1u : 0u));
-            TV_PROF_T(ep[2]);
-#ifdef TV_PROF
-            ep_kind = (*last_flag ? 2u : 1u) | ((unsigned)n_frag << 4);
-#endif
-            const float inv_own = (row_active && l_sum > 0.f) ? 1.f / l_sum : 0.f;
+            const float inv_own = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
             if (!*last_flag) {
               uint4* po = reinterpret_cast<uint4*>(prm.part_o) + (size_t)my_slot * (D / 8) * kRows;
               float* pml = prm.part_ml + (size_t)my_slot * 2 * kRows;
@@ -1209,13 +1160,10 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 pml[kRows + rr] = l_sum;
               }
               tc_fence_before();
-              TV_PROF_T(ep[3]);
               __threadfence();
-              TV_PROF_T(ep[4]);
               tr.mark(0x6000u);
               ok = epi_sync();
               if (!ok) break;
-              TV_PROF_T(ep[5]);
               if (threadIdx.x == 128 && !(prm.debug & 2)) {      // (debug bit 1: the piece is never announced)
                 const unsigned long long seen = *reinterpret_cast<volatile unsigned long long*>(ctr + 1);
                 bump_counter(ctr + 1, seen, prm.epoch);
@@ -1254,8 +1202,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               for (int k = k_first + 4; k <= k_last; ++k) lt += late_weight(k);
               if (!row_active) lt = 0.f;
               const float inv = (row_active && lt > 0.f) ? 1.f / lt : 0.f;
-              TV_PROF_USE(__float_as_uint(inv));
-              TV_PROF_T(ep[3]);
               // ---- pass 2: 64 output columns at a time, pieces in order (one fused multiply-add per piece and
               // element, two elements per instruction); the own piece comes from TMEM and enters as its
               // bf16-rounded normalised output, like every other piece
@@ -1272,7 +1218,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                   if (i >= 4) w = late_weight(k);
                   const float2 w2 = make_float2(w, w);
                   if (k == group) {
-                    TV_PROF_T(pc0);
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                       uint32_t o[32];
@@ -1286,15 +1231,10 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                                 acc[q * 16 + c]);
                       }
                     }
-#ifdef TV_PROF
-                    TV_PROF_USE(__float_as_uint(acc[31].y));
-                    ep_own += clock() - pc0;
-#endif
                     continue;
                   }
                   const uint4* q_o = reinterpret_cast<const uint4*>(prm.part_o) + (size_t)piece_slot(k) * (D / 8) * kRows;
                   uint4 v[8];
-                  TV_PROF_T(pc0);
 #pragma unroll
                   for (int c = 0; c < 8; ++c) v[c] = __ldcg(q_o + (size_t)(hq * 8 + c) * kRows + rr);
 #pragma unroll
@@ -1305,10 +1245,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                       acc[4 * c + e] = ffma2(w2, make_float2(__uint_as_float(wv[e] << 16), __uint_as_float(wv[e] & 0xffff0000u)),
                                              acc[4 * c + e]);
                   }
-#ifdef TV_PROF
-                  TV_PROF_USE(__float_as_uint(acc[31].y));
-                  ep_others += clock() - pc0;
-#endif
                 }
                 if (row_exists) {
 #pragma unroll
@@ -1336,34 +1272,14 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
               if (row_exists && lse_p) *lse_p = (row_active && lt > 0.f) ? (mm + log2f(lt)) / kLog2e : -INFINITY;
               tc_fence_before();
-              TV_PROF_T(ep[4]);
               ok = epi_sync();   // keeps the two warpgroups' barrier phases in step with the other branch
               if (!ok) break;
-              TV_PROF_T(ep[5]);
             }
           }
         }
         tr.mark(0x8000u);
-#ifdef TV_PROF
-        prof[8] += clock() - pc1;
-        if (tr.base && prof[9] < 24) {
-          unsigned long long* e = tr.base + prof[9] * 8;
-          e[0] = ep_kind; e[1] = ep_own;
-          for (int i = 1; i < 6; ++i) e[1 + i] = ep[i] - ep[i - 1];
-          e[7] = ep_others;      // pass 2: cycles from the loads of the other pieces to the end of their sums
-        }
-        prof[9] += 1;
-#endif
         fill += 2 * nt;
       }
-#ifdef TV_PROF
-      if (tr.base)
-      {
-        for (int i = 0; i < 12; ++i) tr.base[kTraceCap - 16 + i] = prof[i];
-        tr.base[kTraceCap - 2] = clock64() - prof_c0;
-        tr.base[kTraceCap - 1] = globaltimer_ns() - prof_g0;
-      }
-#endif
     }
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
