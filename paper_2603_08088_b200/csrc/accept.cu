@@ -270,15 +270,7 @@ __global__ void node_scores_kernel(const tv_bf16* __restrict__ logits, const int
 int scan_chunks(int V) { return (V + kChunkElems - 1) / kChunkElems; }
 
 // CTAs of the persistent scan: three per SM (what its registers allow).
-int scan_ctas() {
-  static int n = [] {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148 * 3;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 148 * 3;
-    return sms * 3;
-  }();
-  return n;
-}
+int scan_ctas() { return 3 * tv::sm_count(); }
 
 // Scratch of tree_accept_noalloc: a fixed device array that lives in the library image, so that callers
 // who may not allocate device memory can still run the accept step.  Every GPU that loads the library

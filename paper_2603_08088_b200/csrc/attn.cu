@@ -1336,16 +1336,6 @@ struct Geometry {
   size_t ml_off, o_off, counters_off, counters_per_layer, total;
 };
 
-int sm_count() {
-  static int sms = [] {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-    return n;
-  }();
-  return sms;
-}
-
 constexpr int kCounterLayers = 32;      // layers whose counters the workspace of tv_attn_workspace_bytes holds
 
 Geometry geometry(int B, int Nmax, int Hq, int Hkv, int d, bool query_device) {
@@ -1355,7 +1345,7 @@ Geometry geometry(int B, int Nmax, int Hq, int Hkv, int d, bool query_device) {
   g.n_row_tiles = (Nmax + g.NPT - 1) / g.NPT;
   g.MT = g.n_row_tiles > 1 ? 2 : 1;
   g.NP = (g.n_row_tiles + g.MT - 1) / g.MT;
-  g.sms = query_device ? sm_count() : 148;
+  g.sms = query_device ? tv::sm_count() : 148;
   g.groups = g.sms / g.NP > 0 ? g.sms / g.NP : 1;
   g.grid = g.groups * g.NP;
   // workspace: (m,l) pairs, partial O (both sized for 160 SMs so the size does not depend on the device), then

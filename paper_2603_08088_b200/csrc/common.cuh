@@ -59,6 +59,9 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 #endif
 
+// Streaming multiprocessors of the current device (of the first device asked about: the library is for one GPU model).
+int sm_count();
+
 // Process-wide count of kernels this library has launched (diagnostics only).
 void count_launches(int n);
 

@@ -6,22 +6,23 @@
 // child passes, the next token is drawn from what is left of p by inversion of the cumulative sum in
 // vocabulary order at u_bonus.  p = softmax(logits / T) of the current node's row.
 //
-// Phase 1 (row_stats_kernel) streams logits[B,Nmax,V] once, like the argmax scan: every CTA reduces one
-// vocabulary chunk of one row to (max, sum of 2^((l - max) k)), k = log2(e) / T.  Phase 2
-// (sample_walk_kernel), one CTA per sequence: folds the chunk pairs per row in chunk order, gathers the mass
-// of every node's token in its parent's row, walks the tree with one thread, and then all threads draw the
-// next token from the last node's row (segment sums in vocabulary order, a serial prefix over the segments,
-// a rescan of the segment that holds the target).  All arithmetic in fp32.
+// Phase 1 (row_stats_kernel) streams logits[B,Nmax,V] once: every warp reduces one vocabulary chunk of one row to
+// (max, sum of 2^((l - max) k)), k = log2(e) / T.  Phase 2 (sample_walk_kernel), one CTA per sequence: folds the
+// chunk pairs per row, gathers the mass of every node's token in its parent's row, walks the tree with one warp, and
+// draws the next token from the last node's row by two scans in vocabulary order: over the masses of its chunks, then
+// over the entries of the chunk that holds the target.  All arithmetic in fp32.
 #include "common.cuh"
+#include "logits.cuh"
 
 #include <cuda_bf16.h>
 
 namespace {
 
 constexpr int kStatThreads = 256;
-constexpr int kStatVecPerThread = 4;
-constexpr int kStatChunk = kStatThreads * kStatVecPerThread * 8;      // 8192 logits per CTA
-constexpr int kWalkThreads = 256;
+constexpr int kStatVecs = 8;                                          // 16-byte loads in flight per lane
+constexpr int kStatChunk = 32 * kStatVecs * 8;                        // 2048 logits per warp and item
+constexpr int kWalkThreads = 1024;
+constexpr int kLanesPerRow = 8;                                       // lanes that fold one row's chunk pairs
 constexpr int kMaxNodes = 256;
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -53,63 +54,120 @@ __device__ __forceinline__ void merge_pair(float& m, float& s, float mo, float s
   }
 }
 
-__global__ void __launch_bounds__(kStatThreads)
+// Persistent scan, one warp per (row, chunk) item, no barrier anywhere: a warp requests the vectors of its next item
+// before it reduces the ones it holds, takes the chunk's maximum first (packed bf16) and then one exponential per
+// logit.  Bounds: the logits once through HBM (295 MB: 45 us), one special-function result per logit (147 M: 32 us).
+// Chunks of 2048 per warp, three CTAs an SM: with one chunk of 8192 per CTA and a block reduction this kernel took 99 us,
+// with two CTAs an SM a call takes 2 us more, with four loads a lane and four CTAs 7 us more; 128.6 -> 65.6 us a call,
+// both kernels (16 x 60 rows of 153600).
+__global__ void __launch_bounds__(kStatThreads, 3)
 row_stats_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict__ n_nodes, int Nmax, int V,
-                 int n_chunks, float k, RowStat* __restrict__ stats) {
-  const int row = blockIdx.y;
-  const int b = row / Nmax, i = row - b * Nmax;
-  if (i >= n_nodes[b]) return;
-  const int c0 = blockIdx.x * kStatChunk;
-  const int c1 = min(V, c0 + kStatChunk);
-  const uint16_t* base = reinterpret_cast<const uint16_t*>(logits) + (size_t)row * V;
-  const int tid = threadIdx.x;
-  // the chunk's values of this thread stay in registers between the two passes (maximum, then sum)
-  float vals[kStatVecPerThread * 8];
-  const bool vec_ok = ((V & 7) == 0) && ((reinterpret_cast<uintptr_t>(logits) & 15u) == 0);
+                 int n_chunks, int n_items, float k, RowStat* __restrict__ stats) {
+  tv::pdl_enter();
+  const int lane = threadIdx.x & 31;
+  const int n_warps = gridDim.x * (kStatThreads / 32);
+  auto locate = [&](int item, int& row, int& chunk) -> bool {
+    if (item >= n_items) return false;
+    row = item / n_chunks;
+    chunk = item - row * n_chunks;
+    const int b = row / Nmax;
+    return row - b * Nmax < n_nodes[b];
+  };
+  auto fetch = [&](int row, int chunk, uint4* u) {
+    const tv::LogitsRow r(logits, row, V);
 #pragma unroll
-  for (int q = 0; q < kStatVecPerThread; ++q) {
-    const int v0 = c0 + (q * kStatThreads + tid) * 8;
-    if (vec_ok && v0 + 8 <= c1) {
-      const uint4 u = __ldcs(reinterpret_cast<const uint4*>(base + v0));
-      const uint32_t e[4] = {u.x, u.y, u.z, u.w};
+    for (int q = 0; q < kStatVecs; ++q) u[q] = r.vector((chunk * kStatVecs + q) * 32 + lane);
+  };
+  int item = blockIdx.x * (kStatThreads / 32) + (threadIdx.x >> 5);
+  int row = 0, chunk = 0;
+  bool active = locate(item, row, chunk);
+  uint4 u[kStatVecs];
+  if (active) fetch(row, chunk, u);
+  while (item < n_items) {
+    const int nitem = item + n_warps;
+    int nrow = 0, nchunk = 0;
+    const bool nactive = locate(nitem, nrow, nchunk);
+    uint4 un[kStatVecs];
+    if (nactive) fetch(nrow, nchunk, un);
+    if (active) {
+      __nv_bfloat162 mx = *reinterpret_cast<const __nv_bfloat162*>(&u[0].x);
 #pragma unroll
-      for (int t = 0; t < 8; ++t) vals[q * 8 + t] = bf16_to_float((t & 1) ? (e[t >> 1] >> 16) : (e[t >> 1] & 0xffffu));
-    } else {
+      for (int q = 0; q < kStatVecs; ++q) {
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u[q]);
+        mx = __hmax2(mx, __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3])));
+      }
+      // entries outside the row's whole vectors, in the chunk they lie in
+      float rest = -INFINITY;
+      if (lane < 16 && (chunk == 0 || chunk >= n_chunks - 2)) {
+        const tv::LogitsRow r(logits, row, V);
+        const int v = r.edge(lane);
+        if (v >= 0 && (v + r.off) / kStatChunk == chunk) rest = bf16_to_float(r.row[v]);
+      }
+      float m = fmaxf(fmaxf(__low2float(mx), __high2float(mx)), rest);      // max of a NaN and x is x: only NaNs give a NaN
+      if (!(m == m)) m = -INFINITY;
 #pragma unroll
-      for (int t = 0; t < 8; ++t) vals[q * 8 + t] = (v0 + t < c1) ? bf16_to_float(base[v0 + t]) : -INFINITY;
+      for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+      float s = 0.f;
+      if (m > -INFINITY) {
+        const float2 k2 = make_float2(k, k), mk2 = make_float2(-m * k, -m * k);
+        float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < kStatVecs; ++q) {
+          const uint32_t e[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            float2 x = __ffma2_rn(make_float2(__uint_as_float(e[t] << 16), __uint_as_float(e[t] & 0xffff0000u)), k2, mk2);
+            x.x = ex2_approx(fmaxf(x.x, -150.f));
+            x.y = ex2_approx(fmaxf(x.y, -150.f));
+            sum = __fadd2_rn(sum, x);
+          }
+        }
+        s = sum.x + sum.y + mass_of(rest, m, k);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      }
+      if (lane == 0) {
+        RowStat out;
+        out.m = m;
+        out.s = s;
+        stats[(size_t)row * n_chunks + chunk] = out;
+      }
     }
-  }
-  // per thread, then per warp (pairs merged by shuffles), then one barrier and a fold of the eight warp pairs
-  float m = -INFINITY;
+    item = nitem;
+    row = nrow;
+    chunk = nchunk;
+    active = nactive;
 #pragma unroll
-  for (int t = 0; t < kStatVecPerThread * 8; ++t) m = fmaxf(m, vals[t]);      // a NaN never becomes the maximum
-  float s = 0.f;
-  if (m > -INFINITY) {
-#pragma unroll
-    for (int t = 0; t < kStatVecPerThread * 8; ++t) s += mass_of(vals[t], m, k);
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float mo = __shfl_xor_sync(0xffffffffu, m, off);
-    const float so = __shfl_xor_sync(0xffffffffu, s, off);
-    merge_pair(m, s, mo, so, k);
-  }
-  __shared__ float red_m[kStatThreads / 32], red_s[kStatThreads / 32];
-  if ((tid & 31) == 0) {
-    red_m[tid >> 5] = m;
-    red_s[tid >> 5] = s;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < kStatThreads / 32; ++w) merge_pair(m, s, red_m[w], red_s[w], k);
-    RowStat out;
-    out.m = m;
-    out.s = s;
-    stats[(size_t)row * n_chunks + blockIdx.x] = out;
+    for (int q = 0; q < kStatVecs; ++q) u[q] = un[q];
   }
 }
 
+// Inclusive scan over the CTA in thread order; `total` is the sum over all threads.  Two barriers.
+__device__ __forceinline__ float block_scan(float v, float* warp_sums, float& total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const float o = __shfl_up_sync(0xffffffffu, v, off);
+    if (lane >= off) v += o;
+  }
+  if (lane == 31) warp_sums[warp] = v;
+  __syncthreads();
+  float w = warp_sums[lane];                   // kWalkThreads / 32 = 32 warps
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const float o = __shfl_up_sync(0xffffffffu, w, off);
+    if (lane >= off) w += o;
+  }
+  total = __shfl_sync(0xffffffffu, w, 31);
+  const float before = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
+  __syncthreads();
+  return v + (warp > 0 ? before : 0.f);
+}
 
+// One CTA per sequence.  A chain of dependent round trips, so everything that does not depend on the row statistics
+// (tree, tokens, uniforms, the token logits) is fetched while row_stats_kernel still runs: that kernel lets this one
+// start only after every earlier kernel of the stream has completed, and the loads bypass L1.  The draw reads one chunk
+// of the row (4 KB) and not the row up to the crossing (walk and draw took 37 us before).
 __global__ void __launch_bounds__(kWalkThreads)
 sample_walk_kernel(const tv_bf16* __restrict__ logits, const RowStat* __restrict__ stats, int n_chunks,
                    const int32_t* __restrict__ tokens, const int32_t* __restrict__ parent,
@@ -117,90 +175,111 @@ sample_walk_kernel(const tv_bf16* __restrict__ logits, const RowStat* __restrict
                    const float* __restrict__ u_bonus, float k, int Nmax, int V, int Dp1,
                    int32_t* __restrict__ accept_len, int32_t* __restrict__ accepted_nodes,
                    int32_t* __restrict__ next_token, int32_t* __restrict__ status) {
+  static_assert(kWalkThreads == 1024 && kMaxNodes <= kWalkThreads, "block_scan and the node arrays rely on it");
   __shared__ float sM[kMaxNodes], sZ[kMaxNodes], sE[kMaxNodes], sU[kMaxNodes];   // row max, row sum, token mass, uniform
   __shared__ int sPar[kMaxNodes], sTok[kMaxNodes], sRej[kMaxNodes];
+  __shared__ float sRejE[kMaxNodes];
   __shared__ float sWarp[kWalkThreads / 32];
-  __shared__ int sLast, sNrej, sHit, sBad;
-  __shared__ float sTarget;
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int n = n_nodes[b];
+  __shared__ int sLast, sNrej, sChunk, sHit, sLastMass;
+  __shared__ float sTarget, sExcl;
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  int n = __ldcg(n_nodes + b);
   n = n < 0 ? 0 : (n > Nmax ? Nmax : n);
   const uint16_t* lg = reinterpret_cast<const uint16_t*>(logits) + (size_t)b * Nmax * V;
-  if (tid == 0) sBad = 0;
-  // ---- per-row maximum and sum: the chunk pairs folded in chunk order (one pass, rescaling as the maximum grows)
-  for (int i = tid; i < n; i += kWalkThreads) {
-    const RowStat* rs = stats + ((size_t)b * Nmax + i) * n_chunks;
-    float M = -INFINITY, Z = 0.f;
-    for (int c = 0; c < n_chunks; ++c) {
-      const RowStat r = rs[c];
-      if (r.m > -INFINITY) {
-        const float Mn = fmaxf(M, r.m);
-        Z = Z * exp2f((M - Mn) * k) + r.s * exp2f((r.m - Mn) * k);       // M = -inf the first time: 0 * 0
-        M = Mn;
-      }
+  float tok_logit = -INFINITY;
+  bool bad = false;
+  if (tid < n) {
+    const int p = __ldcg(parent + (size_t)b * Nmax + tid), x = __ldcg(tokens + (size_t)b * Nmax + tid);
+    const int sp = (p >= 0 && p < n) ? p : 0;            // dummy-root remap (Section 3.2)
+    sPar[tid] = sp;
+    sTok[tid] = x;
+    sU[tid] = __ldcg(u_node + (size_t)b * Nmax + tid);
+    if (tid >= 1) {
+      bad = x < 0 || x >= V;
+      if (!bad) tok_logit = bf16_to_float(__ldcg(lg + (size_t)sp * V + x));
     }
-    sM[i] = M;
-    sZ[i] = Z;
-    const int p = parent[(size_t)b * Nmax + i];
-    sPar[i] = (p >= 0 && p < n) ? p : 0;                 // dummy-root remap (Section 3.2)
-    sTok[i] = tokens[(size_t)b * Nmax + i];
-    sU[i] = u_node[(size_t)b * Nmax + i];
+  }
+  const float ub = __ldcg(u_bonus + b);
+  if (tid == 0) {
+    sChunk = sHit = sLastMass = -1;
+  }
+  tv::pdl_enter();
+  const bool any_bad = __syncthreads_or(bad);
+  // ---- per-row maximum and sum: kLanesPerRow lanes fold a row's chunk pairs
+  for (int i0 = 0; i0 < n; i0 += kWalkThreads / kLanesPerRow) {
+    const int i = i0 + tid / kLanesPerRow;
+    float M = -INFINITY, Z = 0.f;
+    if (i < n) {
+      const RowStat* rs = stats + ((size_t)b * Nmax + i) * n_chunks;
+#pragma unroll 8
+      for (int c = tid % kLanesPerRow; c < n_chunks; c += kLanesPerRow) merge_pair(M, Z, rs[c].m, rs[c].s, k);
+    }
+#pragma unroll
+    for (int off = kLanesPerRow / 2; off > 0; off >>= 1) {
+      const float mo = __shfl_xor_sync(0xffffffffu, M, off), so = __shfl_xor_sync(0xffffffffu, Z, off);
+      merge_pair(M, Z, mo, so, k);
+    }
+    if (i < n && tid % kLanesPerRow == 0) {
+      sM[i] = M;
+      sZ[i] = Z;
+    }
   }
   __syncthreads();
   // ---- mass of every node's token in its parent's row (the node score of Section 3.3, exponentiated)
-  for (int i = tid; i < n; i += kWalkThreads) {
-    float e = 0.f;
-    if (i >= 1) {
-      const int x = sTok[i];
-      if (x >= 0 && x < V) {
-        e = mass_of(bf16_to_float(lg[(size_t)sPar[i] * V + x]), sM[sPar[i]], k);
-      } else {
-        sBad = 1;            // benign race: every writer stores 1
-      }
-    }
-    sE[i] = e;
-  }
+  if (tid < n) sE[tid] = (tid >= 1 && !bad) ? mass_of(tok_logit, sM[sPar[tid]], k) : 0.f;
   __syncthreads();
-  // ---- the walk (one thread, shared memory only; at most Nmax steps in all)
-  if (tid == 0) {
+  // ---- the walk (one warp): the children of a node are found 32 nodes at a time and tried in node order
+  if (tid < 32) {
     int c = 0, depth = 0, nrej = 0;
     float rem = n > 0 ? sZ[0] : 0.f;
-    for (int j = 0; j < Dp1; ++j) accepted_nodes[(size_t)b * Dp1 + j] = 0;
+    for (int j = lane; j < Dp1; j += 32) accepted_nodes[(size_t)b * Dp1 + j] = 0;
+    __syncwarp();
     while (depth < Dp1 - 1) {
       int acc = -1;
-      for (int kk = c + 1; kk < n; ++kk) {
-        if (sPar[kk] != c) continue;
-        const int x = sTok[kk];
-        if (x < 0 || x >= V) continue;
-        bool dup = false;
-        for (int r = 0; r < nrej; ++r) dup |= (sRej[r] == x);
-        if (dup) continue;
-        const float prob = rem > 0.f ? sE[kk] / rem : 0.f;
-        if (sU[kk] < prob) {
-          acc = kk;
-          break;
+      for (int base = (c + 1) & ~31; base < n && acc < 0; base += 32) {
+        const int kk = base + lane;
+        bool child = kk > c && kk < n && sPar[kk] == c;
+        if (child) child = sTok[kk] >= 0 && sTok[kk] < V;
+        unsigned todo = __ballot_sync(0xffffffffu, child);
+        while (todo) {
+          const int cand = base + __ffs(todo) - 1;
+          todo &= todo - 1;
+          const int x = sTok[cand];
+          bool dup = false;
+          for (int r0 = 0; r0 < nrej; r0 += 32) dup |= __any_sync(0xffffffffu, r0 + lane < nrej && sRej[r0 + lane] == x);
+          if (dup) continue;
+          const float prob = rem > 0.f ? sE[cand] / rem : 0.f;
+          if (sU[cand] < prob) {
+            acc = cand;
+            break;
+          }
+          if (lane == 0) {
+            sRej[nrej] = x;
+            sRejE[nrej] = sE[cand];
+          }
+          __syncwarp();
+          ++nrej;
+          rem -= sE[cand];
         }
-        sRej[nrej++] = x;
-        rem -= sE[kk];
       }
       if (acc < 0) break;
       ++depth;
-      accepted_nodes[(size_t)b * Dp1 + depth] = acc;
+      if (lane == 0) accepted_nodes[(size_t)b * Dp1 + depth] = acc;
       c = acc;
       nrej = 0;
       rem = sZ[c];
     }
-    accept_len[b] = depth;
-    sLast = c;
-    sNrej = nrej;
-    sTarget = u_bonus[b] * fmaxf(rem, 0.f);       // in units of the remaining (unnormalised) mass
-    sHit = -1;
-    if (sBad) atomicOr(status + b, TV_ST_BAD_INDEX);
+    if (lane == 0) {
+      accept_len[b] = depth;
+      sLast = c;
+      sNrej = nrej;
+      sTarget = ub * fmaxf(rem, 0.f);       // in units of the remaining (unnormalised) mass
+      if (any_bad) atomicOr(status + b, TV_ST_BAD_INDEX);
+    }
   }
   __syncthreads();
-  // ---- next token: the first entry of row c, rejected tokens left out, whose cumulative mass in vocabulary
-  // order exceeds the target.  The row is streamed 64 entries per thread and step (one 128-byte line each, a
-  // warp reads 4 KB in a row); the running sum passes from step to step through a block-wide scan.
+  // ---- next token: the first entry of row c, rejected tokens left out, whose cumulative mass in vocabulary order
+  // exceeds the target.
   if (n == 0) {
     if (tid == 0) next_token[b] = -1;       // no row to draw from
     return;
@@ -208,101 +287,81 @@ sample_walk_kernel(const tv_bf16* __restrict__ logits, const RowStat* __restrict
   const int c = sLast, nrej = sNrej;
   const float M = sM[c], target = sTarget;
   const uint16_t* row = lg + (size_t)c * V;
-  const bool vec_ok = ((V & 7) == 0) && ((reinterpret_cast<uintptr_t>(logits) & 15u) == 0);
-  constexpr int kPerThread = 64;
-  float carried = 0.f;                 // cumulative mass of everything before this step
-  int last_with_mass = -1;             // fallback when rounding leaves the target above the scanned total
-  for (int base = 0; base < V; base += kWalkThreads * kPerThread) {
-    const int v0 = base + tid * kPerThread;
-    float vals[kPerThread];
-    if (vec_ok && v0 + kPerThread <= V) {
-#pragma unroll
-      for (int q = 0; q < kPerThread / 8; ++q) {
-        const uint4 u = __ldg(reinterpret_cast<const uint4*>(row + v0) + q);
-        const uint32_t e[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int t = 0; t < 8; ++t) vals[q * 8 + t] = bf16_to_float((t & 1) ? (e[t >> 1] >> 16) : (e[t >> 1] & 0xffffu));
-      }
-    } else {
-#pragma unroll
-      for (int t = 0; t < kPerThread; ++t) vals[t] = (v0 + t < V) ? bf16_to_float(row[v0 + t]) : -INFINITY;
+  const int off = tv::LogitsRow(logits, (long long)b * Nmax + c, V).off;       // chunk q holds entries q * kStatChunk - off ...
+  // first the chunk: cumulative masses of the chunks, rejected tokens subtracted
+  float carried = 0.f;
+  for (int q0 = 0; q0 < n_chunks; q0 += kWalkThreads) {
+    const int q = q0 + tid;
+    float mass = 0.f;
+    if (q < n_chunks) {
+      const RowStat r = stats[((size_t)b * Nmax + c) * n_chunks + q];
+      if (r.m > -INFINITY) mass = r.s * ex2_approx(fmaxf((r.m - M) * k, -150.f));
+      for (int x = 0; x < nrej; ++x)
+        if ((sRej[x] + off) / kStatChunk == q) mass -= sRejE[x];
+      mass = fmaxf(mass, 0.f);
     }
-    float sum = 0.f;
+    float total;
+    const float incl = carried + block_scan(mass, sWarp, total);
+    if (mass > 0.f) {
+      if (target < incl) atomicMin(reinterpret_cast<unsigned*>(&sChunk), (unsigned)q);      // -1 is the largest unsigned
+      atomicMax(&sLastMass, q);
+    }
+    carried += total;
+    __syncthreads();
+    if (sChunk >= 0) {                                 // uniform: read after the barrier
+      if (q == sChunk) sExcl = incl - mass;
+      break;
+    }
+  }
+  // rounding can leave the target above the scanned total (u_bonus close to 1): the last chunk with mass then, and the
+  // last of its entries that has mass
+  const int chunk = sChunk >= 0 ? sChunk : max(sLastMass, 0);
+  auto entry_mass = [&](int v) -> float {
+    if (v < 0 || v >= V) return 0.f;
+    for (int x = 0; x < nrej; ++x)
+      if (sRej[x] == v) return 0.f;
+    return mass_of(bf16_to_float(row[v]), M, k);
+  };
+  __syncthreads();
+  const float excl = sChunk >= 0 ? sExcl : INFINITY;
+  if (tid == 0) sLastMass = -1;
+  __syncthreads();
+  {
+    constexpr int kPer = kStatChunk / kWalkThreads;       // entries per thread, in vocabulary order
+    const int v0 = chunk * kStatChunk - off + tid * kPer;
+    float vals[kPer], sum = 0.f;
 #pragma unroll
-    for (int t = 0; t < kPerThread; ++t) {
-      vals[t] = mass_of(vals[t], M, k);
+    for (int t = 0; t < kPer; ++t) {
+      vals[t] = entry_mass(v0 + t);
       sum += vals[t];
     }
-    for (int r = 0; r < nrej; ++r) {               // rejected tokens that fall into this thread's 64 entries
-      const int off = sRej[r] - v0;
-      if (off >= 0 && off < kPerThread) {
-        float m_r = 0.f;
+    float total;
+    float cum = excl + (block_scan(sum, sWarp, total) - sum);
+    int first = -1, last = -1;
 #pragma unroll
-        for (int t = 0; t < kPerThread; ++t) m_r = (t == off) ? vals[t] : m_r;
-        sum -= m_r;
-#pragma unroll
-        for (int t = 0; t < kPerThread; ++t) vals[t] = (t == off) ? 0.f : vals[t];
+    for (int t = 0; t < kPer; ++t) {
+      cum += vals[t];
+      if (vals[t] > 0.f) {
+        last = v0 + t;
+        if (first < 0 && cum > target) first = v0 + t;
       }
     }
-    sum = fmaxf(sum, 0.f);
-    // block-wide inclusive scan of the thread sums, in thread (= vocabulary) order
-    float incl = sum;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const float o = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += o;
-    }
-    if (lane == 31) sWarp[warp] = incl;
-    __syncthreads();
-    float before = carried;
-    for (int w = 0; w < warp; ++w) before += sWarp[w];
-    float step_total = 0.f;
-    for (int w = 0; w < kWalkThreads / 32; ++w) step_total += sWarp[w];
-    const float excl = before + incl - sum;          // cumulative mass before this thread's entries
-    if (excl <= target && target < excl + sum) {     // the crossing lies in this thread's entries
-      float cum = excl;
-      int hit = -1;
-#pragma unroll
-      for (int t = 0; t < kPerThread; ++t) {
-        cum += vals[t];
-        if (hit < 0 && cum > target) hit = v0 + t;
-      }
-      if (hit < 0) {                                 // rounding inside the 64 entries: the last one with mass
-#pragma unroll
-        for (int t = 0; t < kPerThread; ++t)
-          if (vals[t] > 0.f) hit = v0 + t;
-      }
-      if (hit >= 0) sHit = hit;
-    }
-    {
-      int lw = -1;
-#pragma unroll
-      for (int t = 0; t < kPerThread; ++t)
-        if (vals[t] > 0.f) lw = v0 + t;
-      last_with_mass = max(last_with_mass, lw);
-    }
-    carried += step_total;
-    __syncthreads();
-    if (sHit >= 0) break;                            // uniform: read after the barrier
+    if (excl == INFINITY) first = -1;
+    if (first >= 0) atomicMin(reinterpret_cast<unsigned*>(&sHit), (unsigned)first);
+    if (last >= 0) atomicMax(&sLastMass, last);
   }
-  if (sHit < 0) {
-    // the target was not below the scanned total (u_bonus close to 1 and rounding): the last entry with mass
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) last_with_mass = max(last_with_mass, __shfl_xor_sync(0xffffffffu, last_with_mass, off));
-    __shared__ int sLastMass[kWalkThreads / 32];
-    if (lane == 0) sLastMass[warp] = last_with_mass;
+  __syncthreads();
+  if (sHit < 0 && sLastMass < 0) {      // the chunk's mass was a rounding residue of a rejected token: last entry of the row
     __syncthreads();
-    if (tid == 0) {
-      int lm = -1;
-      for (int w = 0; w < kWalkThreads / 32; ++w) lm = max(lm, sLastMass[w]);
-      sHit = lm >= 0 ? lm : V - 1;
-    }
+    for (int v = tid; v < V; v += kWalkThreads)
+      if (entry_mass(v) > 0.f) atomicMax(&sLastMass, v);
     __syncthreads();
   }
-  if (tid == 0) next_token[b] = sHit;
+  if (tid == 0) next_token[b] = sHit >= 0 ? sHit : (sLastMass >= 0 ? sLastMass : V - 1);
 }
 
-int stat_chunks(int V) { return (V + kStatChunk - 1) / kStatChunk; }
+// A row may start anywhere inside a 16-byte vector, so up to seven entries of it fall into one more vector.
+int stat_chunks(int V) { return (int)(((long long)V + 7 + kStatChunk - 1) / kStatChunk); }
 
 }  // namespace
 
@@ -332,11 +391,16 @@ extern "C" int tree_accept_sample(const tv_bf16* logits, const int32_t* tokens, 
   const float k = kLog2e / temperature;
   RowStat* stats = static_cast<RowStat*>(workspace);
   cudaStream_t s = (cudaStream_t)stream;
-  row_stats_kernel<<<dim3(n_chunks, B * Nmax), kStatThreads, 0, s>>>(logits, n_nodes, Nmax, V, n_chunks, k, stats);
-  TV_CUDA_OK(cudaGetLastError());
-  sample_walk_kernel<<<B, kWalkThreads, 0, s>>>(logits, stats, n_chunks, tokens, parent, n_nodes, u_node, u_bonus, k,
-                                                Nmax, V, Dp1, accept_len, accepted_nodes, next_token, status);
-  TV_CUDA_OK(cudaGetLastError());
+  const long long n_items = (long long)B * Nmax * n_chunks;
+  TV_REQUIRE(n_items < (1ll << 31) - (1 << 20), "tree_accept_sample: B * Nmax * ceil(V / 2048) must stay below 2^31");
+  constexpr int kWarps = kStatThreads / 32;
+  const int resident = 3 * tv::sm_count();
+  const long long want = (n_items + kWarps - 1) / kWarps;
+  const int grid = (int)(want < resident ? want : resident);
+  TV_CUDA_OK(tv::launch_pdl(row_stats_kernel, dim3(grid), dim3(kStatThreads), 0, s, logits, n_nodes, Nmax, V, n_chunks,
+                            (int)n_items, k, stats));
+  TV_CUDA_OK(tv::launch_pdl(sample_walk_kernel, dim3(B), dim3(kWalkThreads), 0, s, logits, stats, n_chunks, tokens, parent,
+                            n_nodes, u_node, u_bonus, k, Nmax, V, Dp1, accept_len, accepted_nodes, next_token, status));
   tv::count_launches(2);
   return TV_OK;
 }

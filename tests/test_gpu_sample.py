@@ -171,3 +171,10 @@ def test_sample_accept_flags_and_edges():
     assert (g1["accept_len"] == 0).all()
     with pytest.raises(tv.TreeVerifyError):
         run_gpu(lt, tokens, parent, n, u_node, u_bonus, 0.0, 4)
+
+
+@pytest.mark.parametrize("V", [43, 2041, 2047, 2049, 4096, 6145, 10003])
+def test_vocabularies_around_the_chunk_and_vector_edges(V):
+    """Rows whose start lies anywhere inside a 16-byte vector, chunks of 2048 entries with every kind of remainder."""
+    lt, tokens, parent, n, u_node, u_bonus = make_inputs(70 + V, 6, 17, 5, V, ragged=True)
+    check(lt, tokens, parent, n, u_node, u_bonus, 1.0, 6, min_fraction=0.5)
