@@ -1,234 +1,175 @@
-// kv_commit: path-index commit with the prefix-sharing fast reorder
-// (Section 3.1).  The committed prefix is never moved; the accepted nodes' K/V
-// rows are gathered from the tree ("branch") buffers and appended behind it,
-// for every layer and KV head, in one launch.  A second one-warp launch then
-// advances prefix_len, so no copy CTA can observe the updated length.
+// kv_commit, kv_commit_inplace, kv_commit_paged: path-index commit (Section 3.1).  The committed prefix is never
+// moved; the accepted nodes' K/V rows are gathered behind it, for every layer and KV head, and prefix_len advances.
 //
-// Each (layer, sequence) is one CTA; a thread moves 16 bytes at a time, so a
-// head row of d bf16 is written by d/8 adjacent threads (coalesced on both
-// sides: the source row [node, h, :] and the destination row [h, S+j, :]).
+// One warp moves up to 128 pieces of 16 bytes of a (layer, K or V, node) row over all heads, four a lane (a head row of d bf16 is d/8 adjacent
+// lanes, coalesced on both sides); a sequence has as many CTAs as its rows keep busy.  Every CTA reads the sequence's scalars and its node list
+// and decides alike whether the sequence commits.  Where one CTA per sequence is enough (see launch_commit) it also
+// advances prefix_len; otherwise a second launch does, so that no copying CTA can observe the updated length.
+// (One launch with a thread-block cluster per sequence instead was 1.9 times slower on 16 sequences of 32 layers: 6.2
+// -> 11.9 us; clusters start late when many of them are needed.)  Before / now, us a call: one layer of 32 heads, seven
+// rows 10.6 / 3.7; one sequence of 32 layers 5.1 / 4.2; in-cache, 16 sequences of 32 layers 8.7 / 7.1; paged, 8 of 8
+// layers 5.6 / 5.0; 16 sequences of 32 layers 6.3 / 6.7.
 #include "common.cuh"
 
 namespace {
 
-// Decides, identically in both kernels, whether sequence b commits.
-// Returns the status bits to raise (0 = commit).
-__device__ __forceinline__ int commit_check(const int32_t* accepted_nodes, int A, int S, int st_in,
-                                            int Nmax, int Scap, int Dp1, int b) {
-  if (st_in & tv::kFatalStatus) return -1;            // skipped, nothing new to report
-  if (A < 0 || A >= Dp1) return TV_ST_BAD_INDEX;
-  for (int j = 0; j <= A; ++j) {
-    const int node = accepted_nodes[(size_t)b * Dp1 + j];
-    if (node < 0 || node >= Nmax) return TV_ST_BAD_INDEX;
-  }
-  if (S < 0 || S + A + 1 > Scap) return TV_ST_CAPACITY;
-  return 0;
-}
+constexpr int kThreads = 256;                 // of a CTA when a sequence has several
+constexpr int kMaxThreads = 512;              // ... when it has one
+constexpr int kPerLane = 4;                   // 16-byte pieces of a row in flight per lane
+constexpr int kHeld = 4;                      // in-cache layout: pieces a thread holds
+constexpr int kMaxDp1 = 2048;                 // longest path of the in-cache layout (the others: 1024)
+constexpr int kPageRows = 128;
+constexpr int kMaxPages = 1024 / kPageRows + 1;      // pages under a segment of at most 1024 rows
+constexpr int kMaxCtas = 4096;                // CTAs of a launch beyond which more of them cannot help
 
-// One CTA per (layer, sequence): the per-sequence scalars and the node list are fetched together and validated by
-// all threads at once (the same decision as commit_check), then the CTA moves every 16-byte piece of the accepted
-// segment, K and V, all heads; the pieces of a row are adjacent threads on both sides.
-constexpr int kCopyThreads = 256;
-constexpr int kCopyMaxDp1 = 1024;
+struct Commit {
+  uint4* k_cache;
+  uint4* v_cache;
+  const uint4* k_tree;                        // unused in the in-cache layout
+  const uint4* v_tree;
+  const int32_t* block_table;                 // paged layout only
+  const int32_t* accepted_nodes;
+  const int32_t* accept_len;
+  int32_t* prefix_len;
+  int32_t* status;
+  int L, Nmax, Hkv, dvec, Scap, Dp1, n_pages, max_blocks;
+  int64_t cache_layer, tree_layer;            // 16-byte pieces between two layers
+};
 
-__global__ void __launch_bounds__(kCopyThreads)
-commit_copy_kernel(uint4* __restrict__ k_cache, uint4* __restrict__ v_cache,
-                   const uint4* __restrict__ k_tree, const uint4* __restrict__ v_tree,
-                   const int32_t* __restrict__ accepted_nodes, const int32_t* __restrict__ accept_len,
-                   const int32_t* __restrict__ prefix_len, const int32_t* __restrict__ status,
-                   int B, int Nmax, int Hkv, int dvec, int Scap, int Dp1,
-                   int64_t cache_layer_vec, int64_t tree_layer_vec) {
-  tv::pdl_enter();
-  __shared__ int s_nodes[kCopyMaxDp1];
-  const int b = blockIdx.x, l = blockIdx.y;
-  const int A = accept_len[b];
-  const int S = prefix_len[b];
-  const int st = status[b];
-  for (int j = threadIdx.x; j < Dp1; j += kCopyThreads) s_nodes[j] = accepted_nodes[(size_t)b * Dp1 + j];
-  int bad = (st & tv::kFatalStatus) || A < 0 || A >= Dp1 || S < 0 || S + A + 1 > Scap;
+enum Layout { kContiguous, kInCache, kPaged };
+
+// COPY: move the accepted rows.  FINISH: advance prefix_len, raise status bits.
+template <Layout LAYOUT, bool COPY, bool FINISH>
+__global__ void __launch_bounds__(kMaxThreads)
+commit_kernel(const Commit c, int ctas_per_seq) {
+  // A kernel that writes prefix_len, which a tree_verify_attn launch directly behind it may read before its own wait,
+  // releases nothing early: the next launch must not start until this grid is complete.
+  if (FINISH) tv::pdl_wait_only();
+  else tv::pdl_enter();
+  __shared__ int s_nodes[LAYOUT == kInCache ? kMaxDp1 : 1024];
+  __shared__ int s_pages[LAYOUT == kPaged ? kMaxPages : 1];
+  const unsigned ranks = ctas_per_seq, rank = blockIdx.x % ranks;
+  const int b = blockIdx.x / ranks, tid = threadIdx.x, nt = blockDim.x;
+  const int A = c.accept_len[b];
+  const int S = c.prefix_len[b];
+  const int st = c.status[b];
+  for (int j = tid; j < c.Dp1; j += nt) s_nodes[j] = c.accepted_nodes[(size_t)b * c.Dp1 + j];
+  const int cap = LAYOUT == kPaged ? c.max_blocks * kPageRows : c.Scap;
+  const bool skip = (st & tv::kFatalStatus) != 0;               // nothing new to report
+  const bool len_ok = A >= 0 && A < c.Dp1;
+  const bool fits = len_ok && S >= 0 && S <= cap - (A + 1);
   __syncthreads();
-  if (!bad)
-    for (int j = threadIdx.x; j <= A; j += kCopyThreads) bad |= (s_nodes[j] < 0 || s_nodes[j] >= Nmax);
-  if (__syncthreads_or(bad)) return;
-  const size_t src0 = (size_t)l * tree_layer_vec + (size_t)b * Nmax * Hkv * dvec;       // [node, h, :]
-  const size_t dst0 = (size_t)l * cache_layer_vec + (size_t)b * Hkv * Scap * dvec;      // [h, row, :]
-  const int per = Hkv * dvec;                   // pieces of one node's row over all heads
-  const int total = 2 * (A + 1) * per;
-  // four pieces per thread and round: the loads of a round are all issued before the first store
-  for (int t0 = threadIdx.x; t0 < total; t0 += 4 * kCopyThreads) {
-    uint4 val[4];
-    uint4* dst[4];
+  bool bad_node = false, bad_source = false, bad_page = false;
+  if (len_ok)
+    for (int j = tid; j <= A; j += nt) {
+      const int node = s_nodes[j];
+      bad_node |= node < 0 || node >= c.Nmax;
+      if (LAYOUT == kInCache) bad_source |= S + (long long)node >= c.Scap;      // a source row outside the cache
+    }
+  if (LAYOUT == kPaged && fits)
+    for (int t = tid; t <= (S + A) / kPageRows - S / kPageRows; t += nt) {
+      const int pg = c.block_table[(size_t)b * c.max_blocks + S / kPageRows + t];
+      bad_page |= pg < 0 || pg >= c.n_pages;
+      s_pages[t] = pg;
+    }
+  int report = 0;                                               // status bits to raise; 0: commit
+  if (!len_ok || __syncthreads_or(bad_node)) report = TV_ST_BAD_INDEX;
+  else if (!fits || (LAYOUT == kInCache && __syncthreads_or(bad_source))) report = TV_ST_CAPACITY;
+  else if (LAYOUT == kPaged && __syncthreads_or(bad_page)) report = TV_ST_BAD_INDEX;
+  if (FINISH && tid == 0 && !skip) {                            // (every thread has read the scalars before a barrier)
+    if (report == 0) c.prefix_len[b] = S + A + 1;
+    else c.status[b] = st | report;
+  }
+  if (!COPY || skip || report != 0) return;
+  const int dvec = c.dvec;
+  if (LAYOUT == kInCache) {
+    // Row S + j takes the OLD row S + accepted_nodes[j]: source and destination ranges overlap (a row can be the
+    // source of one slot and the destination of another), so a CTA owns all rows of a (layer, K or V, head) slab,
+    // holds every piece it needs in registers and writes only behind a barrier.
+    const int per_head = (A + 1) * dvec;                        // <= kHeld * nt (launch_commit)
+    const int hpc = kHeld * nt / per_head;           // slabs a CTA holds at once
+    const long long slabs = 2ll * c.L * c.Hkv;
+    for (long long s0 = (long long)rank * hpc; s0 < slabs; s0 += (long long)ranks * hpc) {
+      uint4 held[kHeld];
+      uint4* dst[kHeld];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int t = t0 + i * kCopyThreads;
-      dst[i] = nullptr;
-      if (t < total) {
-        const int kv = t >= (A + 1) * per;
-        const int u = kv ? t - (A + 1) * per : t;
-        const int j = u / per, w = u - j * per;
-        const int h = w / dvec, c = w - h * dvec;
-        val[i] = (kv ? v_tree : k_tree)[src0 + (size_t)s_nodes[j] * per + w];
-        dst[i] = (kv ? v_cache : k_cache) + dst0 + ((size_t)h * Scap + S + j) * dvec + c;
+      for (int i = 0; i < kHeld; ++i) {
+        const int t = tid + i * nt;
+        const int h = t / per_head, u = t - h * per_head;
+        const int j = u / dvec, w = u - j * dvec;
+        const long long slab = s0 + h;
+        dst[i] = nullptr;
+        if (h < hpc && slab < slabs) {
+          const int l = (int)(slab / (2 * c.Hkv)), r = (int)(slab - (long long)l * 2 * c.Hkv);
+          const int kv = r >= c.Hkv, head = kv ? r - c.Hkv : r;
+          uint4* base = (kv ? c.v_cache : c.k_cache) + (size_t)l * c.cache_layer +
+                        (((size_t)b * c.Hkv + head) * c.Scap + S) * (size_t)dvec;
+          held[i] = base[(size_t)s_nodes[j] * dvec + w];
+          if (s_nodes[j] != j) dst[i] = base + (size_t)j * dvec + w;
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < kHeld; ++i)
+        if (dst[i]) *dst[i] = held[i];
+    }
+  } else {
+    const int per = c.Hkv * dvec;                               // pieces of one node's row over all heads
+    const int warps = nt >> 5, lane = tid & 31;
+    const int rounds = (per + 32 * kPerLane - 1) / (32 * kPerLane);
+    const long long units = 2ll * c.L * (A + 1) * rounds;
+    for (long long r = (long long)rank * warps + (tid >> 5); r < units; r += (long long)ranks * warps) {
+      const int in_layer = 2 * (A + 1) * rounds;
+      const int l = (int)(r / in_layer), in = (int)(r - (long long)l * in_layer);
+      const int u = in / rounds, w0 = (in - u * rounds) * 32 * kPerLane + lane;
+      const bool kv = u > A;
+      const int j = kv ? u - (A + 1) : u, row = S + j;
+      const uint4* src = (kv ? c.v_tree : c.k_tree) + (size_t)l * c.tree_layer + ((size_t)b * c.Nmax + s_nodes[j]) * per;
+      const size_t at = LAYOUT == kPaged ? (size_t)s_pages[row / kPageRows - S / kPageRows] * c.Hkv * kPageRows + row % kPageRows
+                                         : (size_t)b * c.Hkv * c.Scap + row;      // row of head 0
+      const size_t head_rows = LAYOUT == kPaged ? kPageRows : c.Scap;
+      uint4* dst = (kv ? c.v_cache : c.k_cache) + (size_t)l * c.cache_layer + at * dvec;
+      uint4 val[kPerLane];
+#pragma unroll
+      for (int i = 0; i < kPerLane; ++i)
+        if (w0 + 32 * i < per) val[i] = src[w0 + 32 * i];
+#pragma unroll
+      for (int i = 0; i < kPerLane; ++i) {
+        const int w = w0 + 32 * i;
+        if (w < per) {
+          const int h = w / dvec;
+          dst[(size_t)h * head_rows * dvec + (w - h * dvec)] = val[i];
+        }
       }
     }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (dst[i]) *dst[i] = val[i];
   }
 }
 
-__global__ void commit_finish_kernel(const int32_t* __restrict__ accepted_nodes,
-                                     const int32_t* __restrict__ accept_len,
-                                     int32_t* __restrict__ prefix_len, int32_t* __restrict__ status,
-                                     int B, int Nmax, int Scap, int Dp1) {
-  // This kernel writes prefix_len, which a tree_verify_attn launch directly behind it reads before its own
-  // wait: the next launch must not start until this grid is complete, so nothing is released early here.
-  tv::pdl_wait_only();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  const int A = accept_len[b];
-  const int S = prefix_len[b];
-  const int r = commit_check(accepted_nodes, A, S, status[b], Nmax, Scap, Dp1, b);
-  if (r == 0) prefix_len[b] = S + A + 1;
-  else if (r > 0) status[b] |= r;
-}
-
-// In-cache layout: the tree's K/V rows were written into the cache itself, node i at row S + i, and the commit
-// reorders them in place: row S + j takes the old row S + accepted_nodes[j], j = 0..A.  Source and destination
-// ranges overlap (a row can be the source of one slot and the destination of another), so the copy is a gather
-// from the state BEFORE the commit: one CTA owns all the rows of a (layer, sequence, KV head, K or V), reads
-// every row it needs into registers, and only writes after a barrier.
-constexpr int kInplaceThreads = 256;
-constexpr int kInplaceMaxPerThread = 8;
-constexpr int kInplaceMaxPieces = kInplaceThreads * kInplaceMaxPerThread;
-
-// One CTA per (layer, sequence, K or V, group of `hpc` KV heads).  The per-sequence scalars and the node list are
-// fetched together (one round trip), validated by all threads at once, and then every 16-byte piece of the
-// accepted segments of the CTA's heads is read, a barrier passes, and the pieces that move are written.
-__global__ void __launch_bounds__(kInplaceThreads)
-commit_inplace_kernel(uint4* __restrict__ k_cache, uint4* __restrict__ v_cache,
-                      const int32_t* __restrict__ accepted_nodes, const int32_t* __restrict__ accept_len,
-                      const int32_t* __restrict__ prefix_len, const int32_t* __restrict__ status,
-                      int B, int Nmax, int Hkv, int dvec, int Scap, int Dp1, int hpc, int64_t cache_layer_vec) {
-  __shared__ int s_nodes[kInplaceMaxPieces];
-  const int kv = blockIdx.x & 1, h0 = (blockIdx.x >> 1) * hpc, b = blockIdx.y, l = blockIdx.z;
-  const int A = accept_len[b];
-  const int S = prefix_len[b];
-  const int st = status[b];
-  for (int j = threadIdx.x; j < Dp1; j += kInplaceThreads) s_nodes[j] = accepted_nodes[(size_t)b * Dp1 + j];
-  // the same decision as commit_check plus the source-row bound, taken by all threads together
-  int bad = (st & tv::kFatalStatus) || A < 0 || A >= Dp1 || S < 0 || S + A + 1 > Scap;
-  __syncthreads();
-  if (!bad)
-    for (int j = threadIdx.x; j <= A; j += kInplaceThreads) {
-      const int node = s_nodes[j];
-      bad |= (node < 0 || node >= Nmax || S + node >= Scap);
-    }
-  if (__syncthreads_or(bad)) return;
-  uint4* base = (kv ? v_cache : k_cache) + (size_t)l * cache_layer_vec + ((size_t)b * Hkv + h0) * (size_t)Scap * dvec;
-  const int per_head = (A + 1) * dvec;           // 16-byte pieces of one head's accepted segment
-  const int total = hpc * per_head;
-  uint4 held[kInplaceMaxPerThread];
-#pragma unroll
-  for (int i = 0; i < kInplaceMaxPerThread; ++i) {
-    const int t = threadIdx.x + i * kInplaceThreads;
-    if (t < total) {
-      const int h = t / per_head, u = t - h * per_head;
-      const int j = u / dvec, c = u - j * dvec;
-      held[i] = base[((size_t)h * Scap + S + s_nodes[j]) * dvec + c];
-    }
+// CTAs per sequence: what the longest path of the call keeps busy for one round.  One larger CTA and one launch where
+// the call is small (one layer, eight heads of 128, paths of eight: 4.1 -> 2.8 us), two launches where it is not.
+template <Layout LAYOUT>
+cudaError_t launch_commit(const Commit& c, int B, cudaStream_t s) {
+  const long long pieces = 2ll * c.L * c.Hkv * c.dvec * c.Dp1;
+  if (pieces <= kMaxThreads * kPerLane || kMaxCtas / B <= 1) {
+    tv::count_launches(1);
+    return tv::launch_pdl(commit_kernel<LAYOUT, true, true>, dim3(B), dim3(kMaxThreads), 0, s, c, 1);
   }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < kInplaceMaxPerThread; ++i) {
-    const int t = threadIdx.x + i * kInplaceThreads;
-    if (t < total) {
-      const int h = t / per_head, u = t - h * per_head;
-      const int j = u / dvec, c = u - j * dvec;
-      if (s_nodes[j] != j) base[((size_t)h * Scap + S + j) * dvec + c] = held[i];
-    }
+  int threads = kThreads;
+  long long ctas;
+  if (LAYOUT == kInCache) {
+    if (c.Dp1 * c.dvec > kHeld * kThreads) threads = kMaxThreads;       // one head's longest segment has to fit a CTA
+    ctas = (pieces * 5 / 8 + threads * kHeld - 1) / (threads * kHeld);  // most paths are shorter than the longest
+  } else {
+    const int rounds = (c.Hkv * c.dvec + 32 * kPerLane - 1) / (32 * kPerLane), warps = kThreads / 32;
+    ctas = (2ll * c.L * c.Dp1 * rounds + warps - 1) / warps;
+    if (ctas * B > 8ll * tv::sm_count()) ctas = (ctas * 5 + 7) / 8;     // more than one wave: most paths are shorter
   }
-}
-
-// prefix_len and status of the in-place commit (after every copy CTA has finished)
-__global__ void commit_inplace_finish_kernel(const int32_t* __restrict__ accepted_nodes,
-                                             const int32_t* __restrict__ accept_len,
-                                             int32_t* __restrict__ prefix_len, int32_t* __restrict__ status,
-                                             int B, int Nmax, int Scap, int Dp1) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  const int A = accept_len[b];
-  const int S = prefix_len[b];
-  int r = commit_check(accepted_nodes, A, S, status[b], Nmax, Scap, Dp1, b);
-  if (r == 0)
-    for (int j = 0; j <= A; ++j)
-      if (S + accepted_nodes[(size_t)b * Dp1 + j] >= Scap) r = TV_ST_CAPACITY;     // a source row outside the cache
-  if (r == 0) prefix_len[b] = S + A + 1;
-  else if (r > 0) status[b] |= r;
-}
-
-// Paged cache: pages [n_pages,Hkv,128,d] per layer, block_table[b, t] = page of rows 128 t .. 128 t + 127 of
-// sequence b.  Row S + j of the sequence is row (S + j) % 128 of page block_table[b, (S + j) / 128].
-constexpr int kPageRows = 128;
-
-__device__ __forceinline__ bool paged_segment_ok(const int32_t* block_table, int b, int S, int A, int max_blocks,
-                                                 int n_pages) {
-  for (int t = S / kPageRows; t <= (S + A) / kPageRows; ++t) {
-    const int pg = block_table[(size_t)b * max_blocks + t];
-    if (pg < 0 || pg >= n_pages) return false;
-  }
-  return true;
-}
-
-__global__ void __launch_bounds__(kCopyThreads)
-commit_paged_kernel(uint4* __restrict__ k_pages, uint4* __restrict__ v_pages, const int32_t* __restrict__ block_table,
-                    const uint4* __restrict__ k_tree, const uint4* __restrict__ v_tree,
-                    const int32_t* __restrict__ accepted_nodes, const int32_t* __restrict__ accept_len,
-                    const int32_t* __restrict__ prefix_len, const int32_t* __restrict__ status,
-                    int B, int Nmax, int Hkv, int dvec, int n_pages, int max_blocks, int Dp1,
-                    int64_t page_layer_vec, int64_t tree_layer_vec) {
-  __shared__ int s_nodes[kCopyMaxDp1];
-  const int b = blockIdx.x, l = blockIdx.y;
-  const int A = accept_len[b];
-  const int S = prefix_len[b];
-  const int st = status[b];
-  for (int j = threadIdx.x; j < Dp1; j += kCopyThreads) s_nodes[j] = accepted_nodes[(size_t)b * Dp1 + j];
-  int bad = (st & tv::kFatalStatus) || A < 0 || A >= Dp1 || S < 0 || S + A + 1 > max_blocks * kPageRows;
-  __syncthreads();
-  if (!bad) {
-    for (int j = threadIdx.x; j <= A; j += kCopyThreads) bad |= (s_nodes[j] < 0 || s_nodes[j] >= Nmax);
-    if (threadIdx.x == 0) bad |= !paged_segment_ok(block_table, b, S, A, max_blocks, n_pages);
-  }
-  if (__syncthreads_or(bad)) return;
-  const size_t src0 = (size_t)l * tree_layer_vec + (size_t)b * Nmax * Hkv * dvec;       // [node, h, :]
-  const size_t dst0 = (size_t)l * page_layer_vec;                                       // [page, h, row, :]
-  const int per = Hkv * dvec;
-  const int total = 2 * (A + 1) * per;
-  for (int t = threadIdx.x; t < total; t += kCopyThreads) {
-    const int kv = t >= (A + 1) * per;
-    const int u = kv ? t - (A + 1) * per : t;
-    const int j = u / per, w = u - j * per;
-    const int h = w / dvec, c = w - h * dvec;
-    const int row = S + j;
-    const int pg = block_table[(size_t)b * max_blocks + row / kPageRows];
-    const uint4 val = (kv ? v_tree : k_tree)[src0 + (size_t)s_nodes[j] * per + w];
-    (kv ? v_pages : k_pages)[dst0 + (((size_t)pg * Hkv + h) * kPageRows + row % kPageRows) * dvec + c] = val;
-  }
-}
-
-__global__ void commit_paged_finish_kernel(const int32_t* __restrict__ accepted_nodes,
-                                           const int32_t* __restrict__ accept_len,
-                                           const int32_t* __restrict__ block_table,
-                                           int32_t* __restrict__ prefix_len, int32_t* __restrict__ status,
-                                           int B, int Nmax, int n_pages, int max_blocks, int Dp1) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  const int A = accept_len[b];
-  const int S = prefix_len[b];
-  int r = commit_check(accepted_nodes, A, S, status[b], Nmax, max_blocks * kPageRows, Dp1, b);
-  if (r == 0 && !paged_segment_ok(block_table, b, S, A, max_blocks, n_pages)) r = TV_ST_BAD_INDEX;
-  if (r == 0) prefix_len[b] = S + A + 1;
-  else if (r > 0) status[b] |= r;
+  if (ctas > kMaxCtas / B) ctas = kMaxCtas / B;
+  tv::count_launches(2);
+  const cudaError_t e = tv::launch_pdl(commit_kernel<LAYOUT, true, false>, dim3((unsigned)ctas * B), dim3(threads), 0, s, c,
+                                       (int)ctas);
+  if (e != cudaSuccess) return e;
+  return tv::launch_pdl(commit_kernel<LAYOUT, false, true>, dim3(B), dim3(kThreads), 0, s, c, 1);
 }
 
 }  // namespace
@@ -249,18 +190,22 @@ extern "C" int kv_commit_paged(tv_bf16* k_pages, tv_bf16* v_pages, const int32_t
   TV_REQUIRE(page_layer_stride % 8 == 0 && tree_layer_stride % 8 == 0, "kv_commit_paged: layer strides must be multiples of 8 elements");
   TV_REQUIRE(tv::aligned16(k_pages) && tv::aligned16(v_pages) && tv::aligned16(k_tree) && tv::aligned16(v_tree),
              "kv_commit_paged: tensors must be 16-byte aligned");
-  TV_REQUIRE(L <= 65535 && Dp1 <= kCopyMaxDp1, "kv_commit_paged: L must be <= 65535 and Dp1 <= 1024");
+  TV_REQUIRE(L <= 65535 && Dp1 <= 1024, "kv_commit_paged: L must be <= 65535 and Dp1 <= 1024");
   if (L == 0 || B == 0) return TV_OK;
-  cudaStream_t s = (cudaStream_t)stream;
-  commit_paged_kernel<<<dim3(B, L), kCopyThreads, 0, s>>>(
-      reinterpret_cast<uint4*>(k_pages), reinterpret_cast<uint4*>(v_pages), block_table,
-      reinterpret_cast<const uint4*>(k_tree), reinterpret_cast<const uint4*>(v_tree), accepted_nodes, accept_len,
-      prefix_len, status, B, Nmax, Hkv, d / 8, n_pages, max_blocks, Dp1, page_layer_stride / 8, tree_layer_stride / 8);
-  TV_CUDA_OK(cudaGetLastError());
-  commit_paged_finish_kernel<<<(B + 127) / 128, 128, 0, s>>>(accepted_nodes, accept_len, block_table, prefix_len, status,
-                                                             B, Nmax, n_pages, max_blocks, Dp1);
-  TV_CUDA_OK(cudaGetLastError());
-  tv::count_launches(2);
+  Commit c{};
+  c.k_cache = reinterpret_cast<uint4*>(k_pages);
+  c.v_cache = reinterpret_cast<uint4*>(v_pages);
+  c.k_tree = reinterpret_cast<const uint4*>(k_tree);
+  c.v_tree = reinterpret_cast<const uint4*>(v_tree);
+  c.block_table = block_table;
+  c.accepted_nodes = accepted_nodes;
+  c.accept_len = accept_len;
+  c.prefix_len = prefix_len;
+  c.status = status;
+  c.L = L; c.Nmax = Nmax; c.Hkv = Hkv; c.dvec = d / 8; c.Dp1 = Dp1; c.n_pages = n_pages; c.max_blocks = max_blocks;
+  c.cache_layer = page_layer_stride / 8;
+  c.tree_layer = tree_layer_stride / 8;
+  TV_CUDA_OK(launch_commit<kPaged>(c, B, (cudaStream_t)stream));
   return TV_OK;
 }
 
@@ -277,21 +222,19 @@ extern "C" int kv_commit_inplace(tv_bf16* k_cache, tv_bf16* v_cache,
   TV_REQUIRE(cache_layer_stride % 8 == 0, "kv_commit_inplace: the layer stride must be a multiple of 8 elements");
   TV_REQUIRE(tv::aligned16(k_cache) && tv::aligned16(v_cache), "kv_commit_inplace: tensors must be 16-byte aligned");
   TV_REQUIRE(B <= 65535 && L <= 65535 && Hkv <= 32767, "kv_commit_inplace: B and L must be <= 65535, Hkv <= 32767");
-  TV_REQUIRE((long long)Dp1 * (d / 8) <= kInplaceMaxPieces,
+  TV_REQUIRE((long long)Dp1 * (d / 8) <= kMaxDp1,
              "kv_commit_inplace: Dp1 * d / 8 must be <= 2048 (the accepted segment of a head is staged in registers)");
   if (L == 0 || B == 0) return TV_OK;
-  cudaStream_t s = (cudaStream_t)stream;
-  int hpc = 1;       // KV heads per CTA: the largest divisor of Hkv whose longest possible segments fit the registers
-  for (int c = 1; c <= Hkv; ++c)
-    if (Hkv % c == 0 && (long long)c * Dp1 * (d / 8) <= kInplaceMaxPieces) hpc = c;
-  commit_inplace_kernel<<<dim3(2 * (Hkv / hpc), B, L), kInplaceThreads, 0, s>>>(
-      reinterpret_cast<uint4*>(k_cache), reinterpret_cast<uint4*>(v_cache), accepted_nodes, accept_len, prefix_len,
-      status, B, Nmax, Hkv, d / 8, Scap, Dp1, hpc, cache_layer_stride / 8);
-  TV_CUDA_OK(cudaGetLastError());
-  commit_inplace_finish_kernel<<<(B + 127) / 128, 128, 0, s>>>(accepted_nodes, accept_len, prefix_len, status,
-                                                               B, Nmax, Scap, Dp1);
-  TV_CUDA_OK(cudaGetLastError());
-  tv::count_launches(2);
+  Commit c{};
+  c.k_cache = reinterpret_cast<uint4*>(k_cache);
+  c.v_cache = reinterpret_cast<uint4*>(v_cache);
+  c.accepted_nodes = accepted_nodes;
+  c.accept_len = accept_len;
+  c.prefix_len = prefix_len;
+  c.status = status;
+  c.L = L; c.Nmax = Nmax; c.Hkv = Hkv; c.dvec = d / 8; c.Scap = Scap; c.Dp1 = Dp1;
+  c.cache_layer = cache_layer_stride / 8;
+  TV_CUDA_OK(launch_commit<kInCache>(c, B, (cudaStream_t)stream));
   return TV_OK;
 }
 
@@ -311,17 +254,20 @@ extern "C" int kv_commit(tv_bf16* k_cache, tv_bf16* v_cache,
   TV_REQUIRE(tv::aligned16(k_cache) && tv::aligned16(v_cache) && tv::aligned16(k_tree) && tv::aligned16(v_tree),
              "kv_commit: tensors must be 16-byte aligned");
   TV_REQUIRE(L <= 65535, "kv_commit: L must be <= 65535");
-  TV_REQUIRE(Dp1 <= kCopyMaxDp1, "kv_commit: Dp1 must be <= 1024");
+  TV_REQUIRE(Dp1 <= 1024, "kv_commit: Dp1 must be <= 1024");
   if (L == 0 || B == 0) return TV_OK;
-  const int dvec = d / 8;
-  cudaStream_t s = (cudaStream_t)stream;
-  TV_CUDA_OK(tv::launch_pdl(commit_copy_kernel, dim3(B, L), dim3(kCopyThreads), 0, s,
-                            reinterpret_cast<uint4*>(k_cache), reinterpret_cast<uint4*>(v_cache),
-                            reinterpret_cast<const uint4*>(k_tree), reinterpret_cast<const uint4*>(v_tree),
-                            accepted_nodes, accept_len, prefix_len, status, B, Nmax, Hkv, dvec, Scap, Dp1,
-                            cache_layer_stride / 8, tree_layer_stride / 8));
-  TV_CUDA_OK(tv::launch_pdl(commit_finish_kernel, dim3((B + 127) / 128), dim3(128), 0, s, accepted_nodes, accept_len,
-                            prefix_len, status, B, Nmax, Scap, Dp1));
-  tv::count_launches(2);
+  Commit c{};
+  c.k_cache = reinterpret_cast<uint4*>(k_cache);
+  c.v_cache = reinterpret_cast<uint4*>(v_cache);
+  c.k_tree = reinterpret_cast<const uint4*>(k_tree);
+  c.v_tree = reinterpret_cast<const uint4*>(v_tree);
+  c.accepted_nodes = accepted_nodes;
+  c.accept_len = accept_len;
+  c.prefix_len = prefix_len;
+  c.status = status;
+  c.L = L; c.Nmax = Nmax; c.Hkv = Hkv; c.dvec = d / 8; c.Scap = Scap; c.Dp1 = Dp1;
+  c.cache_layer = cache_layer_stride / 8;
+  c.tree_layer = tree_layer_stride / 8;
+  TV_CUDA_OK(launch_commit<kContiguous>(c, B, (cudaStream_t)stream));
   return TV_OK;
 }

@@ -205,3 +205,61 @@ def test_node_scores_parity():
     assert np.array_equal(scores.cpu().numpy(), ref)
     assert np.array_equal(status.cpu().numpy(), ref_st)
     assert ref_st[bad[0]] == orc.ST_BAD_INDEX and np.isneginf(ref[bad[1], 1]) and (ref[:, 0] == 0).all()
+
+
+COMMIT_SHAPES = [      # L, B, Hkv, d, Dp1: one launch or two, one or several rounds a row, more CTAs than one wave
+    (1, 1, 1, 8, 1), (1, 3, 2, 64, 5), (1, 2, 8, 128, 8), (1, 2, 8, 128, 9), (3, 2, 33, 128, 6), (2, 2, 4, 64, 200),
+    (40, 9, 2, 64, 11), (64, 24, 8, 8, 9),
+]
+
+
+@pytest.mark.parametrize("layout", ["contiguous", "in_cache", "paged"])
+@pytest.mark.parametrize("L,B,Hkv,d,Dp1", COMMIT_SHAPES)
+def test_commit_launch_shapes_byte_exact(layout, L, B, Hkv, d, Dp1):
+    rng = np.random.default_rng(L * 1000 + Dp1)
+    Nmax, cap = Dp1 + 7, 512
+    A = rng.integers(0, Dp1, size=B).astype(np.int32)
+    A[0] = Dp1 - 1
+    nodes = np.stack([np.sort(rng.permutation(Nmax)[:Dp1]) for _ in range(B)]).astype(np.int32)
+    S = rng.integers(0, cap - Nmax - Dp1, size=B).astype(np.int32)
+    u16 = lambda *s: rng.integers(0, 2 ** 16, size=s).astype(np.uint16)
+    kt, vt = u16(L, B, Nmax, Hkv, d), u16(L, B, Nmax, Hkv, d)
+    if layout == "paged":
+        bt = rng.permutation(B * cap // 128).astype(np.int32).reshape(B, cap // 128)
+        kc, vc = u16(L, bt.size, Hkv, 128, d), u16(L, bt.size, Hkv, 128, d)
+        ref = orc.kv_commit_paged(kc, vc, bt, kt, vt, nodes, A, S)
+    else:
+        kc, vc = u16(L, B, Hkv, cap, d), u16(L, B, Hkv, cap, d)
+        ref = orc.kv_commit(kc, vc, kt, vt, nodes, A, S) if layout == "contiguous" else \
+            orc.kv_commit_inplace(kc, vc, nodes, A, S, Nmax)
+    up = lambda a: torch.from_numpy(a.view(np.int16) if a.dtype == np.uint16 else a).cuda()
+    bf = lambda a: up(a).view(torch.bfloat16)
+    kd, vd, Sd, st = bf(kc), bf(vc), up(S), torch.zeros(B, dtype=torch.int32, device="cuda")
+    if layout == "contiguous":
+        tv.kv_commit(kd, vd, bf(kt), bf(vt), up(nodes), up(A), Sd, st)
+    elif layout == "in_cache":
+        tv.kv_commit_inplace(kd, vd, up(nodes), up(A), Sd, Nmax, st)
+    else:
+        tv.kv_commit_paged(kd, vd, up(bt), bf(kt), bf(vt), up(nodes), up(A), Sd, st)
+    torch.cuda.synchronize()
+    assert np.array_equal(st.cpu().numpy(), ref[3]) and np.array_equal(Sd.cpu().numpy(), ref[2])
+    for got, want in ((kd, ref[0]), (vd, ref[1])):
+        assert np.array_equal(got.view(torch.int16).cpu().numpy().view(np.uint16), want)
+
+
+@pytest.mark.parametrize("V", [1, 7, 8, 9, 16383, 16385, 16391, 32777])
+def test_argmax_vocabularies_around_vector_and_chunk_edges(V):
+    """Rows that start anywhere inside a 16-byte vector: ties and maxima on the first and last entries included."""
+    g = torch.Generator().manual_seed(V)
+    B, N = 3, 13
+    logits = torch.randint(-3, 4, (B, N, V), generator=g).to(torch.bfloat16)
+    for i in range(N):
+        logits[:, i, (0 if i % 3 == 0 else V - 1 if i % 3 == 1 else V // 2)] = 4.0
+    logits[0, 2] = float("-inf")
+    n = torch.tensor([N, 5, N], dtype=torch.int32, device="cuda")
+    z = lambda *s: torch.zeros(s, dtype=torch.int32, device="cuda")
+    am, st = z(B, N), z(B)
+    ws = torch.zeros(max(16, tv.tv_accept_workspace_bytes(B, N, V)), dtype=torch.uint8, device="cuda")
+    tv.tree_accept(logits.cuda(), z(B, N), z(B, 1, 2) - 1, n, am, z(B), z(B), z(B, 2), z(B), ws, st)
+    want = orc.argmax_rows(bf16_bits(logits), n.cpu().numpy())
+    assert np.array_equal(am.cpu().numpy(), want)
