@@ -33,8 +33,10 @@
 // is cut evenly over the CTA groups (a group = the CTAs that hold the row
 // tiles of the same unit and walk the same keys together, so the second reader
 // hits L2).  A unit cut in pieces leaves partials (normalised O in bf16, m, l) in the
-// workspace; the piece that draws the last ticket on the unit's counter merges them.
-// Counters carry a per-call epoch, so the workspace needs no initialisation.
+// workspace; the CTA that holds the unit's first piece merges them.  Groups run
+// downwards over the block index, so a merging CTA waits only for CTAs with a lower
+// block index, which were started before it.  Flags carry a per-call epoch, so the
+// workspace needs no initialisation.
 //
 // Every wait on an mbarrier is bounded: on expiry the CTA raises
 // TV_ST_TIMEOUT for all sequences, all roles leave their loops, outstanding
@@ -330,8 +332,8 @@ struct AttnParams {
   float* lse;
   int32_t* status;
   tv_bf16* part_o;               // [slots][D/8][MT*128][8] bf16 normalised outputs, column-group major
-  float* part_ml;                // [slots][2][MT*128]  (m in log2 units, then l)
-  unsigned long long* counters;  // [B*Hkv*NP][2]: tickets claimed, partials ready (epoch-tagged)
+  float* part_ml;                // [slots][2][MT*128]  (m in log2 units, then l); one slot per CTA
+  unsigned long long* counters;  // [L*B*Hkv*NP][2], epoch-tagged: the unit's second piece is ready, count of later ones
   unsigned long long epoch;      // 48-bit tag of this call
   int B, Nmax, Hq, Hkv, Scap, G, NPT, NP, W, groups;
   int TT;                        // key tiles of the tree's own K/V: ceil(Nmax / 128), 1 or 2
@@ -395,7 +397,7 @@ struct SmemLayout {
   // beside P0 P1 O0 O1), two buffers otherwise.
   static constexpr int kTmemS0 = 0, kTmemP0 = 128, kTmemO0 = 256;
   static constexpr int kTmemS1 = (D == 128 && MT == 2) ? kTmemS0 : 384;
-  static constexpr int kMisc = kBars + NBARS * 8;          // tmem ptr, abort flag, last flag
+  static constexpr int kMisc = kBars + NBARS * 8;          // tmem ptr, abort flag
   static constexpr int kCum = kMisc + 16;
   static constexpr int kGs = kCum + (kMaxB + 1) * 4;
   static constexpr int kTotal = kGs + (kMaxGroups + 1) * 4;
@@ -414,7 +416,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t bars = sbase + L::kBars;
   auto bar = [&](int i) { return bars + 8u * i; };
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMisc + 4);
-  volatile int* last_flag = reinterpret_cast<volatile int*>(smem + L::kMisc + 8);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + L::kMisc);
   int* cum = reinterpret_cast<int*>(smem + L::kCum);
   int* gs = reinterpret_cast<int*>(smem + L::kGs);
@@ -427,6 +428,30 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_vc) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_kt) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_vt) : "memory");
+  }
+  if (threadIdx.x == 32) {
+    mbar_init(bar(L::Q_FULL), 1);
+    mbar_init(bar(L::Q_EMPTY), 1);
+#pragma unroll 1
+    for (int s = 0; s < kSlots; ++s) {
+      mbar_init(bar(L::KV_FULL + s), 1);
+      mbar_init(bar(L::KV_EMPTY + s), 1);
+    }
+    for (int s = 0; s < 2; ++s) {                // index = row tile, or parity of the key tile with one row tile
+      mbar_init(bar(L::S_FULL + s), 1);
+      mbar_init(bar(L::S_FREE + s), 4);
+      mbar_init(bar(L::P_READY + s), 4);
+      mbar_init(bar(L::ITEM_DONE + s), 1);
+    }
+    mbar_init(bar(L::O_DONE), 1);
+    mbar_init(bar(L::EPI), MT * 128);
+    *abort_flag = ((sbase & 1023u) != 0) ? 1 : 0;   // swizzled tiles need a 1024-byte aligned base
+    fence_barrier_init();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32((const void*)tmem_slot))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   // Without the caller's promise nothing of the problem is read before every earlier kernel of the stream has
   // finished (a kernel in front may still be writing prefix_len, and lines of it cached by an earlier launch on
@@ -453,31 +478,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       run += __shfl_sync(0xffffffffu, inc, 31);
     }
     if (lane == 0) cum[prm.B] = run;
-  }
-  if (threadIdx.x == 32) {
-    mbar_init(bar(L::Q_FULL), 1);
-    mbar_init(bar(L::Q_EMPTY), 1);
-#pragma unroll 1
-    for (int s = 0; s < kSlots; ++s) {
-      mbar_init(bar(L::KV_FULL + s), 1);
-      mbar_init(bar(L::KV_EMPTY + s), 1);
-    }
-    for (int s = 0; s < 2; ++s) {                // index = row tile, or parity of the key tile with one row tile
-      mbar_init(bar(L::S_FULL + s), 1);
-      mbar_init(bar(L::S_FREE + s), 4);
-      mbar_init(bar(L::P_READY + s), 4);
-      mbar_init(bar(L::ITEM_DONE + s), 1);
-    }
-    mbar_init(bar(L::O_DONE), 1);
-    mbar_init(bar(L::EPI), MT * 128);
-    *abort_flag = ((sbase & 1023u) != 0) ? 1 : 0;   // swizzled tiles need a 1024-byte aligned base
-    *last_flag = 0;
-    fence_barrier_init();
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32((const void*)tmem_slot))
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
@@ -506,9 +506,12 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   __syncthreads();
 
   Sched sch{cum, gs, prm.B, prm.Hkv, prm.Hkv * cum[prm.B] * prm.L, prm.Hkv * cum[prm.B]};
-  const int group = blockIdx.x / prm.NP;
+  // Downwards over the block index (see "Work split"); groups past the last used one get an empty range, and the CTAs
+  // that are started first (on SMs the kernel in front does not use) get work.
+  const int place = (int)(blockIdx.x / prm.NP);
+  const int group = place < groups ? groups - 1 - place : place;
   const int pair = blockIdx.x % prm.NP;
-  const int g_begin = sch.group_start(group, groups);        // groups past the last used one get an empty range
+  const int g_begin = sch.group_start(group, groups);
   const int g_end = sch.group_start(group + 1, groups);
 
   // Walks the items of this CTA's range; identical in every role.
@@ -865,25 +868,12 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const bool row_active = row_exists && node < it.n;
         float m_used = -INFINITY;      // running reference maximum, in log2 units (score * scale * log2e)
         float l_sum = 0.f;
-        // A piece of a cut unit draws its ticket early (thread 128 only): the counter is read at the start of
-        // the item and the compare-and-swap is issued when the last key tile begins, so that both round trips
-        // are hidden behind the softmax of that tile; the outcome is looked at in the epilogue.
-        const bool piece = !(it.j0 == 0 && it.j1 == it.len);
-        unsigned long long* claim_ctr =
-            prm.counters + ((((size_t)it.layer * prm.B + it.b) * prm.Hkv + it.hk) * prm.NP + pair) * 2;
-        unsigned long long claim_assumed = 0, claim_ret = 1;
-        int claim_cnt = 0;
-        if (piece && threadIdx.x == 128) claim_assumed = *reinterpret_cast<volatile unsigned long long*>(claim_ctr);
         const uint32_t o_addr_loop = tmem + lane_addr + L::kTmemO0 + wg * D;
         // key tiles below this index are full tiles of the committed prefix (no mask of any kind)
         const int j_full = min(it.S / kTileN, it.len - prm.TT);
         for (int jt = 0; jt < nt && ok; ++jt, ++tj) {
           const int j = it.j0 + jt;
           const bool masked = j >= j_full;
-          if (piece && threadIdx.x == 128 && jt == nt - 1) {
-            claim_cnt = ((claim_assumed >> 16) == prm.epoch) ? (int)(claim_assumed & 0xffffu) : 0;
-            claim_ret = atomicCAS(claim_ctr, claim_assumed, (prm.epoch << 16) | (unsigned long long)(claim_cnt + 1));
-          }
           uint32_t vis[4] = {0u, 0u, 0u, 0u};      // masked tiles: visible keys of this row
           if (masked) {
             const int tt = j - (it.len - prm.TT);      // >= 0: index of the tree key tile
@@ -1092,15 +1082,14 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               *lse_p = (row_active && m_used > -INFINITY) ? (m_used + log2f(l_sum)) / kLog2e : -INFINITY;
             tc_fence_before();
           } else {
-            // ---- a piece of a unit.  The pieces of a unit draw tickets on the unit's "claimed" counter (the
-            // draw was started while the last key tile was still being processed): the piece with the last
-            // ticket becomes the merger and keeps its O in TMEM; every other piece leaves its normalised
-            // output O/l (bf16) and (m, l) in its CTA's slot and then bumps the unit's "ready" counter.  The
-            // merger waits (bounded) until all other pieces are ready - they hold tickets, so they are in
-            // their epilogue - and combines out = sum_p w_p O_p / sum_p w_p with w_p = l_p 2^(m_p - max m).
-            // Every piece enters the sum as its bf16-rounded normalised output, the merger's own included,
-            // and the sum runs in piece order with one fused multiply-add per piece, so the result does not
-            // depend on which piece merges.  Both counters carry the call's epoch: no initialisation needed.
+            // ---- a piece of a unit.  The first piece (the one with the unit's first key tile, always the last thing
+            // its CTA does) merges; every other piece leaves its normalised output O/l (bf16) and (m, l) in its CTA's
+            // slot and raises its flag.  The merger waits (bounded) for the flags and combines
+            // out = sum_p w_p O_p / sum_p w_p with w_p = l_p 2^(m_p - max m).  Every piece enters the sum as its
+            // bf16-rounded normalised output, the merger's own included, in piece order with one fused multiply-add
+            // per piece.  What bounds this is dependent round trips to L2 (some 2 K cycles each under load): a fixed
+            // merger needs no ticket, its pieces are usually ready long before, and a piece's whole row is requested at
+            // once, the first one's beside its (m, l).  The sum stays in tensor memory between two pieces.
             // Partial outputs are stored column-group major, [slot][D/8][MT*128 rows][8 bf16]: a warp writes
             // and reads 512 contiguous bytes per instruction.
             constexpr int kRows = MT * 128;
@@ -1113,167 +1102,131 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             int k_first = group, k_last = group;
             while (gs[k_first] > real0) --k_first;
             while (gs[k_last + 1] < uend) ++k_last;
-            const int n_frag = k_last - k_first + 1;
-            // slot of the piece CTA group k holds: slot 1 of its CTA if the unit starts in that group, else slot 0
-            auto piece_slot = [&](int k) -> int { return (k * prm.NP + pair) * 2 + (k == k_first ? 1 : 0); };
-            const int my_slot = piece_slot(group);
-            unsigned long long* ctr = claim_ctr;
-            if (threadIdx.x == 128) {
-              int ticket;
-              if (claim_ret == claim_assumed) {
-                ticket = claim_cnt + 1;                      // the early draw went through
-              } else {
-                ticket = bump_counter(ctr, claim_ret, prm.epoch);
-              }
-              const int merger = (ticket == n_frag) ? 1 : 0;
-              if (merger) {
-                // wait until the other n_frag - 1 pieces have published their partials
-                const unsigned long long t0 = globaltimer_ns();
-                while (true) {
-                  const unsigned long long v = *reinterpret_cast<volatile unsigned long long*>(ctr + 1);
-                  const int ready = ((v >> 16) == prm.epoch) ? (int)(v & 0xffffu) : 0;
-                  if (ready >= n_frag - 1) break;
-                  if (*abort_flag || globaltimer_ns() - t0 > wait_limit) {
-                    *abort_flag = 1;
-                    break;
-                  }
-                }
-                __threadfence();
-                // every piece has drawn its ticket and published: nobody touches the two counters again in
-                // this launch.  Clearing them lets the same launch be replayed with the same epoch (a captured
-                // CUDA graph) and find them unused.
-                *reinterpret_cast<volatile unsigned long long*>(ctr) = 0ull;
-                *reinterpret_cast<volatile unsigned long long*>(ctr + 1) = 0ull;
-              }
-              *last_flag = merger;
-            }
-            ok = epi_sync();
-            if (!ok || *abort_flag) { ok = false; break; }
-            tr.mark(0x7000u | (*last_flag ? 1u : 0u));
+            const int n_other = k_last - k_first;
+            unsigned long long* flags = prm.counters + ((((size_t)it.layer * prm.B + it.b) * prm.Hkv + it.hk) * prm.NP + pair) * 2;
+            const unsigned long long tag = prm.epoch << 16;
             const float inv_own = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
-            if (!*last_flag) {
-              uint4* po = reinterpret_cast<uint4*>(prm.part_o) + (size_t)my_slot * (D / 8) * kRows;
-              float* pml = prm.part_ml + (size_t)my_slot * 2 * kRows;
-              store_rows(po + rr, kRows, inv_own, row_active, false);
+            if (group != k_first) {
+              const size_t slot = (size_t)group * prm.NP + pair;
+              uint4* po = reinterpret_cast<uint4*>(prm.part_o) + slot * (D / 8) * kRows;
+              float* pml = prm.part_ml + slot * 2 * kRows;
               if (row_active) {
                 pml[rr] = m_used;
                 pml[kRows + rr] = l_sum;
               }
+              store_rows(po + rr, kRows, inv_own, row_active, false);
               tc_fence_before();
               __threadfence();
               tr.mark(0x6000u);
               ok = epi_sync();
               if (!ok) break;
               if (threadIdx.x == 128 && !(prm.debug & 2)) {      // (debug bit 1: the piece is never announced)
-                const unsigned long long seen = *reinterpret_cast<volatile unsigned long long*>(ctr + 1);
-                bump_counter(ctr + 1, seen, prm.epoch);
+                const int i = group - k_first;
+                if (i == 1) *reinterpret_cast<volatile unsigned long long*>(flags) = tag | 1u;
+                else if (n_other == 2) *reinterpret_cast<volatile unsigned long long*>(flags + 1) = tag | 1u;
+                else bump_counter(flags + 1, *reinterpret_cast<volatile unsigned long long*>(flags + 1), prm.epoch);
               }
             } else {
-              // ---- pass 1: reference maximum and total weight of the row.  (m, l) of the first four pieces
-              // are fetched together (one round trip; a unit rarely has more), the rest one by one.  Loads are
-              // issued by every thread (row rr always lies inside a slot; rows that are not active read stale
-              // bytes and are masked by selects): no thread-divergent branch sits between the warp-wide TMEM ops.
-              float pm[4], w4[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int k = k_first + i;
-                const bool other = k <= k_last && k != group;
-                const float* q_ml = prm.part_ml + (size_t)piece_slot(other ? k : group) * 2 * kRows;
-                const float m_k = __ldcg(q_ml + rr), l_k = __ldcg(q_ml + kRows + rr);
-                pm[i] = other ? m_k : (k == group ? m_used : -INFINITY);
-                w4[i] = other ? l_k : (k == group ? l_sum : 0.f);
-              }
-              float mm = fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3]));
-#pragma unroll 1
-              for (int k = k_first + 4; k <= k_last; ++k)
-                mm = fmaxf(mm, k == group ? m_used : __ldcg(prm.part_ml + (size_t)piece_slot(k) * 2 * kRows + rr));
-              float lt = 0.f;
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {       // weights w_p = l_p 2^(m_p - mm), summed in piece order
-                w4[i] *= fast_exp2(pm[i] - mm);
-                lt += w4[i];
-              }
-              auto late_weight = [&](int k) -> float {     // pieces past the fourth
-                if (k == group) return l_sum * fast_exp2(m_used - mm);
-                const float* q_ml = prm.part_ml + (size_t)piece_slot(k) * 2 * kRows;
-                return __ldcg(q_ml + kRows + rr) * fast_exp2(__ldcg(q_ml + rr) - mm);
-              };
-#pragma unroll 1
-              for (int k = k_first + 4; k <= k_last; ++k) lt += late_weight(k);
-              if (!row_active) lt = 0.f;
-              const float inv = (row_active && lt > 0.f) ? 1.f / lt : 0.f;
-              // ---- pass 2: 64 output columns at a time, pieces in order (one fused multiply-add per piece and
-              // element, two elements per instruction); the own piece comes from TMEM and enters as its
-              // bf16-rounded normalised output, like every other piece
-              const float2 inv_own2 = make_float2(inv_own, inv_own), inv2 = make_float2(inv, inv);
-#pragma unroll 1
-              for (int hq = 0; hq < D / 64; ++hq) {
-                float2 acc[32];
-#pragma unroll
-                for (int c = 0; c < 32; ++c) acc[c] = make_float2(0.f, 0.f);
-#pragma unroll 1
-                for (int k = k_first; k <= k_last; ++k) {
-                  const int i = k - k_first;
-                  float w = i == 0 ? w4[0] : (i == 1 ? w4[1] : (i == 2 ? w4[2] : w4[3]));
-                  if (i >= 4) w = late_weight(k);
-                  const float2 w2 = make_float2(w, w);
-                  if (k == group) {
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                      uint32_t o[32];
-                      tmem_ld32(o_addr + (hq * 2 + q) * 32, o);
-                      tmem_wait_ld();
-#pragma unroll
-                      for (int c = 0; c < 16; ++c) {
-                        const float2 t = __fmul2_rn(make_float2(__uint_as_float(o[2 * c]), __uint_as_float(o[2 * c + 1])), inv_own2);
-                        const uint32_t own = pack_bf16(t.x, t.y);
-                        acc[q * 16 + c] = ffma2(w2, make_float2(__uint_as_float(own << 16), __uint_as_float(own & 0xffff0000u)),
-                                                acc[q * 16 + c]);
-                      }
+              if (warp == 4) {
+                // wait until the other pieces have published their partials: lane 0 the second, lane 1 the later ones
+                if (lane < 2 && lane < n_other) {
+                  const int want = lane == 0 ? 1 : n_other - 1;
+                  const unsigned long long t0 = globaltimer_ns();
+                  while (true) {
+                    const unsigned long long v = *reinterpret_cast<volatile unsigned long long*>(flags + lane);
+                    if ((v >> 16) == prm.epoch && (int)(v & 0xffffu) >= want) break;
+                    if (*abort_flag || globaltimer_ns() - t0 > wait_limit) {
+                      *abort_flag = 1;
+                      break;
                     }
-                    continue;
                   }
-                  const uint4* q_o = reinterpret_cast<const uint4*>(prm.part_o) + (size_t)piece_slot(k) * (D / 8) * kRows;
-                  uint4 v[8];
-#pragma unroll
-                  for (int c = 0; c < 8; ++c) v[c] = __ldcg(q_o + (size_t)(hq * 8 + c) * kRows + rr);
-#pragma unroll
-                  for (int c = 0; c < 8; ++c) {
-                    const uint32_t wv[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                      acc[4 * c + e] = ffma2(w2, make_float2(__uint_as_float(wv[e] << 16), __uint_as_float(wv[e] & 0xffff0000u)),
-                                             acc[4 * c + e]);
-                  }
+                  // nobody touches the flag again in this launch.  Clearing it lets the same launch be replayed with the
+                  // same epoch (a captured CUDA graph) and find it unused.
+                  *reinterpret_cast<volatile unsigned long long*>(flags + lane) = 0ull;
                 }
-                if (row_exists) {
+                __threadfence();
+              }
+              ok = epi_sync();
+              if (!ok || *abort_flag) { ok = false; break; }
+              tr.mark(0x7001u);
+              // Loads are issued by every thread (row rr always lies inside a slot; rows that are not active read stale
+              // bytes and are masked by selects): no thread-divergent branch sits between the warp-wide TMEM ops.
+              auto slot_of = [&](int i) -> size_t { return (size_t)(k_first + i) * prm.NP + pair; };       // i-th other piece, i >= 1
+              auto ml_of = [&](int i) -> const float* { return prm.part_ml + slot_of(i) * 2 * kRows + rr; };
+              auto o_of = [&](int i) -> const uint4* { return reinterpret_cast<const uint4*>(prm.part_o) + slot_of(i) * (D / 8) * kRows + rr; };
+              uint4 v[D / 8];                              // one row of a piece
+              auto fetch = [&](int i) {
+                const uint4* q_o = o_of(i);
 #pragma unroll
-                  for (int c = 0; c < 8; c += 2) {
-                    uint4 v[2];
+                for (int c = 0; c < D / 8; ++c) v[c] = __ldcg(q_o + (size_t)c * kRows);
+              };
+              const float m_1 = __ldcg(ml_of(1)), l_1 = __ldcg(ml_of(1) + kRows);
+              fetch(1);
+              float mm = fmaxf(m_used, m_1);
+#pragma unroll 4
+              for (int i = 2; i <= n_other; ++i) mm = fmaxf(mm, __ldcg(ml_of(i)));
+              const float mref = mm == -INFINITY ? 0.f : mm;
+              auto weight = [&](int i) -> float { return __ldcg(ml_of(i) + kRows) * fast_exp2(__ldcg(ml_of(i)) - mref); };
+              const float w_own = l_sum * fast_exp2(m_used - mref);
+              float w = l_1 * fast_exp2(m_1 - mref), lt = w_own + w;
+#pragma unroll 4
+              for (int i = 2; i <= n_other; ++i) lt += weight(i);
+              const bool any_key = row_active && mm > -INFINITY;
+              const float inv = any_key ? 1.f / lt : 0.f;
+#pragma unroll 1
+              for (int i = 1; i <= n_other; ++i) {
+                if (i > 1) {
+                  fetch(i);
+                  w = weight(i);
+                }
+                const float2 w2 = make_float2(w, w), own2 = make_float2(w_own, w_own), inv_own2 = make_float2(inv_own, inv_own);
+                const float2 inv2 = make_float2(inv, inv);
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                      float2 t[4];
+                for (int q = 0; q < D / 32; ++q) {
+                  uint32_t o[32];
+                  tmem_ld32(o_addr + q * 32, o);
+                  tmem_wait_ld();
 #pragma unroll
-                      for (int x = 0; x < 4; ++x) t[x] = __fmul2_rn(acc[4 * (c + e) + x], inv2);
-                      v[e].x = pack_bf16(t[0].x, t[0].y);
-                      v[e].y = pack_bf16(t[1].x, t[1].y);
-                      v[e].z = pack_bf16(t[2].x, t[2].y);
-                      v[e].w = pack_bf16(t[3].x, t[3].y);
-                      if (!row_active) v[e] = make_uint4(0, 0, 0, 0);
+                  for (int c = 0; c < 16; ++c) {
+                    float2 acc = make_float2(__uint_as_float(o[2 * c]), __uint_as_float(o[2 * c + 1]));
+                    if (i == 1) {
+                      const float2 t = __fmul2_rn(acc, inv_own2);
+                      const uint32_t own = pack_bf16(t.x, t.y);
+                      acc = __fmul2_rn(own2, make_float2(__uint_as_float(own << 16), __uint_as_float(own & 0xffff0000u)));
+                    }
+                    const uint4 vv = v[q * 4 + (c >> 2)];
+                    const uint32_t x = (c & 3) == 0 ? vv.x : ((c & 3) == 1 ? vv.y : ((c & 3) == 2 ? vv.z : vv.w));
+                    acc = ffma2(w2, make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)), acc);
+                    o[2 * c] = __float_as_uint(acc.x);
+                    o[2 * c + 1] = __float_as_uint(acc.y);
+                  }
+                  if (i < n_other) {
+                    tmem_st32(o_addr + q * 32, o);
+                  } else if (row_exists) {
+                    uint4 r[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                      uint32_t pk4[4];
+#pragma unroll
+                      for (int e = 0; e < 4; ++e) {
+                        const float2 t = __fmul2_rn(make_float2(__uint_as_float(o[8 * c + 2 * e]), __uint_as_float(o[8 * c + 2 * e + 1])), inv2);
+                        pk4[e] = any_key ? pack_bf16(t.x, t.y) : 0u;
+                      }
+                      r[c] = make_uint4(pk4[0], pk4[1], pk4[2], pk4[3]);
                     }
                     if (prm.out_al32) {
-                      st_global_32B(orow + hq * 64 + c * 8, v[0], v[1]);
+                      st_global_32B(orow + q * 32, r[0], r[1]);
+                      st_global_32B(orow + q * 32 + 16, r[2], r[3]);
                     } else {
-                      *reinterpret_cast<uint4*>(orow + hq * 64 + c * 8) = v[0];
-                      *reinterpret_cast<uint4*>(orow + hq * 64 + c * 8 + 8) = v[1];
+#pragma unroll
+                      for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(orow + q * 32 + c * 8) = r[c];
                     }
                   }
                 }
+                tmem_wait_st();
               }
-              if (row_exists && lse_p) *lse_p = (row_active && lt > 0.f) ? (mm + log2f(lt)) / kLog2e : -INFINITY;
+              if (row_exists && lse_p) *lse_p = any_key ? (mm + log2f(lt)) / kLog2e : -INFINITY;
               tc_fence_before();
-              ok = epi_sync();   // keeps the two warpgroups' barrier phases in step with the other branch
-              if (!ok) break;
             }
           }
         }
@@ -1353,10 +1306,10 @@ Geometry geometry(int B, int Nmax, int Hq, int Hkv, int d, bool query_device) {
   const size_t max_ctas = 160 > g.grid ? 160 : g.grid;
   size_t off = 0;
   g.ml_off = off;
-  off += max_ctas * 2 * (size_t)g.MT * 128 * 2 * sizeof(float);
+  off += max_ctas * (size_t)g.MT * 128 * 2 * sizeof(float);
   off = (off + 255) & ~size_t(255);
   g.o_off = off;
-  off += max_ctas * 2 * (size_t)g.MT * 128 * d * sizeof(tv_bf16);
+  off += max_ctas * (size_t)g.MT * 128 * d * sizeof(tv_bf16);
   off = (off + 255) & ~size_t(255);
   g.counters_off = off;
   g.counters_per_layer = ((size_t)B * Hkv * g.NP * 2 * sizeof(unsigned long long) + 255) & ~size_t(255);

@@ -513,3 +513,19 @@ def test_layers_call_with_padded_layer_strides_is_bit_equal_to_the_dense_call():
     per = B * N * Hq * d                       # the gaps between the layers of the output were left alone
     gaps = torch.as_strided(out_p, (L, 24), (per + 24, 1), per)
     assert (gaps == 7.0).all()
+
+
+@pytest.mark.parametrize("S", [700, 1100, 2600, 6000])
+@pytest.mark.parametrize("G,d", [(2, 64), (4, 128)])
+@pytest.mark.parametrize("B", [1, 3])
+def test_units_cut_in_two_to_many_pieces(S, G, d, B):
+    """Prefixes that are cut in two, three and more pieces (one KV head, few units): sums that stay in tensor memory
+    between two pieces, and both kinds of flags, twice with the same workspace contents."""
+    cfg = CONFIGS[0].scaled(B=B, Hq=G, Hkv=1, d=d, S_lo=S - 130, S_hi=S, Scap=S + 200, N=40, D=6, V=0, tree="uniform")
+    case = make_case(cfg, seed=S + G + B, ragged_nodes=True, with_logits=False)
+    dcase = to_device(case)
+    out, lse, bits, dense = gpu_attention(dcase)
+    ref_out, ref_lse = oracle_attention(case_to_numpy(case), dense.cpu().numpy())
+    assert_attention_close(out, lse, ref_out, ref_lse, f"S={S}")
+    out2, lse2, _, _ = gpu_attention(dcase)
+    assert torch.equal(out, out2) and torch.equal(lse, lse2)
