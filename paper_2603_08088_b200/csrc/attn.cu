@@ -38,6 +38,11 @@
 // block index, which were started before it.  Flags carry a per-call epoch, so the
 // workspace needs no initialisation.
 //
+// Few units (CL = true).  A unit is shared by a thread-block cluster instead: its CTAs
+// take equal shares of the unit's key tiles, leave their partials in their own shared
+// memory and, behind a cluster barrier, each merges a share of the rows through
+// distributed shared memory.  No tile table, no workspace, no flags; see cluster_size.
+//
 // Every wait on an mbarrier is bounded: on expiry the CTA raises
 // TV_ST_TIMEOUT for all sequences, all roles leave their loops, outstanding
 // copies are given time to land, TMEM is freed and the kernel returns.
@@ -79,6 +84,8 @@ constexpr int kMaxGroups = 160;
 #define TV_MIN_VT 6
 #endif
 constexpr int kMinVirtualTilesPerGroup = TV_MIN_VT;
+constexpr int kMaxCluster = 8;     // CTAs that share a unit (16 is not portable; few clusters of 16 fit the GPU at once: 21.7 us
+                                   // instead of 10.8 us a launch for eight units of 12 key tiles)
 constexpr int kTraceCap = 256;     // events per (CTA, role) kept by the optional trace
 
 // ---------------------------------------------------------------- PTX helpers
@@ -148,6 +155,31 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void st_global_32B(void* p, uint4 a, uint4 b) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w),
                "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
+}
+// Thread-block clusters: barrier over all threads, and reads of another CTA's shared memory (32-bit cluster addresses).
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_size_x() {
+  uint32_t n;
+  asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));
+  return n;
+}
+__device__ __forceinline__ uint32_t peer_smem(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float ld_peer_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 ld_peer_16B(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -401,10 +433,12 @@ struct SmemLayout {
   static constexpr int kCum = kMisc + 16;
   static constexpr int kGs = kCum + (kMaxB + 1) * 4;
   static constexpr int kTotal = kGs + (kMaxGroups + 1) * 4;
+  static constexpr int kMl = kCum;                         // cluster kernel: (m, l) of every row, in place of the tile table
+  static_assert(kMl + MT * 128 * 8 <= kTotal && kMl % 8 == 0, "(m, l) pairs fit the room of the tile table");
 };
 
 // ---------------------------------------------------------------- the kernel
-template <int D, int MT>
+template <int D, int MT, bool CL>
 __global__ void __launch_bounds__(kThreads, 1)
 tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kc,
                  const __grid_constant__ CUtensorMap map_vc, const __grid_constant__ CUtensorMap map_kt,
@@ -457,7 +491,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // finished (a kernel in front may still be writing prefix_len, and lines of it cached by an earlier launch on
   // this SM are only dropped by the wait).
   if (!prm.early) gdc_wait();
-  if (warp == 0) {
+  if (!CL && warp == 0) {
     int run = 0;
 #pragma unroll 1
     for (int base = 0; base < prm.B; base += 32) {
@@ -485,8 +519,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t tmem = *tmem_slot;
   // Small problems use fewer CTA groups, so that a unit is cut into few pieces (each piece costs a partial
   // write and a merge) and every group still gets a worthwhile share of tiles.
-  int groups;
-  {
+  int groups = 1;
+  if (!CL) {
     const unsigned total = (unsigned)(prm.Hkv * cum[prm.B]) * (unsigned)prm.L;
     const unsigned want = total / (unsigned)kMinVirtualTilesPerGroup;
     groups = want < 1u ? 1 : (want < (unsigned)prm.groups ? (int)want : prm.groups);
@@ -503,19 +537,38 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     for (int k = threadIdx.x; k <= prm.groups; k += kThreads)
       gs[k] = k <= groups ? (int)(k * q + (k * r) / (unsigned)groups) : (int)total;
   }
-  __syncthreads();
+  if (!CL) __syncthreads();
 
-  Sched sch{cum, gs, prm.B, prm.Hkv, prm.Hkv * cum[prm.B] * prm.L, prm.Hkv * cum[prm.B]};
+  const int per_layer = CL ? 0 : prm.Hkv * cum[prm.B];
+  Sched sch{cum, gs, prm.B, prm.Hkv, per_layer * prm.L, per_layer};
   // Downwards over the block index (see "Work split"); groups past the last used one get an empty range, and the CTAs
   // that are started first (on SMs the kernel in front does not use) get work.
+  const int unit = CL ? (int)(blockIdx.x / cluster_size_x()) : 0;      // cluster kernel: (layer, sequence, KV head, pair)
   const int place = (int)(blockIdx.x / prm.NP);
   const int group = place < groups ? groups - 1 - place : place;
-  const int pair = blockIdx.x % prm.NP;
-  const int g_begin = sch.group_start(group, groups);
-  const int g_end = sch.group_start(group + 1, groups);
+  const int pair = CL ? unit % prm.NP : (int)(blockIdx.x % prm.NP);
+  const int g_begin = CL ? 0 : sch.group_start(group, groups);
+  const int g_end = CL ? 1 : sch.group_start(group + 1, groups);
 
   // Walks the items of this CTA's range; identical in every role.
   auto next_item = [&](int& g, Item& it) -> bool {
+    if (CL) {                      // one item: this CTA's share of the key tiles of its cluster's unit (may be empty)
+      if (g > 0) return false;
+      g = 1;
+      const int u = unit / prm.NP;
+      it.hk = u % prm.Hkv;
+      it.b = u / prm.Hkv % prm.B;
+      it.layer = u / prm.Hkv / prm.B;
+      int S = prm.prefix_len[it.b];
+      it.S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
+      int n = prm.n_nodes[it.b];
+      it.n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
+      it.len = (it.S + kTileN - 1) / kTileN + prm.TT;
+      const int size = (int)cluster_size_x(), rank = (int)(blockIdx.x % size);
+      it.j0 = it.len * rank / size;
+      it.j1 = it.len * (rank + 1) / size;
+      return it.j1 > it.j0;
+    }
     while (g < g_end) {
       const int layer = (int)((unsigned)g / (unsigned)sch.per_layer);
       const int gl = g - layer * sch.per_layer;                   // place inside the layer
@@ -657,6 +710,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     } else {
       gdc_wait();
       if (elect_one()) gdc_launch_dependents();
+    }
+    if (CL) {
+      __syncwarp();
+      cluster_sync();
+      cluster_sync();
     }
   } else if (warp == 1) {
     // =========================================================== MMA issuer
@@ -817,6 +875,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         ++item_idx;
       }
     }
+    if (CL) {
+      __syncwarp();
+      cluster_sync();
+      cluster_sync();
+    }
   } else if (warp >= 4) {
     // =========================================================== softmax / epilogue warpgroups
     // Register budget: the CTA starts with 168 registers per thread; warps 0-3 give up 96 each (168 -> 72) and
@@ -839,6 +902,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
         if (S + prm.n_nodes[b] > prm.Scap) atomicOr(prm.status + b, TV_ST_CAPACITY);
       }
+    float m_fin = -INFINITY, l_fin = 0.f;            // cluster kernel: (m, l) of the row; no key tile: weight 0
     if (wg_active && !*abort_flag && !(prm.debug & 4)) {
       int g = g_begin;
       Item it;
@@ -1075,7 +1139,30 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
             }
           };
-          if (whole) {
+          if (CL) {
+            // ---- the partial of this CTA: normalised bf16 rows over the Q tile (every QK^T of the item is done), 16-byte
+            // pieces of a row swizzled by the row so that neither the writes nor the reads collide; (m, l) beside them
+            const float inv = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
+            uint8_t* mine = smem + L::kQ + wg * L::kTileBytes + row * (D * 2);
+#pragma unroll 1
+            for (int q = 0; q < D / 32; ++q) {
+              uint32_t o[32];
+              tmem_ld32(o_addr + q * 32, o);
+              tmem_wait_ld();
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                uint4 v;
+                v.x = pack_bf16(__uint_as_float(o[8 * c + 0]) * inv, __uint_as_float(o[8 * c + 1]) * inv);
+                v.y = pack_bf16(__uint_as_float(o[8 * c + 2]) * inv, __uint_as_float(o[8 * c + 3]) * inv);
+                v.z = pack_bf16(__uint_as_float(o[8 * c + 4]) * inv, __uint_as_float(o[8 * c + 5]) * inv);
+                v.w = pack_bf16(__uint_as_float(o[8 * c + 6]) * inv, __uint_as_float(o[8 * c + 7]) * inv);
+                *reinterpret_cast<uint4*>(mine + (((q * 4 + c) ^ (row & 7)) * 16)) = v;
+              }
+            }
+            m_fin = m_used;
+            l_fin = l_sum;
+            tc_fence_before();
+          } else if (whole) {
             const float inv = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
             store_rows(reinterpret_cast<uint4*>(orow), 1, inv, row_exists, !row_active);
             if (row_exists && lse_p)
@@ -1234,8 +1321,78 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         fill += 2 * nt;
       }
     }
+    if (CL) {
+      // ---- merge of the cluster's partials: each CTA takes a share of the rows, 16 bytes of a row per thread; out =
+      // sum_p w_p O_p / sum_p w_p, w_p = l_p 2^(m_p - max m), in rank order.  A piece without keys has weight 0 (its rows
+      // were not written and are not used).
+      if (wg_active) *reinterpret_cast<float2*>(smem + L::kMl + (wg * 128 + row) * 8) = make_float2(m_fin, l_fin);
+      __syncwarp();
+      cluster_sync();
+      if (!*abort_flag && !(prm.debug & 4)) {
+        constexpr int kVecs = D / 8;
+        const int size = (int)cluster_size_x(), rank = (int)(blockIdx.x % size);
+        const int u = unit / prm.NP, hk = u % prm.Hkv, b = u / prm.Hkv % prm.B, layer = u / prm.Hkv / prm.B;
+        int n = prm.n_nodes[b];
+        n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
+        const int nodes = max(0, min(MT * prm.NPT, prm.Nmax - pair * MT * prm.NPT));      // nodes of this pair of row tiles
+        const int total = nodes * prm.G * kVecs;
+        for (int x = rank * 256 + (int)threadIdx.x - 128; x < total; x += size * 256) {
+          const int r = x / kVecs, c = x - r * kVecs;              // row among the existing ones, piece of the row
+          const int node_l = r / prm.G, gm = r - node_l * prm.G;
+          const int t = MT == 2 && node_l >= prm.NPT ? 1 : 0, in_tile = (node_l - t * prm.NPT) * prm.G + gm;
+          const uint32_t ml = sbase + L::kMl + (t * 128 + in_tile) * 8;
+          const uint32_t at = sbase + L::kQ + t * L::kTileBytes + in_tile * (D * 2) + ((c ^ (in_tile & 7)) * 16);
+          float pm[kMaxCluster], w[kMaxCluster];
+          uint4 v[kMaxCluster];
+#pragma unroll
+          for (int k = 0; k < kMaxCluster; ++k)
+            if (k < size) {
+              const uint32_t pml = peer_smem(ml, k);
+              pm[k] = ld_peer_f32(pml);
+              w[k] = ld_peer_f32(pml + 4);
+              v[k] = ld_peer_16B(peer_smem(at, k));
+            }
+          float mm = -INFINITY;
+#pragma unroll
+          for (int k = 0; k < kMaxCluster; ++k)
+            if (k < size) mm = fmaxf(mm, pm[k]);
+          float lt = 0.f, acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int k = 0; k < kMaxCluster; ++k)
+            if (k < size) {
+              const float wk = pm[k] > -INFINITY ? w[k] * fast_exp2(pm[k] - mm) : 0.f;
+              lt += wk;
+              const uint32_t e[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+              if (wk > 0.f)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  acc[2 * i] = fmaf(wk, __uint_as_float(e[i] << 16), acc[2 * i]);
+                  acc[2 * i + 1] = fmaf(wk, __uint_as_float(e[i] & 0xffff0000u), acc[2 * i + 1]);
+                }
+            }
+          const int node = pair * MT * prm.NPT + node_l, h = hk * prm.G + gm;
+          const bool any_key = node < n && mm > -INFINITY;
+          const float inv = any_key ? 1.f / lt : 0.f;
+          uint4 o;
+          o.x = pack_bf16(acc[0] * inv, acc[1] * inv);
+          o.y = pack_bf16(acc[2] * inv, acc[3] * inv);
+          o.z = pack_bf16(acc[4] * inv, acc[5] * inv);
+          o.w = pack_bf16(acc[6] * inv, acc[7] * inv);
+          if (!any_key) o = make_uint4(0, 0, 0, 0);
+          *reinterpret_cast<uint4*>(prm.out + (size_t)layer * prm.out_layer_stride + (((size_t)b * prm.Nmax + node) * prm.Hq + h) * D + c * 8) = o;
+          if (c == 0 && prm.lse)
+            prm.lse[(((size_t)layer * prm.B + b) * prm.Hq + h) * prm.Nmax + node] = any_key ? (mm + log2f(lt)) / kLog2e : -INFINITY;
+        }
+      }
+      __syncwarp();
+      cluster_sync();            // nobody leaves while its shared memory may still be read
+    }
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    if (CL) {
+      cluster_sync();
+      cluster_sync();
+    }
   }
 
   // ---- teardown
@@ -1327,31 +1484,99 @@ unsigned long long next_epoch() {
   return ctr.fetch_add(1, std::memory_order_relaxed) & 0xffffffffffffull;
 }
 
-template <int D, int MT>
-cudaError_t launch(const Geometry& g, const CUtensorMap* maps, const AttnParams& prm, cudaStream_t s) {
-  using L = SmemLayout<D, MT>;
+// Allows the kernel its shared memory, once per device.
+template <int D, int MT, bool CL>
+cudaError_t configure(int dev) {
   static std::atomic<bool> configured[64];
-  auto kern = tree_attn_kernel<D, MT>;
+  if (dev >= 0 && dev < 64 && configured[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(tree_attn_kernel<D, MT, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             SmemLayout<D, MT>::kTotal);
+  if (e == cudaSuccess && dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
+  return e;
+}
+
+struct LaunchConfig {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  LaunchConfig(unsigned grid, unsigned cluster, size_t smem, cudaStream_t s) {
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    // Programmatic stream serialisation: this launch may be scheduled while the kernel in front is still
+    // running (if that kernel allows it); the kernel itself waits before it touches anything that kernel writes.
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+  }
+};
+
+// Clusters of 2, 4 and 8 CTAs that the device runs at the same time (asked once per device and size; 0: none).
+template <int D, int MT>
+int clusters_at_once(int dev, int log2_size) {
+  static std::atomic<int> known[64][4];          // value + 1
+  if (dev < 0 || dev >= 64) return 0;
+  int v = known[dev][log2_size].load(std::memory_order_relaxed);
+  if (v == 0) {
+    int n = 0;
+    const unsigned size = 1u << log2_size;
+    LaunchConfig lc(size, size, SmemLayout<D, MT>::kTotal, nullptr);
+    if (configure<D, MT, true>(dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, tree_attn_kernel<D, MT, true>, &lc.cfg) != cudaSuccess)
+      n = 0;
+    v = n + 1;
+    known[dev][log2_size].store(v, std::memory_order_relaxed);
+  }
+  return v - 1;
+}
+
+// CTAs per unit for the cluster kernel, 1: the even cut over all CTAs.  `units`: (layer, sequence, KV head, row-tile pair);
+// `tiles`: key tiles of the longest unit the call can have (the lengths themselves are on the device).  The largest
+// cluster for which all units run at once; then the rule weighs a CTA's share of the tiles against the share of the even
+// cut plus what that pays beyond its tiles: flags and partials through L2 (about six tiles' time) and the serial merge of
+// a unit's pieces (about one tile's each).  Measured (32 query heads, d = 128; cluster / even cut, us a launch): 8 KV
+// heads, 17 nodes, one sequence of 200: 8.9 / 15.6, 1392: 10.9 / 18.3, 8192: 18.3 / 31.1, 32768: 44 / 54; 60 nodes, 65536:
+// 110 / 89; 32 KV heads, 60 nodes, 2048: 14.2 / 20.6, 32768: 85 / 90.  Several sequences may differ in length, which only
+// the even cut can level: they take the cluster kernel only while a share is short (4 sequences of 2048 ... 256: 13.9 /
+// 20.1, of 4096 ... 512: 18.5 / 24.4; four equal ones of 4096: 19.0 / 25.0).
+template <int D, int MT>
+int cluster_size(long long units, int B, int tiles, int sms) {
+  if (units * 2 > sms) return 1;
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
+  for (int lg = 3; lg >= 1; --lg) {
+    const int size = 1 << lg;
+    if (units * size > sms || (size > 2 && size / 2 >= tiles) || clusters_at_once<D, MT>(dev, lg) < units) continue;
+    const int share = (tiles + size - 1) / size;
+    if (B > 1) return share <= 12 ? size : 1;
+    return share <= units * tiles / sms + 6 + sms / units ? size : 1;
   }
-  // Programmatic stream serialisation: this launch may be scheduled while the kernel in front is still
-  // running (if that kernel allows it); the kernel itself waits before it touches anything that kernel writes.
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(g.grid);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = L::kTotal;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
+  return 1;
+}
+
+// cluster = 1: the even cut
+template <int D, int MT, bool CL>
+cudaError_t launch_kernel(unsigned grid, unsigned cluster, const CUtensorMap* maps, const AttnParams& prm, cudaStream_t s) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const cudaError_t e = configure<D, MT, CL>(dev);
+  if (e != cudaSuccess) return e;
+  LaunchConfig lc(grid, cluster, SmemLayout<D, MT>::kTotal, s);
+  return cudaLaunchKernelEx(&lc.cfg, tree_attn_kernel<D, MT, CL>, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
+}
+
+template <int D, int MT>
+cudaError_t launch(const Geometry& g, const CUtensorMap* maps, const AttnParams& prm, cudaStream_t s) {
+  const long long units = (long long)prm.L * prm.B * prm.Hkv * prm.NP;
+  // (the test entries exercise the waits of the even cut)
+  const int cluster = prm.debug ? 1 : cluster_size<D, MT>(units, prm.B, (prm.Scap + kTileN - 1) / kTileN + prm.TT, g.sms);
+  if (cluster > 1) return launch_kernel<D, MT, true>((unsigned)(units * cluster), (unsigned)cluster, maps, prm, s);
+  return launch_kernel<D, MT, false>((unsigned)g.grid, 1, maps, prm, s);
 }
 
 struct AttnOptions {

@@ -529,3 +529,26 @@ def test_units_cut_in_two_to_many_pieces(S, G, d, B):
     assert_attention_close(out, lse, ref_out, ref_lse, f"S={S}")
     out2, lse2, _, _ = gpu_attention(dcase)
     assert torch.equal(out, out2) and torch.equal(lse, lse2)
+
+
+CLUSTERS = [      # B, Hkv, G, N, S, d: units shared by 8, 4 and 2 CTAs; fewer key tiles than CTAs; one and two row tiles; padding
+    (1, 1, 1, 1, 0, 64), (1, 2, 4, 17, 1, 128), (1, 8, 4, 17, 130, 128), (1, 8, 4, 33, 1000, 128), (2, 8, 3, 60, 900, 128),
+    (1, 32, 1, 60, 1300, 128), (3, 4, 8, 40, 513, 64), (1, 64, 1, 9, 700, 128), (1, 5, 4, 200, 777, 128), (8, 8, 1, 256, 300, 64),
+    (1, 1, 128, 5, 600, 128), (1, 1, 4, 60, 6200, 64),
+]
+
+
+@pytest.mark.parametrize("B,Hkv,G,N,S,d", CLUSTERS)
+def test_units_shared_by_a_cluster(B, Hkv, G, N, S, d):
+    cfg = CONFIGS[0].scaled(B=B, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=S // 3 if B > 1 else S, S_hi=S, Scap=S + N + 40, N=N,
+                            D=min(6, N - 1), V=0, tree="uniform")
+    case = make_case(cfg, seed=S + G + N, ragged_nodes=True, with_logits=False)
+    dcase = to_device(case)
+    for b in range(B):                       # rows behind the prefix hold NaN: nothing of them may reach an output
+        dcase["k_cache"][0, b, :, int(case["prefix_len"][b]):] = float("nan")
+        dcase["v_cache"][0, b, :, int(case["prefix_len"][b]):] = float("nan")
+    out, lse, bits, dense = gpu_attention(dcase)
+    ref_out, ref_lse = oracle_attention(case_to_numpy(case), dense.cpu().numpy())
+    assert_attention_close(out, lse, ref_out, ref_lse, "cluster")
+    out2, lse2, _, _ = gpu_attention(dcase)
+    assert torch.equal(out, out2) and torch.equal(lse, lse2)
