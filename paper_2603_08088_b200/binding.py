@@ -1,6 +1,8 @@
-"""ctypes binding of libtreeverify.so: the same entry points as
-include/treeverify.h, taking torch tensors (device memory) and doing argument
-marshalling only.  There is no fallback of any kind: if the shared library is
+"""Binding of libtreeverify.so: the same entry points as include/treeverify.h,
+taking torch tensors (device memory) and doing argument marshalling only.  The
+calls of a step go through _calls.so (csrc/calls.cpp, which finds pointers, sizes
+and the current stream natively: a step is many small calls), everything else
+through ctypes.  There is no fallback of any kind: if a shared library is
 missing or a call fails, an exception is raised.
 """
 import ctypes
@@ -43,11 +45,12 @@ class StepHostArgs(ctypes.Structure):
 
 
 _lib = None
+_calls = None
 
 
 def load():
-    """Load the shared library (once).  Raises if it has not been built."""
-    global _lib
+    """Load the shared libraries (once).  Raises if they have not been built."""
+    global _lib, _calls
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -110,8 +113,16 @@ def load():
     if hasattr(lib, "tv_debug_attn_simt"):
         lib.tv_debug_attn_simt.restype = _c_int
         lib.tv_debug_attn_simt.argtypes = [_c_vp] * 8 + [_c_int] * 6 + [_c_f, _c_vp, _c_vp, _c_vp]
+    from . import _calls as native        # links to the library loaded above
+    _calls = native
     _lib = lib
     return lib
+
+
+def _native():
+    if _calls is None:
+        load()
+    return _calls
 
 
 def _ptr(t):
@@ -156,56 +167,29 @@ def tv_step_staging_bytes(L, B, Nmax, Hq, Hkv, d, Scap, V, P, Dp1):
 
 def tree_build_mask(parent, n_nodes, Dcap, Pcap, anc_bits, status, dense_mask=None, depth=None,
                     anc_table=None, retrieve_indices=None, n_paths=None, stream=None):
-    B, Nmax = parent.shape
-    _check(load().tree_build_mask(_ptr(parent), _ptr(n_nodes), B, Nmax, Dcap, Pcap, _ptr(anc_bits),
-                                  _ptr(dense_mask), _ptr(depth), _ptr(anc_table), _ptr(retrieve_indices),
-                                  _ptr(n_paths), _ptr(status), _stream(stream)))
+    _check((_calls or _native()).tree_build_mask(parent, n_nodes, Dcap, Pcap, anc_bits, dense_mask, depth, anc_table,
+                                                 retrieve_indices, n_paths, status, stream))
 
 
 def tree_verify_attn(q, k_cache, v_cache, k_tree, v_tree, prefix_len, n_nodes, anc_bits, scale, out,
                      workspace, status, lse=None, stream=None):
-    B, Nmax, Hq, d = q.shape
-    _, Hkv, Scap, _ = k_cache.shape
-    _check(load().tree_verify_attn(_ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(k_tree), _ptr(v_tree),
-                                   _ptr(prefix_len), _ptr(n_nodes), _ptr(anc_bits), B, Nmax, Hq, Hkv, d, Scap,
-                                   float(scale), _ptr(out), _ptr(lse), _ptr(workspace),
-                                   workspace.numel() * workspace.element_size(), _ptr(status), _stream(stream)))
+    _check((_calls or _native()).tree_verify_attn(q, k_cache, v_cache, k_tree, v_tree, prefix_len, n_nodes, anc_bits, scale,
+                                                  out, workspace, status, lse, stream))
 
 
 def tree_verify_attn_layers(q, k_cache, v_cache, k_tree, v_tree, prefix_len, n_nodes, anc_bits, scale, out,
                             workspace, status, lse=None, flags=0, stream=None):
     """All layers of a step in one call: q, out [L,B,Nmax,Hq,d], k_cache, v_cache [L,B,Hkv,Scap,d], k_tree, v_tree
     [L,B,Nmax,Hkv,d] (or None: in-cache layout), lse [L,B,Hq,Nmax] or None; layer strides are taken from the tensors."""
-    L, B, Nmax, Hq, d = q.shape
-    _, _, Hkv, Scap, _ = k_cache.shape
-    for t in (q, k_cache, v_cache, k_tree, v_tree, out, lse):
-        assert t is None or t.shape[0] == L
-        assert t is None or t[0].is_contiguous(), "treeverify takes dense layers"
-    assert k_cache.stride(0) == v_cache.stride(0) and (k_tree is None or k_tree.stride(0) == v_tree.stride(0))
-    assert lse is None or lse.is_contiguous()
-    _check(load().tree_verify_attn_layers(q.data_ptr(), k_cache.data_ptr(), v_cache.data_ptr(),
-                                          None if k_tree is None else k_tree.data_ptr(),
-                                          None if v_tree is None else v_tree.data_ptr(), _ptr(prefix_len), _ptr(n_nodes),
-                                          _ptr(anc_bits), L, B, Nmax, Hq, Hkv, d, Scap, float(scale), q.stride(0),
-                                          k_cache.stride(0), 0 if k_tree is None else k_tree.stride(0), out.data_ptr(),
-                                          out.stride(0), None if lse is None else lse.data_ptr(), _ptr(workspace),
-                                          workspace.numel() * workspace.element_size(), _ptr(status), int(flags),
-                                          _stream(stream)))
+    _check((_calls or _native()).tree_verify_attn_layers(q, k_cache, v_cache, k_tree, v_tree, prefix_len, n_nodes, anc_bits,
+                                                         scale, out, workspace, status, lse, flags, stream))
 
 
 def tree_verify_attn_paged_layers(q, k_pages, v_pages, block_table, k_tree, v_tree, prefix_len, n_nodes, anc_bits, scale,
                                   out, workspace, status, lse=None, flags=0, stream=None):
     """All layers over a paged cache: k_pages, v_pages [L,n_pages,Hkv,128,d], one block table [B,max_blocks]."""
-    L, B, Nmax, Hq, d = q.shape
-    _, n_pages, Hkv, _, _ = k_pages.shape
-    assert lse is None or lse.is_contiguous()
-    _check(load().tree_verify_attn_paged_layers(q.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(), _ptr(block_table),
-                                                k_tree.data_ptr(), v_tree.data_ptr(), _ptr(prefix_len), _ptr(n_nodes),
-                                                _ptr(anc_bits), L, B, Nmax, Hq, Hkv, d, n_pages, block_table.shape[1],
-                                                float(scale), q.stride(0), k_pages.stride(0), k_tree.stride(0),
-                                                out.data_ptr(), out.stride(0), None if lse is None else lse.data_ptr(),
-                                                _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                                _ptr(status), int(flags), _stream(stream)))
+    _check((_calls or _native()).tree_verify_attn_paged_layers(q, k_pages, v_pages, block_table, k_tree, v_tree, prefix_len,
+                                                               n_nodes, anc_bits, scale, out, workspace, status, lse, flags, stream))
 
 
 def tv_debug_attn_expire(q, k_cache, v_cache, k_tree, v_tree, prefix_len, n_nodes, anc_bits, scale, out, workspace, status,
@@ -245,13 +229,8 @@ def tv_debug_attn_simt(q, k_cache, v_cache, k_tree, v_tree, prefix_len, n_nodes,
 
 def tree_accept(logits, tokens, retrieve_indices, n_nodes, argmax_tok, accept_len, best_path, accepted_nodes,
                 next_token, workspace, status, safe_idx=None, candidates=None, stream=None):
-    B, Nmax, V = logits.shape
-    P, Dp1 = retrieve_indices.shape[1], retrieve_indices.shape[2]
-    _check(load().tree_accept(_ptr(logits), _ptr(tokens), _ptr(retrieve_indices) if P > 0 else None, _ptr(n_nodes),
-                              B, Nmax, V, P, Dp1, _ptr(argmax_tok), _ptr(safe_idx), _ptr(candidates),
-                              _ptr(accept_len), _ptr(best_path), _ptr(accepted_nodes), _ptr(next_token),
-                              _ptr(workspace), workspace.numel() * workspace.element_size(), _ptr(status),
-                              _stream(stream)))
+    _check((_calls or _native()).tree_accept(logits, tokens, retrieve_indices, n_nodes, argmax_tok, safe_idx, candidates,
+                                             accept_len, best_path, accepted_nodes, next_token, workspace, status, stream))
 
 
 def tree_node_scores(logits, tokens, parent, n_nodes, scores, status, stream=None):
@@ -261,9 +240,7 @@ def tree_node_scores(logits, tokens, parent, n_nodes, scores, status, stream=Non
 
 
 def tree_merge_partials(o_parts, lse_parts, out, lse=None, stream=None):
-    R, B, Nmax, Hq, d = o_parts.shape
-    _check(load().tree_merge_partials(_ptr(o_parts), _ptr(lse_parts), R, B, Nmax, Hq, d, _ptr(out),
-                                      _ptr(lse) if lse is not None else None, _stream(stream)))
+    _check((_calls or _native()).tree_merge_partials(o_parts, lse_parts, out, lse, stream))
 
 
 def tv_sample_workspace_bytes(B, Nmax, V):
@@ -273,11 +250,8 @@ def tv_sample_workspace_bytes(B, Nmax, V):
 def tree_accept_sample(logits, tokens, parent, n_nodes, u_node, u_bonus, temperature, accept_len, accepted_nodes,
                        next_token, workspace, status, stream=None):
     """Sampling-mode acceptance over the tree; u_node [B,Nmax] and u_bonus [B] are float32 uniforms in [0,1)."""
-    B, Nmax, V = logits.shape
-    _check(load().tree_accept_sample(_ptr(logits), _ptr(tokens), _ptr(parent), _ptr(n_nodes), _ptr(u_node),
-                                     _ptr(u_bonus), float(temperature), B, Nmax, V, accepted_nodes.shape[1],
-                                     _ptr(accept_len), _ptr(accepted_nodes), _ptr(next_token), _ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _ptr(status), _stream(stream)))
+    _check((_calls or _native()).tree_accept_sample(logits, tokens, parent, n_nodes, u_node, u_bonus, temperature,
+                                                    accept_len, accepted_nodes, next_token, workspace, status, stream))
 
 
 def tv_accept_noalloc_max_bytes():
@@ -297,46 +271,29 @@ def tree_accept_noalloc(logits, tokens, retrieve_indices, n_nodes, argmax_tok, a
 
 
 def kv_commit(k_cache, v_cache, k_tree, v_tree, accepted_nodes, accept_len, prefix_len, status, stream=None):
-    L, B, Hkv, Scap, d = k_cache.shape
-    Nmax = k_tree.shape[2]
-    Dp1 = accepted_nodes.shape[1]
-    _check(load().kv_commit(_ptr(k_cache), _ptr(v_cache), _ptr(k_tree), _ptr(v_tree), _ptr(accepted_nodes),
-                            _ptr(accept_len), _ptr(prefix_len), L, B, Nmax, Hkv, d, Scap, Dp1,
-                            k_cache.stride(0), k_tree.stride(0), _ptr(status), _stream(stream)))
+    _check((_calls or _native()).kv_commit(k_cache, v_cache, k_tree, v_tree, accepted_nodes, accept_len, prefix_len, status,
+                                           stream))
 
 
 def tree_verify_attn_paged(q, k_pages, v_pages, block_table, k_tree, v_tree, prefix_len, n_nodes, anc_bits, scale, out,
                            workspace, status, lse=None, stream=None):
     """k_pages, v_pages [n_pages,Hkv,128,d] (one layer), block_table [B,max_blocks] int32."""
-    B, Nmax, Hq, d = q.shape
-    n_pages, Hkv = k_pages.shape[0], k_pages.shape[1]
-    assert k_pages.shape[2] == 128 and block_table.shape[0] == B
-    _check(load().tree_verify_attn_paged(_ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(block_table), _ptr(k_tree),
-                                         _ptr(v_tree), _ptr(prefix_len), _ptr(n_nodes), _ptr(anc_bits), B, Nmax, Hq,
-                                         Hkv, d, n_pages, block_table.shape[1], float(scale), _ptr(out), _ptr(lse),
-                                         _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                         _ptr(status), _stream(stream)))
+    _check((_calls or _native()).tree_verify_attn_paged(q, k_pages, v_pages, block_table, k_tree, v_tree, prefix_len,
+                                                        n_nodes, anc_bits, scale, out, workspace, status, lse, stream))
 
 
 def kv_commit_paged(k_pages, v_pages, block_table, k_tree, v_tree, accepted_nodes, accept_len, prefix_len, status,
                     stream=None):
     """k_pages, v_pages [L,n_pages,Hkv,128,d]."""
-    L, n_pages, Hkv, _, d = k_pages.shape
-    B, Nmax = k_tree.shape[1], k_tree.shape[2]
-    _check(load().kv_commit_paged(_ptr(k_pages), _ptr(v_pages), _ptr(block_table), _ptr(k_tree), _ptr(v_tree),
-                                  _ptr(accepted_nodes), _ptr(accept_len), _ptr(prefix_len), L, B, Nmax, Hkv, d,
-                                  n_pages, block_table.shape[1], accepted_nodes.shape[1], k_pages.stride(0),
-                                  k_tree.stride(0), _ptr(status), _stream(stream)))
+    _check((_calls or _native()).kv_commit_paged(k_pages, v_pages, block_table, k_tree, v_tree, accepted_nodes, accept_len,
+                                                 prefix_len, status, stream))
 
 
 def kv_commit_inplace(k_cache, v_cache, accepted_nodes, accept_len, prefix_len, Nmax, status, stream=None):
     """In-cache layout: node i's K/V are rows prefix_len[b] + i of the cache; the accepted path is gathered to
     the front of that region and prefix_len advances."""
-    L, B, Hkv, Scap, d = k_cache.shape
-    Dp1 = accepted_nodes.shape[1]
-    _check(load().kv_commit_inplace(_ptr(k_cache), _ptr(v_cache), _ptr(accepted_nodes), _ptr(accept_len),
-                                    _ptr(prefix_len), L, B, Nmax, Hkv, d, Scap, Dp1, k_cache.stride(0),
-                                    _ptr(status), _stream(stream)))
+    _check((_calls or _native()).kv_commit_inplace(k_cache, v_cache, accepted_nodes, accept_len, prefix_len, Nmax, status,
+                                                   stream))
 
 
 def tv_verify_step_host(host, k_cache, v_cache, prefix_len, staging, scale, V, stream=None):

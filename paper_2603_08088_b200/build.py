@@ -3,13 +3,15 @@
     python -m paper_2603_08088_b200.build [--force] [--verbose]
 
 Every .cu under csrc/ is compiled to an object file under csrc/build/ and
-linked into paper_2603_08088_b200/libtreeverify.so.  Objects are rebuilt when
-their source or a header is newer.
+linked into paper_2603_08088_b200/libtreeverify.so; csrc/calls.cpp (argument
+marshalling for Python) becomes paper_2603_08088_b200/_calls.so, which links to
+it.  Objects are rebuilt when their source or a header is newer.
 """
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -17,6 +19,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(PKG, "libtreeverify.so")
+CALLS = os.path.join(PKG, "_calls.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -30,6 +33,24 @@ def _nvcc():
     if not os.path.exists(exe):
         raise RuntimeError("nvcc not found; the treeverify library cannot be built")
     return exe
+
+
+def _calls_commands():
+    """Compile and link commands of _calls.so (torch's headers and libraries are those of the running Python)."""
+    import torch
+    root = os.path.dirname(torch.__file__)
+    lib, inc = os.path.join(root, "lib"), os.path.join(root, "include")
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    obj = os.path.join(OBJ, "calls.o")
+    abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
+    compile_cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={abi}",
+                   "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(cuda, "include"),
+                   "-isystem", sysconfig.get_paths()["include"]]
+    compile_cmd += ["-isystem", inc, "-isystem", os.path.join(inc, "torch", "csrc", "api", "include")]
+    compile_cmd += ["-c", os.path.join(CSRC, "calls.cpp"), "-o", obj]
+    link_cmd = ["g++", "-shared", "-o", CALLS, obj, "-L", PKG, "-l:libtreeverify.so", "-L", lib, "-ltorch_python", "-ltorch_cpu",
+                "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + lib]
+    return obj, compile_cmd, link_cmd
 
 
 def _newest_header():
@@ -62,13 +83,24 @@ def build(force=False, verbose=False):
         if r.returncode != 0 or verbose:
             sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
         if r.returncode != 0:
-            raise RuntimeError("nvcc failed for " + cmd[-3])
+            raise RuntimeError(cmd[0] + " failed for " + cmd[-3])
+
+    calls_src = os.path.join(CSRC, "calls.cpp")
+    calls_obj, calls_compile, calls_link = _calls_commands()
+    calls_stale = (force or not os.path.exists(calls_obj)
+                   or os.path.getmtime(calls_obj) < max(os.path.getmtime(calls_src),
+                                                        os.path.getmtime(os.path.join(ROOT, "include", "treeverify.h"))))
+    cu_jobs = len(jobs)
+    if calls_stale:
+        jobs.append(calls_compile)
 
     with ThreadPoolExecutor(max_workers=min(8, max(1, len(jobs)))) as ex:
         list(ex.map(run, jobs))
-    if jobs or not os.path.exists(LIB):
+    if cu_jobs or not os.path.exists(LIB):
         cmd = [nvcc, "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a", "-lcudart_static", "-ldl", "-lrt", "-lpthread"]
         run(cmd)
+    if calls_stale or not os.path.exists(CALLS):
+        run(calls_link)
     return LIB
 
 
