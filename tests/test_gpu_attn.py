@@ -552,3 +552,37 @@ def test_units_shared_by_a_cluster(B, Hkv, G, N, S, d):
     assert_attention_close(out, lse, ref_out, ref_lse, "cluster")
     out2, lse2, _, _ = gpu_attention(dcase)
     assert torch.equal(out, out2) and torch.equal(lse, lse2)
+
+
+@pytest.mark.parametrize("N", [65, 129])
+def test_last_row_tile_in_a_launch_of_its_own(N):
+    """Odd numbers of row tiles (three and five) on enough key tiles: two launches, equal to the one-launch calls of the
+    single layers up to the rounding of the partials and to the oracle on sampled heads."""
+    cfg = CONFIGS[0].scaled(B=10, L=4, Hq=32, Hkv=8, d=64, S_lo=20, S_hi=400, Scap=4096, N=N, D=6, V=0, tree="uniform")
+    case = make_case(cfg, seed=N, device="cuda", ragged_nodes=True, with_logits=False)
+    B, L, Hq, Hkv, d = cfg.B, cfg.L, cfg.Hq, cfg.Hkv, cfg.d
+    bits = torch.zeros(B, N, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    st = torch.zeros(B, dtype=torch.int32, device="cuda")
+    tv.tree_build_mask(case["parent"], case["n_nodes"], N - 1, 1, bits, st)
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(B, N, Hq, Hkv, d, cfg.Scap), dtype=torch.uint8, device="cuda")
+
+    def run(flags):
+        out = torch.full((L, B, N, Hq, d), 3.0, dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((L, B, Hq, N), 3.0, dtype=torch.float32, device="cuda")
+        n0 = tv.tv_launch_count()
+        tv.tree_verify_attn_layers(case["q"], case["k_cache"], case["v_cache"], case["k_tree"], case["v_tree"],
+                                   case["prefix_len"], case["n_nodes"], bits, d ** -0.5, out, ws, st, lse=lse, flags=flags)
+        torch.cuda.synchronize()
+        return out, lse, tv.tv_launch_count() - n0
+
+    out, lse, launches = run(0)
+    one, _, per_layer = run(tv.TV_ATTN_LAUNCH_PER_LAYER)
+    assert launches == 2 and per_layer == L and (st == 0).all()
+    assert (out.float() - one.float()).abs().max().item() <= 2.0 ** -5
+    cn = case_to_numpy(case)
+    vis = oracle_visibility(case["parent"], case["n_nodes"], bits_gpu=bits)[:, 0]
+    G = Hq // Hkv
+    for l, b, hk in ((0, 0, 0), (1, 4, 3), (3, 9, 7)):
+        ref_out, ref_lse = oracle_attention_slice(cn, l, b, hk, G, vis, d ** -0.5)
+        assert_attention_close(out[l][b:b + 1, :, hk * G:(hk + 1) * G], lse[l][b:b + 1, hk * G:(hk + 1) * G], ref_out, ref_lse,
+                               f"{l} {b} {hk}")
