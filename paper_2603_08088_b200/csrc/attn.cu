@@ -71,10 +71,11 @@ constexpr float kRescaleThreshold = 8.0f;            // in log2 units
 #define TV_POLY_SEL(i) ((((i) & 7) == 3) || (((i) & 15) == 7))
 #endif
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
-// virtual tiles charged per unit by the scheduler (32-layer shape, five seeds: 2 is 0.2-2 % faster than 4,
-// 0 and 1 are slower)
+// Virtual tiles charged per unit by the scheduler: what a CTA pays for one more item (epilogue, masked tiles, refill) is
+// some 5 us, three to four tiles' time.  Eight shapes, one and 32 layers a launch: 4 is 1 to 3 % faster than 2 and 1 to 2 %
+// faster than 1 and 5 on all but the ragged batch (1.8 % slower than 2); 3 is level with 4.
 #ifndef TV_SETUP_COST
-#define TV_SETUP_COST 2
+#define TV_SETUP_COST 4
 #endif
 constexpr int kSetupCost = TV_SETUP_COST;
 constexpr int kMaxGroups = 160;
@@ -425,13 +426,14 @@ struct SmemLayout {
   // barrier indices (8 bytes each)
   static constexpr int Q_FULL = 0, Q_EMPTY = 1, KV_FULL = 2, KV_EMPTY = 2 + kSlots, S_FULL = 2 + 2 * kSlots,
                        S_FREE = S_FULL + 2, P_READY = S_FREE + 2, O_DONE = P_READY + 2, ITEM_DONE = O_DONE + 1,
-                       EPI = ITEM_DONE + 2, NBARS = EPI + 1;
+                       EPI = ITEM_DONE + 2, ITEM_READ = EPI + 1, NBARS = ITEM_READ + 1;
   // Tensor memory columns.  One S buffer for two row tiles of 128-wide heads (there is no room for a second one
   // beside P0 P1 O0 O1), two buffers otherwise.
   static constexpr int kTmemS0 = 0, kTmemP0 = 128, kTmemO0 = 256;
   static constexpr int kTmemS1 = (D == 128 && MT == 2) ? kTmemS0 : 384;
   static constexpr int kMisc = kBars + NBARS * 8;          // tmem ptr, abort flag
-  static constexpr int kCum = kMisc + 16;
+  static constexpr int kItems = kMisc + 16;                // the producer's current and next item (see publish)
+  static constexpr int kCum = kItems + 2 * 32;
   static constexpr int kGs = kCum + (kMaxB + 1) * 4;
   static constexpr int kTotal = kGs + (kMaxGroups + 1) * 4;
   static constexpr int kMl = kCum;                         // cluster kernel: (m, l) of every row, in place of the tile table
@@ -451,6 +453,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t bars = sbase + L::kBars;
   auto bar = [&](int i) { return bars + 8u * i; };
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMisc + 4);
+  Item* items = reinterpret_cast<Item*>(smem + L::kItems);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + L::kMisc);
   int* cum = reinterpret_cast<int*>(smem + L::kCum);
   int* gs = reinterpret_cast<int*>(smem + L::kGs);
@@ -480,6 +483,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     mbar_init(bar(L::O_DONE), 1);
     mbar_init(bar(L::EPI), MT * 128);
+    mbar_init(bar(L::ITEM_READ), MT * 4);
     *abort_flag = ((sbase & 1023u) != 0) ? 1 : 0;   // swizzled tiles need a 1024-byte aligned base
     fence_barrier_init();
   }
@@ -551,7 +555,10 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const int g_begin = CL ? 0 : sch.group_start(group, groups);
   const int g_end = CL ? 1 : sch.group_start(group + 1, groups);
 
-  // Walks the items of this CTA's range; identical in every role.
+  // Walks the items of this CTA's range (producer warp).  It publishes every item to the other roles through shared
+  // memory, in front of the arrival on Q_FULL that they wait for; entries are used in turn, and an item is published only
+  // when the softmax warps have read the one before (a parity wait cannot tell phases two apart).  (Walking in every role cost each of them a division, a search and two L2 round trips per item: about
+  // 1.5 us between the epilogue of an item and its successor's first tile.)
   auto next_item = [&](int& g, Item& it) -> bool {
     if (CL) {                      // one item: this CTA's share of the key tiles of its cluster's unit (may be empty)
       if (g > 0) return false;
@@ -632,8 +639,14 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         __syncwarp();
         synced = true;
       };
+      auto publish = [&](const Item& x) {
+        if (item_idx > 0 && !(prm.debug & 4)) ok = mbar_wait(bar(L::ITEM_READ), (item_idx - 1) & 1, abort_flag, wait_limit);
+        if (ok && elect_one()) items[(item_idx & 1)] = x;
+        __syncwarp();
+      };
       auto load_q = [&]() {
-        if (elect_one()) {
+        publish(it);
+        if (ok && elect_one()) {
           mbar_expect_tx(bar(L::Q_FULL), MT * (D / 64) * prm.q_box_bytes);
 #pragma unroll
           for (int t = 0; t < MT; ++t)
@@ -651,7 +664,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         tr.mark(0x1000u | item_idx);
         bool q_pending = !synced;          // first item: Q goes out after the first prefix tiles
         if (!q_pending) load_q();
-        ++item_idx;
+        if (!ok) break;
         // paged cache: the page of a prefix key tile comes from the block table, fetched one tile ahead of its use
         auto page_of = [&](int jj) -> int {
           if (!prm.block_table || jj >= it.len - prm.TT || jj >= it.j1) return 0;
@@ -706,6 +719,12 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           sync_with_predecessor();
           load_q();
         }
+        ++item_idx;
+      }
+      if (ok) ok = mbar_wait(bar(L::Q_EMPTY), (item_idx & 1) ^ 1, abort_flag, wait_limit);
+      if (ok) {                            // no more items
+        publish(Item{});
+        if (ok && elect_one()) mbar_arrive(bar(L::Q_FULL));
       }
       if (!synced) sync_with_predecessor();        // a CTA without work still has to let the next kernel go
     } else {
@@ -730,8 +749,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     //   one row tile (buffers alternate by key tile):  S(j+1), O += P(j) V(j).
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (!*abort_flag) {      // the whole warp walks the items; one elected lane issues
-      int g = g_begin;
-      Item it;
       uint32_t item_idx = 0, fill = 0, tj = 0;
       bool ok = true;
       Tracer tr;
@@ -770,10 +787,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         __syncwarp();
       };
-      while (ok && next_item(g, it)) {
-        const int nt = it.j1 - it.j0;
+      while (true) {
         ok = mbar_wait(bar(L::Q_FULL), item_idx & 1, abort_flag, wait_limit);
         if (!ok) break;
+        const int nt = items[item_idx & 1].j1 - items[item_idx & 1].j0;
+        if (nt == 0) break;
         tr.mark(0x1000u | item_idx);
         if (prm.debug & 4) {       // stream only: every tile of the item is released as soon as it has landed
 #pragma unroll 1
@@ -905,8 +923,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
     float m_fin = -INFINITY, l_fin = 0.f;            // cluster kernel: (m, l) of the row; no key tile: weight 0
     if (wg_active && !*abort_flag && !(prm.debug & 4)) {
-      int g = g_begin;
-      Item it;
       uint32_t fill = 0, tj = 0, epi_phase = 0, item_cnt = 0;   // tj: key tiles handled so far (all items)
       uint32_t od_phase = 0;                                    // items of more than one key tile so far
       bool ok = true;
@@ -925,8 +941,14 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         ++epi_phase;
         return r;
       };
-      while (ok && next_item(g, it)) {
+      while (true) {
+        ok = wwait(bar(L::Q_FULL), item_cnt & 1);
+        if (!ok) break;
+        const Item it = items[item_cnt & 1];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(L::ITEM_READ));
         const int nt = it.j1 - it.j0;
+        if (nt == 0) break;
         const int node = (prm.tile0 + pair * MT + wg) * prm.NPT + row / prm.G;
         const int gm = row % prm.G;
         const bool row_exists = row < prm.NPT * prm.G && node < prm.Nmax;
@@ -934,6 +956,12 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // One row tile: a warp without an active row takes part in the barriers only.  (With two row tiles the test costs
         // the loop more than it saves: 32-layer shape 1296 -> 1314 us.)
         const bool warp_active = MT == 2 || __any_sync(0xffffffffu, row_active);
+        // the row's ancestor words are wanted on the last tile(s): fetched into L1 now, not a round trip in front of that tile
+        if (row_active) {
+          const uint32_t* words = prm.anc_bits + ((size_t)it.b * prm.Nmax + node) * prm.W;
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(words));
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(words + prm.W - 1));
+        }
         float m_used = -INFINITY;      // running reference maximum, in log2 units (score * scale * log2e)
         float l_sum = 0.f;
         const uint32_t o_addr_loop = tmem + lane_addr + L::kTmemO0 + wg * D;
@@ -1184,7 +1212,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // bf16-rounded normalised output, the merger's own included, in piece order with one fused multiply-add
             // per piece.  What bounds this is dependent round trips to L2 (some 2 K cycles each under load): a fixed
             // merger needs no ticket, its pieces are usually ready long before, and a piece's whole row is requested at
-            // once, the first one's beside its (m, l).  The sum stays in tensor memory between two pieces.
+            // once, the first one's beside its (m, l), a later one's as the row before it is used up.  The sum stays in
+            // tensor memory between two pieces.
             // Partial outputs are stored column-group major, [slot][D/8][MT*128 rows][8 bf16]: a warp writes
             // and reads 512 contiguous bytes per instruction.
             constexpr int kRows = MT * 128;
@@ -1270,9 +1299,10 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               const float inv = any_key ? 1.f / lt : 0.f;
 #pragma unroll 1
               for (int i = 1; i <= n_other; ++i) {
-                if (i > 1) {
-                  fetch(i);
-                  w = weight(i);
+                float m_next = 0.f, l_next = 0.f;
+                if (i < n_other) {
+                  m_next = __ldcg(ml_of(i + 1));
+                  l_next = __ldcg(ml_of(i + 1) + kRows);
                 }
                 const float2 w2 = make_float2(w, w), own2 = make_float2(w_own, w_own), inv_own2 = make_float2(inv_own, inv_own);
                 const float2 inv2 = make_float2(inv, inv);
@@ -1297,6 +1327,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                   }
                   if (i < n_other) {
                     tmem_st32(o_addr + q * 32, o);
+                    const uint4* q_o = o_of(i + 1);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) v[q * 4 + c] = __ldcg(q_o + (size_t)(q * 4 + c) * kRows);
                   } else if (row_exists) {
                     uint4 r[4];
 #pragma unroll
@@ -1319,6 +1352,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                   }
                 }
                 tmem_wait_st();
+                w = l_next * fast_exp2(m_next - mref);
               }
               if (row_exists && lse_p) *lse_p = any_key ? (mm + log2f(lt)) / kLog2e : -INFINITY;
               tc_fence_before();
