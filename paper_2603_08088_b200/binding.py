@@ -299,19 +299,4 @@ def kv_commit_inplace(k_cache, v_cache, accepted_nodes, accept_len, prefix_len, 
 def tv_verify_step_host(host, k_cache, v_cache, prefix_len, staging, scale, V, stream=None):
     """``host``: dict of pinned CPU tensors parent, n_nodes, tokens, retrieve_indices (or None), q, k_tree,
     v_tree, logits and outputs out, accept_len, accepted_nodes, next_token, status."""
-    L, B, Nmax, Hq, d = host["q"].shape
-    Hkv, Scap = k_cache.shape[2], k_cache.shape[3]
-    Dp1 = host["accepted_nodes"].shape[1]
-    r = host.get("retrieve_indices")
-    P = r.shape[1] if r is not None else host["P"]
-    a = StepHostArgs()
-    for name in ("parent", "n_nodes", "tokens", "q", "k_tree", "v_tree", "logits", "out", "accept_len",
-                 "accepted_nodes", "next_token", "status"):
-        setattr(a, name, _ptr(host[name]))
-    a.retrieve_indices = _ptr(r)
-    a.k_cache, a.v_cache, a.prefix_len = _ptr(k_cache), _ptr(v_cache), _ptr(prefix_len)
-    a.staging, a.staging_bytes = _ptr(staging), staging.numel() * staging.element_size()
-    a.L, a.B, a.Nmax, a.Hq, a.Hkv, a.d, a.Scap, a.V, a.P, a.Dp1 = L, B, Nmax, Hq, Hkv, d, Scap, V, P, Dp1
-    a.scale = float(scale)
-    a.stream = _stream(stream)
-    _check(load().tv_verify_step_host(ctypes.byref(a)))
+    _check((_calls or _native()).tv_verify_step_host(host, k_cache, v_cache, prefix_len, staging, scale, V, stream))

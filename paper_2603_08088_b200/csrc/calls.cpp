@@ -326,6 +326,56 @@ PyObject* commit_inplace(PyObject* const* a, Py_ssize_t n) {
   return call([&] { return kv_commit_inplace(pk, pv, nodes, al, S, L, B, N, Hkv, d, Scap, Dp1, cl, st, s); });
 }
 
+// host (dict of pinned tensors), k_cache, v_cache, prefix_len, staging, scale, V, stream
+PyObject* step_host(PyObject* const* a, Py_ssize_t n) {
+  Args x(a, n, 8);
+  if (!PyDict_Check(a[0])) raise(PyExc_TypeError, "treeverify: the host buffers are a dict of tensors");
+  static const char* const names[] = {"parent", "n_nodes", "tokens", "retrieve_indices", "q", "k_tree", "v_tree", "logits", "out",
+                                      "accept_len", "accepted_nodes", "next_token", "status", "P"};
+  PyObject* h[14];
+  for (int i = 0; i < 14; ++i) {
+    h[i] = PyDict_GetItemString(a[0], names[i]);
+    if (!h[i]) {
+      if (i != 3 && i != 13) raise(PyExc_KeyError, names[i]);
+      h[i] = Py_None;
+    }
+  }
+  Args y(h, 14, 14);
+  const at::Tensor &q = y.tensor(4, 5), &kc = x.tensor(1, 5), &acc = y.tensor(10, 2);
+  tv_step_host_args s{};
+  s.parent = y.ptr<int32_t>(0);
+  s.n_nodes = y.ptr<int32_t>(1);
+  s.tokens = y.ptr<int32_t>(2);
+  s.retrieve_indices = y.ptr<int32_t>(3);
+  s.q = y.ptr<tv_bf16>(4);
+  s.k_tree = y.ptr<tv_bf16>(5);
+  s.v_tree = y.ptr<tv_bf16>(6);
+  s.logits = y.ptr<tv_bf16>(7);
+  s.out = y.ptr<tv_bf16>(8);
+  s.accept_len = y.ptr<int32_t>(9);
+  s.accepted_nodes = y.ptr<int32_t>(10);
+  s.next_token = y.ptr<int32_t>(11);
+  s.status = y.ptr<int32_t>(12);
+  s.k_cache = x.ptr<tv_bf16>(1);
+  s.v_cache = x.ptr<tv_bf16>(2);
+  s.prefix_len = x.ptr<int32_t>(3);
+  s.staging = x.ptr(4);
+  s.staging_bytes = x.bytes(4);
+  s.L = q.size(0);
+  s.B = q.size(1);
+  s.Nmax = q.size(2);
+  s.Hq = q.size(3);
+  s.d = q.size(4);
+  s.Hkv = kc.size(2);
+  s.Scap = kc.size(3);
+  s.V = x.integer(6);
+  s.P = y.none(3) ? y.integer(13) : (int)y.tensor(3, 3).size(1);
+  s.Dp1 = acc.size(1);
+  s.scale = x.number(5);
+  s.stream = x.stream(7);
+  return call([&] { return tv_verify_step_host(&s); });
+}
+
 #define TV_METHOD(name, body) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&guarded<body>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
     TV_METHOD("tree_build_mask", build_mask),
@@ -339,6 +389,7 @@ PyMethodDef methods[] = {
     TV_METHOD("kv_commit", commit),
     TV_METHOD("kv_commit_paged", commit_paged),
     TV_METHOD("kv_commit_inplace", commit_inplace),
+    TV_METHOD("tv_verify_step_host", step_host),
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

@@ -119,3 +119,45 @@ def test_host_buffer_step_matches_device_step():
     assert np.array_equal(host["status"].numpy(), ref["status"])
     assert np.array_equal(bf16_bits(kc), ref["k_cache"]) and np.array_equal(bf16_bits(vc), ref["v_cache"])
     assert np.array_equal(i32(S), ref["prefix_len"])
+
+
+def _host_step(cfg, seed, given_rows, stream=None):
+    case = make_case(cfg, seed=seed)
+    ref = orc.verify_step(case_to_numpy(case), cfg.d ** -0.5, use_given_retrieve=given_rows)
+    P, Dp1 = case["retrieve"].shape[1], cfg.D + 1
+    pin = lambda t: t.contiguous().pin_memory()
+    host = {k: pin(case[k]) for k in ("parent", "n_nodes", "tokens", "q", "k_tree", "v_tree", "logits")}
+    host["retrieve_indices"], host["P"] = (pin(case["retrieve"]) if given_rows else None), P
+    host["out"] = torch.zeros(cfg.L, cfg.B, cfg.N, cfg.Hq, cfg.d, dtype=torch.bfloat16).pin_memory()
+    for k, shape in (("accept_len", (cfg.B,)), ("accepted_nodes", (cfg.B, Dp1)), ("next_token", (cfg.B,)), ("status", (cfg.B,))):
+        host[k] = torch.full(shape, -5, dtype=torch.int32).pin_memory()
+    kc, vc, S = case["k_cache"].cuda(), case["v_cache"].cuda(), case["prefix_len"].cuda()
+    staging = torch.zeros(tv.tv_step_staging_bytes(cfg.L, cfg.B, cfg.N, cfg.Hq, cfg.Hkv, cfg.d, cfg.Scap, cfg.V, P, Dp1),
+                          dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    tv.tv_verify_step_host(host, kc, vc, S, staging, cfg.d ** -0.5, cfg.V, stream=stream)
+    assert np.abs(host["out"].float().numpy() - ref["out"]).max() <= ATTN_ATOL
+    for k in ("accept_len", "accepted_nodes", "next_token"):
+        assert np.array_equal(host[k].numpy(), ref["accept"][k]), k
+    assert np.array_equal(bf16_bits(kc), ref["k_cache"]) and np.array_equal(bf16_bits(vc), ref["v_cache"])
+    assert np.array_equal(i32(S), ref["prefix_len"])
+
+
+HOST_STEPS = [
+    dict(B=4, L=5, Hq=16, Hkv=4, S_lo=50, S_hi=200, Scap=256, V=1003),              # stages of 2, 2 and 1 layers
+    dict(B=40, L=1, Hq=2, Hkv=1, d=64, S_lo=5, S_hi=60, Scap=80, V=512, P=60),      # small arrays above 64 KB
+]
+
+
+@pytest.mark.parametrize("over", HOST_STEPS, ids=["stages", "large_rows"])
+@pytest.mark.parametrize("given_rows", [True, False])
+def test_host_buffer_step_stages_and_blocks(over, given_rows):
+    _host_step(CONFIGS[4].scaled(**over), 77, given_rows)
+
+
+def test_host_buffer_steps_from_several_threads():
+    from concurrent.futures import ThreadPoolExecutor
+    cfg = CONFIGS[4].scaled(B=2, L=2, Hq=4, Hkv=2, d=64, S_lo=20, S_hi=90, Scap=128, V=777)
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    with ThreadPoolExecutor(4) as ex:
+        list(ex.map(lambda i: _host_step(cfg, 500 + i, i % 2 == 0, streams[i % 4]), range(12)))
