@@ -2,7 +2,9 @@
 // context-split group), from the per-range outputs and log-sum-exps (Section 6, "Limitations and future
 // work": longer-context, multi-device serving; the attention is Section 2.4).  For every query row
 //   out = sum_r w_r O_r / sum_r w_r,  w_r = exp(lse_r - max_r lse_r),  lse = max + log sum_r w_r.
-// Pure streaming: R reads of the partials, one write; one thread per (row, 8 output columns).
+// Pure streaming: R reads of the partials, one write; one thread per (row, 8 output columns), four ranges' weights and
+// payloads requested together.  Eight ranges of 4 x 128 nodes x 32 heads (38 MB, 5.8 us at the copy rate): 11.0 -> 8.4 us,
+// two ranges 5.9 -> 4.8; with eight ranges in flight 9.2 and 6.5 (fewer threads fit an SM).
 #include "common.cuh"
 
 #include <cuda_bf16.h>
@@ -17,50 +19,59 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return r;
 }
 
-__global__ void merge_partials_kernel(const uint4* __restrict__ o_parts, const float* __restrict__ lse_parts, int R,
-                                      int B, int Nmax, int Hq, int d8, uint4* __restrict__ out,
-                                      float* __restrict__ lse_out) {
-  const long long total = (long long)B * Nmax * Hq * d8;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+constexpr int kThreads = 128;
+constexpr int kHold = 4;          // ranges whose loads are in flight together
+
+// Index: 32 bits wherever the number of threads fits (five 64-bit divisions per thread took longer than its loads).
+template <typename Index>
+__global__ void __launch_bounds__(kThreads)
+merge_partials_kernel(const uint4* __restrict__ o_parts, const float* __restrict__ lse_parts, int R,
+                      int B, int Nmax, int Hq, int d8, uint4* __restrict__ out, float* __restrict__ lse_out) {
+  tv::pdl_enter();
+  const Index total = (Index)B * Nmax * Hq * d8;
+  const Index t = (Index)blockIdx.x * kThreads + threadIdx.x;
   if (t >= total) return;
-  const int cg = (int)(t % d8);
-  const long long row = t / d8;                       // (b * Nmax + node) * Hq + h
-  const int h = (int)(row % Hq);
-  const long long bn = row / Hq;
-  const int node = (int)(bn % Nmax);
-  const int b = (int)(bn / Nmax);
+  const Index row = t / (Index)d8;                    // (b * Nmax + node) * Hq + h
+  const int cg = (int)(t - row * (Index)d8);
+  const Index bn = row / (Index)Hq;
+  const int h = (int)(row - bn * (Index)Hq);
+  const int b = (int)(bn / (Index)Nmax);
+  const int node = (int)(bn - (Index)b * (Index)Nmax);
   const long long rows = (long long)B * Nmax * Hq;
   const long long lse_idx = ((long long)b * Hq + h) * Nmax + node;
-  float m = -INFINITY;
-#pragma unroll 4
-  for (int r = 0; r < R; ++r) m = fmaxf(m, __ldg(lse_parts + (long long)r * rows + lse_idx));
+  const float* lp = lse_parts + lse_idx;
+  const uint4* op = o_parts + t;
+  float m = -INFINITY;                                 // running maximum: more than kHold ranges rescale what they find
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   float tot = 0.f;
-  if (m > -INFINITY) {
-    // four ranges at a time: all loads of a group are in flight together; the payload of an empty range
-    // (weight 0) may be anything, so it is replaced by zeros rather than multiplied
-    for (int r0 = 0; r0 < R; r0 += 4) {
-      float w[4];
-      uint4 v[4];
+  for (int r0 = 0; r0 < R; r0 += kHold) {
+    float w[kHold];
+    uint4 v[kHold];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int r = r0 + k < R ? r0 + k : R - 1;
-        w[k] = __ldg(lse_parts + (long long)r * rows + lse_idx);
-        v[k] = __ldg(o_parts + ((long long)r * rows + row) * d8 + cg);
-      }
+    for (int k = 0; k < kHold; ++k) w[k] = r0 + k < R ? __ldcs(lp + (r0 + k) * rows) : -INFINITY;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float wk = (r0 + k < R) ? expf(w[k] - m) : 0.f;
-        if (!(wk > 0.f)) v[k] = make_uint4(0u, 0u, 0u, 0u);
+    for (int k = 0; k < kHold; ++k)
+      if (r0 + k < R) v[k] = __ldcs(op + (r0 + k) * rows * d8);
+    float mx = m;
+#pragma unroll
+    for (int k = 0; k < kHold; ++k) mx = fmaxf(mx, w[k]);
+    if (mx == -INFINITY) continue;
+    const float keep = expf(m - mx);                   // 0 the first time
+    m = mx;
+    tot *= keep;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] *= keep;
+#pragma unroll
+    for (int k = 0; k < kHold; ++k) {
+      const float wk = expf(w[k] - mx);
+      if (wk > 0.f) {                                  // the payload of an empty range (weight 0) may be anything
         tot += wk;
-        acc[0] = fmaf(wk, bf16_lo(v[k].x), acc[0]);
-        acc[1] = fmaf(wk, bf16_hi(v[k].x), acc[1]);
-        acc[2] = fmaf(wk, bf16_lo(v[k].y), acc[2]);
-        acc[3] = fmaf(wk, bf16_hi(v[k].y), acc[3]);
-        acc[4] = fmaf(wk, bf16_lo(v[k].z), acc[4]);
-        acc[5] = fmaf(wk, bf16_hi(v[k].z), acc[5]);
-        acc[6] = fmaf(wk, bf16_lo(v[k].w), acc[6]);
-        acc[7] = fmaf(wk, bf16_hi(v[k].w), acc[7]);
+        const uint32_t e[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          acc[2 * i] = fmaf(wk, bf16_lo(e[i]), acc[2 * i]);
+          acc[2 * i + 1] = fmaf(wk, bf16_hi(e[i]), acc[2 * i + 1]);
+        }
       }
     }
   }
@@ -70,7 +81,7 @@ __global__ void merge_partials_kernel(const uint4* __restrict__ o_parts, const f
   o.y = pack_bf16(acc[2] * inv, acc[3] * inv);
   o.z = pack_bf16(acc[4] * inv, acc[5] * inv);
   o.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-  out[row * d8 + cg] = o;
+  out[t] = o;
   if (lse_out && cg == 0) lse_out[lse_idx] = tot > 0.f ? m + logf(tot) : -INFINITY;
 }
 
@@ -84,10 +95,13 @@ extern "C" int tree_merge_partials(const tv_bf16* o_parts, const float* lse_part
   TV_REQUIRE(tv::aligned16(o_parts) && tv::aligned16(out), "tree_merge_partials: tensors must be 16-byte aligned");
   if (B == 0) return TV_OK;
   const long long total = (long long)B * Nmax * Hq * (d / 8);
-  TV_REQUIRE((total + 255) / 256 < (1ll << 31), "tree_merge_partials: problem too large for one launch");
-  merge_partials_kernel<<<(unsigned)((total + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
-      reinterpret_cast<const uint4*>(o_parts), lse_parts, R, B, Nmax, Hq, d / 8, reinterpret_cast<uint4*>(out), lse);
-  TV_CUDA_OK(cudaGetLastError());
+  TV_REQUIRE((total + kThreads - 1) / kThreads < (1ll << 31), "tree_merge_partials: problem too large for one launch");
+  const auto launch = [&](auto kernel) {
+    return tv::launch_pdl(kernel, dim3((unsigned)((total + kThreads - 1) / kThreads)), dim3(kThreads), 0, (cudaStream_t)stream,
+                          reinterpret_cast<const uint4*>(o_parts), lse_parts, R, B, Nmax, Hq, d / 8,
+                          reinterpret_cast<uint4*>(out), lse);
+  };
+  TV_CUDA_OK(total < (1ll << 31) ? launch(merge_partials_kernel<unsigned>) : launch(merge_partials_kernel<long long>));
   tv::count_launches(1);
   return TV_OK;
 }

@@ -113,3 +113,23 @@ def test_context_split_attention_single_process_is_plain_attention():
                         case["prefix_len"], case["n_nodes"], bits, d ** -0.5, ref, ws, status)
     torch.cuda.synchronize()
     assert torch.equal(out.view(torch.int16), ref.view(torch.int16))      # one part, weight 1: unchanged
+
+
+@pytest.mark.parametrize("R", [1, 3, 4, 5, 8, 11])
+def test_merge_counts_around_the_ranges_in_flight(R):
+    """Maxima that grow from range to range (what was summed is rescaled), an empty range first and last."""
+    g = torch.Generator().manual_seed(R)
+    B, N, Hq, d = 2, 7, 3, 64
+    o = torch.randn(R, B, N, Hq, d, generator=g).to(torch.bfloat16)
+    lse = torch.randn(R, B, Hq, N, generator=g) * 3 + torch.arange(R).view(R, 1, 1, 1) * 9.0
+    if R > 2:
+        lse[0], lse[-1] = float("-inf"), float("-inf")
+        o[0], o[-1] = float("nan"), float("nan")
+    out = torch.empty(B, N, Hq, d, dtype=torch.bfloat16, device="cuda")
+    lout = torch.empty(B, Hq, N, device="cuda")
+    tv.tree_merge_partials(o.cuda(), lse.cuda(), out, lout)
+    w = torch.softmax(lse.double(), 0).permute(0, 1, 3, 2)[..., None]
+    want = (w * torch.nan_to_num(o.double())).sum(0)
+    # one bf16 rounding of the result (2^-9 of it) and fp32 sums (2^-20 of the largest term)
+    assert ((out.double().cpu() - want).abs() <= 2.0 ** -8 * want.abs() + 1e-4).all()
+    assert (lout.double().cpu() - torch.logsumexp(lse.double(), 0)).abs().max() <= 1e-4
