@@ -8,19 +8,24 @@
 //
 // Pipeline (one CTA per SM, 12 warps):
 //   warp 0      TMA producer: Q tiles once per work item, then K and V tiles
-//               through a 5-slot shared-memory ring (128-byte swizzled boxes).
+//               through a shared-memory ring of 5 or 10 slots (128-byte swizzled
+//               boxes).
 //   warp 1      tcgen05.mma issuer (one thread): S = Q K^T for a whole 128-key
 //               tile (N = 128; 64-key MMAs re-read Q from shared memory twice as
 //               often and run at 2/3 of the rate), O += P V with P read from
 //               TMEM; completion goes to mbarriers with tcgen05.commit.  With
 //               two row tiles it serves them in turn, so the softmax of one row
 //               tile runs while the tensor pipe works for the other.
-//   warps 4-7   softmax warpgroup for row tile 0: one thread per row, online
-//   warps 8-11  softmax with lazy rescale; tile 1 likewise.  The ancestor
+//   warps 4-7   two softmax warpgroups, one thread per row, online softmax with
+//   warps 8-11  lazy rescale, one for each row tile.  With one row tile and
+//               64-wide heads (KS) one takes the even and one the odd key tiles of
+//               an item, each with an O of its own (combined in the epilogue);
+//               with 128-wide heads, whose K/V stream sets the pace, the second
+//               one idles.  The ancestor
 //               bitmask of the row is applied only on the tree tile(s), the
 //               prefix length only on the ragged last prefix tile.
 // TMEM: S0 (128 columns) | P0 P1 (bf16, 64 columns each) | O0 O1 (D columns each),
-// and S1 where O1 leaves room for it (see SmemLayout).  With one row tile the S and
+// and S1 where O1 leaves room for it (see SmemLayout).  With one warpgroup the S and
 // P buffers alternate by key tile.
 //
 // Code size matters here: instruction fetches compete with the K/V stream for
@@ -59,7 +64,6 @@ namespace {
 
 constexpr int kTileN = 128;        // keys per tile
 constexpr int kTileM = 128;        // rows per row tile
-constexpr int kSlots = 5;          // K/V ring slots
 constexpr int kThreads = 384;
 constexpr int kMaxB = 512;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -420,6 +424,7 @@ template <int D, int MT>
 struct SmemLayout {
   static constexpr int kHalf = 64 * 128 * 2;               // one 64-column, 128-row swizzled box: 16 KB
   static constexpr int kTileBytes = (D / 64) * kHalf;      // a 128 x D bf16 tile
+  static constexpr int kSlots = D == 64 ? 10 : 5;             // K/V ring slots
   static constexpr int kQ = 0;
   static constexpr int kRing = MT * kTileBytes;
   static constexpr int kBars = kRing + kSlots * kTileBytes;
@@ -435,7 +440,10 @@ struct SmemLayout {
   static constexpr int kItems = kMisc + 16;                // the producer's current and next item (see publish)
   static constexpr int kCum = kItems + 2 * 32;
   static constexpr int kGs = kCum + (kMaxB + 1) * 4;
-  static constexpr int kTotal = kGs + (kMaxGroups + 1) * 4;
+  static constexpr int kXch = (kGs + (kMaxGroups + 1) * 4 + 7) & ~7;      // KS: (m, l) of both warpgroups' rows
+  static constexpr bool kKeySplit = MT == 1 && D == 64;
+  static constexpr int kTotal = kKeySplit ? kXch + 256 * 8 : kGs + (kMaxGroups + 1) * 4;
+  static_assert(kTotal <= 232448, "shared memory of a CTA");
   static constexpr int kMl = kCum;                         // cluster kernel: (m, l) of every row, in place of the tile table
   static_assert(kMl + MT * 128 * 8 <= kTotal && kMl % 8 == 0, "(m, l) pairs fit the room of the tile table");
 };
@@ -447,6 +455,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                  const __grid_constant__ CUtensorMap map_vc, const __grid_constant__ CUtensorMap map_kt,
                  const __grid_constant__ CUtensorMap map_vt, const AttnParams prm) {
   using L = SmemLayout<D, MT>;
+  // One row tile.  KS: the two softmax warpgroups share the keys of an item, tile by tile.  A 64-wide head's key tile is
+  // 32 KB, 0.7 us of the HBM rate, and one warpgroup needs 1 us for it (16 sequences of 8000, G = 4, 24 nodes: 72.7 ->
+  // 59.5 us a launch).  ONE: a 128-wide head's tile takes 1.5 us to arrive; there the second tile in hand only takes ring
+  // slots away from the stream (16 sequences of 1000, 17 nodes: 22.5 -> 25.7 us), and one warpgroup does it all.
+  constexpr bool KS = L::kKeySplit, ONE = MT == 1 && !KS;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -471,19 +484,19 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     mbar_init(bar(L::Q_FULL), 1);
     mbar_init(bar(L::Q_EMPTY), 1);
 #pragma unroll 1
-    for (int s = 0; s < kSlots; ++s) {
+    for (int s = 0; s < L::kSlots; ++s) {
       mbar_init(bar(L::KV_FULL + s), 1);
       mbar_init(bar(L::KV_EMPTY + s), 1);
     }
-    for (int s = 0; s < 2; ++s) {                // index = row tile, or parity of the key tile with one row tile
+    for (int s = 0; s < 2; ++s) {                // index = softmax warpgroup, or parity of the key tile with one warpgroup
       mbar_init(bar(L::S_FULL + s), 1);
       mbar_init(bar(L::S_FREE + s), 4);
       mbar_init(bar(L::P_READY + s), 4);
       mbar_init(bar(L::ITEM_DONE + s), 1);
     }
     mbar_init(bar(L::O_DONE), 1);
-    mbar_init(bar(L::EPI), MT * 128);
-    mbar_init(bar(L::ITEM_READ), MT * 4);
+    mbar_init(bar(L::EPI), ONE ? 128 : 256);
+    mbar_init(bar(L::ITEM_READ), ONE ? 4 : 8);
     *abort_flag = ((sbase & 1023u) != 0) ? 1 : 0;   // swizzled tiles need a 1024-byte aligned base
     fence_barrier_init();
   }
@@ -686,8 +699,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const int slab = (prm.block_table ? page : it.b) * prm.Hkv + it.hk;               // (page or sequence, KV head)
 #pragma unroll
           for (int kv = 0; kv < 2; ++kv) {
-            const uint32_t slot = fill % kSlots, round = fill / kSlots;
-            if (q_pending && (tree || fill >= (uint32_t)kSlots)) {      // before the first wait for a ring slot
+            const uint32_t slot = fill % L::kSlots, round = fill / L::kSlots;
+            if (q_pending && (tree || fill >= (uint32_t)L::kSlots)) {      // before the first wait for a ring slot
               sync_with_predecessor();
               load_q();
               q_pending = false;
@@ -746,10 +759,12 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // (32-layer shape: 1342 -> 1312 us a launch, power-capped 1583 -> 1540 us, against P overlaying its S).
     //   two row tiles:  S_0(j+1), O_0 += P_0(j) V(j), S_1(j+1), O_1 += P_1(j) V(j): each S as soon as the other row
     //     tile's S has been taken out of the buffer, each PV as soon as its P is there;
-    //   one row tile (buffers alternate by key tile):  S(j+1), O += P(j) V(j).
+    //   KS:  S(j+2), O_w += P(j) V(j), w = j mod 2 the warpgroup of key tile j;
+    //   one warpgroup (buffers alternate by key tile):  S(j+1), O += P(j) V(j).
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (!*abort_flag) {      // the whole warp walks the items; one elected lane issues
       uint32_t item_idx = 0, fill = 0, tj = 0;
+      uint32_t done[2] = {0, 0};             // KS: key tiles of each warpgroup in earlier items
       bool ok = true;
       Tracer tr;
       tr.init(lane == 0 ? prm.trace : nullptr, 1);
@@ -783,7 +798,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int ks = 0; ks < 8; ++ks)            // 16 keys = 16 rows of 128 bytes = 8 packed P columns
             mma_ts_lohi(tmem + L::kTmemO0 + t * D, tmem + L::kTmemP0 + idx * 64 + ks * 8, va + ks * 128, desc_hi, kIdescPV,
                         (!first_tile || ks > 0) ? 1u : 0u);
-          if (MT == 1) mma_commit(bar(L::O_DONE));
+          if (ONE) mma_commit(bar(L::O_DONE));
         }
         __syncwarp();
       };
@@ -797,8 +812,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll 1
           for (int f = 0; f < 2 * nt && ok; ++f) {
             const uint32_t ff = fill + f;
-            ok = mbar_wait(bar(L::KV_FULL + ff % kSlots), (ff / kSlots) & 1, abort_flag, wait_limit);
-            if (ok && elect_one()) mbar_arrive(bar(L::KV_EMPTY + ff % kSlots));
+            ok = mbar_wait(bar(L::KV_FULL + ff % L::kSlots), (ff / L::kSlots) & 1, abort_flag, wait_limit);
+            if (ok && elect_one()) mbar_arrive(bar(L::KV_EMPTY + ff % L::kSlots));
             __syncwarp();
           }
           if (elect_one()) mbar_arrive(bar(L::Q_EMPTY));
@@ -807,35 +822,97 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ++item_idx;
           continue;
         }
+        if (KS) {
+          auto phase = [&](int i) -> uint32_t { return (done[i & 1] + (i >> 1)) & 1u; };      // of key tile i's barriers
+          auto next_s = [&](int i) {       // S of key tile i, i < nt; its buffer was last filled for tile i - 1 (or i - 2)
+            const uint32_t f = fill + 2 * i, slot = f % L::kSlots;
+            ok = mbar_wait(bar(L::KV_FULL + slot), (f / L::kSlots) & 1, abort_flag, wait_limit);
+            const int before = L::kTmemS1 == L::kTmemS0 ? i - 1 : i - 2;
+            if (ok && before >= 0) ok = mbar_wait(bar(L::S_FREE + (before & 1)), phase(before), abort_flag, wait_limit);
+            if (!ok) return;
+            tc_fence_after();
+            issue_qk(0, i & 1, slot);
+            if (elect_one()) {
+              mma_commit(bar(L::KV_EMPTY + slot));
+              if (i + 1 == nt) mma_commit(bar(L::Q_EMPTY));
+            }
+            __syncwarp();
+          };
+          // The S buffers are free: the P of every earlier key tile has been waited for, hence its S was taken.
+          next_s(0);
+          if (ok && nt > 1) next_s(1);
+#pragma unroll 1
+          for (int i = 0; i < nt && ok; ++i) {
+            if (i + 2 < nt) next_s(i + 2);
+            const uint32_t f = fill + 2 * i + 1, slot = f % L::kSlots;
+            if (ok) ok = mbar_wait(bar(L::P_READY + (i & 1)), phase(i), abort_flag, wait_limit);
+            if (ok) ok = mbar_wait(bar(L::KV_FULL + slot), (f / L::kSlots) & 1, abort_flag, wait_limit);
+            if (!ok) break;
+            tc_fence_after();
+            tr.mark(0x4000u | (i & 0xfffu));
+            issue_pv(i & 1, i & 1, slot, i < 2);
+            if (elect_one()) {
+              if (i + 3 == nt) mma_commit(bar(L::O_DONE));      // no S follows the PV behind the last key tile's predecessor
+              if (i + 1 == nt) mma_commit(bar(L::ITEM_DONE));
+              mma_commit(bar(L::KV_EMPTY + slot));
+            }
+            __syncwarp();
+          }
+          done[0] += (nt + 1) / 2;
+          done[1] += nt / 2;
+          fill += 2 * nt;
+          ++item_idx;
+          if (!ok) break;
+          continue;
+        }
         {
           // The S buffers are free: the P of every earlier key tile has been waited for, hence its S was taken.
-          const uint32_t slot = fill % kSlots;
-          ok = mbar_wait(bar(L::KV_FULL + slot), (fill / kSlots) & 1, abort_flag, wait_limit);
+          const uint32_t slot = fill % L::kSlots;
+          ok = mbar_wait(bar(L::KV_FULL + slot), (fill / L::kSlots) & 1, abort_flag, wait_limit);
           if (!ok) break;
           tc_fence_after();
-          if (MT == 2) {
+          if (ONE) {
+            issue_qk(0, tj & 1, slot);
+          } else {
             issue_qk(0, 0, slot);
             if (L::kTmemS1 == L::kTmemS0) ok = mbar_wait(bar(L::S_FREE + 0), tj & 1, abort_flag, wait_limit);
             if (!ok) break;
             tc_fence_after();
             issue_qk(1, 1, slot);
-          } else {
-            issue_qk(0, tj & 1, slot);
           }
           if (elect_one()) mma_commit(bar(L::KV_EMPTY + slot));
           if (nt == 1 && elect_one()) mma_commit(bar(L::Q_EMPTY));
         }
         for (int jt = 0; jt < nt && ok; ++jt, ++tj) {
-          const uint32_t fv = fill + 2 * jt + 1, vslot = fv % kSlots;
-          const uint32_t fk = fv + 1, kslot = fk % kSlots;
+          const uint32_t fv = fill + 2 * jt + 1, vslot = fv % L::kSlots;
+          const uint32_t fk = fv + 1, kslot = fk % L::kSlots;
           const bool more = jt + 1 < nt;
-          if (MT == 2) {
+          if (ONE) {
+            const int buf = tj & 1;
+            if (more) {
+              ok = mbar_wait(bar(L::KV_FULL + kslot), (fk / L::kSlots) & 1, abort_flag, wait_limit);
+              if (!ok) break;
+              tc_fence_after();
+              issue_qk(0, buf ^ 1, kslot);       // the P of the key tile before has been waited for: its S was taken
+            }
+            ok = mbar_wait(bar(L::P_READY + buf), (tj >> 1) & 1, abort_flag, wait_limit);
+            if (ok) ok = mbar_wait(bar(L::KV_FULL + vslot), (fv / L::kSlots) & 1, abort_flag, wait_limit);
+            if (!ok) break;
+            tc_fence_after();
+            issue_pv(0, buf, vslot, jt == 0);
+            if (elect_one()) {
+              if (!more) mma_commit(bar(L::ITEM_DONE));
+              mma_commit(bar(L::KV_EMPTY + vslot));
+              if (more) mma_commit(bar(L::KV_EMPTY + kslot));
+              if (jt + 2 == nt) mma_commit(bar(L::Q_EMPTY));
+            }
+          } else {
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
               // S_t(j+1): the buffer was last filled for the other row tile (or, with two buffers, for S_t(j))
               if (more) {
                 if (t == 0) {
-                  ok = mbar_wait(bar(L::KV_FULL + kslot), (fk / kSlots) & 1, abort_flag, wait_limit);
+                  ok = mbar_wait(bar(L::KV_FULL + kslot), (fk / L::kSlots) & 1, abort_flag, wait_limit);
                   if (!ok) break;
                 }
                 if (L::kTmemS1 == L::kTmemS0)
@@ -853,7 +930,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
               tr.mark(0x2000u | ((2 * tj + t) & 0xfffu));
               ok = mbar_wait(bar(L::P_READY + t), tj & 1, abort_flag, wait_limit);
-              if (ok && t == 0) ok = mbar_wait(bar(L::KV_FULL + vslot), (fv / kSlots) & 1, abort_flag, wait_limit);
+              if (ok && t == 0) ok = mbar_wait(bar(L::KV_FULL + vslot), (fv / L::kSlots) & 1, abort_flag, wait_limit);
               if (!ok) break;
               tc_fence_after();
               tr.mark(0x4000u | ((2 * tj + t) & 0xfffu));
@@ -865,27 +942,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (elect_one()) {
               if (jt + 2 == nt) mma_commit(bar(L::O_DONE));
               mma_commit(bar(L::KV_EMPTY + vslot));
-            }
-          } else {
-            const int buf = tj & 1;
-            if (more) {
-              ok = mbar_wait(bar(L::KV_FULL + kslot), (fk / kSlots) & 1, abort_flag, wait_limit);
-              if (!ok) break;
-              tc_fence_after();
-              issue_qk(0, buf ^ 1, kslot);       // the P of the key tile before has been waited for: its S was taken
-            }
-            ok = mbar_wait(bar(L::P_READY + buf), (tj >> 1) & 1, abort_flag, wait_limit);
-            if (ok) ok = mbar_wait(bar(L::KV_FULL + vslot), (fv / kSlots) & 1, abort_flag, wait_limit);
-            if (!ok) break;
-            tc_fence_after();
-            tr.mark(0x4000u | (tj & 0xfffu));
-            issue_pv(0, buf, vslot, jt == 0);
-            if (!more && elect_one()) mma_commit(bar(L::ITEM_DONE));
-            tr.mark(0x2000u | (tj & 0xfffu));
-            if (elect_one()) {
-              mma_commit(bar(L::KV_EMPTY + vslot));
-              if (more) mma_commit(bar(L::KV_EMPTY + kslot));
-              if (jt + 2 == nt) mma_commit(bar(L::Q_EMPTY));
             }
           }
           __syncwarp();
@@ -906,10 +962,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // other warpgroup has released enough, so any other split has to keep 4 (168 - low) >= 8 (high - 168) or the
     // kernel never gets past this instruction.
     asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
-    const int wg = (warp - 4) >> 2;                  // row tile of this warpgroup
+    const int wg = (warp - 4) >> 2;                  // its row tile, or parity of its key tiles
     const int row = ((warp & 3) << 5) | lane;        // TMEM lane = row inside the tile
     const uint32_t lane_addr = (uint32_t)((warp & 3) << 5) << 16;
-    const bool wg_active = wg < MT;
     gdc_wait();      // anc_bits, the workspace and the outputs may belong to the kernel in front until it is done
     // in-cache layout: a tree that does not fit behind its prefix is reported, not read past the capacity (rows
     // past Scap arrive as zeros and the sequence's output is unspecified).  Raised after the wait: status[] may
@@ -922,9 +977,10 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (S + prm.n_nodes[b] > prm.Scap) atomicOr(prm.status + b, TV_ST_CAPACITY);
       }
     float m_fin = -INFINITY, l_fin = 0.f;            // cluster kernel: (m, l) of the row; no key tile: weight 0
-    if (wg_active && !*abort_flag && !(prm.debug & 4)) {
-      uint32_t fill = 0, tj = 0, epi_phase = 0, item_cnt = 0;   // tj: key tiles handled so far (all items)
-      uint32_t od_phase = 0;                                    // items of more than one key tile so far
+    if (!(ONE && wg) && !*abort_flag && !(prm.debug & 4)) {
+      uint32_t fill = 0, tj = 0, epi_phase = 0, item_cnt = 0;   // tj: key tiles of this warpgroup so far (all items)
+      uint32_t to = 0;                                          // KS: those of the other one in earlier items
+      uint32_t od_phase = 0;                                    // completions of O_DONE so far
       bool ok = true;
       Tracer tr;
       tr.init((threadIdx.x & 127) == 0 ? prm.trace : nullptr, 2 + wg);
@@ -949,7 +1005,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (lane == 0) mbar_arrive(bar(L::ITEM_READ));
         const int nt = it.j1 - it.j0;
         if (nt == 0) break;
-        const int node = (prm.tile0 + pair * MT + wg) * prm.NPT + row / prm.G;
+        const int node = (prm.tile0 + pair * MT + (MT == 1 ? 0 : wg)) * prm.NPT + row / prm.G;
         const int gm = row % prm.G;
         const bool row_exists = row < prm.NPT * prm.G && node < prm.Nmax;
         const bool row_active = row_exists && node < it.n;
@@ -967,7 +1023,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t o_addr_loop = tmem + lane_addr + L::kTmemO0 + wg * D;
         // key tiles below this index are full tiles of the committed prefix (no mask of any kind)
         const int j_full = min(it.S / kTileN, it.len - prm.TT);
-        for (int jt = 0; jt < nt && ok; ++jt, ++tj) {
+        for (int jt = KS ? wg : 0; jt < nt && ok; jt += KS ? 2 : 1, ++tj) {
           const int j = it.j0 + jt;
           const bool masked = j >= j_full;
           uint32_t vis[4] = {0u, 0u, 0u, 0u};      // masked tiles: visible keys of this row
@@ -992,8 +1048,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // outside the tensor arrive as zeros from the copy itself: a tree tile whose tree is full (the
             // usual case) needs nothing.
             if (valid_keys < kTileN && !(tree && !prm.tree_in_cache && tt * kTileN + valid_keys >= prm.Nmax)) {
-              const uint32_t f = fill + 2 * jt + 1, slot = f % kSlots;
-              ok = wwait(bar(L::KV_FULL + slot), (f / kSlots) & 1);
+              const uint32_t f = fill + 2 * jt + 1, slot = f % L::kSlots;
+              ok = wwait(bar(L::KV_FULL + slot), (f / L::kSlots) & 1);
               if (!ok) break;
               if (row >= valid_keys) {
                 uint8_t* vrow = smem + L::kRing + slot * L::kTileBytes + row * 128;
@@ -1006,24 +1062,33 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               fence_proxy_async_smem();
             }
           }
-          // S and P of this key tile: index = row tile, or parity of the key tile when the CTA has one row tile
-          const int idx = (MT == 2) ? wg : (int)(tj & 1u);
-          const uint32_t use_par = (MT == 2) ? (tj & 1u) : ((tj >> 1) & 1u);
-          // Completion of the PV of the key tile before this one (for the first key tile of an item: nothing to wait
-          // for).  MT = 2: the pipe works in issue order, and S_1(j) is issued behind O_0 += P_0(j-1) V, S_0(j+1) behind
-          // O_1 += P_1(j-1) V; where no S_0(j+1) follows, that PV has a commit of its own (once per item).
+          // Completion of the PV of this warpgroup's key tile before this one (for its first key tile of an item: nothing to
+          // wait for).  The pipe works in issue order.  Two row tiles: S_1(j) is issued behind O_0 += P_0(j-1) V, S_0(j+1)
+          // behind O_1 += P_1(j-1) V; KS: S(j+1) behind O += P(j-2) V.  Where no such S follows, that PV has a commit of its
+          // own (once per item).  One warpgroup: each PV has one.
           auto previous_pv_done = [&]() -> bool {
+            if (KS) {
+              if (jt < 2) return true;
+              return jt + 1 < nt ? wwait(bar(L::S_FULL + (wg ^ 1)), (to + ((jt + 1) >> 1)) & 1u) : wwait(bar(L::O_DONE), od_phase & 1u);
+            }
             if (jt == 0) return true;
-            if (MT == 1) return wwait(bar(L::O_DONE), (tj - 1) & 1u);
+            if (ONE) return wwait(bar(L::O_DONE), (tj - 1) & 1u);
             if (wg == 0) return wwait(bar(L::S_FULL + 1), tj & 1u);
             return jt + 1 < nt ? wwait(bar(L::S_FULL + 0), (tj + 1) & 1u) : wwait(bar(L::O_DONE), od_phase & 1u);
           };
+          // S and P of this key tile: index = warpgroup, or parity of the key tile when there is one
+          const int idx = ONE ? (int)(tj & 1u) : wg;
           tr.mark(0x0800u | (tj & 0x7ffu));
-          ok = wwait(bar(L::S_FULL + idx), use_par);
+          ok = wwait(bar(L::S_FULL + idx), (ONE ? tj >> 1 : tj) & 1u);
           if (!ok) break;
           tc_fence_after();
           tr.mark(0x1000u | (tj & 0xfffu));
           if (MT == 1 && !warp_active) {      // nothing of S is looked at; P and O keep whatever tensor memory holds there
+            if (KS) {
+              if (lane == 0) mbar_arrive(bar(L::S_FREE + wg));
+              ok = previous_pv_done();        // or this warp could arrive for P twice in one phase
+              if (!ok) break;
+            }
             if (lane == 0) mbar_arrive(bar(L::P_READY + idx));
             continue;
           }
@@ -1036,10 +1101,10 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             tmem_ld32(s_base + 64, sall + 64);
             tmem_ld32(s_base + 96, sall + 96);
             tmem_wait_ld();
-            if (MT == 2) {
+            if (!ONE) {
               tc_fence_before();
               __syncwarp();
-              if (lane == 0) mbar_arrive(bar(L::S_FREE + idx));
+              if (lane == 0) mbar_arrive(bar(L::S_FREE + wg));
             }
           }
           float* sa = reinterpret_cast<float*>(sall);
@@ -1065,7 +1130,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               const float alpha = (moves && m_used > -INFINITY) ? fast_exp2(m_used - mx2) : 1.f;
               if (moves) m_used = mx2;
               l_sum *= alpha;
-              if (jt > 0) {
+              if (jt > (KS ? 1 : 0)) {
                 ok = previous_pv_done();
                 if (!ok) break;
                 tc_fence_after();
@@ -1112,9 +1177,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 if (!((vis[i >> 4] >> ((2 * i + 1) & 31)) & 1u)) pkk[i] &= 0x0000ffffu;
               }
           }
-          // ---- P into its columns once the PV that read them last is done: with two row tiles that of the key tile
-          // before; with one (two P buffers in turn) it was issued in front of the S this tile has waited for
-          if (MT == 2) {
+          // ---- P into its columns once the PV that read them last is done; with one warpgroup (two P buffers in turn) that
+          // was issued in front of the S this tile has waited for
+          if (!ONE) {
             ok = previous_pv_done();
             if (!ok) break;
             tc_fence_after();
@@ -1130,19 +1195,52 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (lane == 0) mbar_arrive(bar(L::P_READY + idx));
           tr.mark(0x2000u | (tj & 0xfffu));
         }
-        if (nt > 1) ++od_phase;
+        if (nt > (KS ? 2 : 1)) ++od_phase;
+        to += (nt + wg) / 2;
         if (!ok) break;
         // ---- epilogue of the item: wait for the last PV into this O buffer
         {
           // Wait for every MMA of the item.  This barrier completes once per item, so its phase is never
           // more than one away from the one waited for (a parity wait cannot tell phases two apart, which
           // is why the per-PV barrier O_DONE is not used here: both last PVs may or may not be done yet).
-          ok = wwait(bar(L::ITEM_DONE + wg), item_cnt & 1);
+          ok = wwait(bar(L::ITEM_DONE + (MT == 1 ? 0 : wg)), item_cnt & 1);
           ++item_cnt;
           if (!ok) break;
           tc_fence_after();
           tr.mark(0x5000u);
-          const uint32_t o_addr = o_addr_loop;
+          // KS: the two warpgroups have half of the keys each.  They exchange (m, l), and each of them finishes half
+          // of the columns: O = e_0 O_0 + e_1 O_1 with e_w = 2^(m_w - max m); a warpgroup without keys has weight 0 (its O was
+          // not written).
+          float e_0 = 1.f, e_1 = 0.f;
+          if (KS) {
+            float2* xch = reinterpret_cast<float2*>(smem + L::kXch);
+            xch[wg * 128 + row] = make_float2(m_used, l_sum);
+            ok = epi_sync();
+            if (!ok) break;
+            const float2 a = xch[row], b = xch[128 + row];
+            m_used = fmaxf(a.x, b.x);
+            e_0 = a.x > -INFINITY ? fast_exp2(a.x - m_used) : 0.f;
+            e_1 = b.x > -INFINITY ? fast_exp2(b.x - m_used) : 0.f;
+            l_sum = e_0 * a.y + e_1 * b.y;
+          }
+          constexpr int kGroups = KS ? D / 64 : D / 32;                // groups of 32 columns that this warpgroup finishes,
+          const int q0 = KS ? wg * kGroups : 0;                        // from this one on
+          const uint32_t o_addr = MT == 1 ? tmem + lane_addr + L::kTmemO0 : o_addr_loop;
+          auto load_own = [&](int q, uint32_t* o) {
+            tmem_ld32(o_addr + q * 32, o);
+            if (KS) {
+              uint32_t o1[32];
+              tmem_ld32(o_addr + D + q * 32, o1);
+              tmem_wait_ld();
+#pragma unroll
+              for (int c = 0; c < 32; ++c) {
+                const float x = e_0 > 0.f ? e_0 * __uint_as_float(o[c]) : 0.f;
+                o[c] = __float_as_uint(e_1 > 0.f ? fmaf(e_1, __uint_as_float(o1[c]), x) : x);
+              }
+            } else {
+              tmem_wait_ld();
+            }
+          };
           const bool whole = (it.j0 == 0 && it.j1 == it.len);
           const int h = it.hk * prm.G + gm;
           tv_bf16* orow = prm.out + (size_t)it.layer * prm.out_layer_stride + (((size_t)it.b * prm.Nmax + node) * prm.Hq + h) * D;
@@ -1151,10 +1249,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           // epilogue is cold code, fetched while the other CTAs still stream K/V).
           auto store_rows = [&](uint4* dst, size_t stride_u4, float inv, bool do_store, bool zero) {
 #pragma unroll 1
-            for (int q = 0; q < D / 32; ++q) {
+            for (int q = q0; q < q0 + kGroups; ++q) {
               uint32_t o[32];
-              tmem_ld32(o_addr + q * 32, o);
-              tmem_wait_ld();
+              load_own(q, o);
               if (do_store) {
                 uint4 v[4];
 #pragma unroll
@@ -1179,12 +1276,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // ---- the partial of this CTA: normalised bf16 rows over the Q tile (every QK^T of the item is done), 16-byte
             // pieces of a row swizzled by the row so that neither the writes nor the reads collide; (m, l) beside them
             const float inv = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
-            uint8_t* mine = smem + L::kQ + wg * L::kTileBytes + row * (D * 2);
+            uint8_t* mine = smem + L::kQ + (MT == 1 ? 0 : wg) * L::kTileBytes + row * (D * 2);
 #pragma unroll 1
-            for (int q = 0; q < D / 32; ++q) {
+            for (int q = q0; q < q0 + kGroups; ++q) {
               uint32_t o[32];
-              tmem_ld32(o_addr + q * 32, o);
-              tmem_wait_ld();
+              load_own(q, o);
 #pragma unroll
               for (int c = 0; c < 4; ++c) {
                 uint4 v;
@@ -1201,7 +1297,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           } else if (whole) {
             const float inv = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
             store_rows(reinterpret_cast<uint4*>(orow), 1, inv, row_exists, !row_active);
-            if (row_exists && lse_p)
+            if (row_exists && lse_p && !(KS && wg))
               *lse_p = (row_active && m_used > -INFINITY) ? (m_used + log2f(l_sum)) / kLog2e : -INFINITY;
             tc_fence_before();
           } else {
@@ -1217,7 +1313,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // Partial outputs are stored column-group major, [slot][D/8][MT*128 rows][8 bf16]: a warp writes
             // and reads 512 contiguous bytes per instruction.
             constexpr int kRows = MT * 128;
-            const int rr = wg * 128 + row;
+            const int rr = (MT == 1 ? 0 : wg * 128) + row;
             // The unit's real tiles occupy [real0, uend) of the virtual tile space.  CTA groups k_first..k_last
             // hold them, one piece each (a group between the two lies wholly inside the unit), and this CTA's
             // group is one of them: two short walks over the cut table find both ends.
@@ -1234,7 +1330,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               const size_t slot = (size_t)group * prm.NP + pair;
               uint4* po = reinterpret_cast<uint4*>(prm.part_o) + slot * (D / 8) * kRows;
               float* pml = prm.part_ml + slot * 2 * kRows;
-              if (row_active) {
+              if (row_active && !(KS && wg)) {
                 pml[rr] = m_used;
                 pml[kRows + rr] = l_sum;
               }
@@ -1278,11 +1374,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               auto slot_of = [&](int i) -> size_t { return (size_t)(k_first + i) * prm.NP + pair; };       // i-th other piece, i >= 1
               auto ml_of = [&](int i) -> const float* { return prm.part_ml + slot_of(i) * 2 * kRows + rr; };
               auto o_of = [&](int i) -> const uint4* { return reinterpret_cast<const uint4*>(prm.part_o) + slot_of(i) * (D / 8) * kRows + rr; };
-              uint4 v[D / 8];                              // one row of a piece
+              uint4 v[kGroups * 4];                        // one row of a piece, the columns of this warpgroup
               auto fetch = [&](int i) {
-                const uint4* q_o = o_of(i);
+                const uint4* q_o = o_of(i) + (size_t)q0 * 4 * kRows;
 #pragma unroll
-                for (int c = 0; c < D / 8; ++c) v[c] = __ldcg(q_o + (size_t)c * kRows);
+                for (int c = 0; c < kGroups * 4; ++c) v[c] = __ldcg(q_o + (size_t)c * kRows);
               };
               const float m_1 = __ldcg(ml_of(1)), l_1 = __ldcg(ml_of(1) + kRows);
               fetch(1);
@@ -1307,10 +1403,15 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 const float2 w2 = make_float2(w, w), own2 = make_float2(w_own, w_own), inv_own2 = make_float2(inv_own, inv_own);
                 const float2 inv2 = make_float2(inv, inv);
 #pragma unroll
-                for (int q = 0; q < D / 32; ++q) {
+                for (int x = 0; x < kGroups; ++x) {
+                  const int q = q0 + x;
                   uint32_t o[32];
-                  tmem_ld32(o_addr + q * 32, o);
-                  tmem_wait_ld();
+                  if (i == 1) {
+                    load_own(q, o);
+                  } else {
+                    tmem_ld32(o_addr + q * 32, o);
+                    tmem_wait_ld();
+                  }
 #pragma unroll
                   for (int c = 0; c < 16; ++c) {
                     float2 acc = make_float2(__uint_as_float(o[2 * c]), __uint_as_float(o[2 * c + 1]));
@@ -1319,9 +1420,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                       const uint32_t own = pack_bf16(t.x, t.y);
                       acc = __fmul2_rn(own2, make_float2(__uint_as_float(own << 16), __uint_as_float(own & 0xffff0000u)));
                     }
-                    const uint4 vv = v[q * 4 + (c >> 2)];
-                    const uint32_t x = (c & 3) == 0 ? vv.x : ((c & 3) == 1 ? vv.y : ((c & 3) == 2 ? vv.z : vv.w));
-                    acc = ffma2(w2, make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)), acc);
+                    const uint4 vv = v[x * 4 + (c >> 2)];
+                    const uint32_t pv = (c & 3) == 0 ? vv.x : ((c & 3) == 1 ? vv.y : ((c & 3) == 2 ? vv.z : vv.w));
+                    acc = ffma2(w2, make_float2(__uint_as_float(pv << 16), __uint_as_float(pv & 0xffff0000u)), acc);
                     o[2 * c] = __float_as_uint(acc.x);
                     o[2 * c + 1] = __float_as_uint(acc.y);
                   }
@@ -1329,7 +1430,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                     tmem_st32(o_addr + q * 32, o);
                     const uint4* q_o = o_of(i + 1);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) v[q * 4 + c] = __ldcg(q_o + (size_t)(q * 4 + c) * kRows);
+                    for (int c = 0; c < 4; ++c) v[x * 4 + c] = __ldcg(q_o + (size_t)(q * 4 + c) * kRows);
                   } else if (row_exists) {
                     uint4 r[4];
 #pragma unroll
@@ -1354,10 +1455,14 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 tmem_wait_st();
                 w = l_next * fast_exp2(m_next - mref);
               }
-              if (row_exists && lse_p) *lse_p = any_key ? (mm + log2f(lt)) / kLog2e : -INFINITY;
+              if (row_exists && lse_p && !(KS && wg)) *lse_p = any_key ? (mm + log2f(lt)) / kLog2e : -INFINITY;
               tc_fence_before();
             }
           }
+        }
+        if (KS) {      // both warpgroups have read both O: the next item may write them
+          ok = epi_sync();
+          if (!ok) break;
         }
         tr.mark(0x8000u);
         fill += 2 * nt;
@@ -1367,7 +1472,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // ---- merge of the cluster's partials: each CTA takes a share of the rows, 16 bytes of a row per thread; out =
       // sum_p w_p O_p / sum_p w_p, w_p = l_p 2^(m_p - max m), in rank order.  A piece without keys has weight 0 (its rows
       // were not written and are not used).
-      if (wg_active) *reinterpret_cast<float2*>(smem + L::kMl + (wg * 128 + row) * 8) = make_float2(m_fin, l_fin);
+      if (MT == 2 || wg == 0) *reinterpret_cast<float2*>(smem + L::kMl + (wg * 128 + row) * 8) = make_float2(m_fin, l_fin);
       __syncwarp();
       cluster_sync();
       if (!*abort_flag && !(prm.debug & 4)) {

@@ -586,3 +586,19 @@ def test_last_row_tile_in_a_launch_of_its_own(N):
         ref_out, ref_lse = oracle_attention_slice(cn, l, b, hk, G, vis, d ** -0.5)
         assert_attention_close(out[l][b:b + 1, :, hk * G:(hk + 1) * G], lse[l][b:b + 1, hk * G:(hk + 1) * G], ref_out, ref_lse,
                                f"{l} {b} {hk}")
+
+
+@pytest.mark.parametrize("G,N,d", [(2, 40, 64), (4, 40, 64), (2, 40, 128), (4, 40, 128)])
+@pytest.mark.parametrize("longest", [900, 2100, 6000])
+def test_long_unit_among_many_is_cut_in_many_pieces(G, N, d, longest):
+    """Too many units for clusters, one of them far longer than the rest: its pieces are two, several and many, next to
+    whole units of one to three key tiles; one and two row tiles, both head widths."""
+    cfg = CONFIGS[0].scaled(B=80, Hq=G, Hkv=1, d=d, S_lo=0, S_hi=260, Scap=longest + 64, N=N, D=6, V=0, tree="uniform")
+    case = make_case(cfg, seed=longest + G + d, ragged_nodes=True, with_logits=False)
+    case["prefix_len"][33] = longest
+    dcase = to_device(case)
+    out, lse, bits, dense = gpu_attention(dcase)
+    ref_out, ref_lse = oracle_attention(case_to_numpy(case), dense.cpu().numpy())
+    assert_attention_close(out, lse, ref_out, ref_lse, f"longest={longest}")
+    out2, lse2, _, _ = gpu_attention(dcase)
+    assert torch.equal(out, out2) and torch.equal(lse, lse2)
