@@ -166,6 +166,11 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The same without ordering any memory access: for a barrier that only keeps a CTA's shared memory alive.
+__device__ __forceinline__ void cluster_sync_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t cluster_size_x() {
   uint32_t n;
   asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));
@@ -176,9 +181,9 @@ __device__ __forceinline__ uint32_t peer_smem(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ float ld_peer_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+__device__ __forceinline__ float2 ld_peer_8B(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
   return v;
 }
 __device__ __forceinline__ uint4 ld_peer_16B(uint32_t addr) {
@@ -507,8 +512,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   }
   // Without the caller's promise nothing of the problem is read before every earlier kernel of the stream has
   // finished (a kernel in front may still be writing prefix_len, and lines of it cached by an earlier launch on
-  // this SM are only dropped by the wait).
-  if (!prm.early) gdc_wait();
+  // this SM are only dropped by the wait).  The cluster kernel has no table to build: its roles wait where they read.
+  if (!CL && !prm.early) gdc_wait();
   if (!CL && warp == 0) {
     int run = 0;
 #pragma unroll 1
@@ -747,7 +752,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (CL) {
       __syncwarp();
       cluster_sync();
-      cluster_sync();
+      cluster_sync_relaxed();
     }
   } else if (warp == 1) {
     // =========================================================== MMA issuer
@@ -953,7 +958,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (CL) {
       __syncwarp();
       cluster_sync();
-      cluster_sync();
+      cluster_sync_relaxed();
     }
   } else if (warp >= 4) {
     // =========================================================== softmax / epilogue warpgroups
@@ -1473,18 +1478,19 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // sum_p w_p O_p / sum_p w_p, w_p = l_p 2^(m_p - max m), in rank order.  A piece without keys has weight 0 (its rows
       // were not written and are not used).
       if (MT == 2 || wg == 0) *reinterpret_cast<float2*>(smem + L::kMl + (wg * 128 + row) * 8) = make_float2(m_fin, l_fin);
+      const int size = (int)cluster_size_x(), rank = (int)(blockIdx.x % size);
+      const int u = unit / prm.NP, hk = u % prm.Hkv, b = u / prm.Hkv % prm.B, layer = u / prm.Hkv / prm.B;
+      int n = prm.n_nodes[b];                                      // (on its way while the barrier is waited for)
       __syncwarp();
       cluster_sync();
       if (!*abort_flag && !(prm.debug & 4)) {
         constexpr int kVecs = D / 8;
-        const int size = (int)cluster_size_x(), rank = (int)(blockIdx.x % size);
-        const int u = unit / prm.NP, hk = u % prm.Hkv, b = u / prm.Hkv % prm.B, layer = u / prm.Hkv / prm.B;
-        int n = prm.n_nodes[b];
         n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
         const int node0 = (prm.tile0 + pair * MT) * prm.NPT;
         const int nodes = max(0, min(MT * prm.NPT, prm.Nmax - node0));      // nodes of this pair of row tiles
         const int total = nodes * prm.G * kVecs;
-        for (int x = rank * 256 + (int)threadIdx.x - 128; x < total; x += size * 256) {
+        const int share = (total + size - 1) / size, x_end = min(total, (rank + 1) * share);
+        for (int x = rank * share + (int)threadIdx.x - 128; x < x_end; x += 256) {
           const int r = x / kVecs, c = x - r * kVecs;              // row among the existing ones, piece of the row
           const int node_l = r / prm.G, gm = r - node_l * prm.G;
           const int t = MT == 2 && node_l >= prm.NPT ? 1 : 0, in_tile = (node_l - t * prm.NPT) * prm.G + gm;
@@ -1495,9 +1501,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
           for (int k = 0; k < kMaxCluster; ++k)
             if (k < size) {
-              const uint32_t pml = peer_smem(ml, k);
-              pm[k] = ld_peer_f32(pml);
-              w[k] = ld_peer_f32(pml + 4);
+              const float2 p = ld_peer_8B(peer_smem(ml, k));
+              pm[k] = p.x;
+              w[k] = p.y;
               v[k] = ld_peer_16B(peer_smem(at, k));
             }
           float mm = -INFINITY;
@@ -1533,13 +1539,13 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
       }
       __syncwarp();
-      cluster_sync();            // nobody leaves while its shared memory may still be read
+      cluster_sync_relaxed();    // nobody leaves while its shared memory may still be read
     }
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (CL) {
       cluster_sync();
-      cluster_sync();
+      cluster_sync_relaxed();
     }
   }
 
