@@ -288,6 +288,21 @@ TV_API int tree_accept(const tv_bf16* logits, const int32_t* tokens,
                 int32_t* status, tv_stream stream);
 
 /*
+ * tree_accept for a call directly behind tree_verify_attn (any of its variants) on the same stream, whose inputs that
+ * launch leaves alone: logits, tokens, retrieve_indices and n_nodes are complete when the attention starts.  The
+ * vocabulary scan may then start on SMs the attention has left; it ends after the attention, so everything behind
+ * this call is ordered as behind tree_accept.  Arguments and results are those of tree_accept.
+ */
+TV_API int tree_accept_behind_attn(const tv_bf16* logits, const int32_t* tokens,
+                const int32_t* retrieve_indices, const int32_t* n_nodes,
+                int B, int Nmax, int V, int P, int Dp1,
+                int32_t* argmax_tok, int32_t* safe_idx, int32_t* candidates,
+                int32_t* accept_len, int32_t* best_path, int32_t* accepted_nodes,
+                int32_t* next_token,
+                void* workspace, size_t workspace_bytes,
+                int32_t* status, tv_stream stream);
+
+/*
  * Node verification scores (Section 3.3, "Mapping teacher outputs to node
  * verification scores"): the teacher's logit of every node's proposed token,
  * taken from the logits row of the node's parent slot (that row predicts the

@@ -20,7 +20,7 @@ TV_ATTN_LAUNCH_PER_LAYER = 2
 
 EXPORTS = ["tv_last_error", "tv_version", "tv_launch_count", "tree_build_mask", "tv_attn_workspace_bytes", "tree_verify_attn",
            "tree_verify_attn_layers", "tree_verify_attn_paged_layers",
-           "tv_accept_workspace_bytes", "tree_accept", "tree_node_scores", "tree_merge_partials", "tv_accept_noalloc_max_bytes", "tree_accept_noalloc",
+           "tv_accept_workspace_bytes", "tree_accept", "tree_accept_behind_attn", "tree_node_scores", "tree_merge_partials", "tv_accept_noalloc_max_bytes", "tree_accept_noalloc",
            "tv_sample_workspace_bytes", "tree_accept_sample",
            "kv_commit", "kv_commit_inplace", "tree_verify_attn_paged", "kv_commit_paged", "tv_step_staging_bytes",
            "tv_verify_step_host"]
@@ -230,7 +230,14 @@ def tv_debug_attn_simt(q, k_cache, v_cache, k_tree, v_tree, prefix_len, n_nodes,
 def tree_accept(logits, tokens, retrieve_indices, n_nodes, argmax_tok, accept_len, best_path, accepted_nodes,
                 next_token, workspace, status, safe_idx=None, candidates=None, stream=None):
     _check((_calls or _native()).tree_accept(logits, tokens, retrieve_indices, n_nodes, argmax_tok, safe_idx, candidates,
-                                             accept_len, best_path, accepted_nodes, next_token, workspace, status, stream))
+                                             accept_len, best_path, accepted_nodes, next_token, workspace, status, 0, stream))
+
+
+def tree_accept_behind_attn(logits, tokens, retrieve_indices, n_nodes, argmax_tok, accept_len, best_path, accepted_nodes,
+                            next_token, workspace, status, safe_idx=None, candidates=None, stream=None):
+    """tree_accept directly behind an attention call that does not write its inputs: the scan may overlap it."""
+    _check((_calls or _native()).tree_accept(logits, tokens, retrieve_indices, n_nodes, argmax_tok, safe_idx, candidates,
+                                             accept_len, best_path, accepted_nodes, next_token, workspace, status, 1, stream))
 
 
 def tree_node_scores(logits, tokens, parent, n_nodes, scores, status, stream=None):

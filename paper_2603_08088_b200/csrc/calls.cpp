@@ -233,9 +233,9 @@ PyObject* verify_attn_paged_layers(PyObject* const* a, Py_ssize_t n) {
 }
 
 // logits, tokens, retrieve_indices, n_nodes, argmax_tok, safe_idx, candidates, accept_len, best_path, accepted_nodes,
-// next_token, workspace, status, stream
+// next_token, workspace, status, behind_attn, stream
 PyObject* accept(PyObject* const* a, Py_ssize_t n) {
-  Args x(a, n, 14);
+  Args x(a, n, 15);
   const at::Tensor &lg = x.tensor(0, 3), &r = x.tensor(2, 3);
   const int B = lg.size(0), N = lg.size(1), V = lg.size(2), P = r.size(1), Dp1 = r.size(2);
   const auto* logits = x.ptr<tv_bf16>(0);
@@ -245,9 +245,10 @@ PyObject* accept(PyObject* const* a, Py_ssize_t n) {
   void* ws = x.ptr(11);
   const size_t wsb = x.bytes(11);
   auto* st = x.ptr<int32_t>(12);
-  const tv_stream s = x.stream(13);
+  const auto entry = x.integer(13) ? tree_accept_behind_attn : tree_accept;
+  const tv_stream s = x.stream(14);
   return call([&] {
-    return tree_accept(logits, tok, rows, nn, B, N, V, P, Dp1, am, safe, cand, al, best, nodes, next, ws, wsb, st, s);
+    return entry(logits, tok, rows, nn, B, N, V, P, Dp1, am, safe, cand, al, best, nodes, next, ws, wsb, st, s);
   });
 }
 

@@ -62,9 +62,10 @@ def verify_step(case, buf: StepBuffers, scale, retrieve=None, commit=True, strea
                                buf.status, lse=buf.lse, flags=tv.TV_ATTN_STABLE_INPUTS, stream=stream)
     if V > 0 and "logits" in case:
         rows = buf.retrieve if own_rows else retrieve
-        tv.tree_accept(case["logits"], case["tokens"], rows, case["n_nodes"], buf.argmax_tok, buf.accept_len,
-                       buf.best_path, buf.accepted_nodes, buf.next_token, buf.accept_ws, buf.status,
-                       safe_idx=buf.safe_idx, candidates=buf.candidates, stream=stream)
+        # (the logits were there before the step: the scan may fill the SMs that the attention leaves)
+        tv.tree_accept_behind_attn(case["logits"], case["tokens"], rows, case["n_nodes"], buf.argmax_tok, buf.accept_len,
+                                   buf.best_path, buf.accepted_nodes, buf.next_token, buf.accept_ws, buf.status,
+                                   safe_idx=buf.safe_idx, candidates=buf.candidates, stream=stream)
         if commit and in_cache:
             tv.kv_commit_inplace(case["k_cache"], case["v_cache"], buf.accepted_nodes, buf.accept_len,
                                  case["prefix_len"], Nmax, buf.status, stream=stream)

@@ -82,3 +82,44 @@ def test_status_bits_raised_by_a_one_layer_attention_survive_the_mask_kernel():
     for rep, (st1, st2) in enumerate(statuses):
         assert i32(st1).tolist() == [tv.TV_ST_CAPACITY, 0], f"repetition {rep}: {i32(st1).tolist()}"
         assert i32(st2).tolist() == [0, tv.TV_ST_BAD_INDEX], f"repetition {rep}: {i32(st2).tolist()}"
+
+
+@pytest.mark.parametrize("in_cache", [False, True])
+@pytest.mark.parametrize("B,L,S", [(1, 1, 1500), (12, 3, 2500)])
+def test_scan_beside_the_attention_changes_nothing(B, L, S, in_cache):
+    """verify_step lets the vocabulary scan overlap the attention in front of it.  Three steps in a row without a
+    synchronisation, each on the cache and the lengths the one before has left, give bit for bit what the same calls
+    with the ordered tree_accept give (acceptance and commit wait for the attention in both)."""
+    cfg = CONFIGS[2].scaled(B=B, L=L, Hq=16, Hkv=4, S_lo=S // 2, S_hi=S, Scap=S + 300, V=30001, N=33, D=6)
+    case = to_device(make_case(cfg, seed=B + L))
+
+    def steps(ordered):
+        c = {k: (v.clone() if isinstance(v, torch.Tensor) else v) for k, v in case.items()}
+        P, Dp1 = cfg.N, cfg.D + 1
+        outs = []
+        for _ in range(3):
+            buf = tv.StepBuffers(L, B, cfg.N, cfg.Hq, cfg.Hkv, cfg.d, cfg.Scap, cfg.V, P, Dp1)
+            if not ordered:
+                tv.verify_step(c, buf, cfg.d ** -0.5, in_cache=in_cache)
+            else:
+                tv.tree_build_mask(c["parent"], c["n_nodes"], Dp1 - 1, P, buf.anc_bits, buf.status, depth=buf.depth,
+                                   anc_table=buf.anc_table, retrieve_indices=buf.retrieve, n_paths=buf.n_paths)
+                tv.tree_verify_attn_layers(c["q"], c["k_cache"], c["v_cache"], None if in_cache else c["k_tree"],
+                                           None if in_cache else c["v_tree"], c["prefix_len"], c["n_nodes"], buf.anc_bits,
+                                           cfg.d ** -0.5, buf.out, buf.attn_ws, buf.status, flags=tv.TV_ATTN_STABLE_INPUTS)
+                torch.cuda.synchronize()
+                tv.tree_accept(c["logits"], c["tokens"], buf.retrieve, c["n_nodes"], buf.argmax_tok, buf.accept_len,
+                               buf.best_path, buf.accepted_nodes, buf.next_token, buf.accept_ws, buf.status)
+                if in_cache:
+                    tv.kv_commit_inplace(c["k_cache"], c["v_cache"], buf.accepted_nodes, buf.accept_len, c["prefix_len"],
+                                         cfg.N, buf.status)
+                else:
+                    tv.kv_commit(c["k_cache"], c["v_cache"], c["k_tree"], c["v_tree"], buf.accepted_nodes, buf.accept_len,
+                                 c["prefix_len"], buf.status)
+                torch.cuda.synchronize()
+            outs.append((buf.out, buf.status, buf.argmax_tok, buf.accept_len, buf.accepted_nodes, buf.next_token))
+        torch.cuda.synchronize()
+        return [t for o in outs for t in o] + [c["k_cache"], c["v_cache"], c["prefix_len"]]
+
+    for a, b in zip(steps(False), steps(True)):
+        assert torch.equal(a, b)
