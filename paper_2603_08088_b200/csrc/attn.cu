@@ -1319,9 +1319,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // out = sum_p w_p O_p / sum_p w_p with w_p = l_p 2^(m_p - max m).  Every piece enters the sum as its
             // bf16-rounded normalised output, the merger's own included, in piece order with one fused multiply-add
             // per piece.  What bounds this is dependent round trips to L2 (some 2 K cycles each under load): a fixed
-            // merger needs no ticket, its pieces are usually ready long before, and a piece's whole row is requested at
-            // once, the first one's beside its (m, l), a later one's as the row before it is used up.  The sum stays in
-            // tensor memory between two pieces.
+            // merger needs no ticket, its pieces are usually ready long before, and two pieces' whole rows are requested
+            // at once beside their (m, l) (one piece at a time: 4 sequences of 4096, 128 nodes 42.6 -> 41.7 us, 32 of 1024
+            // 50.6 -> 50.1 us a launch; three do not fit the registers).  The sum stays in tensor memory between two pairs.
+            // The code is cold, so the columns go in two equal turns, each in the first half of the registers (unrolled
+            // over all of them: +1 %, over a quarter of them: +1 %).
             // Partial outputs are stored column-group major, [slot][D/8][MT*128 rows][8 bf16]: a warp writes
             // and reads 512 contiguous bytes per instruction.
             constexpr int kRows = MT * 128;
@@ -1385,86 +1387,110 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               auto slot_of = [&](int i) -> size_t { return (size_t)(k_first + i) * prm.NP + pair; };       // i-th other piece, i >= 1
               auto ml_of = [&](int i) -> const float* { return prm.part_ml + slot_of(i) * 2 * kRows + rr; };
               auto o_of = [&](int i) -> const uint4* { return reinterpret_cast<const uint4*>(prm.part_o) + slot_of(i) * (D / 8) * kRows + rr; };
-              uint4 v[kGroups * 4];                        // one row of a piece, the columns of this warpgroup
+              // two pieces at a time: (m, l) of the row and the columns of this warpgroup
+              float m_a = 0.f, l_a = 0.f, m_b = 0.f, l_b = 0.f;
+              constexpr int kTurn = kGroups > 2 ? 2 : kGroups;      // groups of 32 columns in a turn
+              uint4 va[kGroups * 4], vb[kGroups * 4];
               auto fetch = [&](int i) {
-                const uint4* q_o = o_of(i) + (size_t)q0 * 4 * kRows;
+                m_a = __ldcg(ml_of(i));
+                l_a = __ldcg(ml_of(i) + kRows);
+                const uint4* a_o = o_of(i) + (size_t)q0 * 4 * kRows;
 #pragma unroll
-                for (int c = 0; c < kGroups * 4; ++c) v[c] = __ldcg(q_o + (size_t)c * kRows);
+                for (int c = 0; c < kGroups * 4; ++c) va[c] = __ldcg(a_o + (size_t)c * kRows);
+                m_b = -INFINITY;
+                l_b = 0.f;
+                if (i < n_other) {
+                  m_b = __ldcg(ml_of(i + 1));
+                  l_b = __ldcg(ml_of(i + 1) + kRows);
+                  const uint4* b_o = o_of(i + 1) + (size_t)q0 * 4 * kRows;
+#pragma unroll
+                  for (int c = 0; c < kGroups * 4; ++c) vb[c] = __ldcg(b_o + (size_t)c * kRows);
+                } else {
+#pragma unroll
+                  for (int c = 0; c < kGroups * 4; ++c) vb[c] = make_uint4(0, 0, 0, 0);
+                }
               };
-              const float m_1 = __ldcg(ml_of(1)), l_1 = __ldcg(ml_of(1) + kRows);
               fetch(1);
-              float mm = fmaxf(m_used, m_1);
+              float mm = fmaxf(m_used, fmaxf(m_a, m_b));
 #pragma unroll 4
-              for (int i = 2; i <= n_other; ++i) mm = fmaxf(mm, __ldcg(ml_of(i)));
+              for (int i = 3; i <= n_other; ++i) mm = fmaxf(mm, __ldcg(ml_of(i)));
               const float mref = mm == -INFINITY ? 0.f : mm;
-              auto weight = [&](int i) -> float { return __ldcg(ml_of(i) + kRows) * fast_exp2(__ldcg(ml_of(i)) - mref); };
               const float w_own = l_sum * fast_exp2(m_used - mref);
-              float w = l_1 * fast_exp2(m_1 - mref), lt = w_own + w;
+              float w_a = l_a * fast_exp2(m_a - mref), w_b = l_b * fast_exp2(m_b - mref), lt = w_own + w_a + w_b;
 #pragma unroll 4
-              for (int i = 2; i <= n_other; ++i) lt += weight(i);
+              for (int i = 3; i <= n_other; ++i) lt += __ldcg(ml_of(i) + kRows) * fast_exp2(__ldcg(ml_of(i)) - mref);
               const bool any_key = row_active && mm > -INFINITY;
               const float inv = any_key ? 1.f / lt : 0.f;
+              const float2 own2 = make_float2(w_own, w_own), inv_own2 = make_float2(inv_own, inv_own), inv2 = make_float2(inv, inv);
 #pragma unroll 1
-              for (int i = 1; i <= n_other; ++i) {
-                float m_next = 0.f, l_next = 0.f;
-                if (i < n_other) {
-                  m_next = __ldcg(ml_of(i + 1));
-                  l_next = __ldcg(ml_of(i + 1) + kRows);
-                }
-                const float2 w2 = make_float2(w, w), own2 = make_float2(w_own, w_own), inv_own2 = make_float2(inv_own, inv_own);
-                const float2 inv2 = make_float2(inv, inv);
+              for (int i = 1; i <= n_other; i += 2) {
+                const float2 wa2 = make_float2(w_a, w_a), wb2 = make_float2(w_b, w_b);
+                const bool more = i + 2 <= n_other;
+#pragma unroll 1
+                for (int xo = 0; xo < kGroups; xo += kTurn) {
 #pragma unroll
-                for (int x = 0; x < kGroups; ++x) {
-                  const int q = q0 + x;
-                  uint32_t o[32];
-                  if (i == 1) {
-                    load_own(q, o);
-                  } else {
-                    tmem_ld32(o_addr + q * 32, o);
-                    tmem_wait_ld();
-                  }
-#pragma unroll
-                  for (int c = 0; c < 16; ++c) {
-                    float2 acc = make_float2(__uint_as_float(o[2 * c]), __uint_as_float(o[2 * c + 1]));
+                  for (int x = 0; x < kTurn; ++x) {
+                    const int q = q0 + xo + x;
+                    uint32_t o[32];
                     if (i == 1) {
-                      const float2 t = __fmul2_rn(acc, inv_own2);
-                      const uint32_t own = pack_bf16(t.x, t.y);
-                      acc = __fmul2_rn(own2, make_float2(__uint_as_float(own << 16), __uint_as_float(own & 0xffff0000u)));
-                    }
-                    const uint4 vv = v[x * 4 + (c >> 2)];
-                    const uint32_t pv = (c & 3) == 0 ? vv.x : ((c & 3) == 1 ? vv.y : ((c & 3) == 2 ? vv.z : vv.w));
-                    acc = ffma2(w2, make_float2(__uint_as_float(pv << 16), __uint_as_float(pv & 0xffff0000u)), acc);
-                    o[2 * c] = __float_as_uint(acc.x);
-                    o[2 * c + 1] = __float_as_uint(acc.y);
-                  }
-                  if (i < n_other) {
-                    tmem_st32(o_addr + q * 32, o);
-                    const uint4* q_o = o_of(i + 1);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) v[x * 4 + c] = __ldcg(q_o + (size_t)(q * 4 + c) * kRows);
-                  } else if (row_exists) {
-                    uint4 r[4];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                      uint32_t pk4[4];
-#pragma unroll
-                      for (int e = 0; e < 4; ++e) {
-                        const float2 t = __fmul2_rn(make_float2(__uint_as_float(o[8 * c + 2 * e]), __uint_as_float(o[8 * c + 2 * e + 1])), inv2);
-                        pk4[e] = any_key ? pack_bf16(t.x, t.y) : 0u;
-                      }
-                      r[c] = make_uint4(pk4[0], pk4[1], pk4[2], pk4[3]);
-                    }
-                    if (prm.out_al32) {
-                      st_global_32B(orow + q * 32, r[0], r[1]);
-                      st_global_32B(orow + q * 32 + 16, r[2], r[3]);
+                      load_own(q, o);
                     } else {
+                      tmem_ld32(o_addr + q * 32, o);
+                      tmem_wait_ld();
+                    }
 #pragma unroll
-                      for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(orow + q * 32 + c * 8) = r[c];
+                    for (int c = 0; c < 16; ++c) {
+                      float2 acc = make_float2(__uint_as_float(o[2 * c]), __uint_as_float(o[2 * c + 1]));
+                      if (i == 1) {
+                        const float2 t = __fmul2_rn(acc, inv_own2);
+                        const uint32_t own = pack_bf16(t.x, t.y);
+                        acc = __fmul2_rn(own2, make_float2(__uint_as_float(own << 16), __uint_as_float(own & 0xffff0000u)));
+                      }
+                      const uint4 aa = va[x * 4 + (c >> 2)], bb = vb[x * 4 + (c >> 2)];
+                      const uint32_t pa = (c & 3) == 0 ? aa.x : ((c & 3) == 1 ? aa.y : ((c & 3) == 2 ? aa.z : aa.w));
+                      const uint32_t pb = (c & 3) == 0 ? bb.x : ((c & 3) == 1 ? bb.y : ((c & 3) == 2 ? bb.z : bb.w));
+                      acc = ffma2(wa2, make_float2(__uint_as_float(pa << 16), __uint_as_float(pa & 0xffff0000u)), acc);
+                      acc = ffma2(wb2, make_float2(__uint_as_float(pb << 16), __uint_as_float(pb & 0xffff0000u)), acc);
+                      o[2 * c] = __float_as_uint(acc.x);
+                      o[2 * c + 1] = __float_as_uint(acc.y);
+                    }
+                    if (more) {
+                      tmem_st32(o_addr + q * 32, o);
+                    } else if (row_exists) {
+                      uint4 r[4];
+#pragma unroll
+                      for (int c = 0; c < 4; ++c) {
+                        uint32_t pk4[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                          const float2 t = __fmul2_rn(make_float2(__uint_as_float(o[8 * c + 2 * e]), __uint_as_float(o[8 * c + 2 * e + 1])), inv2);
+                          pk4[e] = any_key ? pack_bf16(t.x, t.y) : 0u;
+                        }
+                        r[c] = make_uint4(pk4[0], pk4[1], pk4[2], pk4[3]);
+                      }
+                      if (prm.out_al32) {
+                        st_global_32B(orow + q * 32, r[0], r[1]);
+                        st_global_32B(orow + q * 32 + 16, r[2], r[3]);
+                      } else {
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(orow + q * 32 + c * 8) = r[c];
+                      }
+                    }
+                  }
+                  if (kTurn < kGroups) {
+#pragma unroll
+                    for (int c = 0; c + 4 * kTurn < kGroups * 4; ++c) {
+                      va[c] = va[c + 4 * kTurn];
+                      vb[c] = vb[c + 4 * kTurn];
                     }
                   }
                 }
-                tmem_wait_st();
-                w = l_next * fast_exp2(m_next - mref);
+                if (more) {
+                  tmem_wait_st();
+                  fetch(i + 2);
+                  w_a = l_a * fast_exp2(m_a - mref);
+                  w_b = l_b * fast_exp2(m_b - mref);
+                }
               }
               if (row_exists && lse_p && !(KS && wg)) *lse_p = any_key ? (mm + log2f(lt)) / kLog2e : -INFINITY;
               tc_fence_before();

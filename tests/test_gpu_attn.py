@@ -589,7 +589,7 @@ def test_last_row_tile_in_a_launch_of_its_own(N):
 
 
 @pytest.mark.parametrize("G,N,d", [(2, 40, 64), (4, 40, 64), (2, 40, 128), (4, 40, 128)])
-@pytest.mark.parametrize("longest", [900, 2100, 6000])
+@pytest.mark.parametrize("longest", [900, 1400, 2100, 2800, 6000])
 def test_long_unit_among_many_is_cut_in_many_pieces(G, N, d, longest):
     """Too many units for clusters, one of them far longer than the rest: its pieces are two, several and many, next to
     whole units of one to three key tiles; one and two row tiles, both head widths."""
