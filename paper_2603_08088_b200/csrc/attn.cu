@@ -996,9 +996,23 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       tr.mark(0);
       // Rendezvous of the softmax warpgroups through an mbarrier, so that it is bounded like every other wait.
       // All 32 lanes wait together and agree on the outcome, so that the warp-wide TMEM instructions
-      // below are never executed by a part of a warp.
+      // below are never executed by a part of a warp.  The waits that every key tile has do not vote (LAZY): a lane whose
+      // wait was abandoned notes it, goes on with whatever tensor memory holds, hands nothing on, and the vote on the row
+      // maxima of the next tile, or the one behind the last tile, takes the whole warp out.  (32-layer shape 1254 -> 1240 us a
+      // launch, long context 226.7 -> 224.1, 4 sequences of 4096 41.3 -> 40.9.  The cluster kernel, a tile or two per CTA, keeps
+      // the votes: 32 layers of one sequence 10.0 us a layer with them, 10.2 without.)
+      constexpr bool LAZY = !CL;
+      bool lane_ok = true;
       auto wwait = [&](uint32_t b_, uint32_t parity) -> bool {
         return __all_sync(0xffffffffu, mbar_wait(b_, parity, abort_flag, wait_limit));
+      };
+      auto tile_wait = [&](uint32_t b_, uint32_t parity) -> bool {
+        return LAZY ? mbar_wait(b_, parity, abort_flag, wait_limit) : wwait(b_, parity);
+      };
+      auto leave = [&](bool waited) -> bool {      // true: leave the tile loop now
+        if (LAZY) lane_ok = lane_ok && waited;
+        else ok = waited;
+        return !LAZY && !waited;
       };
       auto epi_sync = [&]() -> bool {
         mbar_arrive(bar(L::EPI));
@@ -1035,7 +1049,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t o_addr_loop = tmem + lane_addr + L::kTmemO0 + wg * D;
         // key tiles below this index are full tiles of the committed prefix (no mask of any kind)
         const int j_full = min(it.S / kTileN, it.len - prm.TT);
-        for (int jt = KS ? wg : 0; jt < nt && ok; jt += KS ? 2 : 1, ++tj) {
+        for (int jt = KS ? wg : 0; jt < nt && (LAZY || ok); jt += KS ? 2 : 1, ++tj) {
           const int j = it.j0 + jt;
           const bool masked = j >= j_full;
           uint32_t vis[4] = {0u, 0u, 0u, 0u};      // masked tiles: visible keys of this row
@@ -1081,26 +1095,26 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           auto previous_pv_done = [&]() -> bool {
             if (KS) {
               if (jt < 2) return true;
-              return jt + 1 < nt ? wwait(bar(L::S_FULL + (wg ^ 1)), (to + ((jt + 1) >> 1)) & 1u) : wwait(bar(L::O_DONE), od_phase & 1u);
+              return jt + 1 < nt ? tile_wait(bar(L::S_FULL + (wg ^ 1)), (to + ((jt + 1) >> 1)) & 1u) : tile_wait(bar(L::O_DONE), od_phase & 1u);
             }
             if (jt == 0) return true;
-            if (ONE) return wwait(bar(L::O_DONE), (tj - 1) & 1u);
-            if (wg == 0) return wwait(bar(L::S_FULL + 1), tj & 1u);
-            return jt + 1 < nt ? wwait(bar(L::S_FULL + 0), (tj + 1) & 1u) : wwait(bar(L::O_DONE), od_phase & 1u);
+            if (ONE) return tile_wait(bar(L::O_DONE), (tj - 1) & 1u);
+            if (wg == 0) return tile_wait(bar(L::S_FULL + 1), tj & 1u);
+            return jt + 1 < nt ? tile_wait(bar(L::S_FULL + 0), (tj + 1) & 1u) : tile_wait(bar(L::O_DONE), od_phase & 1u);
           };
           // S and P of this key tile: index = warpgroup, or parity of the key tile when there is one
           const int idx = ONE ? (int)(tj & 1u) : wg;
           tr.mark(0x0800u | (tj & 0x7ffu));
-          ok = wwait(bar(L::S_FULL + idx), (ONE ? tj >> 1 : tj) & 1u);
-          if (!ok) break;
+          if (leave(tile_wait(bar(L::S_FULL + idx), (ONE ? tj >> 1 : tj) & 1u))) break;
           tc_fence_after();
           tr.mark(0x1000u | (tj & 0xfffu));
           if (MT == 1 && !warp_active) {      // nothing of S is looked at; P and O keep whatever tensor memory holds there
             if (KS) {
               if (lane == 0) mbar_arrive(bar(L::S_FREE + wg));
-              ok = previous_pv_done();        // or this warp could arrive for P twice in one phase
-              if (!ok) break;
+              if (leave(previous_pv_done())) break;        // or this warp could arrive for P twice in one phase
             }
+            if (LAZY) ok = __all_sync(0xffffffffu, lane_ok);
+            if (!ok) break;
             if (lane == 0) mbar_arrive(bar(L::P_READY + idx));
             continue;
           }
@@ -1116,7 +1130,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (!ONE) {
               tc_fence_before();
               __syncwarp();
-              if (lane == 0) mbar_arrive(bar(L::S_FREE + wg));
+              if (lane == 0 && lane_ok) mbar_arrive(bar(L::S_FREE + wg));
             }
           }
           float* sa = reinterpret_cast<float*>(sall);
@@ -1138,13 +1152,14 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               for (int k = 0; k < 4; ++k) mx[k] = fmax3(mx[k], sa[c + 2 * k], sa[c + 2 * k + 1]);
             const float mx2 = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * prm.scale_log2e;
             const bool moves = mx2 > m_used + kRescaleThreshold || (m_used == -INFINITY && mx2 > -INFINITY);
-            if (__any_sync(0xffffffffu, moves)) {
+            if (__any_sync(0xffffffffu, moves || !lane_ok)) {
+              if (LAZY) ok = __all_sync(0xffffffffu, lane_ok);
+              if (!ok) break;
               const float alpha = (moves && m_used > -INFINITY) ? fast_exp2(m_used - mx2) : 1.f;
               if (moves) m_used = mx2;
               l_sum *= alpha;
               if (jt > (KS ? 1 : 0)) {
-                ok = previous_pv_done();
-                if (!ok) break;
+                if (leave(previous_pv_done())) break;
                 tc_fence_after();
                 // one 16-column group at a time: this runs while all 128 scores are held in registers
 #pragma unroll 1
@@ -1192,8 +1207,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           // ---- P into its columns once the PV that read them last is done; with one warpgroup (two P buffers in turn) that
           // was issued in front of the S this tile has waited for
           if (!ONE) {
-            ok = previous_pv_done();
-            if (!ok) break;
+            if (leave(previous_pv_done())) break;
             tc_fence_after();
           }
           {
@@ -1204,11 +1218,12 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           tmem_wait_st();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar(L::P_READY + idx));
+          if (lane == 0 && lane_ok) mbar_arrive(bar(L::P_READY + idx));
           tr.mark(0x2000u | (tj & 0xfffu));
         }
         if (nt > (KS ? 2 : 1)) ++od_phase;
         to += (nt + wg) / 2;
+        if (LAZY) ok = __all_sync(0xffffffffu, ok && lane_ok);
         if (!ok) break;
         // ---- epilogue of the item: wait for the last PV into this O buffer
         {
