@@ -2,10 +2,9 @@
 // logits), the accelerator-safe path gather (Section 2.5 / 3.2) and greedy
 // acceptance along root-to-leaf rows (Section 2.3).
 //
-// Phase 1 (argmax_scan_kernel) streams logits[B,Nmax,V] once with 16-byte
-// streaming loads; every CTA reduces one vocabulary chunk of one row to a (value,
-// index) pair in scratch.  Phase 2 (accept_kernel), one CTA per sequence,
-// folds the chunk pairs in index order, then remaps, gathers and compares.
+// Phase 1 (argmax_stream_kernel, argmax_scan_kernel for few rows) streams logits[B,Nmax,V] once in items of 16384
+// entries of one row and reduces each to a (value, index) pair in scratch.  Phase 2 (accept_kernel), one CTA per
+// sequence, folds the item pairs in index order, then remaps, gathers and compares.
 // Ties resolve to the lowest index at every level of the reduction.
 #include "common.cuh"
 #include "logits.cuh"
@@ -17,8 +16,8 @@
 namespace {
 
 constexpr int kScanThreads = 256;
-constexpr int kVecPerThread = 8;                                   // 16-byte loads in flight per thread
-constexpr int kChunkElems = kScanThreads * kVecPerThread * 8;      // 16384 logits per CTA
+constexpr int kChunkElems = tv::kStreamItem;                       // 16384 logits per item of either scan
+static_assert(kChunkElems == kScanThreads * tv::kStreamVecs * 8, "a CTA of the short scan holds one item");
 
 struct ArgPair {
   float val;
@@ -44,14 +43,43 @@ __device__ __forceinline__ float vec8_max(const uint4& u) {
   return r == r ? r : -INFINITY;                            // an all-NaN vector can never win
 }
 
-// Persistent scan: the (row, vocabulary chunk) items are dealt round-robin to a grid of a few CTAs per SM, and a
-// CTA requests the vectors of its next item before it reduces the ones it holds, so the memory pipe never drains
-// at an item boundary.  A row of any V is read in 16-byte vectors (V = 128257, 8 x 64 rows: 107 -> 28 us a call against
-// 2-byte loads; V = 128256 takes the same 28 us).
+// Best entry among a thread's vectors, number first_vec + k stride of the row: lowest index of the largest value.
+__device__ __forceinline__ void thread_best(const uint4* u, int first_vec, int stride, int off, int V, float& best, int& best_i) {
+  best = -INFINITY;
+  best_i = 0x7fffffff;
+  int best_vec = 0;
+#pragma unroll
+  for (int k = 0; k < tv::kStreamVecs; ++k) {      // increasing index order: strict > keeps the first
+    const float m = vec8_max(u[k]);
+    if (m > best) {
+      best = m;
+      best_vec = k;
+    }
+  }
+  uint4 w = u[0];
+#pragma unroll
+  for (int k = 1; k < tv::kStreamVecs; ++k) if (best_vec == k) w = u[k];
+  const uint32_t e[4] = {w.x, w.y, w.z, w.w};
+  const int first = 8 * (first_vec + best_vec * stride) - off;      // entry of the vector's first half-word
+  best = -INFINITY;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    float f = bf16_bits_to_float((t & 1) ? (e[t >> 1] >> 16) : (e[t >> 1] & 0xffffu));
+    f = f == f ? f : -INFINITY;
+    if (first >= 0 && first <= V - 8) take_better(best, best_i, f, first + t);
+  }
+}
+
+// Both scans are persistent, and a row of any V is read in 16-byte vectors (V = 128257, 8 x 64 rows: 107 -> 28 us a call
+// against 2-byte loads; V = 128256 took the same 28 us).
 // `early` (tree_accept_behind_attn): the kernel in front is a tree_verify_attn launch, which lets this one be scheduled only
 // when everything before it has completed, and it does not write what the scan reads.  The scan then runs beside it, on
 // the SMs it leaves, and waits for it at the end: whoever waits for the scan has waited for the attention too.  A step of
-// the ragged batch (8 x 64 nodes, V = 128256) 90.5 -> 86.4 us, of one sequence with 32 KV heads 27.5 -> 25.9.
+// the ragged batch (8 x 64 nodes, V = 128256) 90.5 -> 86.4 us, of one sequence with 32 KV heads 27.5 -> 25.9
+// (with the short scan).
+//
+// Short scans: the (row, vocabulary chunk) items are dealt round-robin to a grid of a few CTAs per SM, and a CTA requests
+// the vectors of its next item before it reduces the ones it holds.
 __global__ void __launch_bounds__(kScanThreads, 3)
 argmax_scan_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict__ n_nodes,
                    int Nmax, int V, int n_chunks, int n_items, int early, ArgPair* __restrict__ partial) {
@@ -74,47 +102,26 @@ argmax_scan_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict
     const tv::LogitsRow r(logits, row, V);
     const int v0 = chunk * (kChunkElems / 8);
 #pragma unroll
-    for (int k = 0; k < kVecPerThread; ++k) u[k] = r.vector(v0 + k * kScanThreads + tid);
+    for (int k = 0; k < tv::kStreamVecs; ++k) u[k] = r.vector(v0 + k * kScanThreads + tid);
   };
 
   int item = blockIdx.x;
   int row = 0, chunk = 0;
   bool active = locate(item, row, chunk);
-  uint4 u[kVecPerThread];
+  uint4 u[tv::kStreamVecs];
   if (active) fetch(row, chunk, u);
   while (item < n_items) {
     const int nitem = item + gridDim.x;
     int nrow = 0, nchunk = 0;
     const bool nactive = locate(nitem, nrow, nchunk);
-    uint4 un[kVecPerThread];
+    uint4 un[tv::kStreamVecs];
     if (nactive) fetch(nrow, nchunk, un);
     if (active) {
       const tv::LogitsRow r(logits, row, V);
       const int v0 = chunk * (kChunkElems / 8);
-      float best = -INFINITY;
-      int best_vec = 0, best_i = 0x7fffffff;
-#pragma unroll
-      for (int k = 0; k < kVecPerThread; ++k) {      // increasing index order: strict > keeps the first
-        const float m = vec8_max(u[k]);
-        if (m > best) {
-          best = m;
-          best_vec = k;
-        }
-      }
-      {
-        uint4 w = u[0];
-#pragma unroll
-        for (int k = 1; k < kVecPerThread; ++k) if (best_vec == k) w = u[k];
-        const uint32_t e[4] = {w.x, w.y, w.z, w.w};
-        const int first = 8 * (v0 + best_vec * kScanThreads + tid) - r.off;      // entry of the vector's first half-word
-        best = -INFINITY;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          float f = bf16_bits_to_float((t & 1) ? (e[t >> 1] >> 16) : (e[t >> 1] & 0xffffu));
-          f = f == f ? f : -INFINITY;
-          if (first >= 0 && first <= V - 8) take_better(best, best_i, f, first + t);
-        }
-      }
+      float best;
+      int best_i;
+      thread_best(u, v0 + tid, kScanThreads, r.off, V, best, best_i);
       // the row's entries outside its whole vectors go with its first chunk
       if (chunk == 0 && tid < 16) {
         const int v = r.edge(tid);
@@ -150,8 +157,55 @@ argmax_scan_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict
     chunk = nchunk;
     active = nactive;
 #pragma unroll
-    for (int k = 0; k < kVecPerThread; ++k) u[k] = un[k];
+    for (int k = 0; k < tv::kStreamVecs; ++k) u[k] = un[k];
   }
+  if (early) tv::pdl_wait_only();
+}
+
+// Long scans (see stream_rows).  The eight warps of an item leave their pairs as one 64-bit key - the value, then the
+// complement of the index - in a maximum in shared memory; the last of them writes the item's pair.
+__global__ void __launch_bounds__(tv::kStreamThreads, 1)
+argmax_stream_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict__ n_nodes,
+                   int Nmax, int V, int n_chunks, int n_items, int early, ArgPair* __restrict__ partial,
+                   int32_t* __restrict__ status) {
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  else tv::pdl_enter();
+  const int lane = threadIdx.x & 31;
+  __shared__ unsigned long long s_key[tv::kStreamStages];
+  __shared__ unsigned s_count[tv::kStreamStages];
+  if (threadIdx.x < tv::kStreamStages) {
+    s_key[threadIdx.x] = 0;
+    s_count[threadIdx.x] = 0;
+  }                                        // (stream_rows starts with a barrier)
+  tv::stream_rows<false>(logits, n_nodes, Nmax, V, n_chunks, n_items, status,
+                         [&](int row, int chunk, int, int first_vec, const tv::LogitsRow& r, const uint4* u, float rest, int rest_v,
+                             int stage) {
+    float best;
+    int best_i;
+    thread_best(u, first_vec + lane, 32, r.off, V, best, best_i);
+    // the row's entries outside its whole vectors go with its first slice
+    if (rest_v >= 0) take_better(best, best_i, rest == rest ? rest : -INFINITY, rest_v);
+    // the warp's best, then the item's: a float as an unsigned number in the same order (+ 0: one key for both zeros)
+    const uint32_t bits = __float_as_uint(best + 0.f);
+    const uint32_t key = bits & 0x80000000u ? ~bits : bits | 0x80000000u;
+    const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+    const uint32_t low = __reduce_min_sync(0xffffffffu, key == top ? (uint32_t)best_i : 0x7fffffffu);
+    if (lane == 0) {
+      atomicMax(&s_key[stage], (unsigned long long)top << 32 | (uint32_t)~low);
+      __threadfence_block();
+      if (atomicAdd(&s_count[stage], 1u) == tv::kStreamWarps - 1) {
+        __threadfence_block();
+        const unsigned long long all = *reinterpret_cast<volatile unsigned long long*>(&s_key[stage]);
+        const uint32_t t = (uint32_t)(all >> 32);
+        ArgPair out;
+        out.val = __uint_as_float(t & 0x80000000u ? t & 0x7fffffffu : ~t);
+        out.idx = (int32_t)~(uint32_t)all;
+        partial[(size_t)row * n_chunks + chunk] = out;
+        s_key[stage] = 0;
+        s_count[stage] = 0;
+      }
+    }
+  });
   if (early) tv::pdl_wait_only();
 }
 
@@ -286,10 +340,10 @@ __global__ void node_scores_kernel(const tv_bf16* __restrict__ logits, const int
   scores[idx] = val;
 }
 
-int scan_chunks(int V) { return (V + kChunkElems - 1) / kChunkElems; }
-
-// CTAs of the persistent scan: three per SM (what its registers allow).
+// CTAs of the short scan: three per SM (what its registers allow).
 int scan_ctas() { return 3 * tv::sm_count(); }
+
+int scan_chunks(int V) { return (V + kChunkElems - 1) / kChunkElems; }
 
 // Scratch of tree_accept_noalloc: a fixed device array that lives in the library image, so that callers
 // who may not allocate device memory can still run the accept step.  Every GPU that loads the library
@@ -339,9 +393,17 @@ int accept_entry(const tv_bf16* logits, const int32_t* tokens, const int32_t* re
   cudaStream_t s = (cudaStream_t)stream;
   const long long n_items = (long long)B * Nmax * n_chunks;
   TV_REQUIRE(n_items < (1ll << 31), "tree_accept: B * Nmax * ceil(V / 16384) must stay below 2^31");
-  const int scan_grid = (int)(n_items < (long long)scan_ctas() ? n_items : scan_ctas());
-  TV_CUDA_OK(tv::launch_pdl(argmax_scan_kernel, dim3(scan_grid), dim3(kScanThreads), 0, s, logits, n_nodes, Nmax, V,
-                            n_chunks, (int)n_items, behind_attn ? 1 : 0, partial));
+  // The long scan from six items an SM on (us a call, short / long: 4.9 items an SM 9.0 / 8.8, 6.5 10.0 / 10.0, 10.8 13.5 /
+  // 12.3, 21.6 22.4 / 19.2, 43 38.8 / 32.1; below, its rings take longer to set up: 1.6 items 6.0 / 7.0).
+  if (n_items >= 6ll * tv::sm_count()) {
+    TV_CUDA_OK(tv::stream_configure<argmax_stream_kernel>());
+    TV_CUDA_OK(tv::launch_pdl(argmax_stream_kernel, dim3(tv::sm_count()), dim3(tv::kStreamThreads), tv::kStreamSmem, s, logits,
+                              n_nodes, Nmax, V, n_chunks, (int)n_items, behind_attn ? 1 : 0, partial, status));
+  } else {
+    const int scan_grid = (int)(n_items < (long long)scan_ctas() ? n_items : scan_ctas());
+    TV_CUDA_OK(tv::launch_pdl(argmax_scan_kernel, dim3(scan_grid), dim3(kScanThreads), 0, s, logits, n_nodes, Nmax, V,
+                              n_chunks, (int)n_items, behind_attn ? 1 : 0, partial));
+  }
   const long long staged_ints = 2ll * Nmax + (long long)P * Dp1;
   const int staged = staged_ints * 4 <= 47 * 1024 ? 1 : 0;        // what a CTA may have without asking for more
   const size_t smem = (staged ? (size_t)staged_ints : (size_t)Nmax) * sizeof(int32_t);

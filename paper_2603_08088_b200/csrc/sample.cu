@@ -6,7 +6,7 @@
 // child passes, the next token is drawn from what is left of p by inversion of the cumulative sum in
 // vocabulary order at u_bonus.  p = softmax(logits / T) of the current node's row.
 //
-// Phase 1 (row_stats_kernel) streams logits[B,Nmax,V] once: every warp reduces one vocabulary chunk of one row to
+// Phase 1 (row_stats_stream_kernel, row_stats_kernel for few rows) streams logits[B,Nmax,V] once: every warp reduces one vocabulary chunk of one row to
 // (max, sum of 2^((l - max) k)), k = log2(e) / T.  Phase 2 (sample_walk_kernel), one CTA per sequence: folds the
 // chunk pairs per row, gathers the mass of every node's token in its parent's row, walks the tree with one warp, and
 // draws the next token from the last node's row by two scans in vocabulary order: over the masses of its chunks, then
@@ -19,8 +19,7 @@
 namespace {
 
 constexpr int kStatThreads = 256;
-constexpr int kStatVecs = 8;                                          // 16-byte loads in flight per lane
-constexpr int kStatChunk = 32 * kStatVecs * 8;                        // 2048 logits per warp and item
+constexpr int kStatChunk = tv::kStreamSlice;                          // 2048 logits: a warp's share of an item
 constexpr int kWalkThreads = 1024;
 constexpr int kLanesPerRow = 8;                                       // lanes that fold one row's chunk pairs
 constexpr int kMaxNodes = 256;
@@ -54,12 +53,59 @@ __device__ __forceinline__ void merge_pair(float& m, float& s, float mo, float s
   }
 }
 
-// Persistent scan, one warp per (row, chunk) item, no barrier anywhere: a warp requests the vectors of its next item
-// before it reduces the ones it holds, takes the chunk's maximum first (packed bf16) and then one exponential per
-// logit.  Bounds: the logits once through HBM (295 MB: 45 us), one special-function result per logit (147 M: 32 us).
-// Chunks of 2048 per warp, three CTAs an SM: with one chunk of 8192 per CTA and a block reduction this kernel took 99 us,
-// with two CTAs an SM a call takes 2 us more, with four loads a lane and four CTAs 7 us more; 128.6 -> 65.6 us a call,
-// both kernels (16 x 60 rows of 153600).
+// (max, sum) of a chunk whose vectors a converged warp holds, with one more entry in some lanes (-inf: none): the maximum
+// first (packed bf16), then one exponential per logit.
+__device__ __forceinline__ RowStat chunk_stat(const uint4* u, float rest, float k) {
+  __nv_bfloat162 mx = *reinterpret_cast<const __nv_bfloat162*>(&u[0].x);
+#pragma unroll
+  for (int q = 0; q < tv::kStreamVecs; ++q) {
+    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u[q]);
+    mx = __hmax2(mx, __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3])));
+  }
+  RowStat out;
+  out.s = 0.f;
+  out.m = fmaxf(fmaxf(__low2float(mx), __high2float(mx)), rest);      // max of a NaN and x is x: only NaNs give a NaN
+  if (!(out.m == out.m)) out.m = -INFINITY;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) out.m = fmaxf(out.m, __shfl_xor_sync(0xffffffffu, out.m, off));
+  if (out.m > -INFINITY) {
+    const float2 k2 = make_float2(k, k), mk2 = make_float2(-out.m * k, -out.m * k);
+    float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < tv::kStreamVecs; ++q) {
+      const uint32_t e[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        float2 x = __ffma2_rn(make_float2(__uint_as_float(e[t] << 16), __uint_as_float(e[t] & 0xffff0000u)), k2, mk2);
+        x.x = ex2_approx(fmaxf(x.x, -150.f));
+        x.y = ex2_approx(fmaxf(x.y, -150.f));
+        sum = __fadd2_rn(sum, x);
+      }
+    }
+    out.s = sum.x + sum.y + mass_of(rest, out.m, k);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) out.s += __shfl_xor_sync(0xffffffffu, out.s, off);
+  }
+  return out;
+}
+
+// Long scans (see stream_rows).  Bounds: the logits once through HBM (295 MB: 45 us), one special-function result per
+// logit (147 M: 33 us).
+__global__ void __launch_bounds__(tv::kStreamThreads, 1)
+row_stats_stream_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict__ n_nodes, int Nmax, int V, int n_chunks,
+                        int row_items, int n_items, float k, RowStat* __restrict__ stats, int32_t* __restrict__ status) {
+  tv::pdl_enter();
+  tv::stream_rows<true>(logits, n_nodes, Nmax, V, row_items, n_items, status,
+                        [&](int row, int item, int w, int, const tv::LogitsRow&, const uint4* u, float rest, int, int) {
+    const int chunk = item * tv::kStreamWarps + w;
+    if (chunk >= n_chunks) return;
+    const RowStat out = chunk_stat(u, rest, k);
+    if ((threadIdx.x & 31) == 0) stats[(size_t)row * n_chunks + chunk] = out;
+  });
+}
+
+// Short scans: persistent, one warp per (row, chunk) item, no barrier anywhere; a warp requests the vectors of its next item
+// before it reduces the ones it holds.
 __global__ void __launch_bounds__(kStatThreads, 3)
 row_stats_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict__ n_nodes, int Nmax, int V,
                  int n_chunks, int n_items, float k, RowStat* __restrict__ stats) {
@@ -76,26 +122,20 @@ row_stats_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict__
   auto fetch = [&](int row, int chunk, uint4* u) {
     const tv::LogitsRow r(logits, row, V);
 #pragma unroll
-    for (int q = 0; q < kStatVecs; ++q) u[q] = r.vector((chunk * kStatVecs + q) * 32 + lane);
+    for (int q = 0; q < tv::kStreamVecs; ++q) u[q] = r.vector((chunk * tv::kStreamVecs + q) * 32 + lane);
   };
   int item = blockIdx.x * (kStatThreads / 32) + (threadIdx.x >> 5);
   int row = 0, chunk = 0;
   bool active = locate(item, row, chunk);
-  uint4 u[kStatVecs];
+  uint4 u[tv::kStreamVecs];
   if (active) fetch(row, chunk, u);
   while (item < n_items) {
     const int nitem = item + n_warps;
     int nrow = 0, nchunk = 0;
     const bool nactive = locate(nitem, nrow, nchunk);
-    uint4 un[kStatVecs];
+    uint4 un[tv::kStreamVecs];
     if (nactive) fetch(nrow, nchunk, un);
     if (active) {
-      __nv_bfloat162 mx = *reinterpret_cast<const __nv_bfloat162*>(&u[0].x);
-#pragma unroll
-      for (int q = 0; q < kStatVecs; ++q) {
-        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u[q]);
-        mx = __hmax2(mx, __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3])));
-      }
       // entries outside the row's whole vectors, in the chunk they lie in
       float rest = -INFINITY;
       if (lane < 16 && (chunk == 0 || chunk >= n_chunks - 2)) {
@@ -103,42 +143,15 @@ row_stats_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict__
         const int v = r.edge(lane);
         if (v >= 0 && (v + r.off) / kStatChunk == chunk) rest = bf16_to_float(r.row[v]);
       }
-      float m = fmaxf(fmaxf(__low2float(mx), __high2float(mx)), rest);      // max of a NaN and x is x: only NaNs give a NaN
-      if (!(m == m)) m = -INFINITY;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-      float s = 0.f;
-      if (m > -INFINITY) {
-        const float2 k2 = make_float2(k, k), mk2 = make_float2(-m * k, -m * k);
-        float2 sum = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int q = 0; q < kStatVecs; ++q) {
-          const uint32_t e[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            float2 x = __ffma2_rn(make_float2(__uint_as_float(e[t] << 16), __uint_as_float(e[t] & 0xffff0000u)), k2, mk2);
-            x.x = ex2_approx(fmaxf(x.x, -150.f));
-            x.y = ex2_approx(fmaxf(x.y, -150.f));
-            sum = __fadd2_rn(sum, x);
-          }
-        }
-        s = sum.x + sum.y + mass_of(rest, m, k);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-      }
-      if (lane == 0) {
-        RowStat out;
-        out.m = m;
-        out.s = s;
-        stats[(size_t)row * n_chunks + chunk] = out;
-      }
+      const RowStat out = chunk_stat(u, rest, k);
+      if (lane == 0) stats[(size_t)row * n_chunks + chunk] = out;
     }
     item = nitem;
     row = nrow;
     chunk = nchunk;
     active = nactive;
 #pragma unroll
-    for (int q = 0; q < kStatVecs; ++q) u[q] = un[q];
+    for (int q = 0; q < tv::kStreamVecs; ++q) u[q] = un[q];
   }
 }
 
@@ -391,14 +404,22 @@ extern "C" int tree_accept_sample(const tv_bf16* logits, const int32_t* tokens, 
   const float k = kLog2e / temperature;
   RowStat* stats = static_cast<RowStat*>(workspace);
   cudaStream_t s = (cudaStream_t)stream;
-  const long long n_items = (long long)B * Nmax * n_chunks;
-  TV_REQUIRE(n_items < (1ll << 31) - (1 << 20), "tree_accept_sample: B * Nmax * ceil(V / 2048) must stay below 2^31");
-  constexpr int kWarps = kStatThreads / 32;
-  const int resident = 3 * tv::sm_count();
-  const long long want = (n_items + kWarps - 1) / kWarps;
-  const int grid = (int)(want < resident ? want : resident);
-  TV_CUDA_OK(tv::launch_pdl(row_stats_kernel, dim3(grid), dim3(kStatThreads), 0, s, logits, n_nodes, Nmax, V, n_chunks,
-                            (int)n_items, k, stats));
+  const int row_items = (n_chunks + tv::kStreamWarps - 1) / tv::kStreamWarps;
+  const long long n_slices = (long long)B * Nmax * n_chunks, n_items = (long long)B * Nmax * row_items;
+  TV_REQUIRE(n_slices < (1ll << 31) - (1 << 20), "tree_accept_sample: B * Nmax * ceil(V / 2048) must stay below 2^31");
+  // The long scan from 24 items an SM on (us a call, short / long: 13.8 items an SM 22.3 / 23.2, 21.6 29.1 / 29.3, 43 47.1 / 46.2,
+  // 65 68.7 / 63.3): its 800 threads an SM keep the walk from being scheduled beside it.
+  if (n_items >= 24ll * tv::sm_count()) {
+    TV_CUDA_OK(tv::stream_configure<row_stats_stream_kernel>());
+    TV_CUDA_OK(tv::launch_pdl(row_stats_stream_kernel, dim3(tv::sm_count()), dim3(tv::kStreamThreads), tv::kStreamSmem, s, logits,
+                              n_nodes, Nmax, V, n_chunks, row_items, (int)n_items, k, stats, status));
+  } else {
+    constexpr int kWarps = kStatThreads / 32;
+    const int resident = 3 * tv::sm_count();
+    const long long want = (n_slices + kWarps - 1) / kWarps;
+    TV_CUDA_OK(tv::launch_pdl(row_stats_kernel, dim3((int)(want < resident ? want : resident)), dim3(kStatThreads), 0, s, logits,
+                              n_nodes, Nmax, V, n_chunks, (int)n_slices, k, stats));
+  }
   TV_CUDA_OK(tv::launch_pdl(sample_walk_kernel, dim3(B), dim3(kWalkThreads), 0, s, logits, stats, n_chunks, tokens, parent,
                             n_nodes, u_node, u_bonus, k, Nmax, V, Dp1, accept_len, accepted_nodes, next_token, status));
   tv::count_launches(2);

@@ -247,16 +247,17 @@ def test_commit_launch_shapes_byte_exact(layout, L, B, Hkv, d, Dp1):
         assert np.array_equal(got.view(torch.int16).cpu().numpy().view(np.uint16), want)
 
 
+@pytest.mark.parametrize("B,N", [(3, 13), (12, 80)])
 @pytest.mark.parametrize("V", [1, 7, 8, 9, 16383, 16385, 16391, 32777])
-def test_argmax_vocabularies_around_vector_and_chunk_edges(V):
-    """Rows that start anywhere inside a 16-byte vector: ties and maxima on the first and last entries included."""
+def test_argmax_vocabularies_around_vector_and_chunk_edges(V, B, N):
+    """Rows that start anywhere inside a 16-byte vector: ties and maxima on the first and last entries included; few rows
+    and so many that the long scan takes them."""
     g = torch.Generator().manual_seed(V)
-    B, N = 3, 13
     logits = torch.randint(-3, 4, (B, N, V), generator=g).to(torch.bfloat16)
     for i in range(N):
         logits[:, i, (0 if i % 3 == 0 else V - 1 if i % 3 == 1 else V // 2)] = 4.0
     logits[0, 2] = float("-inf")
-    n = torch.tensor([N, 5, N], dtype=torch.int32, device="cuda")
+    n = torch.tensor([N, 5, N] * (B // 3), dtype=torch.int32, device="cuda")
     z = lambda *s: torch.zeros(s, dtype=torch.int32, device="cuda")
     am, st = z(B, N), z(B)
     ws = torch.zeros(max(16, tv.tv_accept_workspace_bytes(B, N, V)), dtype=torch.uint8, device="cuda")

@@ -178,3 +178,10 @@ def test_vocabularies_around_the_chunk_and_vector_edges(V):
     """Rows whose start lies anywhere inside a 16-byte vector, chunks of 2048 entries with every kind of remainder."""
     lt, tokens, parent, n, u_node, u_bonus = make_inputs(70 + V, 6, 17, 5, V, ragged=True)
     check(lt, tokens, parent, n, u_node, u_bonus, 1.0, 6, min_fraction=0.5)
+
+
+@pytest.mark.parametrize("V", [43, 2049, 6145, 16379])
+def test_long_scans_around_the_slice_and_vector_edges(V):
+    """So many rows that the long scan takes them, padded nodes among them."""
+    lt, tokens, parent, n, u_node, u_bonus = make_inputs(90 + V, 64, 60, 5, V, ragged=True)
+    check(lt, tokens, parent, n, u_node, u_bonus, 1.0, 6, min_fraction=0.5)
