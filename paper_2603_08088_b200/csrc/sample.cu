@@ -6,9 +6,9 @@
 // child passes, the next token is drawn from what is left of p by inversion of the cumulative sum in
 // vocabulary order at u_bonus.  p = softmax(logits / T) of the current node's row.
 //
-// Phase 1 (row_stats_stream_kernel, row_stats_kernel for few rows) streams logits[B,Nmax,V] once: every warp reduces one vocabulary chunk of one row to
-// (max, sum of 2^((l - max) k)), k = log2(e) / T.  Phase 2 (sample_walk_kernel), one CTA per sequence: folds the
-// chunk pairs per row, gathers the mass of every node's token in its parent's row, walks the tree with one warp, and
+// Phase 1 (row_stats_stream_kernel, row_stats_kernel for few rows) streams logits[B,Nmax,V] once: every warp reduces one
+// vocabulary chunk of one row to (max, sum of 2^((l - max) k)), k = log2(e) / T.  Phase 2 (sample_walk_kernel), one CTA per
+// sequence: folds the chunk pairs per row, gathers the mass of every node's token in its parent's row, walks the tree with one warp, and
 // draws the next token from the last node's row by two scans in vocabulary order: over the masses of its chunks, then
 // over the entries of the chunk that holds the target.  All arithmetic in fp32.
 #include "common.cuh"
