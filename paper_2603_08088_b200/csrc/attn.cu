@@ -83,6 +83,12 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 #define TV_SETUP_COST 4
 #endif
 constexpr int kSetupCost = TV_SETUP_COST;
+// K/V tiles that a CTA asks for in L2 while the kernel in front is still running.  16 sequences of 512 to 4096, layer after
+// layer: 48.6 us a launch with none, 47.7 with 2, 47.9 with 4, 48.6 with 8 (they take their bandwidth from that kernel's tail).
+#ifndef TV_PREFETCH_TILES
+#define TV_PREFETCH_TILES 2
+#endif
+constexpr int kPrefetchTiles = TV_PREFETCH_TILES;
 constexpr int kMaxGroups = 160;
 // do not spread a small problem over more CTA groups than this allows (measured on the 7B-shaped single
 // sequence: 12 -> 26 us, 6 -> 22 us, 4 -> 23 us per launch)
@@ -151,6 +157,16 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 // this grid has got here or has exited.
 __device__ __forceinline__ void gdc_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void gdc_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Asks for a tile of a tensor in L2.
+__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* map, int c0, int c1, int c2, int c3) {
+  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+               : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_5d(const CUtensorMap* map, int c0, int c1, int c2, int c3, int c4) {
+  asm volatile("cp.async.bulk.prefetch.tensor.5d.L2.global.tile [%0, {%1, %2, %3, %4, %5}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2),
+               "r"(c3), "r"(c4)
+               : "memory");
+}
 // One lane of a converged warp (the compiler keeps what it guards in the uniform datapath).
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
@@ -394,6 +410,7 @@ struct AttnParams {
   unsigned long long wait_limit_ns;   // limit of every bounded wait
   int debug;                     // bit 0: the producer issues no copy at all; bit 1: pieces of cut units store their
                                  // partials but never announce them (both exercise the expiry of a bounded wait);
+                                 // bit 3: the guessed table is built from lengths one tile too long;
                                  // bit 2: the K/V stream alone - the issuing warp only hands every slot back as
                                  // soon as it is full, no MMA, no softmax, no output (what the memory side can do)
   int L;                         // layers in this launch: their units form one tile space, layer after layer
@@ -444,7 +461,7 @@ struct SmemLayout {
   static constexpr int kTmemS1 = (D == 128 && MT == 2) ? kTmemS0 : 384;
   static constexpr int kMisc = kBars + NBARS * 8;          // tmem ptr, abort flag, announcement (see PIECE)
   static constexpr int kItems = kMisc + 16;                // the producer's current and next item (see publish)
-  static constexpr int kCum = kItems + 2 * 32;
+  static constexpr int kCum = kItems + 3 * 32 + 16;
   static constexpr int kGs = kCum + (kMaxB + 1) * 4;
   static constexpr int kXch = (kGs + (kMaxGroups + 1) * 4 + 7) & ~7;      // KS: (m, l) of both warpgroups' rows
   static constexpr bool kKeySplit = MT == 1 && D == 64;
@@ -514,91 +531,25 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // Without the caller's promise nothing of the problem is read before every earlier kernel of the stream has
-  // finished (a kernel in front may still be writing prefix_len, and lines of it cached by an earlier launch on
-  // this SM are only dropped by the wait).  The cluster kernel has no table to build: its roles wait where they read.
-  if (!CL && !prm.early) gdc_wait();
-  if (!CL && warp == 0) {
-    int run = 0;
-#pragma unroll 1
-    for (int base = 0; base < prm.B; base += 32) {
-      const int b = base + lane;
-      int len = 0;
-      if (b < prm.B) {
-        int S = prm.prefix_len[b];
-        S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
-        len = (S + kTileN - 1) / kTileN + prm.TT + kSetupCost;
-      }
-      int inc = len;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-      }
-      if (b < prm.B) cum[b] = run + inc - len;
-      run += __shfl_sync(0xffffffffu, inc, 31);
-    }
-    if (lane == 0) cum[prm.B] = run;
-  }
   tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  // Small problems use fewer CTA groups, so that a unit is cut into few pieces (each piece costs a partial
-  // write and a merge) and every group still gets a worthwhile share of tiles.
-  int groups = 1;
-  if (!CL) {
-    const unsigned total = (unsigned)(prm.Hkv * cum[prm.B]) * (unsigned)prm.L;
-    const unsigned want = total / (unsigned)kMinVirtualTilesPerGroup;
-    groups = want < 1u ? 1 : (want < (unsigned)prm.groups ? (int)want : prm.groups);
-    // A group count just above a multiple of the unit count is rounded down to it: with units of equal length
-    // (one sequence, all heads) every unit is then cut into the same number of equal pieces and no cut falls
-    // just behind a unit boundary.  Not worth more than 1/16 of the groups.
-    {
-      const int units = prm.B * prm.Hkv * prm.L, over = groups % units;
-      if (groups > units && over * 16 <= groups) groups -= over;
-    }
-    // gs[k] = floor(total * k / groups) in 32-bit arithmetic: total = q * groups + r
-    const unsigned q = total / (unsigned)groups, r = total % (unsigned)groups;
-#pragma unroll 1
-    for (int k = threadIdx.x; k <= prm.groups; k += kThreads)
-      gs[k] = k <= groups ? (int)(k * q + (k * r) / (unsigned)groups) : (int)total;
-  }
-  if (!CL) __syncthreads();
-
-  const int per_layer = CL ? 0 : prm.Hkv * cum[prm.B];
-  Sched sch{cum, gs, prm.B, prm.Hkv, per_layer * prm.L, per_layer};
-  // Downwards over the block index (see "Work split"); groups past the last used one get an empty range, and the CTAs
-  // that are started first (on SMs the kernel in front does not use) get work.
-  const int unit = CL ? (int)(blockIdx.x / cluster_size_x()) : 0;      // cluster kernel: (layer, sequence, KV head, pair)
-  const int place = (int)(blockIdx.x / prm.NP);
-  const int group = place < groups ? groups - 1 - place : place;
-  const int pair = CL ? unit % prm.NP : (int)(blockIdx.x % prm.NP);
-  const int g_begin = CL ? 0 : sch.group_start(group, groups);
-  const int g_end = CL ? 1 : sch.group_start(group + 1, groups);
+  // Without the caller's promise nothing of the problem counts before every earlier kernel has finished (a kernel in front may
+  // still be writing prefix_len, and lines of it cached by an earlier launch on this SM are only dropped by the wait).  This
+  // kernel is resident long before that, on SMs that the one in front has left, so it goes by what prefix_len says now, builds
+  // the table, asks for the first K/V tiles of its range in L2, and after the wait compares: only if a length has
+  // changed the table is built again (layers behind one another as above: 50.1 -> 47.8 us a launch, the first S is there 3.5 us
+  // after the wait and not 5; a member of a context split 41.2 -> 40.7; 64-wide heads, one row tile, 16 sequences of 8000,
+  // 24 nodes: 62.8 -> 63.6).  What is asked for in L2 is right whoever writes it until the wait.  The cluster
+  // kernel has no table to build: its roles wait where they read.
+  bool guess = !CL && !prm.early;
+  Sched sch{cum, gs, prm.B, prm.Hkv, 0, 0};
+  int groups = 1, group = 0, g_begin = 0, g_end = 1;
 
   // Walks the items of this CTA's range (producer warp).  It publishes every item to the other roles through shared
   // memory, in front of the arrival on Q_FULL that they wait for; entries are used in turn, and an item is published only
-  // when the softmax warps have read the one before (a parity wait cannot tell phases two apart).  (Walking in every role cost each of them a division, a search and two L2 round trips per item: about
-  // 1.5 us between the epilogue of an item and its successor's first tile.)
-  auto next_item = [&](int& g, Item& it) -> bool {
-    if (CL) {                      // one item: this CTA's share of the key tiles of its cluster's unit (may be empty)
-      if (g > 0) return false;
-      g = 1;
-      const int u = unit / prm.NP;
-      it.hk = u % prm.Hkv;
-      it.b = u / prm.Hkv % prm.B;
-      it.layer = u / prm.Hkv / prm.B;
-      int S = prm.prefix_len[it.b];
-      it.S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
-      int n = prm.n_nodes[it.b];
-      it.n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
-      it.len = (it.S + kTileN - 1) / kTileN + prm.TT;
-      const int size = (int)cluster_size_x(), rank = (int)(blockIdx.x % size);
-      it.j0 = it.len * rank / size;
-      it.j1 = it.len * (rank + 1) / size;
-      return it.j1 > it.j0;
-    }
+  // when the softmax warps have read the one before (a parity wait cannot tell phases two apart).  (Walking in every role
+  // cost each of them a division, a search and two L2 round trips per item: about 1.5 us between the epilogue of an item and its
+  // successor's first tile.)  locate: from the table alone, all but S and n.
+  auto locate = [&](int& g, Item& it) -> bool {
     while (g < g_end) {
       const int layer = (int)((unsigned)g / (unsigned)sch.per_layer);
       const int gl = g - layer * sch.per_layer;                   // place inside the layer
@@ -619,13 +570,146 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       it.j0 = j0;
       it.j1 = j1;
       it.len = lenv - kSetupCost;
-      int S = prm.prefix_len[b];
-      it.S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
-      int n = prm.n_nodes[b];
-      it.n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
       return true;
     }
     return false;
+  };
+  // one warp: Q and the first prefix tiles of this CTA's first item, a box per lane and turn, in the order of their use
+  // (items[2]: that item; at[0]: it is there; at[1]: where the search goes on; at[2]: CTA groups)
+  volatile int* at = reinterpret_cast<volatile int*>(items + 3);
+  auto prefetch_first = [&]() {
+    Item first;
+    int g_first = g_begin;
+    const bool have = locate(g_first, first);
+    if (lane == 0) {
+      at[0] = have;
+      at[1] = g_first;
+      items[2] = first;
+    }
+    __syncwarp();
+    if (!have) return;
+    constexpr int kBoxes = 2 * (D / 64), kQBoxes = MT * (D / 64);
+    const int tiles = min(min(first.j1, first.len - prm.TT) - first.j0, kPrefetchTiles);
+    for (int x = lane; x < kQBoxes + tiles * kBoxes; x += 32) {
+      if (x < kQBoxes) {
+        tma_prefetch_5d(&map_q, x % (D / 64) * 64, first.hk * prm.G, (prm.tile0 + (int)(blockIdx.x % prm.NP) * MT + x / (D / 64)) * prm.NPT, first.b, first.layer);
+        continue;
+      }
+      const int y = x - kQBoxes, j = first.j0 + y / kBoxes, kv = y % kBoxes / (D / 64), h = y % (D / 64);
+      int row0 = j * kTileN, slab = first.b * prm.Hkv + first.hk;
+      if (prm.block_table) {
+        const int pg = __ldcg(prm.block_table + (size_t)first.b * prm.max_blocks + j);
+        if ((unsigned)pg >= (unsigned)prm.n_pages) continue;
+        row0 = 0;
+        slab = pg * prm.Hkv + first.hk;
+      }
+      tma_prefetch_4d(kv ? &map_vc : &map_kc, h * 64, row0, slab, first.layer);
+    }
+    __syncwarp();
+  };
+
+  while (!CL) {
+    if (warp == 0) {
+      int run = 0;
+#pragma unroll 1
+      for (int base = 0; base < prm.B; base += 32) {
+        const int b = base + lane;
+        int len = 0;
+        if (b < prm.B) {
+          int S = !guess ? prm.prefix_len[b] : __ldcg(prm.prefix_len + b) + (prm.debug & 8 ? kTileN : 0);
+          S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
+          len = (S + kTileN - 1) / kTileN + prm.TT + kSetupCost;
+        }
+        int inc = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += t;
+        }
+        if (b < prm.B) cum[b] = run + inc - len;
+        run += __shfl_sync(0xffffffffu, inc, 31);
+      }
+      if (lane == 0) cum[prm.B] = run;
+    }
+    __syncthreads();
+    // Small problems use fewer CTA groups, so that a unit is cut into few pieces (each piece costs a partial
+    // write and a merge) and every group still gets a worthwhile share of tiles.
+    const unsigned total = (unsigned)(prm.Hkv * cum[prm.B]) * (unsigned)prm.L;
+    const unsigned want = total / (unsigned)kMinVirtualTilesPerGroup;
+    groups = want < 1u ? 1 : (want < (unsigned)prm.groups ? (int)want : prm.groups);
+    // A group count just above a multiple of the unit count is rounded down to it: with units of equal length
+    // (one sequence, all heads) every unit is then cut into the same number of equal pieces and no cut falls
+    // just behind a unit boundary.  Not worth more than 1/16 of the groups.
+    {
+      const int units = prm.B * prm.Hkv * prm.L, over = groups % units;
+      if (groups > units && over * 16 <= groups) groups -= over;
+    }
+    // gs[k] = floor(total * k / groups) in 32-bit arithmetic: total = q * groups + r
+    const unsigned q = total / (unsigned)groups, r = total % (unsigned)groups;
+#pragma unroll 1
+    for (int k = threadIdx.x; k <= prm.groups; k += kThreads)
+      gs[k] = k <= groups ? (int)(k * q + (k * r) / (unsigned)groups) : (int)total;
+    if (threadIdx.x == 0) at[2] = groups;
+    __syncthreads();
+    sch.per_layer = prm.Hkv * cum[prm.B];
+    sch.total = sch.per_layer * prm.L;
+    // Downwards over the block index (see "Work split"); groups past the last used one get an empty range, and the CTAs
+    // that are started first (on SMs the kernel in front does not use) get work.
+    const int place = (int)(blockIdx.x / prm.NP);
+    group = place < groups ? groups - 1 - place : place;
+    g_begin = sch.group_start(group, groups);
+    g_end = sch.group_start(group + 1, groups);
+    if (!guess) break;
+    if (warp == 0) prefetch_first();
+    gdc_wait();
+    bool changed = false;
+    if (warp == 0 && at[0]) {
+      const int b = items[2].b;
+      const int S = prm.prefix_len[b], n = prm.n_nodes[b];
+      __syncwarp();
+      if (lane == 0) {
+        items[2].S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
+        items[2].n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
+      }
+    }
+#pragma unroll 1
+    for (int b = threadIdx.x; b < prm.B; b += kThreads) {
+      int S = prm.prefix_len[b];
+      S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
+      changed |= (S + kTileN - 1) / kTileN + prm.TT + kSetupCost != cum[b + 1] - cum[b];
+    }
+    guess = false;
+    if (!__syncthreads_or(changed)) break;
+    if (threadIdx.x == 0) at[0] = 0;
+  }
+  if (CL) __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  const int unit = CL ? (int)(blockIdx.x / cluster_size_x()) : 0;      // cluster kernel: (layer, sequence, KV head, pair)
+  const int pair = CL ? unit % prm.NP : (int)(blockIdx.x % prm.NP);
+  auto next_item = [&](int& g, Item& it) -> bool {
+    if (CL) {                      // one item: this CTA's share of the key tiles of its cluster's unit (may be empty)
+      if (g > 0) return false;
+      g = 1;
+      const int u = unit / prm.NP;
+      it.hk = u % prm.Hkv;
+      it.b = u / prm.Hkv % prm.B;
+      it.layer = u / prm.Hkv / prm.B;
+      const int S = prm.prefix_len[it.b], n = prm.n_nodes[it.b];
+      it.S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
+      it.n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
+      it.len = (it.S + kTileN - 1) / kTileN + prm.TT;
+      const int size = (int)cluster_size_x(), rank = (int)(blockIdx.x % size);
+      it.j0 = it.len * rank / size;
+      it.j1 = it.len * (rank + 1) / size;
+      return it.j1 > it.j0;
+    }
+    if (!locate(g, it)) return false;
+    const int S = prm.prefix_len[it.b], n = prm.n_nodes[it.b];
+    it.S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
+    it.n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
+    return true;
   };
 
   constexpr uint32_t kIdescQK = instr_desc(kTileN, false);
@@ -680,7 +764,13 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         __syncwarp();
       };
       if (!prm.early) sync_with_predecessor();
-      while (ok && next_item(g, it)) {
+      bool have_first = !CL && !prm.early && at[0];
+      if (have_first) {
+        g = at[1];
+        it = items[2];
+      }
+      while (ok && (have_first || next_item(g, it))) {
+        have_first = false;
         ok = mbar_wait(bar(L::Q_EMPTY), (item_idx & 1) ^ 1, abort_flag, wait_limit);
         if (!ok) break;
         tr.mark(0x1000u | item_idx);
@@ -1346,7 +1436,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // The unit's real tiles occupy [real0, uend) of the virtual tile space.  CTA groups k_first..k_last
             // hold them, one piece each (a group between the two lies wholly inside the unit), and this CTA's
             // group is one of them: two short walks over the cut table find both ends.
-            const int real0 = it.layer * sch.per_layer + prm.Hkv * cum[it.b] + it.hk * (it.len + kSetupCost) + kSetupCost;
+            const int place = (int)(blockIdx.x / prm.NP), groups = at[2];      // (read here: registers are short in the loop)
+            const int group = place < groups ? groups - 1 - place : place;
+            const int real0 = it.layer * (prm.Hkv * cum[prm.B]) + prm.Hkv * cum[it.b] + it.hk * (it.len + kSetupCost) + kSetupCost;
             const int uend = real0 + it.len;
             int k_first = group, k_last = group;
             while (gs[k_first] > real0) --k_first;

@@ -602,3 +602,30 @@ def test_long_unit_among_many_is_cut_in_many_pieces(G, N, d, longest):
     assert_attention_close(out, lse, ref_out, ref_lse, f"longest={longest}")
     out2, lse2, _, _ = gpu_attention(dcase)
     assert torch.equal(out, out2) and torch.equal(lse, lse2)
+
+
+@pytest.mark.parametrize("G,N,d", [(2, 40, 64), (4, 40, 64), (2, 40, 128), (4, 40, 128)])
+def test_lengths_that_change_under_the_waiting_launch(G, N, d):
+    """The tile table is built from the lengths a launch finds before the kernel in front is done, and again when they have
+    changed: by a switch that makes every guess one key tile too long, and by a kernel in front that writes them."""
+    cfg = CONFIGS[0].scaled(B=80, Hq=G, Hkv=1, d=d, S_lo=0, S_hi=700, Scap=1400, N=N, D=6, V=0, tree="uniform")
+    case = make_case(cfg, seed=91 + G + d, ragged_nodes=True, with_logits=False)
+    dcase = to_device(case)
+    out, lse, bits, dense = gpu_attention(dcase)
+    ref_out, ref_lse = oracle_attention(case_to_numpy(case), dense.cpu().numpy())
+    assert_attention_close(out, lse, ref_out, ref_lse, "settled lengths")
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(80, N, G, 1, d, 1400), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(80, dtype=torch.int32, device="cuda")
+    args = (dcase["q"][0], dcase["k_cache"][0], dcase["v_cache"][0], dcase["k_tree"][0], dcase["v_tree"][0])
+    got, got_lse = torch.zeros_like(out), torch.zeros_like(lse)
+    tv.tv_debug_attn_expire(*args, dcase["prefix_len"], dcase["n_nodes"], bits, d ** -0.5, got, ws, status, 2_000_000_000, 8,
+                            lse=got_lse)
+    assert torch.equal(got, out) and torch.equal(got_lse, lse)
+    lengths = torch.zeros_like(dcase["prefix_len"])
+    for other in (0, 1400, 333):
+        lengths.fill_(other)
+        tv.tree_verify_attn(*args, lengths, dcase["n_nodes"], bits, d ** -0.5, got, ws, status, lse=got_lse)
+        lengths.copy_(dcase["prefix_len"])
+        tv.tree_verify_attn(*args, lengths, dcase["n_nodes"], bits, d ** -0.5, got, ws, status, lse=got_lse)
+        assert torch.equal(got, out) and torch.equal(got_lse, lse), other
+    assert not status.any()
