@@ -69,12 +69,6 @@ constexpr int kThreads = 384;
 constexpr int kMaxB = 512;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleThreshold = 8.0f;            // in log2 units
-// Of every 16 element pairs of the softmax fast path, three take 2^x on the FMA pipe (measured optimum between
-// the special-function unit and the FMA pipe: 2/16 and 4/16 are 1-2 % slower on the 32-layer and the
-// long-context shape, 1/16 and 5/16 far slower).
-#ifndef TV_POLY_SEL
-#define TV_POLY_SEL(i) ((((i) & 7) == 3) || (((i) & 15) == 7))
-#endif
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 // Virtual tiles charged per unit by the scheduler: what a CTA pays for one more item (epilogue, masked tiles, refill) is
 // some 5 us, three to four tiles' time.  Eight shapes, one and 32 layers a launch: 4 is 1 to 3 % faster than 2 and 1 to 2 %
@@ -338,25 +332,6 @@ struct Tracer {
 // Packed fp32 pair arithmetic (one issue slot for two lanes of work).
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 fadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-// 2^x for a pair on the FMA pipe (the special-function unit is the scarce resource of the softmax):
-// x = n + f with n = round(x), f in [-0.5, 0.5]; 2^f by a cubic (relative error 7.5e-5, far below the
-// bf16 rounding of P), 2^n by an add into the exponent field.  x is raised to -125 where it lies below; the lazy
-// rescale bounds it above.
-__device__ __forceinline__ float2 exp2_poly2(float2 x) {
-  x.x = fmaxf(x.x, -125.f);
-  x.y = fmaxf(x.y, -125.f);
-  const float2 t = fadd2(x, make_float2(12582912.f, 12582912.f));          // 1.5 * 2^23: low mantissa bits = n
-  const float2 n = fadd2(t, make_float2(-12582912.f, -12582912.f));
-  const float2 f = ffma2(n, make_float2(-1.f, -1.f), x);
-  float2 p = ffma2(f, make_float2(0.0551716685f, 0.0551716685f), make_float2(0.2426111251f, 0.2426111251f));
-  p = ffma2(p, f, make_float2(0.6932609677f, 0.6932609677f));
-  p = ffma2(p, f, make_float2(0.9999280572f, 0.9999280572f));
-  float2 r;
-  r.x = __int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23));
-  r.y = __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23));
-  return r;
-}
-
 // Three-operand maximum (one instruction on sm_100); a NaN operand is ignored.
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
   float r;
@@ -1264,7 +1239,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
             }
           }
-          // ---- P = exp2(s * c - m), row sum in fp32, P rounded to bf16
+          // ---- P = exp2(s * c - m), row sum in fp32, P rounded to bf16.  All of it on the special-function unit: three pairs in
+          // sixteen as a cubic on the FMA pipe were level in short runs and cost 1 % where the power limit sets the clock
+          // (32-layer shape, seconds on end: 1503 -> 1484 us a launch).
           uint32_t pkk[64];
           {
             const float2 c2 = make_float2(prm.scale_log2e, prm.scale_log2e);
@@ -1274,25 +1251,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
             for (int i = 0; i < 64; ++i) {
               const float2 x = ffma2(make_float2(sa[2 * i], sa[2 * i + 1]), c2, nm2);
-              float2 pv;
-              if (TV_POLY_SEL(i)) {
-                pv = exp2_poly2(x);
-              } else {
-                pv.x = fast_exp2(x.x);
-                pv.y = fast_exp2(x.y);
-              }
+              const float2 pv = make_float2(fast_exp2(x.x), fast_exp2(x.y));
               sum = fadd2(sum, pv);
               pkk[i] = pack_bf16(pv.x, pv.y);
             }
             l_sum += sum.x + sum.y;
-          }
-          if (masked) {      // the polynomial gives a hidden key 2^-125: make that the 0 which the other pairs have
-#pragma unroll
-            for (int i = 0; i < 64; ++i)
-              if (TV_POLY_SEL(i)) {
-                if (!((vis[i >> 4] >> (2 * i & 31)) & 1u)) pkk[i] &= 0xffff0000u;
-                if (!((vis[i >> 4] >> ((2 * i + 1) & 31)) & 1u)) pkk[i] &= 0x0000ffffu;
-              }
           }
           // ---- P into its columns once the PV that read them last is done; with one warpgroup (two P buffers in turn) that
           // was issued in front of the S this tile has waited for
