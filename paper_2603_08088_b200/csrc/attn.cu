@@ -372,8 +372,8 @@ struct AttnParams {
   int B, Nmax, Hq, Hkv, Scap, G, NPT, NP, W, groups;
   int tile0;                     // first row tile of this launch
   int TT;                        // key tiles of the tree's own K/V: ceil(Nmax / 128), 1 or 2
-  uint32_t q_box_bytes;
-  unsigned long long* trace;     // optional event trace [cta][role 0..3][kTraceCap] of (tag << 48 | ns), or NULL          // bytes of one Q box {64, G, NPT}: 16 KB when G divides 128
+  uint32_t q_box_bytes;          // bytes of one Q box {64, G, NPT}: 16 KB when G divides 128
+  unsigned long long* trace;     // optional event trace [cta][role 0..3][kTraceCap] of (tag << 48 | ns), or NULL
   int tree_in_cache;             // the tree's K/V rows live in the cache behind the prefix (rows S_b + node)
   const int32_t* block_table;    // paged cache: page of key tile j of sequence b at [b * max_blocks + j]; else nullptr
   int max_blocks, n_pages;
@@ -567,7 +567,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int tiles = min(min(first.j1, first.len - prm.TT) - first.j0, kPrefetchTiles);
     for (int x = lane; x < kQBoxes + tiles * kBoxes; x += 32) {
       if (x < kQBoxes) {
-        tma_prefetch_5d(&map_q, x % (D / 64) * 64, first.hk * prm.G, (prm.tile0 + (int)(blockIdx.x % prm.NP) * MT + x / (D / 64)) * prm.NPT, first.b, first.layer);
+        const int tile = prm.tile0 + (int)(blockIdx.x % prm.NP) * MT + x / (D / 64);
+        tma_prefetch_5d(&map_q, x % (D / 64) * 64, first.hk * prm.G, tile * prm.NPT, first.b, first.layer);
         continue;
       }
       const int y = x - kQBoxes, j = first.j0 + y / kBoxes, kv = y % kBoxes / (D / 64), h = y % (D / 64);
