@@ -1064,9 +1064,12 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // All 32 lanes wait together and agree on the outcome, so that the warp-wide TMEM instructions
       // below are never executed by a part of a warp.  The waits that every key tile has do not vote (LAZY): a lane whose
       // wait was abandoned notes it, goes on with whatever tensor memory holds, hands nothing on, and the vote on the row
-      // maxima of the next tile, or the one behind the last tile, takes the whole warp out.  (32-layer shape 1254 -> 1240 us a
-      // launch, long context 226.7 -> 224.1, 4 sequences of 4096 41.3 -> 40.9.  The cluster kernel, a tile or two per CTA, keeps
-      // the votes: 32 layers of one sequence 10.0 us a layer with them, 10.2 without.)
+      // maxima of the next tile, or the one behind the last tile, takes the whole warp out.  The lanes leave such a wait one by
+      // one; the tensor-memory instruction behind it is the same for all of them whatever the wait returned (.aligned), and
+      // waits until the last of them has come (.sync), so no barrier stands in front of it: one after each wait costs as much as
+      // the votes and more (dependent layers of 16 sequences 509 -> 530 us, long context 261 -> 272).  (32-layer shape
+      // 1254 -> 1240 us a launch, long context 226.7 -> 224.1, 4 sequences of 4096 41.3 -> 40.9.  The cluster kernel, a tile or two
+      // per CTA, keeps the votes: 32 layers of one sequence 10.0 us a layer with them, 10.2 without.)
       constexpr bool LAZY = !CL;
       bool lane_ok = true;
       auto wwait = [&](uint32_t b_, uint32_t parity) -> bool {

@@ -64,3 +64,39 @@ def test_expired_wait_ends_the_launch_with_a_status_and_the_next_launch_is_unhar
         after = normal()                                                     # tensor memory was freed, barriers are fresh
         assert (i32(status) == 0).all()
         assert torch.equal(after[0], before[0]) and torch.equal(after[1], before[1])
+
+
+MIDDLE = [(128, 4, 64), (64, 4, 64), (128, 4, 20), (64, 4, 20)]      # d, G, nodes: two row tiles and one, both head widths
+
+
+@pytest.mark.parametrize("d,G,N", MIDDLE)
+def test_waits_that_expire_anywhere_in_the_tile_loop(d, G, N):
+    """Limits of the order of the waits themselves: whichever wait is the first to be longer gives up, in the tile loop too,
+    where the lanes of a softmax warp do so one by one with collective instructions behind the wait.  A launch either
+    finishes or reports; the one behind it is unharmed."""
+    cfg = CONFIGS[0].scaled(B=40, L=1, Hq=2 * G, Hkv=2, d=d, S_lo=2500, S_hi=3000, Scap=3200, N=N, D=6, V=0, tree="uniform")
+    c = make_case(cfg, seed=d + N, device="cuda", with_logits=False)
+    bits = torch.zeros(cfg.B, N, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    status = torch.zeros(cfg.B, dtype=torch.int32, device="cuda")
+    tv.tree_build_mask(c["parent"], c["n_nodes"], N - 1, 1, bits, status)
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(cfg.B, N, cfg.Hq, 2, d, cfg.Scap), dtype=torch.uint8, device="cuda")
+    args = (c["q"][0], c["k_cache"][0], c["v_cache"][0], c["k_tree"][0], c["v_tree"][0], c["prefix_len"], c["n_nodes"], bits,
+            d ** -0.5)
+    before, after = (torch.full((cfg.B, N, cfg.Hq, d), x, dtype=torch.bfloat16, device="cuda") for x in (3.0, 4.0))
+    tv.tree_verify_attn(*args, before, ws, status)
+    torch.cuda.synchronize()
+    assert (i32(status) == 0).all()
+    expired = 0
+    for limit in (0, 1000, 2000, 4000, 8000, 16000, 500_000_000):
+        got = torch.zeros_like(before)
+        tv.tv_debug_attn_expire(*args, got, ws, status, limit, 0)
+        torch.cuda.synchronize()
+        st = i32(status)
+        assert (st == st[0]).all() and st[0] in (0, tv.TV_ST_TIMEOUT)
+        assert st[0] != 0 or torch.equal(got, before)
+        expired += st[0] != 0
+        status.zero_()
+        tv.tree_verify_attn(*args, after, ws, status)
+        torch.cuda.synchronize()
+        assert (i32(status) == 0).all() and torch.equal(before, after)
+    assert expired >= 1
