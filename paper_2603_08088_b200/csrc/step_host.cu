@@ -66,16 +66,54 @@ Staging layout(int L, int B, int Nmax, int Hq, int Hkv, int d, int Scap, int V, 
   return s;
 }
 
-// The small arrays of a step cross the link in one copy each way, through a pinned block: a copy of its own costs each of
-// them some 6 us in front of the step or behind it (8 + 20 us of a small model's step).
+// The small arrays of a step cross the link together: a copy of its own costs each of them some 6 us in front of the step
+// or behind it (8 + 20 us of a small model's step).  The results come back in one copy to a pinned block.  The inputs may
+// still be written by work that is queued on the caller's stream (a drafter's copies to the host, say), so the host must
+// not read them when the call is made: a kernel on that stream reads them where they are, if they are pinned.
 constexpr size_t kBlockBytes = 64 << 10;
 
-// Per-device copy streams, a growing pool of timing-free events and two pinned blocks, created on first use and kept.  A
+struct SmallInputs {
+  const int32_t* src[4];
+  int32_t* dst[4];
+  int count[4];
+};
+
+constexpr int kFetchThreads = 256;
+
+// Bound by one round trip over the host link: every thread has one load in flight, 64 KB take 64 CTAs.
+__global__ void __launch_bounds__(kFetchThreads)
+fetch_small_kernel(const SmallInputs a) {
+  tv::pdl_enter();
+  int i = blockIdx.x * kFetchThreads + threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (i >= 0 && i < a.count[k]) a.dst[k][i] = __ldcv(a.src[k] + i);
+    i -= a.count[k];
+  }
+}
+
+// Address under which kernels of this device read `bytes` of pinned host memory, or nullptr.
+const int32_t* mapped(const int32_t* host, size_t bytes) {
+  if ((reinterpret_cast<uintptr_t>(host) & 3u) != 0) return nullptr;
+  const char* ends[2] = {reinterpret_cast<const char*>(host), reinterpret_cast<const char*>(host) + bytes - 1};
+  cudaPointerAttributes attr[2];
+  for (int i = 0; i < 2; ++i) {
+    if (cudaPointerGetAttributes(&attr[i], ends[i]) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    if (attr[i].type != cudaMemoryTypeHost || !attr[i].devicePointer) return nullptr;
+  }
+  const char* first = static_cast<const char*>(attr[0].devicePointer);
+  if (static_cast<const char*>(attr[1].devicePointer) != first + bytes - 1) return nullptr;
+  return reinterpret_cast<const int32_t*>(first);
+}
+
+// Per-device copy streams, a growing pool of timing-free events and a pinned block, created on first use and kept.  A
 // step holds `busy` while it uses them (the call is synchronous).
 struct Pipes {
   std::mutex busy;
   cudaStream_t in = nullptr, out = nullptr;
-  char* block_in = nullptr;
   char* block_out = nullptr;
   std::vector<cudaEvent_t> events;
 };
@@ -92,11 +130,8 @@ cudaError_t get_pipes(int n_events, Pipes** result, std::unique_lock<std::mutex>
     if ((e = cudaStreamCreateWithFlags(&p.in, cudaStreamNonBlocking)) != cudaSuccess) return e;
     if ((e = cudaStreamCreateWithFlags(&p.out, cudaStreamNonBlocking)) != cudaSuccess) return e;
   }
-  if (!p.block_in) {
-    char* both = nullptr;
-    if ((e = cudaHostAlloc(reinterpret_cast<void**>(&both), 2 * kBlockBytes, cudaHostAllocDefault)) != cudaSuccess) return e;
-    p.block_in = both;
-    p.block_out = both + kBlockBytes;
+  if (!p.block_out) {
+    if ((e = cudaHostAlloc(reinterpret_cast<void**>(&p.block_out), kBlockBytes, cudaHostAllocDefault)) != cudaSuccess) return e;
   }
   while ((int)p.events.size() < n_events) {
     cudaEvent_t ev;
@@ -174,16 +209,27 @@ extern "C" int tv_verify_step_host(const tv_step_host_args* a) {
                       {const_cast<int32_t*>(a->n_nodes), s.n_nodes, sizeof(int32_t) * B},
                       {const_cast<int32_t*>(a->tokens), s.tokens, sizeof(int32_t) * B * Nmax},
                       {const_cast<int32_t*>(a->retrieve_indices), s.retrieve, a->retrieve_indices ? sizeof(int32_t) * B * P * Dp1 : 0}};
-  const size_t in_bytes = in[3].at + in[3].bytes - in[0].at;
-  if (in_bytes <= kBlockBytes) {
-    for (const Part& p : in)
-      if (p.bytes) memcpy(pp->block_in + (p.at - in[0].at), p.host, p.bytes);
-    TV_CUDA_OK(cudaMemcpyAsync(dptr(in[0].at), pp->block_in, in_bytes, cudaMemcpyHostToDevice, s_in));
+  SmallInputs small{};
+  size_t in_bytes = 0;
+  bool fetch = true;
+  for (int k = 0; k < 4; ++k) {
+    in_bytes += in[k].bytes;
+    if (!in[k].bytes || !fetch) continue;
+    small.src[k] = in_bytes <= kBlockBytes ? mapped(static_cast<const int32_t*>(in[k].host), in[k].bytes) : nullptr;
+    small.dst[k] = reinterpret_cast<int32_t*>(dptr(in[k].at));
+    small.count[k] = (int)(in[k].bytes / sizeof(int32_t));
+    fetch = small.src[k] != nullptr;
+  }
+  if (fetch) {
+    const unsigned ctas = (unsigned)((in_bytes / sizeof(int32_t) + kFetchThreads - 1) / kFetchThreads);
+    TV_CUDA_OK(tv::launch_pdl(fetch_small_kernel, dim3(ctas), dim3(kFetchThreads), 0, st, small));
+    tv::count_launches(1);
   } else {
     for (const Part& p : in)
       if (p.bytes) TV_CUDA_OK(cudaMemcpyAsync(dptr(p.at), p.host, p.bytes, cudaMemcpyHostToDevice, s_in));
+    TV_CUDA_OK(cudaEventRecord(ev[1], s_in));
+    TV_CUDA_OK(cudaStreamWaitEvent(st, ev[1], 0));
   }
-  TV_CUDA_OK(cudaEventRecord(ev[1], s_in));
   for (int l = 0; l < L; l += per_stage) {
     const size_t n = (size_t)(L - l < per_stage ? L - l : per_stage);
     TV_CUDA_OK(cudaMemcpyAsync(d_q + l * q_layer, a->q + l * q_layer, sizeof(tv_bf16) * n * q_layer, cudaMemcpyHostToDevice, s_in));
@@ -198,7 +244,6 @@ extern "C" int tv_verify_step_host(const tv_step_host_args* a) {
   int32_t* d_status = reinterpret_cast<int32_t*>(dptr(s.status));
   int32_t* d_retrieve = reinterpret_cast<int32_t*>(dptr(s.retrieve));
   uint32_t* d_bits = reinterpret_cast<uint32_t*>(dptr(s.anc_bits));
-  TV_CUDA_OK(cudaStreamWaitEvent(st, ev[1], 0));
   int rc = tree_build_mask(reinterpret_cast<int32_t*>(dptr(s.parent)), d_n_nodes, B, Nmax, Dp1 - 1, P, d_bits,
                            nullptr, nullptr, nullptr, a->retrieve_indices ? nullptr : d_retrieve,
                            reinterpret_cast<int32_t*>(dptr(s.n_paths)), d_status, a->stream);

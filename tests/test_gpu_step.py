@@ -121,7 +121,12 @@ def test_host_buffer_step_matches_device_step():
     assert np.array_equal(i32(S), ref["prefix_len"])
 
 
-def _host_step(cfg, seed, given_rows, stream=None):
+SMALL_INPUTS = ("parent", "n_nodes", "tokens", "retrieve_indices")
+
+
+def _host_step(cfg, seed, given_rows, stream=None, queued=False, pinned=True):
+    """``queued``: the small inputs are still those of another tree when the call is made; copies behind a few
+    milliseconds of work on the same stream bring the right ones."""
     case = make_case(cfg, seed=seed)
     ref = orc.verify_step(case_to_numpy(case), cfg.d ** -0.5, use_given_retrieve=given_rows)
     P, Dp1 = case["retrieve"].shape[1], cfg.D + 1
@@ -134,7 +139,21 @@ def _host_step(cfg, seed, given_rows, stream=None):
     kc, vc, S = case["k_cache"].cuda(), case["v_cache"].cuda(), case["prefix_len"].cuda()
     staging = torch.zeros(tv.tv_step_staging_bytes(cfg.L, cfg.B, cfg.N, cfg.Hq, cfg.Hkv, cfg.d, cfg.Scap, cfg.V, P, Dp1),
                           dtype=torch.uint8, device="cuda")
+    if not pinned:
+        host.update({k: host[k].clone() for k in SMALL_INPUTS if host[k] is not None})
+    if queued:
+        other = make_case(cfg, seed=seed + 1)
+        new = {k: host[k].cuda() for k in SMALL_INPUTS if host[k] is not None}
+        for k in new:
+            host[k].copy_(other["retrieve" if k == "retrieve_indices" else k])
+        busy = torch.zeros(1 << 28, device="cuda")
     torch.cuda.synchronize()
+    if queued:
+        with torch.cuda.stream(stream):
+            for _ in range(12):
+                busy.add_(1.0)
+            for k, t in new.items():
+                host[k].copy_(t, non_blocking=True)
     tv.tv_verify_step_host(host, kc, vc, S, staging, cfg.d ** -0.5, cfg.V, stream=stream)
     assert np.abs(host["out"].float().numpy() - ref["out"]).max() <= ATTN_ATOL
     for k in ("accept_len", "accepted_nodes", "next_token"):
@@ -161,3 +180,15 @@ def test_host_buffer_steps_from_several_threads():
     streams = [torch.cuda.Stream() for _ in range(4)]
     with ThreadPoolExecutor(4) as ex:
         list(ex.map(lambda i: _host_step(cfg, 500 + i, i % 2 == 0, streams[i % 4]), range(12)))
+
+
+@pytest.mark.parametrize("over", HOST_STEPS, ids=["stages", "large_rows"])
+@pytest.mark.parametrize("given_rows", [True, False])
+@pytest.mark.parametrize("own_stream", [True, False])
+def test_host_buffer_step_reads_its_inputs_behind_the_work_in_front(over, given_rows, own_stream):
+    stream = torch.cuda.Stream() if own_stream else torch.cuda.current_stream()
+    _host_step(CONFIGS[4].scaled(**over), 78, given_rows, stream, queued=True)
+
+
+def test_host_buffer_step_with_pageable_small_inputs():
+    _host_step(CONFIGS[4].scaled(**HOST_STEPS[0]), 79, True, pinned=False)
