@@ -126,7 +126,7 @@ argmax_scan_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict
       if (chunk == 0 && tid < 16) {
         const int v = r.edge(tid);
         if (v >= 0) {
-          float f = bf16_bits_to_float(r.row[v]);
+          float f = r.entry(v);
           f = f == f ? f : -INFINITY;
           take_better(best, best_i, f, v);
         }

@@ -12,7 +12,8 @@ namespace tv {
 // The row is covered by the aligned 16-byte vectors of memory it lies in: vector i holds entries 8 i - off .. 8 i - off + 7.
 // vector() gives the vectors that lie wholly inside the row and -inf for all others; edge() gives the entries that are
 // left, at most seven before the first such vector and at most seven behind the last one.  (Putting the outer vectors
-// together inside vector() cost registers and kept a thread's loads from being issued together.)
+// together inside vector() cost registers and kept a thread's loads from being issued together.)  All loads bypass L1: a
+// scan that starts ahead of its wait must not meet a line that an earlier launch on this SM has left there.
 struct LogitsRow {
   const uint16_t* row;
   int off, V;
@@ -21,7 +22,7 @@ struct LogitsRow {
   }
   __device__ __forceinline__ uint4 vector(int i) const {
     const int v = 8 * i - off;
-    return v >= 0 && v <= V - 8 ? __ldcs(reinterpret_cast<const uint4*>(row + v))
+    return v >= 0 && v <= V - 8 ? __ldcg(reinterpret_cast<const uint4*>(row + v))
                                 : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
   }
   // Entry number t (0..15) of those no whole vector holds, or -1.
@@ -31,6 +32,7 @@ struct LogitsRow {
     const int v = t < 8 ? t : tail + t - 8;
     return t < 8 ? (v < head ? v : -1) : (v < V ? v : -1);
   }
+  __device__ __forceinline__ float entry(int v) const { return __uint_as_float((uint32_t)__ldcg(row + v) << 16); }
 };
 
 // Streaming the rows through shared memory: a warp requests stage after stage with bulk copies, 24 others reduce them.  A
@@ -167,7 +169,7 @@ __device__ __forceinline__ void stream_rows(const tv_bf16* __restrict__ logits, 
       if (lane < 16 && (own_slice ? chunk == 0 || chunk + 2 >= n_chunks : chunk == 0 && w == 0)) {
         rest_v = r.edge(lane);
         if (own_slice && rest_v >= 0 && (rest_v + r.off) / kStreamSlice != chunk * kStreamWarps + w) rest_v = -1;
-        if (rest_v >= 0) rest = __uint_as_float((uint32_t)r.row[rest_v] << 16);
+        if (rest_v >= 0) rest = r.entry(rest_v);
       }
       const int in_stage = w * (kStreamSlice / 8), first = chunk * (kStreamItem / 8) + in_stage;
       uint4 u[kStreamVecs];

@@ -141,7 +141,7 @@ row_stats_kernel(const tv_bf16* __restrict__ logits, const int32_t* __restrict__
       if (lane < 16 && (chunk == 0 || chunk >= n_chunks - 2)) {
         const tv::LogitsRow r(logits, row, V);
         const int v = r.edge(lane);
-        if (v >= 0 && (v + r.off) / kStatChunk == chunk) rest = bf16_to_float(r.row[v]);
+        if (v >= 0 && (v + r.off) / kStatChunk == chunk) rest = r.entry(v);
       }
       const RowStat out = chunk_stat(u, rest, k);
       if (lane == 0) stats[(size_t)row * n_chunks + chunk] = out;

@@ -123,3 +123,37 @@ def test_scan_beside_the_attention_changes_nothing(B, L, S, in_cache):
 
     for a, b in zip(steps(False), steps(True)):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("B,N,V", [(1, 17, 30001), (2, 9, 1003), (8, 64, 128257)])
+def test_scan_beside_the_attention_reads_what_the_logits_are_now(B, N, V):
+    """Steps without a synchronisation on one logits and one token buffer that are rewritten between them, with an attention
+    of few units in front (it leaves SMs to the scan at once): short scans and a long one, entries on both sides of the whole
+    vectors of a row.  The argmax of every step is that of the logits of its own step."""
+    cfg = CONFIGS[0].scaled(B=B, L=1, Hq=2, Hkv=1, d=64, S_lo=300, S_hi=300, Scap=1024, N=N, D=min(6, N - 1), V=V, tree="uniform")
+    c = to_device(make_case(cfg, seed=V))
+    g = torch.Generator(device="cuda")
+    g.manual_seed(V)
+    steps = 12
+    logits = [torch.randn(B, N, V, device="cuda", generator=g).to(torch.bfloat16) for _ in range(steps)]
+    ends = list(range(8)) + list(range(V - 8, V))
+    for s, l in enumerate(logits):                       # half of the rows have their maximum at an end of the row
+        for i in range(0, N, 2):
+            l[:, i, ends[(5 * s + i) % 16]] = 16.0 + s
+    tokens = [torch.randint(0, V, (B, N), dtype=torch.int32, device="cuda", generator=g) for _ in range(steps)]
+    buf = [tv.StepBuffers(1, B, N, cfg.Hq, cfg.Hkv, cfg.d, cfg.Scap, V, N, cfg.D + 1) for _ in range(steps)]
+    seen = torch.zeros(steps, B, N, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    for s in range(steps):
+        c["logits"].copy_(logits[s])
+        torch.add(tokens[s], 0, out=c["tokens"])
+        tv.verify_step(c, buf[s], cfg.d ** -0.5)
+        seen[s].copy_(buf[s].argmax_tok)
+    torch.cuda.synchronize()
+    for s in range(steps):
+        l = logits[s].float()
+        first = torch.where(l == l.amax(-1, keepdim=True), torch.arange(V, device="cuda"), V).amin(-1)
+        assert torch.equal(seen[s].long(), first), s
+        ref = orc.greedy_accept(i32(buf[s].retrieve), i32(tokens[s]), i32(c["n_nodes"]), i32(seen[s]))
+        for k in ("accept_len", "accepted_nodes", "next_token"):
+            assert np.array_equal(i32(getattr(buf[s], k)), ref[k]), (s, k)
