@@ -157,3 +157,51 @@ def test_scan_beside_the_attention_reads_what_the_logits_are_now(B, N, V):
         ref = orc.greedy_accept(i32(buf[s].retrieve), i32(tokens[s]), i32(c["n_nodes"]), i32(seen[s]))
         for k in ("accept_len", "accepted_nodes", "next_token"):
             assert np.array_equal(i32(getattr(buf[s], k)), ref[k]), (s, k)
+
+
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("B,Hkv,G", [(80, 1, 4), (2, 2, 4)])      # the even cut, the cluster kernel
+def test_early_reads_see_lengths_and_pages_rewritten_in_place(B, Hkv, G, paged):
+    """Launches under TV_ATTN_STABLE_INPUTS behind the mask kernel, without a synchronisation: the one buffer of lengths, node
+    counts (and pages) is rewritten in front of every mask call.  Each gives the bits it gives alone."""
+    cfg = CONFIGS[0].scaled(B=B, L=1, Hq=G * Hkv, Hkv=Hkv, d=64, S_lo=1, S_hi=1000, Scap=1024, N=20, D=6, V=0, tree="uniform")
+    c = make_case(cfg, seed=B, device="cuda", with_logits=False)
+    N, d, steps = cfg.N, cfg.d, 10
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B)
+    if paged:
+        kp, vp = (c[k].reshape(1, B, Hkv, 8, 128, d).transpose(2, 3).reshape(1, B * 8, Hkv, 128, d).contiguous() for k in ("k_cache", "v_cache"))
+        tables = [torch.randperm(B * 8, device="cuda", generator=g).to(torch.int32).view(B, 8) for _ in range(steps)]
+        table = torch.zeros_like(tables[0])
+    lengths = [torch.randint(0, 1025, (B,), dtype=torch.int32, device="cuda", generator=g) for _ in range(steps)]
+    counts = [torch.randint(1, N + 1, (B,), dtype=torch.int32, device="cuda", generator=g) for _ in range(steps)]
+    S, n = torch.zeros_like(lengths[0]), torch.ones_like(counts[0])
+    bits = torch.zeros(B, N, 1, dtype=torch.int32, device="cuda")
+    status = torch.zeros(B, dtype=torch.int32, device="cuda")
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(B, N, cfg.Hq, Hkv, d, 1024), dtype=torch.uint8, device="cuda")
+
+    def steps_with(sync):
+        outs = [torch.zeros(1, B, N, cfg.Hq, d, dtype=torch.bfloat16, device="cuda") for _ in range(steps)]
+        torch.cuda.synchronize()
+        for s in range(steps):
+            if paged:
+                table.copy_(tables[s])
+            S.copy_(lengths[s])
+            torch.add(counts[s], 0, out=n)
+            sync()
+            tv.tree_build_mask(c["parent"], n, N - 1, 1, bits, status)
+            sync()
+            if paged:
+                tv.tree_verify_attn_paged_layers(c["q"], kp, vp, table, c["k_tree"], c["v_tree"], S, n, bits, d ** -0.5, outs[s],
+                                                 ws, status, flags=tv.TV_ATTN_STABLE_INPUTS)
+            else:
+                tv.tree_verify_attn_layers(c["q"], c["k_cache"], c["v_cache"], c["k_tree"], c["v_tree"], S, n, bits, d ** -0.5,
+                                           outs[s], ws, status, flags=tv.TV_ATTN_STABLE_INPUTS)
+            sync()
+        torch.cuda.synchronize()
+        return outs
+
+    alone, behind = steps_with(torch.cuda.synchronize), steps_with(lambda: None)
+    for s in range(steps):
+        assert torch.equal(alone[s], behind[s]), s
+    assert (i32(status) == 0).all()
