@@ -69,14 +69,16 @@ __device__ __forceinline__ RowStat chunk_stat(const uint4* u, float rest, float 
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) out.m = fmaxf(out.m, __shfl_xor_sync(0xffffffffu, out.m, off));
   if (out.m > -INFINITY) {
-    const float2 k2 = make_float2(k, k), mk2 = make_float2(-out.m * k, -out.m * k);
+    // (l - m) k in this order, as mass_of has it: the mass of the maximum is 1 and the rounding is that of the difference.  As
+    // l k - m k in one FMA the rounding of m k, 2^-24 |m k| of every mass of the chunk, grows without limit as 1 / T.
+    const float2 k2 = make_float2(k, k), m2 = make_float2(-out.m, -out.m);
     float2 sum = make_float2(0.f, 0.f);
 #pragma unroll
     for (int q = 0; q < tv::kStreamVecs; ++q) {
       const uint32_t e[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        float2 x = __ffma2_rn(make_float2(__uint_as_float(e[t] << 16), __uint_as_float(e[t] & 0xffff0000u)), k2, mk2);
+        float2 x = __fmul2_rn(__fadd2_rn(make_float2(__uint_as_float(e[t] << 16), __uint_as_float(e[t] & 0xffff0000u)), m2), k2);
         x.x = ex2_approx(fmaxf(x.x, -150.f));
         x.y = ex2_approx(fmaxf(x.y, -150.f));
         sum = __fadd2_rn(sum, x);

@@ -185,3 +185,33 @@ def test_long_scans_around_the_slice_and_vector_edges(V):
     """So many rows that the long scan takes them, padded nodes among them."""
     lt, tokens, parent, n, u_node, u_bonus = make_inputs(90 + V, 64, 60, 5, V, ragged=True)
     check(lt, tokens, parent, n, u_node, u_bonus, 1.0, 6, min_fraction=0.5)
+
+
+@pytest.mark.parametrize("V", [1003, 5000])
+@pytest.mark.parametrize("rows", [1, 64])        # of 60 nodes: the short scan, the long one
+def test_masses_keep_their_precision_at_low_temperatures(V, rows):
+    """Large logits over a small temperature.  A row whose maximum stands alone accepts its token for every uniform below 1;
+    one whose maximum is shared by two accepts each for uniforms below 1/2 (the sum is 1 or 2 exactly: every other mass is 0)."""
+    rng = np.random.default_rng(V)
+    N = 60
+    parent = np.zeros((rows, N), dtype=np.int32)
+    parent[:, 0] = -1
+    for T in (0.05, 3e-3, 7e-4, 1.3e-5):
+        lt = torch.zeros(rows, N, V)
+        tokens = np.zeros((rows, N), dtype=np.int32)
+        u = np.zeros((rows, N), dtype=np.float32)
+        shared = np.zeros(rows, dtype=bool)
+        want = np.zeros(rows, dtype=np.int32)
+        for b in range(rows):
+            shared[b] = rng.random() < 0.7 if rows > 1 else T != 3e-3
+            a, other = rng.choice(V, 2, replace=False)
+            top = float(rng.integers(130, 255)) / 4.0           # exact in bf16
+            lt[b, 0, a] = top
+            if shared[b]:
+                lt[b, 0, other] = top
+            tokens[b, 1:] = a                                    # one proposal, repeated: skipped once rejected
+            accept = rng.random() < 0.5 if shared[b] else True
+            u[b] = (0.5 - 2.0 ** -20 if accept else 0.5 + 2.0 ** -20) if shared[b] else 1.0 - 2.0 ** -20
+            want[b] = accept
+        got = run_gpu(lt.to(torch.bfloat16), tokens, parent, np.full(rows, N), u, np.zeros(rows), T, 2)
+        assert np.array_equal(got["accept_len"], want), (T, np.flatnonzero(got["accept_len"] != want))
