@@ -182,7 +182,7 @@ __device__ __forceinline__ float block_scan(float v, float* warp_sums, float& to
 // One CTA per sequence.  A chain of dependent round trips, so everything that does not depend on the row statistics
 // (tree, tokens, uniforms, the token logits) is fetched while row_stats_kernel still runs: that kernel lets this one
 // start only after every earlier kernel of the stream has completed, and the loads bypass L1.  The draw reads one chunk
-// of the row (4 KB) and not the row up to the crossing (walk and draw took 37 us before).
+// of the row (4 KB), and the ones with rejected tokens, and not the row up to the crossing (walk and draw took 37 us before).
 __global__ void __launch_bounds__(kWalkThreads)
 sample_walk_kernel(const tv_bf16* __restrict__ logits, const RowStat* __restrict__ stats, int n_chunks,
                    const int32_t* __restrict__ tokens, const int32_t* __restrict__ parent,
@@ -193,10 +193,11 @@ sample_walk_kernel(const tv_bf16* __restrict__ logits, const RowStat* __restrict
   static_assert(kWalkThreads == 1024 && kMaxNodes <= kWalkThreads, "block_scan and the node arrays rely on it");
   __shared__ float sM[kMaxNodes], sZ[kMaxNodes], sE[kMaxNodes], sU[kMaxNodes];   // row max, row sum, token mass, uniform
   __shared__ int sPar[kMaxNodes], sTok[kMaxNodes], sRej[kMaxNodes];
-  __shared__ float sRejE[kMaxNodes];
+  __shared__ float sKept[kMaxNodes];                              // what is left of the chunk that holds rejected token x
+  __shared__ uint32_t sHide[kWalkThreads / 32][kStatChunk / 32];  // per warp: rejected entries of the chunk it sums
   __shared__ float sWarp[kWalkThreads / 32];
   __shared__ int sLast, sNrej, sChunk, sHit, sLastMass;
-  __shared__ float sTarget, sExcl;
+  __shared__ float sExcl;
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
   int n = __ldcg(n_nodes + b);
   n = n < 0 ? 0 : (n > Nmax ? Nmax : n);
@@ -268,10 +269,7 @@ sample_walk_kernel(const tv_bf16* __restrict__ logits, const RowStat* __restrict
             acc = cand;
             break;
           }
-          if (lane == 0) {
-            sRej[nrej] = x;
-            sRejE[nrej] = sE[cand];
-          }
+          if (lane == 0) sRej[nrej] = x;
           __syncwarp();
           ++nrej;
           rem -= sE[cand];
@@ -288,40 +286,92 @@ sample_walk_kernel(const tv_bf16* __restrict__ logits, const RowStat* __restrict
       accept_len[b] = depth;
       sLast = c;
       sNrej = nrej;
-      sTarget = ub * fmaxf(rem, 0.f);       // in units of the remaining (unnormalised) mass
       if (any_bad) atomicOr(status + b, TV_ST_BAD_INDEX);
     }
   }
   __syncthreads();
   // ---- next token: the first entry of row c, rejected tokens left out, whose cumulative mass in vocabulary order
-  // exceeds the target.
+  // exceeds the target, u_bonus of what is left.
   if (n == 0) {
     if (tid == 0) next_token[b] = -1;       // no row to draw from
     return;
   }
   const int c = sLast, nrej = sNrej;
-  const float M = sM[c], target = sTarget;
+  const float M = sM[c];
   const uint16_t* row = lg + (size_t)c * V;
-  const int off = tv::LogitsRow(logits, (long long)b * Nmax + c, V).off;       // chunk q holds entries q * kStatChunk - off ...
-  // first the chunk: cumulative masses of the chunks, rejected tokens subtracted
+  const tv::LogitsRow lr(logits, (long long)b * Nmax + c, V);
+  const int off = lr.off;                                      // chunk q holds entries q * kStatChunk - off ...
+  const RowStat* row_stats = stats + ((size_t)b * Nmax + c) * n_chunks;
+  RowStat st = {-INFINITY, 0.f};
+  if (tid < n_chunks) st = row_stats[tid];
+  // A chunk with rejected tokens is summed again without them, by one warp: taking their masses off its sum would leave the
+  // rounding of that sum, which is more than all other entries where the rejected ones have nearly all of the mass.
+  for (int x = tid >> 5; x < nrej; x += kWalkThreads / 32) {
+    const int q = (sRej[x] + off) / kStatChunk;
+    bool first = true;                                         // of the rejected tokens in this chunk
+    for (int y0 = 0; y0 < x; y0 += 32)
+      first &= !__any_sync(0xffffffffu, y0 + lane < x && (sRej[y0 + lane] + off) / kStatChunk == q);
+    float sum = 0.f;
+    if (first) {
+      uint4 u[tv::kStreamVecs];                                // requested before anything else
+#pragma unroll
+      for (int w = 0; w < tv::kStreamVecs; ++w) u[w] = lr.vector((q * tv::kStreamVecs + w) * 32 + lane);
+      const int v = lane < 16 ? lr.edge(lane) : -1, at_v = v + off - q * kStatChunk;
+      const bool mine = v >= 0 && at_v >= 0 && at_v < kStatChunk;
+      const float rest = mine ? lr.entry(v) : -INFINITY;
+      uint32_t* hide = sHide[tid >> 5];
+      hide[lane] = hide[lane + 32] = 0u;
+      __syncwarp();
+      for (int y = x + lane; y < nrej; y += 32) {
+        const int at = sRej[y] + off - q * kStatChunk;
+        if (at >= 0 && at < kStatChunk) atomicOr(&hide[at >> 5], 1u << (at & 31));
+      }
+      __syncwarp();
+      if (mine && !((hide[at_v >> 5] >> (at_v & 31)) & 1u)) sum = mass_of(rest, M, k);
+#pragma unroll
+      for (int w = 0; w < tv::kStreamVecs; ++w) {
+        const uint32_t hidden = hide[w * 8 + (lane >> 2)] >> ((lane & 3) * 8);
+        const uint32_t e[4] = {u[w].x, u[w].y, u[w].z, u[w].w};
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+          sum += (hidden >> t) & 1u ? 0.f : mass_of(bf16_to_float((t & 1) ? (e[t >> 1] >> 16) : (e[t >> 1] & 0xffffu)), M, k);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      __syncwarp();                                            // (the next round of this warp writes `hide`)
+    }
+    if (lane == 0) sKept[x] = first ? sum : -1.f;
+  }
+  __syncthreads();
+  auto chunk_mass = [&](int q) -> float {                      // st: the chunk's statistics
+    float mass = st.m > -INFINITY ? st.s * ex2_approx(fmaxf((st.m - M) * k, -150.f)) : 0.f;
+    for (int x = 0; x < nrej; ++x)
+      if ((sRej[x] + off) / kStatChunk == q && sKept[x] >= 0.f) mass = sKept[x];
+    return mass;
+  };
+  // first the chunk: cumulative masses of the chunks (rows of at most kWalkThreads of them take one round)
+  float left = 0.f, mass = 0.f, incl = 0.f, total;
+  for (int q0 = 0; q0 < n_chunks; q0 += kWalkThreads) {
+    const int q = q0 + tid;
+    if (q0 > 0 && q < n_chunks) st = row_stats[q];
+    mass = q < n_chunks ? chunk_mass(q) : 0.f;
+    incl = left + block_scan(mass, sWarp, total);
+    left += total;
+  }
+  const float target = ub * left;
   float carried = 0.f;
   for (int q0 = 0; q0 < n_chunks; q0 += kWalkThreads) {
     const int q = q0 + tid;
-    float mass = 0.f;
-    if (q < n_chunks) {
-      const RowStat r = stats[((size_t)b * Nmax + c) * n_chunks + q];
-      if (r.m > -INFINITY) mass = r.s * ex2_approx(fmaxf((r.m - M) * k, -150.f));
-      for (int x = 0; x < nrej; ++x)
-        if ((sRej[x] + off) / kStatChunk == q) mass -= sRejE[x];
-      mass = fmaxf(mass, 0.f);
+    if (n_chunks > kWalkThreads) {
+      if (q < n_chunks) st = row_stats[q];
+      mass = q < n_chunks ? chunk_mass(q) : 0.f;
+      incl = carried + block_scan(mass, sWarp, total);
+      carried += total;
     }
-    float total;
-    const float incl = carried + block_scan(mass, sWarp, total);
     if (mass > 0.f) {
       if (target < incl) atomicMin(reinterpret_cast<unsigned*>(&sChunk), (unsigned)q);      // -1 is the largest unsigned
       atomicMax(&sLastMass, q);
     }
-    carried += total;
     __syncthreads();
     if (sChunk >= 0) {                                 // uniform: read after the barrier
       if (q == sChunk) sExcl = incl - mass;
@@ -366,12 +416,6 @@ sample_walk_kernel(const tv_bf16* __restrict__ logits, const RowStat* __restrict
     if (last >= 0) atomicMax(&sLastMass, last);
   }
   __syncthreads();
-  if (sHit < 0 && sLastMass < 0) {      // the chunk's mass was a rounding residue of a rejected token: last entry of the row
-    __syncthreads();
-    for (int v = tid; v < V; v += kWalkThreads)
-      if (entry_mass(v) > 0.f) atomicMax(&sLastMass, v);
-    __syncthreads();
-  }
   if (tid == 0) next_token[b] = sHit >= 0 ? sHit : (sLastMass >= 0 ? sLastMass : V - 1);
 }
 

@@ -215,3 +215,24 @@ def test_masses_keep_their_precision_at_low_temperatures(V, rows):
             want[b] = accept
         got = run_gpu(lt.to(torch.bfloat16), tokens, parent, np.full(rows, N), u, np.zeros(rows), T, 2)
         assert np.array_equal(got["accept_len"], want), (T, np.flatnonzero(got["accept_len"] != want))
+
+
+@pytest.mark.parametrize("V", [5000, 4099])
+@pytest.mark.parametrize("B,kids", [(6, 1), (6, 39), (64, 59)])      # the last: the long scan
+def test_draw_beside_rejected_tokens_with_nearly_all_of_the_mass(V, B, kids):
+    """The root's first child has all but 10^-4 of the mass and is rejected.  The token is drawn from what is left: 2^-25 of
+    the rejected mass on each of 4000 entries, a part of them in the rejected token's own chunk, where the rounding of the
+    chunk's sum is as large as several of them.  Up to 59 children rejected, in one chunk and in several."""
+    rng = np.random.default_rng(V + kids)
+    N = kids + 1
+    parent = np.zeros((B, N), dtype=np.int32)
+    parent[:, 0] = -1
+    lt = torch.full((B, N, V), -17.25)
+    tokens = np.zeros((B, N), dtype=np.int32)
+    for b in range(B):
+        tokens[b, 1:] = rng.choice(V, kids, replace=False)
+        lt[b, 0, tokens[b, 1]] = 0.0
+    u_node = np.full((B, N), np.float32(1.0 - 2.0 ** -20))
+    u_bonus = rng.random(B).astype(np.float32)
+    u_bonus[0] = 0.0
+    check(lt.to(torch.bfloat16), tokens, parent, np.full(B, N), u_node, u_bonus, 1.0, 2, min_fraction=1.0)
