@@ -514,8 +514,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // changed the table is built again (layers behind one another as above: 50.1 -> 47.8 us a launch, the first S is there 3.5 us
   // after the wait and not 5; a member of a context split 41.2 -> 40.7; 64-wide heads, one row tile, 16 sequences of 8000,
   // 24 nodes: 62.8 -> 63.6).  What is asked for in L2 is right whoever writes it until the wait.  The cluster
-  // kernel has no table to build: its roles wait where they read.  Lengths, node counts and pages that are read before the
-  // wait, here or under the caller's promise, are read past L1.
+  // kernel has no table to build: its roles wait where they read.
   bool guess = !CL && !prm.early;
   Sched sch{cum, gs, prm.B, prm.Hkv, 0, 0};
   int groups = 1, group = 0, g_begin = 0, g_end = 1;
@@ -588,12 +587,16 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   while (!CL) {
     if (warp == 0) {
       int run = 0;
+      // Under the caller's promise this warp reads lengths, node counts and pages before the wait: the fence drops what an
+      // earlier launch on this SM has left of them in L1.  (Loads past L1 in the item walk, which goes on behind the wait,
+      // cost 16 sequences of 600 to 1000 1 to 3 %.)
+      if (prm.early) __threadfence();
 #pragma unroll 1
       for (int base = 0; base < prm.B; base += 32) {
         const int b = base + lane;
         int len = 0;
         if (b < prm.B) {
-          int S = __ldcg(prm.prefix_len + b) + (guess && (prm.debug & 8) ? kTileN : 0);
+          int S = !guess ? prm.prefix_len[b] : __ldcg(prm.prefix_len + b) + (prm.debug & 8 ? kTileN : 0);
           S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
           len = (S + kTileN - 1) / kTileN + prm.TT + kSetupCost;
         }
@@ -665,7 +668,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   const int unit = CL ? (int)(blockIdx.x / cluster_size_x()) : 0;      // cluster kernel: (layer, sequence, KV head, pair)
   const int pair = CL ? unit % prm.NP : (int)(blockIdx.x % prm.NP);
-  auto next_item = [&](int& g, Item& it, bool ahead) -> bool {      // ahead: of the wait for the kernel in front
+  auto next_item = [&](int& g, Item& it) -> bool {
     if (CL) {                      // one item: this CTA's share of the key tiles of its cluster's unit (may be empty)
       if (g > 0) return false;
       g = 1;
@@ -673,8 +676,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       it.hk = u % prm.Hkv;
       it.b = u / prm.Hkv % prm.B;
       it.layer = u / prm.Hkv / prm.B;
-      const int S = ahead ? __ldcg(prm.prefix_len + it.b) : prm.prefix_len[it.b];
-      const int n = ahead ? __ldcg(prm.n_nodes + it.b) : prm.n_nodes[it.b];
+      const int S = __ldcg(prm.prefix_len + it.b), n = __ldcg(prm.n_nodes + it.b);      // (perhaps ahead of the wait: past L1)
       it.S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
       it.n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
       it.len = (it.S + kTileN - 1) / kTileN + prm.TT;
@@ -684,8 +686,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       return it.j1 > it.j0;
     }
     if (!locate(g, it)) return false;
-    const int S = ahead ? __ldcg(prm.prefix_len + it.b) : prm.prefix_len[it.b];
-    const int n = ahead ? __ldcg(prm.n_nodes + it.b) : prm.n_nodes[it.b];
+    const int S = prm.prefix_len[it.b], n = prm.n_nodes[it.b];
     it.S = S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S);
     it.n = n < 0 ? 0 : (n > prm.Nmax ? prm.Nmax : n);
     return true;
@@ -748,7 +749,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         g = at[1];
         it = items[2];
       }
-      while (ok && (have_first || next_item(g, it, !synced))) {
+      while (ok && (have_first || next_item(g, it))) {
         have_first = false;
         ok = mbar_wait(bar(L::Q_EMPTY), (item_idx & 1) ^ 1, abort_flag, wait_limit);
         if (!ok) break;
@@ -760,7 +761,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         auto page_of = [&](int jj) -> int {
           if (!prm.block_table || jj >= it.len - prm.TT || jj >= it.j1) return 0;
           const int32_t* entry = prm.block_table + (size_t)it.b * prm.max_blocks + jj;
-          int pg = synced ? *entry : __ldcg(entry);
+          int pg = CL ? __ldcg(entry) : *entry;
           if ((unsigned)pg >= (unsigned)prm.n_pages) {       // reported; the tile then reads page 0
             if (!synced) bad_page_b = it.b;                  // (only the first item can get here before the wait)
             else if (lane == 0) atomicOr(prm.status + it.b, TV_ST_BAD_INDEX);
