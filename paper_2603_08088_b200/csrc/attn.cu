@@ -90,6 +90,7 @@ constexpr int kMaxGroups = 160;
 #define TV_MIN_VT 6
 #endif
 constexpr int kMinVirtualTilesPerGroup = TV_MIN_VT;
+constexpr int kSplitTilesPerSm = 60;       // from here on an odd last row tile has a launch of its own (see launch)
 constexpr int kMaxCluster = 8;     // CTAs that share a unit (16 is not portable; few clusters of 16 fit the GPU at once: 21.7 us
                                    // instead of 10.8 us a launch for eight units of 12 key tiles)
 constexpr int kTraceCap = 256;     // events per (CTA, role) kept by the optional trace
@@ -371,6 +372,9 @@ struct AttnParams {
   unsigned long long epoch;      // 48-bit tag of this call
   int B, Nmax, Hq, Hkv, Scap, G, NPT, NP, W, groups;
   int tile0;                     // first row tile of this launch
+  int split_tiles;               // > 0: from this many key tiles on (all units of the launch, by the lengths on the device) the
+                                 // odd last row tile belongs to a launch of its own; below, that launch has no work
+  int front_NP, front_groups;    // NP and groups of the launch in front of it then
   int TT;                        // key tiles of the tree's own K/V: ceil(Nmax / 128), 1 or 2
   uint32_t q_box_bytes;          // bytes of one Q box {64, G, NPT}: 16 KB when G divides 128
   unsigned long long* trace;     // optional event trace [cta][role 0..3][kTraceCap] of (tag << 48 | ns), or NULL
@@ -471,6 +475,22 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   int* gs = reinterpret_cast<int*>(smem + L::kGs);
   const unsigned long long wait_limit = prm.wait_limit_ns;
 
+  // Whether an odd last row tile has a launch of its own, from the key tiles of one KV head over all sequences.
+  auto splits = [&](int tiles) -> bool { return (unsigned)(prm.Hkv * tiles) * (unsigned)prm.L >= (unsigned)prm.split_tiles; };
+  if (MT == 1 && !CL && prm.split_tiles > 0) {      // that launch: nothing to do where the one in front has taken it along
+    int tiles = 0;
+#pragma unroll 1
+    for (int b = lane; b < prm.B; b += 32) {
+      const int S = __ldcg(prm.prefix_len + b);
+      tiles += ((S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S)) + kTileN - 1) / kTileN + prm.TT;
+    }
+    if (!splits(__reduce_add_sync(0xffffffffu, tiles))) {
+      gdc_wait();
+      if (threadIdx.x == 0) gdc_launch_dependents();
+      return;
+    }
+  }
+
   // ---- setup: schedule table, barriers, TMEM
   if (threadIdx.x == 64) {     // fetch the five TMA descriptors while the rest of the set-up runs
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
@@ -550,7 +570,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     return false;
   };
   // one warp: Q and the first prefix tiles of this CTA's first item, a box per lane and turn, in the order of their use
-  // (items[2]: that item; at[0]: it is there; at[1]: where the search goes on; at[2]: CTA groups)
+  // (items[2]: that item; at[0]: it is there; at[1]: where the search goes on; at[2]: CTA groups; at[3]: CTAs of a group)
   volatile int* at = reinterpret_cast<volatile int*>(items + 3);
   auto prefetch_first = [&]() {
     Item first;
@@ -567,7 +587,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int tiles = min(min(first.j1, first.len - prm.TT) - first.j0, kPrefetchTiles);
     for (int x = lane; x < kQBoxes + tiles * kBoxes; x += 32) {
       if (x < kQBoxes) {
-        const int tile = prm.tile0 + (int)(blockIdx.x % prm.NP) * MT + x / (D / 64);
+        const int tile = prm.tile0 + (int)(blockIdx.x % (MT == 2 ? at[3] : prm.NP)) * MT + x / (D / 64);
         tma_prefetch_5d(&map_q, x % (D / 64) * 64, first.hk * prm.G, tile * prm.NPT, first.b, first.layer);
         continue;
       }
@@ -616,7 +636,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // write and a merge) and every group still gets a worthwhile share of tiles.
     const unsigned total = (unsigned)(prm.Hkv * cum[prm.B]) * (unsigned)prm.L;
     const unsigned want = total / (unsigned)kMinVirtualTilesPerGroup;
-    groups = want < 1u ? 1 : (want < (unsigned)prm.groups ? (int)want : prm.groups);
+    const bool split = MT == 2 && prm.split_tiles > 0 && splits(cum[prm.B] - prm.B * kSetupCost);
+    const int np = split ? prm.front_NP : prm.NP, max_groups = split ? prm.front_groups : prm.groups;
+    groups = want < 1u ? 1 : (want < (unsigned)max_groups ? (int)want : max_groups);
     // A group count just above a multiple of the unit count is rounded down to it: with units of equal length
     // (one sequence, all heads) every unit is then cut into the same number of equal pieces and no cut falls
     // just behind a unit boundary.  Not worth more than 1/16 of the groups.
@@ -627,15 +649,18 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // gs[k] = floor(total * k / groups) in 32-bit arithmetic: total = q * groups + r
     const unsigned q = total / (unsigned)groups, r = total % (unsigned)groups;
 #pragma unroll 1
-    for (int k = threadIdx.x; k <= prm.groups; k += kThreads)
+    for (int k = threadIdx.x; k <= kMaxGroups; k += kThreads)
       gs[k] = k <= groups ? (int)(k * q + (k * r) / (unsigned)groups) : (int)total;
-    if (threadIdx.x == 0) at[2] = groups;
+    if (threadIdx.x == 0) {
+      at[2] = groups;
+      at[3] = np;
+    }
     __syncthreads();
     sch.per_layer = prm.Hkv * cum[prm.B];
     sch.total = sch.per_layer * prm.L;
     // Downwards over the block index (see "Work split"); groups past the last used one get an empty range, and the CTAs
     // that are started first (on SMs the kernel in front does not use) get work.
-    const int place = (int)(blockIdx.x / prm.NP);
+    const int place = (int)(blockIdx.x / np);
     group = place < groups ? groups - 1 - place : place;
     g_begin = sch.group_start(group, groups);
     g_end = sch.group_start(group + 1, groups);
@@ -667,7 +692,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t tmem = *tmem_slot;
 
   const int unit = CL ? (int)(blockIdx.x / cluster_size_x()) : 0;      // cluster kernel: (layer, sequence, KV head, pair)
-  const int pair = CL ? unit % prm.NP : (int)(blockIdx.x % prm.NP);
+  const int pair = CL ? unit % prm.NP : (int)(blockIdx.x % (MT == 2 ? at[3] : prm.NP));
   auto next_item = [&](int& g, Item& it) -> bool {
     if (CL) {                      // one item: this CTA's share of the key tiles of its cluster's unit (may be empty)
       if (g > 0) return false;
@@ -1408,7 +1433,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // The unit's real tiles occupy [real0, uend) of the virtual tile space.  CTA groups k_first..k_last
             // hold them, one piece each (a group between the two lies wholly inside the unit), and this CTA's
             // group is one of them: two short walks over the cut table find both ends.
-            const int place = (int)(blockIdx.x / prm.NP), groups = at[2];      // (read here: registers are short in the loop)
+            const int np = at[3], place = (int)(blockIdx.x / np), groups = at[2];      // (read here: registers are short in the loop)
             const int group = place < groups ? groups - 1 - place : place;
             const int real0 = it.layer * (prm.Hkv * cum[prm.B]) + prm.Hkv * cum[it.b] + it.hk * (it.len + kSetupCost) + kSetupCost;
             const int uend = real0 + it.len;
@@ -1416,10 +1441,10 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             while (gs[k_first] > real0) --k_first;
             while (gs[k_last + 1] < uend) ++k_last;
             const int n_other = k_last - k_first;
-            unsigned long long* flags = prm.counters + ((((size_t)it.layer * prm.B + it.b) * prm.Hkv + it.hk) * prm.NP + pair) * 2;
+            unsigned long long* flags = prm.counters + ((((size_t)it.layer * prm.B + it.b) * prm.Hkv + it.hk) * np + pair) * 2;
             const float inv_own = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
             if (group != k_first) {
-              const size_t slot = (size_t)group * prm.NP + pair;
+              const size_t slot = (size_t)group * np + pair;
               uint4* po = reinterpret_cast<uint4*>(prm.part_o) + slot * (D / 8) * kRows;
               float* pml = prm.part_ml + slot * 2 * kRows;
               if (row_active && !(KS && wg)) {
@@ -1463,7 +1488,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               tr.mark(0x7001u);
               // Loads are issued by every thread (row rr always lies inside a slot; rows that are not active read stale
               // bytes and are masked by selects): no thread-divergent branch sits between the warp-wide TMEM ops.
-              auto slot_of = [&](int i) -> size_t { return (size_t)(k_first + i) * prm.NP + pair; };       // i-th other piece, i >= 1
+              auto slot_of = [&](int i) -> size_t { return (size_t)(k_first + i) * np + pair; };       // i-th other piece, i >= 1
               auto ml_of = [&](int i) -> const float* { return prm.part_ml + slot_of(i) * 2 * kRows + rr; };
               auto o_of = [&](int i) -> const uint4* { return reinterpret_cast<const uint4*>(prm.part_o) + slot_of(i) * (D / 8) * kRows + rr; };
               // two pieces at a time: (m, l) of the row and the columns of this warpgroup
@@ -1855,14 +1880,20 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
   // An odd number of row tiles leaves the last CTA of a group with an empty one, as expensive as a full one in the time
   // its group takes.  Where the work is long the last row tile gets a launch of its own (one row tile per CTA, two thirds
   // of the time per key tile, every CTA on it): 8 sequences of 65 nodes, 8 layers, G = 4: 305 -> 274 us.  It reads K/V a
-  // second time and costs a fill and a tail of some 12 us, hence the bound on the key tiles per SM.
-  if (MT == 2 && g.n_row_tiles % 2 == 1 && units * tiles >= 60ll * g.sms) {
+  // second time and costs a fill and a tail of some 12 us, hence a bound on the key tiles per SM.  Only the capacity of the
+  // cache is known here: where it allows that many, both launches are made, and both go by the lengths on the device (8
+  // sequences of 65 nodes with prefixes of 300 in a paged cache of 32768, one layer: 34.4 -> 23.2 us against two full launches;
+  // 20.0 in a cache of 512, the difference is the launch that finds nothing to do).
+  if (MT == 2 && g.n_row_tiles % 2 == 1 && units * tiles >= (long long)kSplitTilesPerSm * g.sms) {
     AttnParams front = prm;
-    front.NP = g.n_row_tiles / 2;
-    front.groups = g.sms / front.NP;
-    const cudaError_t e = launch_kernel<D, MT, false>((unsigned)(front.groups * front.NP), 1, maps, front, s);
+    front.split_tiles = kSplitTilesPerSm * g.sms;
+    front.front_NP = g.n_row_tiles / 2;
+    front.front_groups = g.sms / front.front_NP;
+    const int ctas = front.front_groups * front.front_NP;
+    const cudaError_t e = launch_kernel<D, MT, false>((unsigned)(ctas > g.grid ? ctas : g.grid), 1, maps, front, s);
     if (e != cudaSuccess) return e;
     tv::count_launches(1);
+    prm.split_tiles = front.split_tiles;
     prm.tile0 = g.n_row_tiles - 1;
     prm.NP = 1;
     prm.groups = g.sms;

@@ -629,3 +629,63 @@ def test_lengths_that_change_under_the_waiting_launch(G, N, d):
         tv.tree_verify_attn(*args, lengths, dcase["n_nodes"], bits, d ** -0.5, got, ws, status, lse=got_lse)
         assert torch.equal(got, out) and torch.equal(got_lse, lse), other
     assert not status.any()
+
+
+ODD = [(65, 64, False), (65, 128, True), (129, 64, True), (129, 128, False)]      # N, d, paged: three and five row tiles of G = 4
+
+
+@pytest.mark.parametrize("N,d,paged", ODD)
+@pytest.mark.parametrize("what", ["short", "below", "at", "long"])
+def test_last_row_tile_goes_by_the_lengths_and_not_by_the_capacity(N, d, paged, what):
+    """A cache that could hold enough key tiles for two launches.  With short prefixes the call gives the bits it gives in a small
+    cache, where it is one launch; one key tile below the bound, at it and beyond it, the oracle's values on sampled heads."""
+    B, L, Hkv, G, cap = 10, 4, 8, 4, 4480
+    TT = (N + 127) // 128
+    cfg = CONFIGS[0].scaled(B=B, L=L, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=20, S_hi=400, Scap=cap, N=N, D=6, V=0, tree="uniform")
+    case = make_case(cfg, seed=N + d, device="cuda", ragged_nodes=True, with_logits=False)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if what != "short":
+        bound = -(-60 * sms // (L * Hkv))                  # key tiles of the sequences together at which the rule changes
+        total = {"below": bound - 1, "at": bound, "long": bound + 37}[what]
+        tiles = np.full(B, total // B) + (np.arange(B) < total % B)
+        tiles[0] -= 3
+        tiles[1] += 3
+        rows = (tiles - TT) * 128 - np.random.default_rng(N).integers(0, 128, B)
+        assert rows.max() <= cap and rows.min() > 0
+        case["prefix_len"] = torch.from_numpy(rows.astype(np.int32)).cuda()
+    bits = torch.zeros(B, N, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    st = torch.zeros(B, dtype=torch.int32, device="cuda")
+    tv.tree_build_mask(case["parent"], case["n_nodes"], N - 1, 1, bits, st)
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(B, N, cfg.Hq, Hkv, d, cap), dtype=torch.uint8, device="cuda")
+
+    def run(rows):
+        out = torch.full((L, B, N, cfg.Hq, d), 3.0, dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((L, B, cfg.Hq, N), 3.0, dtype=torch.float32, device="cuda")
+        kc, vc = (case[k][:, :, :, :rows].contiguous() for k in ("k_cache", "v_cache"))
+        n0 = tv.tv_launch_count()
+        if paged:
+            kp, vp = (t.reshape(L, B, Hkv, rows // 128, 128, d).transpose(2, 3).reshape(L, -1, Hkv, 128, d).contiguous() for t in (kc, vc))
+            table = torch.arange(B * (rows // 128), dtype=torch.int32, device="cuda").view(B, -1)
+            tv.tree_verify_attn_paged_layers(case["q"], kp, vp, table, case["k_tree"], case["v_tree"], case["prefix_len"],
+                                             case["n_nodes"], bits, d ** -0.5, out, ws, st, lse=lse)
+        else:
+            tv.tree_verify_attn_layers(case["q"], kc, vc, case["k_tree"], case["v_tree"], case["prefix_len"], case["n_nodes"],
+                                       bits, d ** -0.5, out, ws, st, lse=lse)
+        launches = tv.tv_launch_count() - n0
+        torch.cuda.synchronize()
+        assert (st == 0).all()
+        return out, lse, launches
+
+    out, lse, launches = run(cap)
+    assert launches == 2
+    if what == "short":
+        small, small_lse, launches = run(512)
+        assert launches == 1 and torch.equal(out, small) and torch.equal(lse, small_lse)
+    again, again_lse, _ = run(cap)
+    assert torch.equal(out, again) and torch.equal(lse, again_lse)
+    cn = case_to_numpy(case)
+    vis = oracle_visibility(case["parent"], case["n_nodes"], bits_gpu=bits)[:, 0]
+    for l, b, hk in ((0, 0, 0), (L - 1, 1, 7), (L // 2, 9, 3)):
+        ref_out, ref_lse = oracle_attention_slice(cn, l, b, hk, G, vis, d ** -0.5)
+        assert_attention_close(out[l][b:b + 1, :, hk * G:(hk + 1) * G], lse[l][b:b + 1, hk * G:(hk + 1) * G], ref_out, ref_lse,
+                               f"{l} {b} {hk}")
