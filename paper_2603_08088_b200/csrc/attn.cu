@@ -84,12 +84,17 @@ constexpr int kSetupCost = TV_SETUP_COST;
 #endif
 constexpr int kPrefetchTiles = TV_PREFETCH_TILES;
 constexpr int kMaxGroups = 160;
-// do not spread a small problem over more CTA groups than this allows (measured on the 7B-shaped single
-// sequence: 12 -> 26 us, 6 -> 22 us, 4 -> 23 us per launch)
+// do not spread a small problem over more CTA groups than this allows.  Few short units outside the cluster kernel's range, us a
+// call for 6 / 8: 16 sequences of 150 to 600 with 8 KV heads, 60 nodes 22.3 / 25.4, two of 2300 in a cache of 32768 25.6 / 28.3,
+// four of 1000, 17 nodes 17.9 / 19.3.
 #ifndef TV_MIN_VT
 #define TV_MIN_VT 6
 #endif
 constexpr int kMinVirtualTilesPerGroup = TV_MIN_VT;
+// Virtual tiles of a unit up to which equal units stay whole, on one group each.  us a call, cut / whole, 8 KV heads: 8 sequences
+// of 65 nodes, prefixes of 300 19.9 / 16.6, 600 22.8 / 19.4, 1000 26.8 / 23.9, 2300 41.0 / 39.1; 10 of 20 nodes 15.7 / 12.9, 17.5 /
+// 14.6, 20.4 / 17.8, 26.7 / 29.2; 12 of 40 nodes with 64-wide heads 15.2 / 14.2, 19.2 / 17.1, 23.5 / 21.6, 34.4 / 36.8.
+constexpr int kMaxWholeUnit = 13;
 constexpr int kSplitTilesPerSm = 60;       // from here on an odd last row tile has a launch of its own (see launch)
 constexpr int kMaxCluster = 8;     // CTAs that share a unit (16 is not portable; few clusters of 16 fit the GPU at once: 21.7 us
                                    // instead of 10.8 us a launch for eight units of 12 key tiles)
@@ -606,7 +611,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   while (!CL) {
     if (warp == 0) {
-      int run = 0;
+      int run = 0, first_len = 0;
+      bool same = true;      // every unit has the key tiles of the first
       // Under the caller's promise this warp reads lengths, node counts and pages before the wait: the fence drops what an
       // earlier launch on this SM has left of them in L1.  (Loads past L1 in the item walk, which goes on behind the wait,
       // cost 16 sequences of 600 to 1000 1 to 3 %.)
@@ -628,33 +634,38 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         if (b < prm.B) cum[b] = run + inc - len;
         run += __shfl_sync(0xffffffffu, inc, 31);
+        if (base == 0) first_len = __shfl_sync(0xffffffffu, len, 0);
+        same = same && (b >= prm.B || len == first_len);
       }
-      if (lane == 0) cum[prm.B] = run;
+      same = __all_sync(0xffffffffu, same);
+      if (lane == 0) {
+        cum[prm.B] = run;
+        // Small problems use fewer CTA groups, so that a unit is cut into few pieces (each piece costs a partial
+        // write and a merge) and every group still gets a worthwhile share of tiles.
+        const int units = prm.B * prm.Hkv * prm.L;
+        const bool split = MT == 2 && prm.split_tiles > 0 && splits(run - prm.B * kSetupCost);
+        const int np = split ? prm.front_NP : prm.NP, max_groups = split ? prm.front_groups : prm.groups;
+        const int want = (int)((unsigned)(prm.Hkv * run) * (unsigned)prm.L / (unsigned)kMinVirtualTilesPerGroup);
+        int n = want < 1 ? 1 : (want < max_groups ? want : max_groups);
+        // A group count just above a multiple of the unit count is rounded down to it: with units of equal length
+        // (one sequence, all heads) every unit is then cut into the same number of equal pieces and no cut falls
+        // just behind a unit boundary.  Not worth more than 1/16 of the groups, but for short units of equal length:
+        // those stay whole, one a group, because a cut and its merge cost more than the idle groups.
+        const int over = n % units;
+        if (n > units && (over * 16 <= n || (n < 2 * units && same && first_len <= kMaxWholeUnit))) n -= over;
+        at[2] = n;
+        at[3] = np;
+      }
     }
     __syncthreads();
-    // Small problems use fewer CTA groups, so that a unit is cut into few pieces (each piece costs a partial
-    // write and a merge) and every group still gets a worthwhile share of tiles.
     const unsigned total = (unsigned)(prm.Hkv * cum[prm.B]) * (unsigned)prm.L;
-    const unsigned want = total / (unsigned)kMinVirtualTilesPerGroup;
-    const bool split = MT == 2 && prm.split_tiles > 0 && splits(cum[prm.B] - prm.B * kSetupCost);
-    const int np = split ? prm.front_NP : prm.NP, max_groups = split ? prm.front_groups : prm.groups;
-    groups = want < 1u ? 1 : (want < (unsigned)max_groups ? (int)want : max_groups);
-    // A group count just above a multiple of the unit count is rounded down to it: with units of equal length
-    // (one sequence, all heads) every unit is then cut into the same number of equal pieces and no cut falls
-    // just behind a unit boundary.  Not worth more than 1/16 of the groups.
-    {
-      const int units = prm.B * prm.Hkv * prm.L, over = groups % units;
-      if (groups > units && over * 16 <= groups) groups -= over;
-    }
+    const int np = at[3];
+    groups = at[2];
     // gs[k] = floor(total * k / groups) in 32-bit arithmetic: total = q * groups + r
     const unsigned q = total / (unsigned)groups, r = total % (unsigned)groups;
 #pragma unroll 1
     for (int k = threadIdx.x; k <= kMaxGroups; k += kThreads)
       gs[k] = k <= groups ? (int)(k * q + (k * r) / (unsigned)groups) : (int)total;
-    if (threadIdx.x == 0) {
-      at[2] = groups;
-      at[3] = np;
-    }
     __syncthreads();
     sch.per_layer = prm.Hkv * cum[prm.B];
     sch.total = sch.per_layer * prm.L;

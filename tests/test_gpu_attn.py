@@ -689,3 +689,19 @@ def test_last_row_tile_goes_by_the_lengths_and_not_by_the_capacity(N, d, paged, 
         ref_out, ref_lse = oracle_attention_slice(cn, l, b, hk, G, vis, d ** -0.5)
         assert_attention_close(out[l][b:b + 1, :, hk * G:(hk + 1) * G], lse[l][b:b + 1, hk * G:(hk + 1) * G], ref_out, ref_lse,
                                f"{l} {b} {hk}")
+
+
+@pytest.mark.parametrize("G,N,d", [(2, 40, 64), (4, 40, 64), (2, 40, 128), (4, 40, 128)])
+@pytest.mark.parametrize("S,other", [(300, 300), (1024, 1024), (1025, 1025), (300, 100)])
+def test_equal_units_stay_whole_while_they_are_short(S, other, G, N, d):
+    """Fewer units than CTA groups, but more than half: of equal length up to eight prefix tiles (whole, one a group), one row
+    beyond that and with one shorter unit (cut)."""
+    cfg = CONFIGS[0].scaled(B=90, Hq=G, Hkv=1, d=d, S_lo=S, S_hi=S, Scap=S + 64, N=N, D=6, V=0, tree="uniform")
+    case = make_case(cfg, seed=S + G + d + other, ragged_nodes=True, with_logits=False)
+    case["prefix_len"][17] = other
+    dcase = to_device(case)
+    out, lse, bits, dense = gpu_attention(dcase)
+    ref_out, ref_lse = oracle_attention(case_to_numpy(case), dense.cpu().numpy())
+    assert_attention_close(out, lse, ref_out, ref_lse, f"S={S} {other}")
+    out2, lse2, _, _ = gpu_attention(dcase)
+    assert torch.equal(out, out2) and torch.equal(lse, lse2)
