@@ -453,6 +453,7 @@ struct SmemLayout {
   static_assert(kTotal <= 232448, "shared memory of a CTA");
   static constexpr int kMl = kCum;                         // cluster kernel: (m, l) of every row, in place of the tile table
   static_assert(kMl + MT * 128 * 8 <= kTotal && kMl % 8 == 0, "(m, l) pairs fit the room of the tile table");
+  static_assert(MT * 128 * D * 4 <= kSlots * kTileBytes, "fp32 partials of the cluster kernel fit the K/V ring");
 };
 
 // ---------------------------------------------------------------- the kernel
@@ -1328,7 +1329,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           // Wait for every MMA of the item.  This barrier completes once per item, so its phase is never
           // more than one away from the one waited for (a parity wait cannot tell phases two apart, which
           // is why the per-PV barrier O_DONE is not used here: both last PVs may or may not be done yet).
-          ok = wwait(bar(L::ITEM_DONE + (MT == 1 ? 0 : wg)), item_cnt & 1);
+          // (Cluster kernel: of both row tiles, whose V the partials overwrite; the pipe works in issue order.)
+          ok = wwait(bar(L::ITEM_DONE + (MT == 1 ? 0 : (CL ? 1 : wg))), item_cnt & 1);
           ++item_cnt;
           if (!ok) break;
           tc_fence_after();
@@ -1398,23 +1400,18 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             }
           };
           if (CL) {
-            // ---- the partial of this CTA: normalised bf16 rows over the Q tile (every QK^T of the item is done), 16-byte
-            // pieces of a row swizzled by the row so that neither the writes nor the reads collide; (m, l) beside them
-            const float inv = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
-            uint8_t* mine = smem + L::kQ + (MT == 1 ? 0 : wg) * L::kTileBytes + row * (D * 2);
+            // ---- the partial of this CTA: O as it is, fp32 rows over the K/V ring (every MMA of the item is done, and a CTA
+            // has one item), 16-byte pieces of a row swizzled by the row so that neither the writes nor the reads collide;
+            // (m, l) beside them
+            uint8_t* mine = smem + L::kRing + ((MT == 1 ? 0 : wg) * 128 + row) * (D * 4);
 #pragma unroll 1
             for (int q = q0; q < q0 + kGroups; ++q) {
               uint32_t o[32];
               load_own(q, o);
 #pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                uint4 v;
-                v.x = pack_bf16(__uint_as_float(o[8 * c + 0]) * inv, __uint_as_float(o[8 * c + 1]) * inv);
-                v.y = pack_bf16(__uint_as_float(o[8 * c + 2]) * inv, __uint_as_float(o[8 * c + 3]) * inv);
-                v.z = pack_bf16(__uint_as_float(o[8 * c + 4]) * inv, __uint_as_float(o[8 * c + 5]) * inv);
-                v.w = pack_bf16(__uint_as_float(o[8 * c + 6]) * inv, __uint_as_float(o[8 * c + 7]) * inv);
-                *reinterpret_cast<uint4*>(mine + (((q * 4 + c) ^ (row & 7)) * 16)) = v;
-              }
+              for (int c = 0; c < 8; ++c)
+                *reinterpret_cast<uint4*>(mine + (((q * 8 + c) ^ (row & 7)) * 16)) =
+                    make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
             }
             m_fin = m_used;
             l_fin = l_sum;
@@ -1622,8 +1619,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     if (CL) {
       // ---- merge of the cluster's partials: each CTA takes a share of the rows, 16 bytes of a row per thread; out =
-      // sum_p w_p O_p / sum_p w_p, w_p = l_p 2^(m_p - max m), in rank order.  A piece without keys has weight 0 (its rows
-      // were not written and are not used).
+      // sum_p w_p O_p / sum_p w_p l_p, w_p = 2^(m_p - max m), in rank order, all in fp32.  A piece without keys has weight 0
+      // (its rows were not written and are not used).  With normalised bf16 partials outputs were further from 64 bits than
+      // those of units in one piece: relative error 2.70e-3 to 2.87e-3, now 2.12e-3 to 2.34e-3.  A layer of one sequence, 8 KV
+      // heads, 1392 rows: 17 nodes 10.1 us as before, 60 nodes 14.2 -> 15.3 (what is read from other CTAs sets the pace there; the
+      // two halves of a row go to the columns c and D/2 + c, so that eight lanes never meet in a bank).
       if (MT == 2 || wg == 0) *reinterpret_cast<float2*>(smem + L::kMl + (wg * 128 + row) * 8) = make_float2(m_fin, l_fin);
       const int size = (int)cluster_size_x(), rank = (int)(blockIdx.x % size);
       const int u = unit / prm.NP, hk = u % prm.Hkv, b = u / prm.Hkv % prm.B, layer = u / prm.Hkv / prm.B;
@@ -1642,16 +1642,17 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const int node_l = r / prm.G, gm = r - node_l * prm.G;
           const int t = MT == 2 && node_l >= prm.NPT ? 1 : 0, in_tile = (node_l - t * prm.NPT) * prm.G + gm;
           const uint32_t ml = sbase + L::kMl + (t * 128 + in_tile) * 8;
-          const uint32_t at = sbase + L::kQ + t * L::kTileBytes + in_tile * (D * 2) + ((c ^ (in_tile & 7)) * 16);
-          float pm[kMaxCluster], w[kMaxCluster];
-          uint4 v[kMaxCluster];
+          const uint32_t at_lo = sbase + L::kRing + (t * 128 + in_tile) * (D * 4) + ((c ^ (in_tile & 7)) * 16), at_hi = at_lo + kVecs * 16;
+          float pm[kMaxCluster], l[kMaxCluster];
+          uint4 v[kMaxCluster], u[kMaxCluster];
 #pragma unroll
           for (int k = 0; k < kMaxCluster; ++k)
             if (k < size) {
               const float2 p = ld_peer_8B(peer_smem(ml, k));
               pm[k] = p.x;
-              w[k] = p.y;
-              v[k] = ld_peer_16B(peer_smem(at, k));
+              l[k] = p.y;
+              v[k] = ld_peer_16B(peer_smem(at_lo, k));
+              u[k] = ld_peer_16B(peer_smem(at_hi, k));
             }
           float mm = -INFINITY;
 #pragma unroll
@@ -1661,26 +1662,23 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
           for (int k = 0; k < kMaxCluster; ++k)
             if (k < size) {
-              const float wk = pm[k] > -INFINITY ? w[k] * fast_exp2(pm[k] - mm) : 0.f;
-              lt += wk;
-              const uint32_t e[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-              if (wk > 0.f)
+              if (pm[k] > -INFINITY) {
+                const float wk = fast_exp2(pm[k] - mm);
+                lt = fmaf(wk, l[k], lt);
+                const uint32_t e[8] = {v[k].x, v[k].y, v[k].z, v[k].w, u[k].x, u[k].y, u[k].z, u[k].w};
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  acc[2 * i] = fmaf(wk, __uint_as_float(e[i] << 16), acc[2 * i]);
-                  acc[2 * i + 1] = fmaf(wk, __uint_as_float(e[i] & 0xffff0000u), acc[2 * i + 1]);
-                }
+                for (int i = 0; i < 8; ++i) acc[i] = fmaf(wk, __uint_as_float(e[i]), acc[i]);
+              }
             }
           const int node = node0 + node_l, h = hk * prm.G + gm;
           const bool any_key = node < n && mm > -INFINITY;
           const float inv = any_key ? 1.f / lt : 0.f;
-          uint4 o;
-          o.x = pack_bf16(acc[0] * inv, acc[1] * inv);
-          o.y = pack_bf16(acc[2] * inv, acc[3] * inv);
-          o.z = pack_bf16(acc[4] * inv, acc[5] * inv);
-          o.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-          if (!any_key) o = make_uint4(0, 0, 0, 0);
-          *reinterpret_cast<uint4*>(prm.out + (size_t)layer * prm.out_layer_stride + (((size_t)b * prm.Nmax + node) * prm.Hq + h) * D + c * 8) = o;
+          uint2 lo = make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
+          uint2 hi = make_uint2(pack_bf16(acc[4] * inv, acc[5] * inv), pack_bf16(acc[6] * inv, acc[7] * inv));
+          if (!any_key) lo = hi = make_uint2(0, 0);
+          tv_bf16* dst = prm.out + (size_t)layer * prm.out_layer_stride + (((size_t)b * prm.Nmax + node) * prm.Hq + h) * D + c * 4;
+          *reinterpret_cast<uint2*>(dst) = lo;
+          *reinterpret_cast<uint2*>(dst + D / 2) = hi;
           if (c == 0 && prm.lse)
             prm.lse[(((size_t)layer * prm.B + b) * prm.Hq + h) * prm.Nmax + node] = any_key ? (mm + log2f(lt)) / kLog2e : -INFINITY;
         }

@@ -705,3 +705,27 @@ def test_equal_units_stay_whole_while_they_are_short(S, other, G, N, d):
     assert_attention_close(out, lse, ref_out, ref_lse, f"S={S} {other}")
     out2, lse2, _, _ = gpu_attention(dcase)
     assert torch.equal(out, out2) and torch.equal(lse, lse2)
+
+
+@pytest.mark.parametrize("B,Hkv,G,N,S,d", [(1, 2, 2, 15, 128, 64), (1, 8, 4, 17, 1000, 128), (1, 32, 1, 60, 1300, 128),
+                                           (3, 4, 8, 40, 513, 64), (1, 5, 4, 200, 777, 128), (1, 1, 4, 60, 6200, 64)])
+def test_cluster_partials_are_not_rounded(B, Hkv, G, N, S, d):
+    """Zero keys: every weight is 1 and an output is a mean of values in [1, 2).  Units shared by a cluster give the bf16 rounding
+    of the exact mean: partials in 32 bits leave an error of 2^-14 of it at most (2^-23 for each of the up to 500 sums of 16 keys),
+    where partials rounded to bf16 (2^-8 each) miss the right rounding in one element of five."""
+    cfg = CONFIGS[0].scaled(B=B, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=S, S_hi=S, Scap=S + 40, N=N, D=min(6, N - 1), V=0, tree="uniform")
+    case = to_device(make_case(cfg, seed=S + G + N, with_logits=False))
+    g = torch.Generator(device="cuda")
+    g.manual_seed(S)
+    for k in ("k_cache", "k_tree"):
+        case[k].zero_()
+    for k in ("v_cache", "v_tree"):
+        case[k].copy_(torch.rand(case[k].shape, device="cuda", generator=g) * 0.98 + 1.0)
+    out, _, _, dense = gpu_attention(case)
+    vis = dense.reshape(B, N, N).cuda().double()
+    tree = torch.einsum("bij,bjhd->bihd", vis, case["v_tree"][0].double())
+    prefix = case["v_cache"][0][:, :, :S].double().sum(2)                       # [B, Hkv, d]
+    exact = (tree + prefix[:, None]) / (S + vis.sum(-1))[:, :, None, None]      # [B, N, Hkv, d]
+    exact = exact.repeat_interleave(G, dim=2)
+    best = (exact.to(torch.bfloat16).double() - exact).abs()
+    assert ((out.cuda().reshape(exact.shape).double() - exact).abs() <= best + 2.0 ** -14 * exact).all()
