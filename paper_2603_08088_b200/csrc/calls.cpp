@@ -51,12 +51,12 @@ struct Args {
     if (!t.is_contiguous()) raise(PyExc_AssertionError, "treeverify takes dense tensors");
     return static_cast<T*>(t.data_ptr());
   }
-  // ... of a tensor [L, ...] whose layers are dense, L of them.
+  // ... of a tensor [L, ...] whose layers are dense, L of them or (more) at least L.
   template <typename T = void>
-  T* layers(int i, int64_t L) const {
+  T* layers(int i, int64_t L, bool more = false) const {
     if (none(i)) return nullptr;
     const at::Tensor& t = tensor(i);
-    bool dense = t.dim() >= 1 && t.size(0) == L;
+    bool dense = t.dim() >= 1 && (more ? t.size(0) >= L : t.size(0) == L);
     int64_t want = 1;
     for (int64_t d = t.dim() - 1; d >= 1 && dense; --d) {
       dense = t.size(d) == 1 || t.stride(d) == want;
@@ -209,19 +209,20 @@ PyObject* verify_attn_paged_layers(PyObject* const* a, Py_ssize_t n) {
   const at::Tensor &q = x.tensor(0, 5), &kp = x.tensor(1, 5), &table = x.tensor(3, 2);
   const int L = q.size(0), B = q.size(1), N = q.size(2), Hq = q.size(3), d = q.size(4), pages = kp.size(1), Hkv = kp.size(2),
             blocks = table.size(1);
-  const auto *pq = x.layers<tv_bf16>(0, L), *pk = x.layers<tv_bf16>(1, L), *pv = x.layers<tv_bf16>(2, L);
+  // the first L layers of pools, trees and outputs that may have more
+  const auto *pq = x.layers<tv_bf16>(0, L), *pk = x.layers<tv_bf16>(1, L, true), *pv = x.layers<tv_bf16>(2, L, true);
   const auto* bt = x.ptr<int32_t>(3);
-  const auto *kt = x.layers<tv_bf16>(4, L), *vt = x.layers<tv_bf16>(5, L);
-  if (x.layer_stride(1) != x.layer_stride(2) || x.layer_stride(4) != x.layer_stride(5))
+  const auto *kt = x.layers<tv_bf16>(4, L, true), *vt = x.layers<tv_bf16>(5, L, true);
+  if (L > 1 && (x.layer_stride(1) != x.layer_stride(2) || x.layer_stride(4) != x.layer_stride(5)))
     raise(PyExc_AssertionError, "treeverify: K and V need the same layer stride");
   const auto *S = x.ptr<int32_t>(6), *nn = x.ptr<int32_t>(7);
   const auto* bits = x.ptr<uint32_t>(8);
   const float scale = x.number(9);
-  auto* out = x.layers<tv_bf16>(10, L);
+  auto* out = x.layers<tv_bf16>(10, L, true);
   void* ws = x.ptr(11);
   const size_t wsb = x.bytes(11);
   auto* st = x.ptr<int32_t>(12);
-  x.layers(13, L);
+  x.layers(13, L, true);
   auto* lse = x.ptr<float>(13);
   const unsigned flags = (unsigned)x.integer(14);
   const tv_stream s = x.stream(15);

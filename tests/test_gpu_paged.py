@@ -242,3 +242,35 @@ def test_paged_layers_call_equals_layer_by_layer_calls():
                                               case_np["k_tree"][l], case_np["v_tree"][l], case_np["prefix_len"],
                                               case_np["n_nodes"], vis[:, 0], d ** -0.5)
         assert_attention_close(allq[l], lse_all[l], ref_out, ref_lse, f"layer {l}")
+
+
+def test_paged_layers_call_takes_the_first_layers_of_larger_tensors():
+    """Two layers of queries over pools, trees, outputs and log-sum-exps of five; one layer whose K and V pools have layer
+    strides of their own."""
+    cfg = CONFIGS[0].scaled(B=3, L=5, S_lo=0, S_hi=500, Scap=512, N=20, Hq=8, Hkv=2, d=64, V=0)
+    c = to_device(make_case(cfg, seed=5, with_logits=False))
+    B, N, Hq, Hkv, d = cfg.B, cfg.N, cfg.Hq, cfg.Hkv, cfg.d
+    kp, vp = (c[k].reshape(5, B, Hkv, 4, R, d).transpose(2, 3).reshape(5, B * 4, Hkv, R, d).contiguous() for k in ("k_cache", "v_cache"))
+    table = torch.arange(B * 4, dtype=torch.int32, device="cuda").view(B, 4)
+    bits = torch.zeros(B, N, 1, dtype=torch.int32, device="cuda")
+    st = torch.zeros(B, dtype=torch.int32, device="cuda")
+    tv.tree_build_mask(c["parent"], c["n_nodes"], N - 1, 1, bits, st)
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(B, N, Hq, Hkv, d, 512), dtype=torch.uint8, device="cuda")
+
+    def run(L, q, kp, vp, kt, vt, layers):
+        out = torch.full((layers, B, N, Hq, d), 3.0, dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((layers, B, Hq, N), 3.0, device="cuda")
+        tv.tree_verify_attn_paged_layers(q, kp, vp, table, kt, vt, c["prefix_len"], c["n_nodes"], bits, d ** -0.5, out, ws, st, lse=lse)
+        torch.cuda.synchronize()
+        assert (out[L:] == 3.0).all() and (lse[L:] == 3.0).all()
+        return out[:L], lse[:L]
+
+    dense = run(2, c["q"][:2], kp[:2], vp[:2], c["k_tree"][:2], c["v_tree"][:2], 2)
+    larger = run(2, c["q"][:2], kp, vp, c["k_tree"], c["v_tree"], 5)
+    assert all(torch.equal(a, b) for a, b in zip(dense, larger))
+    one = run(1, c["q"][:1], kp[:1], vp[::2][:1], c["k_tree"][:1], c["v_tree"][::3][:1], 1)
+    first = run(1, c["q"][:1], kp[:1], vp[:1], c["k_tree"][:1], c["v_tree"][:1], 1)
+    assert all(torch.equal(a, b) for a, b in zip(one, first))
+    assert (i32(st) == 0).all()
+    with pytest.raises(AssertionError):                    # pools of fewer layers than the queries
+        run(2, c["q"][:2], kp[:1], vp[:1], c["k_tree"], c["v_tree"], 2)
