@@ -306,4 +306,6 @@ def kv_commit_inplace(k_cache, v_cache, accepted_nodes, accept_len, prefix_len, 
 def tv_verify_step_host(host, k_cache, v_cache, prefix_len, staging, scale, V, stream=None):
     """``host``: dict of pinned CPU tensors parent, n_nodes, tokens, retrieve_indices (or None), q, k_tree,
     v_tree, logits and outputs out, accept_len, accepted_nodes, next_token, status."""
+    if not isinstance(host, dict):
+        host = dict(host)
     _check((_calls or _native()).tv_verify_step_host(host, k_cache, v_cache, prefix_len, staging, scale, V, stream))

@@ -2,6 +2,8 @@
 (reduced where the fp64 oracle would take minutes; the attention of the
 full-size configs is covered head-by-head in test_gpu_attn.py), the
 commit-equivalence property, and the host-buffer entry point."""
+import types
+
 import numpy as np
 import pytest
 import torch
@@ -124,7 +126,7 @@ def test_host_buffer_step_matches_device_step():
 SMALL_INPUTS = ("parent", "n_nodes", "tokens", "retrieve_indices")
 
 
-def _host_step(cfg, seed, given_rows, stream=None, queued=False, pinned=True):
+def _host_step(cfg, seed, given_rows, stream=None, queued=False, pinned=True, as_mapping=dict):
     """``queued``: the small inputs are still those of another tree when the call is made; copies behind a few
     milliseconds of work on the same stream bring the right ones."""
     case = make_case(cfg, seed=seed)
@@ -154,7 +156,7 @@ def _host_step(cfg, seed, given_rows, stream=None, queued=False, pinned=True):
                 busy.add_(1.0)
             for k, t in new.items():
                 host[k].copy_(t, non_blocking=True)
-    tv.tv_verify_step_host(host, kc, vc, S, staging, cfg.d ** -0.5, cfg.V, stream=stream)
+    tv.tv_verify_step_host(as_mapping(host), kc, vc, S, staging, cfg.d ** -0.5, cfg.V, stream=stream)
     assert np.abs(host["out"].float().numpy() - ref["out"]).max() <= ATTN_ATOL
     for k in ("accept_len", "accepted_nodes", "next_token"):
         assert np.array_equal(host[k].numpy(), ref["accept"][k]), k
@@ -192,3 +194,7 @@ def test_host_buffer_step_reads_its_inputs_behind_the_work_in_front(over, given_
 
 def test_host_buffer_step_with_pageable_small_inputs():
     _host_step(CONFIGS[4].scaled(**HOST_STEPS[0]), 79, True, pinned=False)
+
+
+def test_host_buffers_in_any_mapping():
+    _host_step(CONFIGS[4].scaled(**HOST_STEPS[0]), 80, True, as_mapping=types.MappingProxyType)
