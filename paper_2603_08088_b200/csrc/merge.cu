@@ -44,6 +44,7 @@ merge_partials_kernel(const uint4* __restrict__ o_parts, const float* __restrict
   float m = -INFINITY;                                 // running maximum: more than kHold ranges rescale what they find
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   float tot = 0.f;
+  bool nan = false;                                    // a log-sum-exp that is NaN: the row is NaN, unless no range has a key
   for (int r0 = 0; r0 < R; r0 += kHold) {
     float w[kHold];
     uint4 v[kHold];
@@ -54,17 +55,20 @@ merge_partials_kernel(const uint4* __restrict__ o_parts, const float* __restrict
       if (r0 + k < R) v[k] = __ldcs(op + (r0 + k) * rows * d8);
     float mx = m;
 #pragma unroll
-    for (int k = 0; k < kHold; ++k) mx = fmaxf(mx, w[k]);
+    for (int k = 0; k < kHold; ++k) {
+      mx = fmaxf(mx, w[k]);
+      nan |= w[k] != w[k];
+    }
     if (mx == -INFINITY) continue;
     const float keep = expf(m - mx);                   // 0 the first time
     m = mx;
     tot *= keep;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] *= keep;
+    for (int i = 0; i < 8; ++i) acc[i] = keep == 0.f ? 0.f : acc[i] * keep;      // (what has no weight left may not be finite)
 #pragma unroll
     for (int k = 0; k < kHold; ++k) {
       const float wk = expf(w[k] - mx);
-      if (wk > 0.f) {                                  // the payload of an empty range (weight 0) may be anything
+      if (wk != 0.f) {                                 // the payload of an empty range (weight 0) may be anything
         tot += wk;
         const uint32_t e[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
@@ -75,6 +79,7 @@ merge_partials_kernel(const uint4* __restrict__ o_parts, const float* __restrict
       }
     }
   }
+  if (nan && m > -INFINITY) tot = acc[0] = acc[1] = acc[2] = acc[3] = acc[4] = acc[5] = acc[6] = acc[7] = NAN;
   const float inv = tot > 0.f ? 1.f / tot : 0.f;
   uint4 o;
   o.x = pack_bf16(acc[0] * inv, acc[1] * inv);

@@ -133,3 +133,32 @@ def test_merge_counts_around_the_ranges_in_flight(R):
     # one bf16 rounding of the result (2^-9 of it) and fp32 sums (2^-20 of the largest term)
     assert ((out.double().cpu() - want).abs() <= 2.0 ** -8 * want.abs() + 1e-4).all()
     assert (lout.double().cpu() - torch.logsumexp(lse.double(), 0)).abs().max() <= 1e-4
+
+
+@pytest.mark.parametrize("R", [2, 4, 5, 9])
+def test_merge_of_values_that_are_not_finite(R):
+    """A NaN or infinite log-sum-exp makes its row NaN wherever it stands, also beside ranges without keys only; the payload of a
+    range whose weight is 0, because it is empty or far below the others, may be anything."""
+    B, N, Hq, d = 1, 6, 2, 16
+    g = torch.Generator().manual_seed(R)
+    inf, nan = float("inf"), float("nan")
+    for at in range(R):
+        o = torch.randn(R, B, N, Hq, d, generator=g).to(torch.bfloat16)
+        lse = torch.randn(R, B, Hq, N, generator=g)
+        lse[at, :, :, 0] = nan
+        lse[at, :, :, 1] = inf
+        lse[at, :, :, 2], o[at, :, 2] = -200.0, inf
+        lse[at, :, :, 3], o[at, :, 3] = -200.0, nan
+        lse[:, :, :, 4], lse[at, :, :, 4] = -inf, nan             # no range has a key
+        out = torch.full((B, N, Hq, d), 3.0, dtype=torch.bfloat16, device="cuda")
+        lout = torch.full((B, Hq, N), 3.0, device="cuda")
+        tv.tree_merge_partials(o.cuda(), lse.cuda(), out, lout)
+        out, lout = out.cpu().double(), lout.cpu()
+        assert torch.isnan(out[:, :2]).all() and torch.isneginf(lout[:, :, :2]).all()
+        assert (out[:, 4] == 0).all() and torch.isneginf(lout[:, :, 4]).all()
+        for n in (2, 3, 5):
+            rest = [r for r in range(R) if n == 5 or r != at]
+            w = torch.softmax(lse[rest][..., n].double(), 0)[..., None]
+            want = (w * o[rest][:, :, n].double()).sum(0)
+            assert ((out[:, n] - want).abs() <= 2.0 ** -8 * want.abs() + 1e-4).all(), (at, n)
+            assert (lout[:, :, n].double() - torch.logsumexp(lse[rest][..., n].double(), 0)).abs().max() <= 1e-4
