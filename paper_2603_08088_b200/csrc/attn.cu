@@ -1346,8 +1346,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (!ok) break;
             const float2 a = xch[row], b = xch[128 + row];
             m_used = fmaxf(a.x, b.x);
-            e_0 = a.x > -INFINITY ? fast_exp2(a.x - m_used) : 0.f;
-            e_1 = b.x > -INFINITY ? fast_exp2(b.x - m_used) : 0.f;
+            e_0 = a.x > -INFINITY ? fast_exp2(a.x - m_used) : a.y * 0.f;      // (0, or NaN for a row of NaN scores)
+            e_1 = b.x > -INFINITY ? fast_exp2(b.x - m_used) : b.y * 0.f;
             l_sum = e_0 * a.y + e_1 * b.y;
           }
           constexpr int kGroups = KS ? D / 64 : D / 32;                // groups of 32 columns that this warpgroup finishes,
@@ -1361,8 +1361,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               tmem_wait_ld();
 #pragma unroll
               for (int c = 0; c < 32; ++c) {
-                const float x = e_0 > 0.f ? e_0 * __uint_as_float(o[c]) : 0.f;
-                o[c] = __float_as_uint(e_1 > 0.f ? fmaf(e_1, __uint_as_float(o1[c]), x) : x);
+                const float x = e_0 != 0.f ? e_0 * __uint_as_float(o[c]) : 0.f;
+                o[c] = __float_as_uint(e_1 != 0.f ? fmaf(e_1, __uint_as_float(o1[c]), x) : x);
               }
             } else {
               tmem_wait_ld();
@@ -1531,7 +1531,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               float w_a = l_a * fast_exp2(m_a - mref), w_b = l_b * fast_exp2(m_b - mref), lt = w_own + w_a + w_b;
 #pragma unroll 4
               for (int i = 3; i <= n_other; ++i) lt += __ldcg(ml_of(i) + kRows) * fast_exp2(__ldcg(ml_of(i)) - mref);
-              const bool any_key = row_active && mm > -INFINITY;
+              const bool any_key = row_active && (mm > -INFINITY || lt != lt);      // (a row of NaN scores stays NaN)
               const float inv = any_key ? 1.f / lt : 0.f;
               const float2 own2 = make_float2(w_own, w_own), inv_own2 = make_float2(inv_own, inv_own), inv2 = make_float2(inv, inv);
 #pragma unroll 1
@@ -1604,7 +1604,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                   w_b = l_b * fast_exp2(m_b - mref);
                 }
               }
-              if (row_exists && lse_p && !(KS && wg)) *lse_p = any_key ? (mm + log2f(lt)) / kLog2e : -INFINITY;
+              if (row_exists && lse_p && !(KS && wg)) *lse_p = any_key && mm > -INFINITY ? (mm + log2f(lt)) / kLog2e : -INFINITY;
               tc_fence_before();
             }
           }
@@ -1662,7 +1662,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
           for (int k = 0; k < kMaxCluster; ++k)
             if (k < size) {
-              if (pm[k] > -INFINITY) {
+              if (pm[k] > -INFINITY || l[k] != l[k]) {      // (a row of NaN scores stays NaN)
                 const float wk = fast_exp2(pm[k] - mm);
                 lt = fmaf(wk, l[k], lt);
                 const uint32_t e[8] = {v[k].x, v[k].y, v[k].z, v[k].w, u[k].x, u[k].y, u[k].z, u[k].w};
@@ -1671,7 +1671,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
             }
           const int node = node0 + node_l, h = hk * prm.G + gm;
-          const bool any_key = node < n && mm > -INFINITY;
+          const bool any_key = node < n && (mm > -INFINITY || lt != lt);
           const float inv = any_key ? 1.f / lt : 0.f;
           uint2 lo = make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
           uint2 hi = make_uint2(pack_bf16(acc[4] * inv, acc[5] * inv), pack_bf16(acc[6] * inv, acc[7] * inv));
@@ -1680,7 +1680,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           *reinterpret_cast<uint2*>(dst) = lo;
           *reinterpret_cast<uint2*>(dst + D / 2) = hi;
           if (c == 0 && prm.lse)
-            prm.lse[(((size_t)layer * prm.B + b) * prm.Hq + h) * prm.Nmax + node] = any_key ? (mm + log2f(lt)) / kLog2e : -INFINITY;
+            prm.lse[(((size_t)layer * prm.B + b) * prm.Hq + h) * prm.Nmax + node] =
+                any_key && mm > -INFINITY ? (mm + log2f(lt)) / kLog2e : -INFINITY;
         }
       }
       __syncwarp();

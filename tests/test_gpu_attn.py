@@ -729,3 +729,23 @@ def test_cluster_partials_are_not_rounded(B, Hkv, G, N, S, d):
     exact = exact.repeat_interleave(G, dim=2)
     best = (exact.to(torch.bfloat16).double() - exact).abs()
     assert ((out.cuda().reshape(exact.shape).double() - exact).abs() <= best + 2.0 ** -14 * exact).all()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,Hkv,G,N,S", [(90, 1, 4, 20, 300), (90, 1, 4, 40, 700), (3, 1, 4, 20, 6000), (1, 2, 4, 20, 700), (1, 4, 8, 40, 1500)])
+def test_nan_queries_and_keys_give_nan_rows(B, Hkv, G, N, S, d):
+    """Whole units, units cut in pieces, clusters, one and two row tiles: a query with a NaN gives a NaN row (as does a key with a
+    NaN to the rows that see it) and changes no bit of another row."""
+    cfg = CONFIGS[0].scaled(B=B, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=S // 2 if B < 90 else S, S_hi=S, Scap=S + 20, N=N, D=6, V=0, tree="uniform")
+    case = to_device(make_case(cfg, seed=S + B + d, with_logits=False))
+    want, _, _, dense = gpu_attention(case)
+    case["q"][0, :, 3, 0, 5] = float("nan")
+    case["q"][0, B - 1, N - 1, :, :] = float("nan")
+    case["k_tree"][0, 0, 2, 0, 7] = float("nan")
+    out, _, _, _ = gpu_attention(case)
+    bad = torch.zeros(B, N, G * Hkv, dtype=torch.bool, device="cuda")
+    bad[:, 3, 0] = True
+    bad[B - 1, N - 1] = True
+    bad[0, :, :G] |= dense.reshape(B, N, N)[0, :, 2].bool().cuda()[:, None]
+    assert torch.isnan(out[bad]).all()
+    assert torch.equal(out[~bad], want[~bad])
