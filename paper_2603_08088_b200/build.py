@@ -5,7 +5,9 @@
 Every .cu under csrc/ is compiled to an object file under csrc/build/ and
 linked into paper_2603_08088_b200/libtreeverify.so; csrc/calls.cpp (argument
 marshalling for Python) becomes paper_2603_08088_b200/_calls.so, which links to
-it.  Objects are rebuilt when their source or a header is newer.
+it.  Objects are rebuilt when their source or a header is newer, _calls.so also
+when it was made for another torch or Python.  The library itself needs neither:
+where torch cannot be imported, _calls.so is left out.
 """
 import os
 import shutil
@@ -41,6 +43,7 @@ def _calls_commands():
     root = os.path.dirname(torch.__file__)
     lib, inc = os.path.join(root, "lib"), os.path.join(root, "include")
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    made_for = f"torch {torch.__version__} {torch.__file__}, Python {sys.version}"
     obj = os.path.join(OBJ, "calls.o")
     abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
     compile_cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={abi}",
@@ -50,7 +53,16 @@ def _calls_commands():
     compile_cmd += ["-c", os.path.join(CSRC, "calls.cpp"), "-o", obj]
     link_cmd = ["g++", "-shared", "-o", CALLS, obj, "-L", PKG, "-l:libtreeverify.so", "-L", lib, "-ltorch_python", "-ltorch_cpu",
                 "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + lib]
-    return obj, compile_cmd, link_cmd
+    return obj, compile_cmd, link_cmd, made_for
+
+
+def _calls_stale(obj, made_for):
+    """Whether _calls.so has to be made again: its sources are newer, or it is for another torch or Python."""
+    stamp = obj + ".for"
+    if not (os.path.exists(CALLS) and os.path.exists(obj) and os.path.exists(stamp)) or open(stamp).read() != made_for:
+        return True
+    sources = (os.path.join(CSRC, "calls.cpp"), os.path.join(ROOT, "include", "treeverify.h"))
+    return os.path.getmtime(obj) < max(os.path.getmtime(s) for s in sources)
 
 
 def _newest_header():
@@ -85,11 +97,12 @@ def build(force=False, verbose=False):
         if r.returncode != 0:
             raise RuntimeError(cmd[0] + " failed for " + cmd[-3])
 
-    calls_src = os.path.join(CSRC, "calls.cpp")
-    calls_obj, calls_compile, calls_link = _calls_commands()
-    calls_stale = (force or not os.path.exists(calls_obj)
-                   or os.path.getmtime(calls_obj) < max(os.path.getmtime(calls_src),
-                                                        os.path.getmtime(os.path.join(ROOT, "include", "treeverify.h"))))
+    try:
+        calls_obj, calls_compile, calls_link, made_for = _calls_commands()
+        calls_stale = force or _calls_stale(calls_obj, made_for)
+    except ImportError as e:
+        sys.stderr.write(f"_calls.so is not built: {e}\n")
+        calls_stale = False
     cu_jobs = len(jobs)
     if calls_stale:
         jobs.append(calls_compile)
@@ -99,8 +112,10 @@ def build(force=False, verbose=False):
     if cu_jobs or not os.path.exists(LIB):
         cmd = [nvcc, "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a", "-lcudart_static", "-ldl", "-lrt", "-lpthread"]
         run(cmd)
-    if calls_stale or not os.path.exists(CALLS):
+    if calls_stale:
         run(calls_link)
+        with open(calls_obj + ".for", "w") as f:
+            f.write(made_for)
     return LIB
 
 

@@ -3,6 +3,8 @@ header declares; host-visible argument errors are reported before any launch."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -83,3 +85,18 @@ def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(binding, "LIB_PATH", "/nonexistent/libtreeverify.so")
     with pytest.raises(ImportError):
         binding.load()
+
+
+def test_library_builds_where_torch_cannot_be_imported(lib, tmp_path):
+    (tmp_path / "torch.py").write_text("raise ImportError('no torch here')\n")
+    r = subprocess.run([sys.executable, os.path.join(ROOT, "paper_2603_08088_b200", "build.py")], capture_output=True, text=True,
+                       env=dict(os.environ, PYTHONPATH=str(tmp_path)), cwd=tmp_path)
+    assert r.returncode == 0 and r.stdout.strip() == tv_build.LIB, r.stderr
+
+
+def test_marshalling_module_is_made_again_for_another_torch(lib, monkeypatch):
+    import torch
+    obj, _, _, made_for = tv_build._calls_commands()
+    assert not tv_build._calls_stale(obj, made_for)
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert tv_build._calls_stale(obj, tv_build._calls_commands()[3])
