@@ -34,6 +34,8 @@ TV_API int tv_debug_attn_simt(const tv_bf16* q, const tv_bf16* k_cache, const tv
  * mode bit 1: the pieces of units that are cut between CTAs store their
  * partials but never announce them, so the poll of the piece that merges
  * expires (a launch without a cut unit is then an ordinary launch).
+ * mode bit 4: a call that tree_verify_attn gives to the cluster kernel goes
+ * there (the other modes take the even cut).
  * mode bit 3: the tile table that is built ahead of the wait for the kernel
  * in front is a wrong one and has to be built again (no result changes).
  * With bit 0 or 1 the launch ends by itself: every role leaves its loop, the tensor

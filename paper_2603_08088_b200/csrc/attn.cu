@@ -395,6 +395,7 @@ struct AttnParams {
   int debug;                     // bit 0: the producer issues no copy at all; bit 1: pieces of cut units store their
                                  // partials but never announce them (both exercise the expiry of a bounded wait);
                                  // bit 3: the guessed table is built from lengths one tile too long;
+                                 // bit 4 (host): the cluster kernel is not left out;
                                  // bit 2: the K/V stream alone - the issuing warp only hands every slot back as
                                  // soon as it is full, no MMA, no softmax, no output (what the memory side can do)
   int L;                         // layers in this launch: their units form one tile space, layer after layer
@@ -1883,8 +1884,8 @@ template <int D, int MT>
 cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, cudaStream_t s) {
   const long long units = (long long)prm.L * prm.B * prm.Hkv;
   const int tiles = (prm.Scap + kTileN - 1) / kTileN + prm.TT;
-  // (the test entries exercise the waits of the even cut)
-  const int cluster = prm.debug ? 1 : cluster_size<D, MT>(units * prm.NP, prm.B, tiles, g.sms);
+  // (the test entries exercise the waits of the even cut, or with bit 4 those of the kernel that the call takes)
+  const int cluster = prm.debug && !(prm.debug & 16) ? 1 : cluster_size<D, MT>(units * prm.NP, prm.B, tiles, g.sms);
   tv::count_launches(1);
   if (cluster > 1) return launch_kernel<D, MT, true>((unsigned)(units * prm.NP * cluster), (unsigned)cluster, maps, prm, s);
   // An odd number of row tiles leaves the last CTA of a group with an empty one, as expensive as a full one in the time

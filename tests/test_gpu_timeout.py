@@ -100,3 +100,28 @@ def test_waits_that_expire_anywhere_in_the_tile_loop(d, G, N):
         torch.cuda.synchronize()
         assert (i32(status) == 0).all() and torch.equal(before, after)
     assert expired >= 1
+
+
+def test_expired_waits_of_the_cluster_kernel():
+    """As above, with a producer that issues nothing: every CTA of a cluster gives up, meets the others at the cluster's barriers
+    and leaves."""
+    cfg = CONFIGS[0].scaled(B=1, L=1, Hq=8, Hkv=2, d=128, S_lo=900, S_hi=900, Scap=1000, N=40, D=6, V=0, tree="uniform")
+    c = make_case(cfg, seed=3, device="cuda", with_logits=False)
+    bits = torch.zeros(1, 40, 2, dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    tv.tree_build_mask(c["parent"], c["n_nodes"], 39, 1, bits, status)
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(1, 40, 8, 2, 128, 1000), dtype=torch.uint8, device="cuda")
+    args = (c["q"][0], c["k_cache"][0], c["v_cache"][0], c["k_tree"][0], c["v_tree"][0], c["prefix_len"], c["n_nodes"], bits, 0.1)
+    before, got = torch.zeros(1, 40, 8, 128, dtype=torch.bfloat16, device="cuda"), torch.zeros(1, 40, 8, 128, dtype=torch.bfloat16, device="cuda")
+    tv.tree_verify_attn(*args, before, ws, status)
+    tv.tv_debug_attn_expire(*args, got, ws, status, 500_000_000, 16)
+    torch.cuda.synchronize()
+    assert (i32(status) == 0).all() and torch.equal(before, got)          # the same kernel, bit for bit
+    for _ in range(3):
+        tv.tv_debug_attn_expire(*args, got, ws, status, 2_000_000, 17)
+        torch.cuda.synchronize()
+        assert i32(status).tolist() == [tv.TV_ST_TIMEOUT]
+        status.zero_()
+        tv.tree_verify_attn(*args, got, ws, status)
+        torch.cuda.synchronize()
+        assert (i32(status) == 0).all() and torch.equal(before, got)
