@@ -29,7 +29,7 @@ METRIC = "tree_verify_steps_per_sec"
 UNIT = "steps/s"
 # DRAM bytes per tree_verify_attn launch from ncu (dram__bytes_read.sum + dram__bytes_write.sum), as a ratio to
 # the algorithmic bytes.  Captured on gqa8b_ragged (164.2 MB / 160.1 MB) and long_context (547.9 MB / 547.4 MB),
-# see profiles/tree_attn_kernel_*.md; full_step_32l holds too much memory for a full capture and takes the ratio of
+# see the captures under profiles/; full_step_32l holds too much memory for a full capture and takes the ratio of
 # a 4-layer launch of its own shape (613.6 MB / 616.1 MB); llama7b_layer holds too little work for
 # a capture larger than L2 and takes the ragged-batch ratio; traffic grows with the sum of (prefix + tree) keys.
 L2_BYTES = 126 * 1024 * 1024

@@ -156,11 +156,18 @@ TV_API size_t tv_attn_workspace_bytes(int B, int Nmax, int Hq, int Hkv, int d, i
  * repeats the call's internal epoch) finds them unused.
  * Stream order: the kernel is launched with programmatic stream serialisation,
  * so it may be scheduled while the kernel in front of it still runs (if that
- * kernel allows it), but it reads and writes nothing of the problem before
- * every earlier kernel of the stream has finished: only its own set-up
- * (barriers, tensor memory, descriptor fetch) overlaps.  Reading
- * the committed prefix earlier than that is what tree_verify_attn_layers
- * offers, under a promise by the caller.
+ * kernel allows it).  It may then read prefix_len and the block table and ask
+ * for Q and cache tiles in L2 before the earlier kernels of the stream have
+ * finished, to prepare itself: these arrays have to be mapped by then, what
+ * they hold does not count.  Every result depends only on what is read when
+ * all earlier kernels have finished, and nothing is written before that.
+ * Using the committed prefix earlier is what tree_verify_attn_layers offers,
+ * under a promise by the caller.
+ * Launches: one kernel, or two (a short last row tile of long problems runs
+ * behind the others; whether it does is decided from the lengths on the
+ * device, in caches whose capacity allows such problems).  How the work is
+ * shared between CTAs follows the shape, the capacity and the lengths;
+ * results agree to the rounding of the partial sums.
  */
 TV_API int tree_verify_attn(const tv_bf16* q,
                      const tv_bf16* k_cache, const tv_bf16* v_cache,
@@ -291,7 +298,9 @@ TV_API int tree_accept(const tv_bf16* logits, const int32_t* tokens,
  * tree_accept for a call directly behind tree_verify_attn (any of its variants) on the same stream, whose inputs that
  * launch leaves alone: logits, tokens, retrieve_indices and n_nodes are complete when the attention starts.  The
  * vocabulary scan may then start on SMs the attention has left; it ends after the attention, so everything behind
- * this call is ordered as behind tree_accept.  Arguments and results are those of tree_accept.
+ * this call is ordered as behind tree_accept.  Arguments and results are those of tree_accept, with two conditions:
+ * workspace must not overlap anything the attention call reads or writes (its workspace, inputs and outputs), and the
+ * attention call must have launched a kernel (L and B > 0; otherwise use tree_accept).
  */
 TV_API int tree_accept_behind_attn(const tv_bf16* logits, const int32_t* tokens,
                 const int32_t* retrieve_indices, const int32_t* n_nodes,
@@ -490,6 +499,10 @@ TV_API int kv_commit_inplace(tv_bf16* k_cache, tv_bf16* v_cache,
  * above run, and the per-step results are copied back; the call returns after
  * the stream has drained.  The KV cache and prefix_len stay resident on the
  * device (they are the committed state, not a per-step input).
+ * All host inputs are read behind the work that is queued on the stream: a
+ * caller may still be copying them from the device on it.  Calls on one device
+ * from several threads take turns (they share the copy streams and a pinned
+ * block for the small results).
  */
 typedef struct tv_step_host_args {
   /* host, pinned memory recommended */

@@ -51,7 +51,9 @@
 //
 // Every wait on an mbarrier is bounded: on expiry the CTA raises
 // TV_ST_TIMEOUT for all sequences, all roles leave their loops, outstanding
-// copies are given time to land, TMEM is freed and the kernel returns.
+// copies are given time to land, TMEM is freed and the kernel returns.  The two
+// barriers of a cluster have no limit of their own: every role of every CTA
+// reaches them, because every wait in front of them ends.
 #include "common.cuh"
 #include "treeverify_debug.h"
 
@@ -1288,7 +1290,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           }
           // ---- P = exp2(s * c - m), row sum in fp32, P rounded to bf16.  All of it on the special-function unit: three pairs in
           // sixteen as a cubic on the FMA pipe were level in short runs and cost 1 % where the power limit sets the clock
-          // (32-layer shape, seconds on end: 1503 -> 1484 us a launch).
+          // (32-layer shape, seconds on end, on one board 1503 -> 1484 us a launch, on another 1462 -> 1441).
           uint32_t pkk[64];
           {
             const float2 c2 = make_float2(prm.scale_log2e, prm.scale_log2e);

@@ -30,9 +30,11 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 #ifdef __CUDACC__
 // Programmatic dependent launch for the small kernels of a step.  Launched with programmatic stream
 // serialisation, such a kernel first waits for everything in front of it in the stream and only then lets the
-// next kernel be scheduled: the next launch overlaps this kernel's body, and no kernel ever runs ahead of data
-// it reads (a kernel that reads inputs before its own wait, as tree_verify_attn does with the committed
-// prefix, can therefore only overtake the body of the kernel directly in front of it).
+// next kernel be scheduled: the next launch overlaps this kernel's body, and what a kernel reads before its own wait
+// (tree_verify_attn the committed prefix, the accept kernels tokens and tree) is complete unless the kernel directly
+// in front of it writes it.  The scan of tree_accept_behind_attn lets the next one go before its own wait: it is itself
+// only scheduled when everything in front of the attention is complete.  Reads ahead of a wait go past L1 or
+// follow a fence that drops it.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
