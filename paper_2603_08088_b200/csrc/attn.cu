@@ -62,6 +62,7 @@
 
 #include <atomic>
 #include <chrono>
+#include <type_traits>
 
 namespace {
 
@@ -1499,7 +1500,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               tr.mark(0x7001u);
               // Loads are issued by every thread (row rr always lies inside a slot; rows that are not active read stale
               // bytes and are masked by selects): no thread-divergent branch sits between the warp-wide TMEM ops.
-              auto slot_of = [&](int i) -> size_t { return (size_t)(k_first + i) * np + pair; };       // i-th other piece, i >= 1
+              // (64-wide heads with many pieces a unit: 32-bit slots 48.3 -> 47.8 us a call; the others keep 64 bits, level or 1 %)
+              using Slot = std::conditional_t<D == 64, uint32_t, size_t>;
+              auto slot_of = [&](int i) -> Slot { return (Slot)(k_first + i) * (Slot)np + (Slot)pair; };       // i-th other piece, i >= 1
               auto ml_of = [&](int i) -> const float* { return prm.part_ml + slot_of(i) * 2 * kRows + rr; };
               auto o_of = [&](int i) -> const uint4* { return reinterpret_cast<const uint4*>(prm.part_o) + slot_of(i) * (D / 8) * kRows + rr; };
               // two pieces at a time: (m, l) of the row and the columns of this warpgroup
