@@ -151,7 +151,7 @@ TV_API size_t tv_attn_workspace_bytes(int B, int Nmax, int Hq, int Hkv, int d, i
  * Hq % Hkv == 0, Hq / Hkv <= 128; B <= 512; all tensors 16-byte aligned;
  * 0 <= prefix_len[b] <= Scap; scale > 0.
  * CUDA graphs: every call of this header only launches on the given stream, so a
- * step can be captured into a CUDA graph and replayed; the split-KV counters in
+ * step can be captured into a CUDA graph and replayed; the split-KV flags in
  * the workspace are cleared by the piece that merges, so a replay (which
  * repeats the call's internal epoch) finds them unused.
  * Stream order: the kernel is launched with programmatic stream serialisation,
@@ -192,9 +192,9 @@ TV_API int tree_verify_attn(const tv_bf16* q,
  * all layers run in ONE launch - their (sequence, KV head) units form one
  * tile space that is cut evenly over the SMs - with one pipeline fill, one
  * tail and at most one cut unit per SM for the whole step instead of per
- * layer.  The workspace of tv_attn_workspace_bytes holds the counters of 32
- * layers per launch; more layers (or a smaller workspace, down to the
- * counters of one layer) are served by more launches.  A caller whose layers
+ * layer.  The workspace of tv_attn_workspace_bytes has room for 32 layers
+ * per launch; more layers (or a smaller workspace, down to the room of
+ * one layer) are served by more launches.  A caller whose layers
  * depend on each other has to issue single-layer calls instead.
  * flags: TV_ATTN_STABLE_INPUTS lets the launch read prefix_len, n_nodes and
  * committed-prefix rows while the kernel in front still runs (see the flag);

@@ -41,7 +41,7 @@
 // hits L2).  A unit cut in pieces leaves partials (normalised O in bf16, m, l) in the
 // workspace; the CTA that holds the unit's first piece merges them.  Groups run
 // downwards over the block index, so a merging CTA waits only for CTAs with a lower
-// block index, which were started before it.  Flags carry a per-call epoch, so the
+// block index, which were started before it.  Flags hold the epoch of the call, so the
 // workspace needs no initialisation.
 //
 // Few units (CL = true).  A unit is shared by a thread-block cluster instead: its CTAs
@@ -354,16 +354,15 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return r;
 }
 
-// Epoch-tagged arrival counter: value = (epoch << 16) | count; a value with another epoch counts as zero, so
-// the counters need no initialisation.  `seen` is a value of the counter read earlier.  Returns the count
-// after this arrival.
-__device__ __forceinline__ int bump_counter(unsigned long long* c, unsigned long long seen, unsigned long long epoch) {
-  while (true) {
-    const unsigned long long assumed = seen;
-    const int cnt = ((assumed >> 16) == epoch) ? (int)(assumed & 0xffffu) : 0;
-    seen = atomicCAS(c, assumed, (epoch << 16) | (unsigned long long)(cnt + 1));
-    if (seen == assumed) return cnt + 1;
-  }
+// Flags between CTAs.  Whoever sees the released value also sees what this thread wrote before, and what threads that it
+// has synchronised with wrote before.
+__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
 }
 
 // ---------------------------------------------------------------- kernel parameters
@@ -376,8 +375,8 @@ struct AttnParams {
   int32_t* status;
   tv_bf16* part_o;               // [slots][D/8][MT*128][8] bf16 normalised outputs, column-group major
   float* part_ml;                // [slots][2][MT*128]  (m in log2 units, then l); one slot per CTA
-  unsigned long long* counters;  // [L*B*Hkv*NP][2], epoch-tagged: the unit's second piece is ready, count of later ones
-  unsigned long long epoch;      // 48-bit tag of this call
+  unsigned long long* flags;     // [slots]: the epoch of the call once the partial in that slot is complete
+  unsigned long long epoch;      // tag of this call
   int B, Nmax, Hq, Hkv, Scap, G, NPT, NP, W, groups;
   int tile0;                     // first row tile of this launch
   int split_tiles;               // > 0: from this many key tiles on (all units of the launch, by the lengths on the device) the
@@ -1453,7 +1452,6 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             while (gs[k_first] > real0) --k_first;
             while (gs[k_last + 1] < uend) ++k_last;
             const int n_other = k_last - k_first;
-            unsigned long long* flags = prm.counters + ((((size_t)it.layer * prm.B + it.b) * prm.Hkv + it.hk) * np + pair) * 2;
             const float inv_own = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
             if (group != k_first) {
               const size_t slot = (size_t)group * np + pair;
@@ -1465,25 +1463,26 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
               store_rows(po + rr, kRows, inv_own, row_active, false);
               tc_fence_before();
-              // Warp 2 announces the piece: the fence behind these stores (a round trip to L2) and the wait for the other
+              // Warp 2 announces the piece: the release behind these stores (a round trip to L2) and the wait for the other
               // warps' stores are not in front of this warp's next item (32 sequences of 1024, one layer: 51.3 -> 50.6 us; 4 of
               // 4096, 128 nodes: 43.5 -> 42.6 us).
-              if (threadIdx.x == 128 && !(prm.debug & 2)) {      // (debug bit 1: the piece is never announced)
-                const int i = group - k_first;
-                *announce = i == 1 ? (unsigned long long)flags | 1u : (unsigned long long)(flags + 1) | (n_other == 2 ? 1u : 2u);
-              }
+              if (threadIdx.x == 128 && !(prm.debug & 2))      // (debug bit 1: the piece is never announced)
+                *announce = reinterpret_cast<unsigned long long>(prm.flags + slot);
               tr.mark(0x6000u);
               __syncwarp();
               if (lane == 0) mbar_arrive(bar(L::PIECE));
             } else {
               if (warp == 4) {
-                // wait until the other pieces have published their partials: lane 0 the second, lane 1 the later ones
-                if (lane < 2 && lane < n_other) {
-                  const int want = lane == 0 ? 1 : n_other - 1;
+                // Wait until the other pieces have published their partials, a lane for each.  A flag per slot, written once
+                // with a release and polled with an acquire: with a counter for all later pieces (a read, a compare-and-swap, a
+                // full fence on either side) the last partial was seen 3 us after its last store, now 2 (us a launch, 8 KV heads:
+                // 8 sequences of 1024 ... 8192 46.9 -> 45.7, 4 of 500 ... 16000 50.7 -> 48.4; 64-wide heads, one row tile, 16 of
+                // 8000 59.8 -> 55.9).
+#pragma unroll 1
+                for (int i = 1 + lane; i <= n_other; i += 32) {
+                  unsigned long long* flag = prm.flags + (size_t)(k_first + i) * np + pair;
                   const unsigned long long t0 = globaltimer_ns();
-                  while (true) {
-                    const unsigned long long v = *reinterpret_cast<volatile unsigned long long*>(flags + lane);
-                    if ((v >> 16) == prm.epoch && (int)(v & 0xffffu) >= want) break;
+                  while (ld_acquire(flag) != prm.epoch) {
                     if (*abort_flag || globaltimer_ns() - t0 > wait_limit) {
                       *abort_flag = 1;
                       break;
@@ -1491,9 +1490,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                   }
                   // nobody touches the flag again in this launch.  Clearing it lets the same launch be replayed with the
                   // same epoch (a captured CUDA graph) and find it unused.
-                  *reinterpret_cast<volatile unsigned long long*>(flags + lane) = 0ull;
+                  *reinterpret_cast<volatile unsigned long long*>(flag) = 0ull;
                 }
-                __threadfence();
+                __syncwarp();
               }
               ok = epi_sync();
               if (!ok || *abort_flag) { ok = false; break; }
@@ -1698,12 +1697,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // Only the first item of a CTA can be a piece whose partials another CTA merges.  Warp 2 waits for every softmax warp to
     // have stored its part (or to have seen that there is none), and then raises the flag.
     if (!CL && warp == 2 && !*abort_flag && !(prm.debug & 4) && mbar_wait(bar(L::PIECE), 0, abort_flag, wait_limit) && lane == 0 &&
-        *announce != 0) {
-      unsigned long long* flag = reinterpret_cast<unsigned long long*>(*announce & ~7ull);
-      __threadfence();
-      if (*announce & 1u) *reinterpret_cast<volatile unsigned long long*>(flag) = prm.epoch << 16 | 1u;
-      else bump_counter(flag, *reinterpret_cast<volatile unsigned long long*>(flag), prm.epoch);
-    }
+        *announce != 0)
+      st_release(reinterpret_cast<unsigned long long*>(*announce), prm.epoch);
     if (CL) {
       cluster_sync();
       cluster_sync_relaxed();
@@ -1758,10 +1753,10 @@ bool encode_map(CUtensorMap* m, const void* base, int rank, const cuuint64_t* di
 
 struct Geometry {
   int G, NPT, n_row_tiles, MT, NP, sms, groups, grid;
-  size_t ml_off, o_off, counters_off, counters_per_layer, total;
+  size_t ml_off, flags_off, o_off, layers_off, per_layer, total;
 };
 
-constexpr int kCounterLayers = 32;      // layers whose counters the workspace of tv_attn_workspace_bytes holds
+constexpr int kWorkspaceLayers = 32;    // layers in one launch with the workspace of tv_attn_workspace_bytes
 
 Geometry geometry(int B, int Nmax, int Hq, int Hkv, int d, bool query_device) {
   Geometry g{};
@@ -1773,30 +1768,28 @@ Geometry geometry(int B, int Nmax, int Hq, int Hkv, int d, bool query_device) {
   g.sms = query_device ? tv::sm_count() : 148;
   g.groups = g.sms / g.NP > 0 ? g.sms / g.NP : 1;
   g.grid = g.groups * g.NP;
-  // workspace: (m,l) pairs, partial O (both sized for 160 SMs so the size does not depend on the device), then
-  // the units' counters, layer after layer: as many layers as fit behind the partials can share one launch
-  const size_t max_ctas = 160 > g.grid ? 160 : g.grid;
-  size_t off = 0;
-  g.ml_off = off;
-  off += max_ctas * (size_t)g.MT * 128 * 2 * sizeof(float);
-  off = (off + 255) & ~size_t(255);
-  g.o_off = off;
-  off += max_ctas * (size_t)g.MT * 128 * d * sizeof(tv_bf16);
-  off = (off + 255) & ~size_t(255);
-  g.counters_off = off;
-  g.counters_per_layer = ((size_t)B * Hkv * g.NP * 2 * sizeof(unsigned long long) + 255) & ~size_t(255);
-  g.total = off + kCounterLayers * g.counters_per_layer;
+  // workspace: (m,l) pairs and partial O, both with 160 slots whatever the device; the flags of the slots in use (one per
+  // CTA) in the (m,l) room of the last ones; then a stretch per layer, none of which is used: how many there are bounds the
+  // layers that share a launch
+  constexpr size_t kSlotsMax = 160;
+  const size_t ml_bytes = (size_t)g.MT * 128 * 2 * sizeof(float);
+  g.ml_off = 0;
+  g.flags_off = (kSlotsMax - 2) * ml_bytes;
+  g.o_off = (kSlotsMax * ml_bytes + 255) & ~size_t(255);
+  g.layers_off = (g.o_off + kSlotsMax * g.MT * 128 * d * sizeof(tv_bf16) + 255) & ~size_t(255);
+  g.per_layer = ((size_t)B * Hkv * g.NP * 2 * sizeof(unsigned long long) + 255) & ~size_t(255);
+  g.total = g.layers_off + kWorkspaceLayers * g.per_layer;
   return g;
 }
 
 std::atomic<unsigned long long*> g_trace{nullptr};
 
-// Tag of a call in its workspace counters (48 bits, never repeated within a process): the only state the
+// Tag of a call in its workspace flags (never repeated within a process, never 0): the only state the
 // library keeps for this entry point besides the cached driver entry point and device attributes.
 unsigned long long next_epoch() {
   static std::atomic<unsigned long long> ctr{
       (unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count() * 2654435761ull};
-  return ctr.fetch_add(1, std::memory_order_relaxed) & 0xffffffffffffull;
+  return ctr.fetch_add(1, std::memory_order_relaxed) | 1ull << 63;
 }
 
 // Allows the kernel its shared memory, once per device.
@@ -1977,7 +1970,7 @@ int attn_launch(const tv_bf16* q, const tv_bf16* k_cache, const tv_bf16* v_cache
   // The launch touches the workspace only after its grid-dependency wait, that is after every earlier kernel of
   // the stream has completed: consecutive launches may share it although they overlap on the device.
   char* ws = static_cast<char*>(workspace);
-  prm.counters = reinterpret_cast<unsigned long long*>(ws + g.counters_off);
+  prm.flags = reinterpret_cast<unsigned long long*>(ws + g.flags_off);
   prm.part_ml = reinterpret_cast<float*>(ws + g.ml_off);
   prm.part_o = reinterpret_cast<tv_bf16*>(ws + g.o_off);
   prm.epoch = next_epoch();
@@ -2032,12 +2025,12 @@ int attn_entry(const tv_bf16* q,
   const Geometry g = geometry(B, Nmax, Hq, Hkv, d, true);
   const long long tiles_per_layer = (long long)B * Hkv * ((Scap + kTileN - 1) / kTileN + 2 + kSetupCost);
   TV_REQUIRE(tiles_per_layer < (1ll << 31), "tree_verify_attn: B * Hkv * Scap is too large for the tile scheduler");
-  if (g.grid > 160) return tv::fail(TV_ERR_INVALID_ARG, "tree_verify_attn: device with more than 160 SMs is not supported");
-  if (workspace_bytes < g.counters_off + g.counters_per_layer)
+  if (g.sms > 158) return tv::fail(TV_ERR_INVALID_ARG, "tree_verify_attn: device with more than 158 SMs is not supported");
+  if (workspace_bytes < g.layers_off + g.per_layer)
     return tv::fail(TV_ERR_WORKSPACE, "tree_verify_attn: workspace of %zu bytes, need %zu", workspace_bytes,
-                    g.counters_off + g.counters_per_layer);
-  // Layers that share a launch: as many as the workspace has counters for and as the 31-bit tile space holds.
-  long long per_launch = (long long)((workspace_bytes - g.counters_off) / g.counters_per_layer);
+                    g.layers_off + g.per_layer);
+  // Layers that share a launch: as many as the workspace has stretches for and as the 31-bit tile space holds.
+  long long per_launch = (long long)((workspace_bytes - g.layers_off) / g.per_layer);
   const long long by_tiles = ((1ll << 31) - 1) / tiles_per_layer;
   if (per_launch > by_tiles) per_launch = by_tiles;
   if (per_launch > 65535) per_launch = 65535;
