@@ -103,7 +103,9 @@ constexpr int kMinTilesPerGroup = TV_MIN_VT;
 // of 65 nodes, prefixes of 300 19.9 / 16.6, 600 22.8 / 19.4, 1000 26.8 / 23.9, 2300 41.0 / 39.1; 10 of 20 nodes 15.7 / 12.9, 17.5 /
 // 14.6, 20.4 / 17.8, 26.7 / 29.2; 12 of 40 nodes with 64-wide heads 15.2 / 14.2, 19.2 / 17.1, 23.5 / 21.6, 34.4 / 36.8.
 constexpr int kMaxWholeUnit = 13;
-constexpr int kSplitTilesPerSm = 60;       // from here on an odd last row tile has a launch of its own (see launch)
+// An odd last row tile has a launch of its own (see launch) where the capacity of the cache allows the first number of key tiles
+// per SM, and the lengths reach the second.
+constexpr int kSplitTilesPerSm = 24, kSplitLengthsPerSm = 12;
 constexpr int kMaxCluster = 8;     // CTAs that share a unit (16 is not portable; few clusters of 16 fit the GPU at once: 21.7 us
                                    // instead of 10.8 us a launch for eight units of 12 key tiles)
 constexpr int kTraceCap = 256;     // events per (CTA, role) kept by the optional trace
@@ -396,6 +398,9 @@ struct AttnParams {
   int out_al32;                  // out is 32-byte aligned: rows can be written 32 bytes per thread and store
   float scale_log2e;             // scale * log2(e)
   float scale;
+  int beside;                    // launched behind the front launch of the same call, to run beside it: everything in front of
+                                 // that one is complete when this one starts, and it reads nothing that the front launch writes;
+                                 // it waits for the front launch where it ends
   int early;                     // the caller promises that the kernel in front leaves prefix_len, n_nodes, the block
                                  // table and the committed rows alone: they are read before the grid-dependency wait
   unsigned long long wait_limit_ns;   // limit of every bounded wait
@@ -499,8 +504,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       tiles += ((S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S)) + kTileN - 1) / kTileN + prm.TT;
     }
     if (!splits(__reduce_add_sync(0xffffffffu, tiles))) {
-      gdc_wait();
       if (threadIdx.x == 0) gdc_launch_dependents();
+      gdc_wait();
       return;
     }
   }
@@ -763,7 +768,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       bool synced = false;
       int bad_page_b = -1;
       auto sync_with_predecessor = [&]() {
-        gdc_wait();
+        if (!prm.beside) gdc_wait();
         if (elect_one()) gdc_launch_dependents();
         if (bad_page_b >= 0 && lane == 0) atomicOr(prm.status + bad_page_b, TV_ST_BAD_INDEX);
         bad_page_b = -1;
@@ -788,7 +793,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         __syncwarp();
       };
-      if (!prm.early) sync_with_predecessor();
+      if (!prm.early || prm.beside) sync_with_predecessor();
       bool have_first = !CL && !prm.early && at[0];
       if (have_first) {
         g = at[1];
@@ -866,7 +871,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       if (!synced) sync_with_predecessor();        // a CTA without work still has to let the next kernel go
     } else {
-      gdc_wait();
+      if (!prm.beside) gdc_wait();
       if (elect_one()) gdc_launch_dependents();
     }
     if (CL) {
@@ -1090,7 +1095,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int wg = (warp - 4) >> 2;                  // its row tile, or parity of its key tiles
     const int row = ((warp & 3) << 5) | lane;        // TMEM lane = row inside the tile
     const uint32_t lane_addr = (uint32_t)((warp & 3) << 5) << 16;
-    gdc_wait();      // anc_bits, the workspace and the outputs may belong to the kernel in front until it is done
+    // anc_bits, the workspace and the outputs may belong to the kernel in front until it is done
+    if (prm.beside) __threadfence();      // (nothing does; the fence drops what an earlier launch has left of anc_bits in L1)
+    else gdc_wait();
     // in-cache layout: a tree that does not fit behind its prefix is reported, not read past the capacity (rows
     // past Scap arrive as zeros and the sequence's output is unspecified).  Raised after the wait: status[] may
     // be written by the kernel in front until then.
@@ -1711,6 +1718,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   }
 
   // ---- teardown
+  if (prm.beside) gdc_wait();      // who waits for this launch waits for the one in front
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -1892,17 +1900,20 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
   tv::count_launches(1);
   if (cluster > 1) return launch_kernel<D, MT, true>((unsigned)(units * prm.NP * cluster), (unsigned)cluster, maps, prm, s);
   // An odd number of row tiles leaves the last CTA of a group with an empty one, as expensive as a full one in the time
-  // its group takes.  Where the work is long the last row tile gets a launch of its own (one row tile per CTA, two thirds
-  // of the time per key tile, every CTA on it): 8 sequences of 65 nodes, 8 layers, G = 4: 305 -> 274 us.  It reads K/V a
-  // second time and costs a fill and a tail of some 12 us, hence a bound on the key tiles per SM.  Only the capacity of the
-  // cache is known here: where it allows that many, both launches are made, and both go by the lengths on the device (8
-  // sequences of 65 nodes with prefixes of 300 in a paged cache of 32768, one layer: 34.4 -> 23.2 us against two full launches;
-  // 20.0 in a cache of 512, the difference is the launch that finds nothing to do).
+  // its group takes.  Where the work is long the last row tile gets a launch of its own, one row tile per CTA, that runs beside
+  // the one with the others: the SMs are shared out between the two by what a key tile costs each (two row tiles 1.3 times as much as
+  // one, with 64-wide heads, whose keys two warpgroups share there, 1.7 times; 1.0 to 2.6 measured).  Behind one another, each on all
+  // SMs, one is bound by tensor work and power while the other waits for memory.  us a call, one launch behind the other / beside,
+  // 8 KV heads, G = 4, 512 ... 4096: 65 nodes, 8 layers 252 / 241, 129 nodes, 4 layers 207 / 193, the same with 64-wide heads 187 / 159; one
+  // layer of 1024 ... 8192, 65 nodes, which was one launch 65.4 / 63.1.  Only the capacity of the cache is known here: where it allows
+  // long work both launches are made, and both go by the lengths on the device (short work: the front launch takes all row tiles,
+  // the other finds nothing to do, some 3 us).
   if (MT == 2 && g.n_row_tiles % 2 == 1 && units * tiles >= (long long)kSplitTilesPerSm * g.sms) {
     AttnParams front = prm;
-    front.split_tiles = kSplitTilesPerSm * g.sms;
+    front.split_tiles = kSplitLengthsPerSm * g.sms;
     front.front_NP = g.n_row_tiles / 2;
-    front.front_groups = g.sms / front.front_NP;
+    const int odd = g.sms * 10 / (10 + (D == 64 ? 17 : 13) * front.front_NP);
+    front.front_groups = (g.sms - odd) / front.front_NP;
     const int ctas = front.front_groups * front.front_NP;
     const cudaError_t e = launch_kernel<D, MT, false>((unsigned)(ctas > g.grid ? ctas : g.grid), 1, maps, front, s);
     if (e != cudaSuccess) return e;
@@ -1910,10 +1921,13 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
     prm.split_tiles = front.split_tiles;
     prm.tile0 = g.n_row_tiles - 1;
     prm.NP = 1;
-    prm.groups = g.sms;
-    prm.early = 1;          // behind a launch of this very call the inputs are stable
+    prm.groups = g.sms - ctas;
+    prm.early = prm.beside = 1;
     prm.epoch = next_epoch();
-    return launch_kernel<D, 1, false>((unsigned)g.sms, 1, maps, prm, s);
+    prm.part_ml += (size_t)ctas * 2 * MT * 128;      // the slots and flags behind those of the front launch
+    prm.part_o += (size_t)ctas * MT * 128 * D;
+    prm.flags += ctas;
+    return launch_kernel<D, 1, false>((unsigned)prm.groups, 1, maps, prm, s);
   }
   return launch_kernel<D, MT, false>((unsigned)g.grid, 1, maps, prm, s);
 }

@@ -691,6 +691,61 @@ def test_last_row_tile_goes_by_the_lengths_and_not_by_the_capacity(N, d, paged, 
                                f"{l} {b} {hk}")
 
 
+@pytest.mark.parametrize("N,d,G", [(65, 64, 4), (65, 128, 4), (129, 128, 4), (160, 64, 4), (44, 128, 8)])
+def test_last_row_tile_beside_the_others_keeps_the_order_of_the_stream(N, d, G):
+    """The two launches of an odd last row tile run at the same time.  Inputs written by the kernels directly in front, outputs
+    overwritten by the one directly behind, call after call, give the bits of a call with the device idle on either side, and so
+    does a replayed graph; three and five row tiles, the last one full, short and nearly empty."""
+    B, Hkv, cap = 14, 8, 4480
+    cfg = CONFIGS[0].scaled(B=B, L=1, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=2600, S_hi=4300, Scap=cap, N=N, D=6, V=0, tree="uniform")
+    cases = [make_case(cfg, seed=N + d + x, device="cuda", ragged_nodes=True, with_logits=False) for x in (0, 1)]
+    names = ("q", "prefix_len", "n_nodes", "parent")
+    here = {k: torch.empty_like(cases[0][k]) for k in names}
+    bits = torch.zeros(B, N, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    st = torch.zeros(B, dtype=torch.int32, device="cuda")
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(B, N, cfg.Hq, Hkv, d, cap), dtype=torch.uint8, device="cuda")
+    out = torch.zeros(B, N, cfg.Hq, d, dtype=torch.bfloat16, device="cuda")
+    kept = torch.zeros(2, *out.shape, dtype=torch.bfloat16, device="cuda")
+    c = cases[0]
+
+    def step(x, idle):
+        for k in names:
+            here[k].copy_(cases[x][k])
+        tv.tree_build_mask(here["parent"], here["n_nodes"], N - 1, 1, bits, st)
+        idle()
+        tv.tree_verify_attn(here["q"][0], c["k_cache"][0], c["v_cache"][0], c["k_tree"][0], c["v_tree"][0], here["prefix_len"],
+                            here["n_nodes"], bits, d ** -0.5, out, ws, st)
+        idle()
+        kept[x].copy_(out)
+        out.fill_(7.0)
+
+    n0 = tv.tv_launch_count()
+    for x in (0, 1):
+        step(x, torch.cuda.synchronize)
+    assert tv.tv_launch_count() - n0 == 6                     # mask and two attention launches each
+    want = kept.clone()
+    for _ in range(4):
+        for x in (0, 1):
+            step(x, lambda: None)
+        torch.cuda.synchronize()
+        assert torch.equal(kept, want)
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.stream(stream), torch.cuda.graph(graph):
+        for x in (0, 1):
+            step(x, lambda: None)
+    for _ in range(3):
+        kept.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(kept, want)
+    assert not st.any()
+    vis = oracle_visibility(cases[0]["parent"], cases[0]["n_nodes"])[:, 0]
+    cn = case_to_numpy(cases[0])
+    for b, hk in ((0, 0), (B - 1, 7)):
+        ref_out, ref_lse = oracle_attention_slice(cn, 0, b, hk, G, vis, d ** -0.5)
+        assert np.abs(want[0][b:b + 1, :, hk * G:(hk + 1) * G].float().cpu().numpy() - ref_out).max() <= 2e-2
+
+
 @pytest.mark.parametrize("G,N,d", [(2, 40, 64), (4, 40, 64), (2, 40, 128), (4, 40, 128)])
 @pytest.mark.parametrize("S,other", [(300, 300), (1024, 1024), (1025, 1025), (300, 100)])
 def test_equal_units_stay_whole_while_they_are_short(S, other, G, N, d):
