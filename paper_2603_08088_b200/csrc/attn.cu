@@ -73,18 +73,16 @@ constexpr int kMaxB = 512;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleThreshold = 8.0f;            // in log2 units
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
-// Virtual tiles charged per unit where the tile space is cut: an item costs its CTA 2.2 us beside its tiles (epilogue, masked
-// tiles, refill) and the first piece of a cut unit 2.5 to 5 (the merge), but a CTA inside a long unit, which pays none of it and
-// gets a full share of tiles, is the one that the merge waits for.  us a launch, charge 1 / 2 / 3 / 4: 16 sequences of 512 ... 4096
-// 43.9 / 44.4 / 46.0 / 46.5, with one row tile 32.7 / 32.8 / 34.2 / 34.5, 8 of 1024 ... 8192 44.6 / 45.0 / 45.6 / 45.7, 12 of 200 ...
-// 2000 with 16 KV heads 41.4 / 39.0 / 38.6 / 39.0, four layers of the first 155 / 152 / 152 / 153.  A second weight for the tiles of units
-// longer than a share, cuts rounded to the nearest tile: level, and 1 us more for the code in front of the first tile.
+// Virtual tiles charged per unit by the scheduler: what a CTA pays for one more item (epilogue, masked tiles, refill) is
+// some 5 us, three to four tiles' time.  Eight shapes, one and 32 layers a launch: 4 is 1 to 3 % faster than 2 and 1 to 2 %
+// faster than 1 and 5 on all but the ragged batch (1.8 % slower than 2); 3 is level with 4.  Of 72 shapes 2 is 1 to 4 %
+// faster than 4 on 33 (one row tile above all), and slower on 9, where every unit, or every second, is cut once: us a launch, 2 / 4, 128-wide
+// heads, 8 sequences of 4096 41.7 / 39.8, 32 of 1024 45.2 / 43.9, 4 of 4096 with 128 nodes 41.7 / 40.8, of 4000 ... 4096
+// 58.1 / 56.2, 32 of 650 ... 4550 with one row tile 65.3 / 63.0; 8 of 1024 ... 8192 47.8 / 46.1.
 #ifndef TV_SETUP_COST
-#define TV_SETUP_COST 2
+#define TV_SETUP_COST 4
 #endif
 constexpr int kSetupCost = TV_SETUP_COST;
-// What a unit counts beside its tiles where the number of CTA groups is chosen.
-constexpr int kUnitCost = 4;
 // K/V tiles that a CTA asks for in L2 while the kernel in front is still running.  16 sequences of 512 to 4096, layer after
 // layer: 48.6 us a launch with none, 47.7 with 2, 47.9 with 4, 48.6 with 8 (they take their bandwidth from that kernel's tail).
 #ifndef TV_PREFETCH_TILES
@@ -98,8 +96,8 @@ constexpr int kMaxGroups = 160;
 #ifndef TV_MIN_VT
 #define TV_MIN_VT 6
 #endif
-constexpr int kMinTilesPerGroup = TV_MIN_VT;
-// Tiles of a unit (kUnitCost among them) up to which equal units stay whole, on one group each.  us a call, cut / whole, 8 KV heads: 8 sequences
+constexpr int kMinVirtualTilesPerGroup = TV_MIN_VT;
+// Virtual tiles of a unit up to which equal units stay whole, on one group each.  us a call, cut / whole, 8 KV heads: 8 sequences
 // of 65 nodes, prefixes of 300 19.9 / 16.6, 600 22.8 / 19.4, 1000 26.8 / 23.9, 2300 41.0 / 39.1; 10 of 20 nodes 15.7 / 12.9, 17.5 /
 // 14.6, 20.4 / 17.8, 26.7 / 29.2; 12 of 40 nodes with 64-wide heads 15.2 / 14.2, 19.2 / 17.1, 23.5 / 21.6, 34.4 / 36.8.
 constexpr int kMaxWholeUnit = 13;
@@ -659,14 +657,14 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int units = prm.B * prm.Hkv * prm.L;
         const bool split = MT == 2 && prm.split_tiles > 0 && splits(run - prm.B * kSetupCost);
         const int np = split ? prm.front_NP : prm.NP, max_groups = split ? prm.front_groups : prm.groups;
-        const int want = (int)((unsigned)(prm.Hkv * (run + prm.B * (kUnitCost - kSetupCost))) * (unsigned)prm.L / (unsigned)kMinTilesPerGroup);
+        const int want = (int)((unsigned)(prm.Hkv * run) * (unsigned)prm.L / (unsigned)kMinVirtualTilesPerGroup);
         int n = want < 1 ? 1 : (want < max_groups ? want : max_groups);
         // A group count just above a multiple of the unit count is rounded down to it: with units of equal length
         // (one sequence, all heads) every unit is then cut into the same number of equal pieces and no cut falls
         // just behind a unit boundary.  Not worth more than 1/16 of the groups, but for short units of equal length:
         // those stay whole, one a group, because a cut and its merge cost more than the idle groups.
         const int over = n % units;
-        if (n > units && (over * 16 <= n || (n < 2 * units && same && first_len + kUnitCost - kSetupCost <= kMaxWholeUnit))) n -= over;
+        if (n > units && (over * 16 <= n || (n < 2 * units && same && first_len <= kMaxWholeUnit))) n -= over;
         at[2] = n;
         at[3] = np;
       }
@@ -2045,7 +2043,7 @@ int attn_entry(const tv_bf16* q,
   TV_REQUIRE((reinterpret_cast<uintptr_t>(workspace) & 255u) == 0, "tree_verify_attn: workspace must be 256-byte aligned");
   if (B == 0 || L == 0) return TV_OK;
   const Geometry g = geometry(B, Nmax, Hq, Hkv, d, true);
-  const long long tiles_per_layer = (long long)B * Hkv * ((Scap + kTileN - 1) / kTileN + 2 + kUnitCost);
+  const long long tiles_per_layer = (long long)B * Hkv * ((Scap + kTileN - 1) / kTileN + 2 + kSetupCost);
   TV_REQUIRE(tiles_per_layer < (1ll << 31), "tree_verify_attn: B * Hkv * Scap is too large for the tile scheduler");
   if (g.sms > 158) return tv::fail(TV_ERR_INVALID_ARG, "tree_verify_attn: device with more than 158 SMs is not supported");
   if (workspace_bytes < g.layers_off + g.per_layer)
