@@ -102,8 +102,10 @@ constexpr int kMinVirtualTilesPerGroup = TV_MIN_VT;
 // 14.6, 20.4 / 17.8, 26.7 / 29.2; 12 of 40 nodes with 64-wide heads 15.2 / 14.2, 19.2 / 17.1, 23.5 / 21.6, 34.4 / 36.8.
 constexpr int kMaxWholeUnit = 13;
 // An odd last row tile has a launch of its own (see launch) where the capacity of the cache allows the first number of key tiles
-// per SM, and the lengths reach the second.
-constexpr int kSplitTilesPerSm = 24, kSplitLengthsPerSm = 12;
+// per SM, and the lengths reach the second.  In a smaller cache the long calls would gain less than the short ones lose to a second
+// launch that finds nothing to do: 65 nodes, 8 sequences, us a call, one launch / two, in a cache of 28 key tiles per SM with lengths of 4
+// 31.1 / 33.7, 10 50.7 / 53.2, 14 64.0 / 60.5, in one of 33 with 22 98.6 / 91.1.
+constexpr int kSplitTilesPerSm = 60, kSplitLengthsPerSm = 12;
 constexpr int kMaxCluster = 8;     // CTAs that share a unit (16 is not portable; few clusters of 16 fit the GPU at once: 21.7 us
                                    // instead of 10.8 us a launch for eight units of 12 key tiles)
 constexpr int kTraceCap = 256;     // events per (CTA, role) kept by the optional trace
@@ -1905,8 +1907,8 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
   // the one with the others: the SMs are shared out between the two by what a key tile costs each (two row tiles 1.3 times as much as
   // one, with 64-wide heads, whose keys two warpgroups share there, 1.7 times; 1.0 to 2.6 measured).  Behind one another, each on all
   // SMs, one is bound by tensor work and power while the other waits for memory.  us a call, one launch behind the other / beside,
-  // 8 KV heads, G = 4, 512 ... 4096: 65 nodes, 8 layers 252 / 241, 129 nodes, 4 layers 207 / 193, the same with 64-wide heads 187 / 159; one
-  // layer of 1024 ... 8192, 65 nodes, which was one launch 65.4 / 63.1.  Only the capacity of the cache is known here: where it allows
+  // 8 KV heads, G = 4, 512 ... 4096: 65 nodes, 8 layers 252 / 241, 129 nodes, 4 layers 207 / 193, the same with 64-wide heads 187 / 159.
+  // Only the capacity of the cache is known here: where it allows
   // long work both launches are made, and both go by the lengths on the device (short work: the front launch takes all row tiles,
   // the other finds nothing to do, some 3 us).
   if (MT == 2 && g.n_row_tiles % 2 == 1 && units * tiles >= (long long)kSplitTilesPerSm * g.sms) {

@@ -691,12 +691,43 @@ def test_last_row_tile_goes_by_the_lengths_and_not_by_the_capacity(N, d, paged, 
                                f"{l} {b} {hk}")
 
 
+@pytest.mark.parametrize("N,d", [(65, 64), (129, 128)])
+@pytest.mark.parametrize("cap,launches", [(59, 1), (60, 2)])
+def test_caches_without_room_for_long_work_have_one_launch(N, d, cap, launches):
+    """Short prefixes in a cache of one key tile per SM less than two launches need, and in one that allows them: the second one
+    is made only there, and the results are the same bits."""
+    B, L, Hkv, G = 4, 2, 2, 4
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = (-(-cap * sms // (B * L * Hkv)) - (N + 127) // 128) * 128
+    cfg = CONFIGS[0].scaled(B=B, L=L, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=200, S_hi=900, Scap=1024, N=N, D=6, V=0, tree="uniform")
+    case = make_case(cfg, seed=N, device="cuda", ragged_nodes=True, with_logits=False)
+    bits = torch.zeros(B, N, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    st = torch.zeros(B, dtype=torch.int32, device="cuda")
+    tv.tree_build_mask(case["parent"], case["n_nodes"], N - 1, 1, bits, st)
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(B, N, cfg.Hq, Hkv, d, rows), dtype=torch.uint8, device="cuda")
+
+    def run(rows):
+        kc, vc = (torch.full((L, B, Hkv, rows, d), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in "kv")
+        kc[:, :, :, :900], vc[:, :, :, :900] = case["k_cache"][:, :, :, :900], case["v_cache"][:, :, :, :900]
+        out = torch.full((L, B, N, cfg.Hq, d), 3.0, dtype=torch.bfloat16, device="cuda")
+        n0 = tv.tv_launch_count()
+        tv.tree_verify_attn_layers(case["q"], kc, vc, case["k_tree"], case["v_tree"], case["prefix_len"], case["n_nodes"], bits,
+                                   d ** -0.5, out, ws, st)
+        torch.cuda.synchronize()
+        return out, tv.tv_launch_count() - n0
+
+    out, n = run(rows)
+    assert n == launches
+    other, n = run(rows // 2)
+    assert n == 1 and torch.equal(out, other) and not st.any()
+
+
 @pytest.mark.parametrize("N,d,G", [(65, 64, 4), (65, 128, 4), (129, 128, 4), (160, 64, 4), (44, 128, 8)])
 def test_last_row_tile_beside_the_others_keeps_the_order_of_the_stream(N, d, G):
     """The two launches of an odd last row tile run at the same time.  Inputs written by the kernels directly in front, outputs
     overwritten by the one directly behind, call after call, give the bits of a call with the device idle on either side, and so
     does a replayed graph; three and five row tiles, the last one full, short and nearly empty."""
-    B, Hkv, cap = 14, 8, 4480
+    B, Hkv, cap = 14, 8, 10240
     cfg = CONFIGS[0].scaled(B=B, L=1, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=2600, S_hi=4300, Scap=cap, N=N, D=6, V=0, tree="uniform")
     cases = [make_case(cfg, seed=N + d + x, device="cuda", ragged_nodes=True, with_logits=False) for x in (0, 1)]
     names = ("q", "prefix_len", "n_nodes", "parent")
