@@ -55,6 +55,7 @@
 // barriers of a cluster have no limit of their own: every role of every CTA
 // reaches them, because every wait in front of them ends.
 #include "common.cuh"
+#include "row_tiles.h"
 #include "treeverify_debug.h"
 
 #include <cuda.h>
@@ -101,11 +102,11 @@ constexpr int kMinVirtualTilesPerGroup = TV_MIN_VT;
 // of 65 nodes, prefixes of 300 19.9 / 16.6, 600 22.8 / 19.4, 1000 26.8 / 23.9, 2300 41.0 / 39.1; 10 of 20 nodes 15.7 / 12.9, 17.5 /
 // 14.6, 20.4 / 17.8, 26.7 / 29.2; 12 of 40 nodes with 64-wide heads 15.2 / 14.2, 19.2 / 17.1, 23.5 / 21.6, 34.4 / 36.8.
 constexpr int kMaxWholeUnit = 13;
-// An odd last row tile has a launch of its own (see launch) where the capacity of the cache allows the first number of key tiles
-// per SM, and the lengths reach the second.  In a smaller cache the long calls would gain less than the short ones lose to a second
+// An odd last row tile has a launch of its own where the capacity of the cache allows this many key tiles per SM, and the lengths
+// reach those of odd_row_tile.  In a smaller cache the long calls would gain less than the short ones lose to a second
 // launch that finds nothing to do: 65 nodes, 8 sequences, us a call, one launch / two, in a cache of 28 key tiles per SM with lengths of 4
 // 31.1 / 33.7, 10 50.7 / 53.2, 14 64.0 / 60.5, in one of 33 with 22 98.6 / 91.1.
-constexpr int kSplitTilesPerSm = 60, kSplitLengthsPerSm = 12;
+constexpr int kSplitTilesPerSm = 60;
 constexpr int kMaxCluster = 8;     // CTAs that share a unit (16 is not portable; few clusters of 16 fit the GPU at once: 21.7 us
                                    // instead of 10.8 us a launch for eight units of 12 key tiles)
 constexpr int kTraceCap = 256;     // events per (CTA, role) kept by the optional trace
@@ -1903,34 +1904,35 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
   tv::count_launches(1);
   if (cluster > 1) return launch_kernel<D, MT, true>((unsigned)(units * prm.NP * cluster), (unsigned)cluster, maps, prm, s);
   // An odd number of row tiles leaves the last CTA of a group with an empty one, as expensive as a full one in the time
-  // its group takes.  Where the work is long the last row tile gets a launch of its own, one row tile per CTA, that runs beside
-  // the one with the others: the SMs are shared out between the two by what a key tile costs each (two row tiles 1.3 times as much as
-  // one, with 64-wide heads, whose keys two warpgroups share there, 1.7 times; 1.0 to 2.6 measured).  Behind one another, each on all
-  // SMs, one is bound by tensor work and power while the other waits for memory.  us a call, one launch behind the other / beside,
-  // 8 KV heads, G = 4, 512 ... 4096: 65 nodes, 8 layers 252 / 241, 129 nodes, 4 layers 207 / 193, the same with 64-wide heads 187 / 159.
-  // Only the capacity of the cache is known here: where it allows
+  // its group takes.  Where the work is long the last row tile gets a launch of its own, one row tile per CTA, beside the one with
+  // the others or behind it (see odd_row_tile).  Only the capacity of the cache is known here: where it allows
   // long work both launches are made, and both go by the lengths on the device (short work: the front launch takes all row tiles,
   // the other finds nothing to do, some 3 us).
   if (MT == 2 && g.n_row_tiles % 2 == 1 && units * tiles >= (long long)kSplitTilesPerSm * g.sms) {
-    AttnParams front = prm;
-    front.split_tiles = kSplitLengthsPerSm * g.sms;
-    front.front_NP = g.n_row_tiles / 2;
-    const int odd = g.sms * 10 / (10 + (D == 64 ? 17 : 13) * front.front_NP);
-    front.front_groups = (g.sms - odd) / front.front_NP;
-    const int ctas = front.front_groups * front.front_NP;
-    const cudaError_t e = launch_kernel<D, MT, false>((unsigned)(ctas > g.grid ? ctas : g.grid), 1, maps, front, s);
-    if (e != cudaSuccess) return e;
-    tv::count_launches(1);
-    prm.split_tiles = front.split_tiles;
-    prm.tile0 = g.n_row_tiles - 1;
-    prm.NP = 1;
-    prm.groups = g.sms - ctas;
-    prm.early = prm.beside = 1;
-    prm.epoch = next_epoch();
-    prm.part_ml += (size_t)ctas * 2 * MT * 128;      // the slots and flags behind those of the front launch
-    prm.part_o += (size_t)ctas * MT * 128 * D;
-    prm.flags += ctas;
-    return launch_kernel<D, 1, false>((unsigned)prm.groups, 1, maps, prm, s);
+    const tv::OddRowTile odd = tv::odd_row_tile(g.sms, g.n_row_tiles, D);
+    if (odd.front_groups > 0) {
+      AttnParams front = prm;
+      front.split_tiles = odd.tiles_per_sm * g.sms;
+      front.front_NP = g.n_row_tiles / 2;
+      front.front_groups = odd.front_groups;
+      const int ctas = front.front_groups * front.front_NP;
+      const cudaError_t e = launch_kernel<D, MT, false>((unsigned)(ctas > g.grid ? ctas : g.grid), 1, maps, front, s);
+      if (e != cudaSuccess) return e;
+      tv::count_launches(1);
+      prm.split_tiles = front.split_tiles;
+      prm.tile0 = g.n_row_tiles - 1;
+      prm.NP = 1;
+      prm.groups = odd.odd_groups;
+      prm.early = 1;          // behind a launch of this very call the inputs are stable
+      prm.epoch = next_epoch();
+      if (odd.beside) {
+        prm.beside = 1;
+        prm.part_ml += (size_t)ctas * 2 * MT * 128;      // the slots and flags behind those of the front launch
+        prm.part_o += (size_t)ctas * MT * 128 * D;
+        prm.flags += ctas;
+      }
+      return launch_kernel<D, 1, false>((unsigned)prm.groups, 1, maps, prm, s);
+    }
   }
   return launch_kernel<D, MT, false>((unsigned)g.grid, 1, maps, prm, s);
 }

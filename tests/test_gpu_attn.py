@@ -722,6 +722,64 @@ def test_caches_without_room_for_long_work_have_one_launch(N, d, cap, launches):
     assert n == 1 and torch.equal(out, other) and not st.any()
 
 
+def torch_attention_slice(case, l, b, h, hk, vis, scale):
+    """One query head in fp32: (out [N,d], lse [N]) of the rows that have a node."""
+    S, n = int(case["prefix_len"][b]), int(case["n_nodes"][b])
+    k, v = (torch.cat([case[c][l][b, hk, :S], case[t][l][b, :n, hk]]).float() for c, t in (("k_cache", "k_tree"), ("v_cache", "v_tree")))
+    s = case["q"][l][b, :n, h].float() @ k.T * scale
+    s[:, S:] += torch.where(torch.from_numpy(vis[b, :n, :n]).cuda() != 0, 0.0, float("-inf"))
+    return torch.softmax(s, -1) @ v, torch.logsumexp(s, -1)
+
+
+@pytest.mark.parametrize("N,G,d", [(145, 32, 64), (149, 64, 128), (149, 128, 64)])      # 37, 75 and 149 row tiles
+@pytest.mark.parametrize("what", ["below", "at", "long"])
+def test_wide_head_groups_have_the_last_row_tile_behind_the_others(N, G, d, what):
+    """With lengths just below the bound the call gives the bits it gives in a cache that is too small for two launches; from the
+    bound on the last row tile comes out of the second launch: fp32 values on heads at both ends."""
+    B, L, Hkv, TT = 3, 4, 2, 2
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    bound = -(-60 * sms // (L * Hkv))                      # key tiles of the sequences together from which the work is split
+    each = (bound - 1) // B                                # a cache of so many key tiles (the tree's among them) has one launch
+    tiles = np.full(B, {"below": each, "at": bound // B, "long": bound // B + 40}[what])
+    if what == "at":
+        tiles[:bound % B] += 1
+    cap = (each - TT) * 128
+    big = (bound // B + 60) * 128
+    cfg = CONFIGS[0].scaled(B=B, L=L, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=cap, S_hi=cap, Scap=big, N=N, D=6, V=0, tree="uniform")
+    case = make_case(cfg, seed=N + G, device="cuda", ragged_nodes=True, with_logits=False)
+    case["prefix_len"] = torch.from_numpy(((tiles - TT) * 128).astype(np.int32)).cuda()
+    case["n_nodes"][0] = N
+    bits = torch.zeros(B, N, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    st = torch.zeros(B, dtype=torch.int32, device="cuda")
+    tv.tree_build_mask(case["parent"], case["n_nodes"], N - 1, 1, bits, st)
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(B, N, cfg.Hq, Hkv, d, big), dtype=torch.uint8, device="cuda")
+
+    def run(rows):
+        out = torch.full((L, B, N, cfg.Hq, d), 3.0, dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((L, B, cfg.Hq, N), 3.0, dtype=torch.float32, device="cuda")
+        kc, vc = (case[k] if rows == big else case[k][:, :, :, :rows].contiguous() for k in ("k_cache", "v_cache"))
+        n0 = tv.tv_launch_count()
+        tv.tree_verify_attn_layers(case["q"], kc, vc, case["k_tree"], case["v_tree"], case["prefix_len"], case["n_nodes"], bits,
+                                   d ** -0.5, out, ws, st, lse=lse)
+        torch.cuda.synchronize()
+        assert not st.any()
+        return out, lse, tv.tv_launch_count() - n0
+
+    out, lse, launches = run(big)
+    assert launches == 2
+    again, again_lse, _ = run(big)
+    assert torch.equal(out, again) and torch.equal(lse, again_lse)
+    if what == "below":
+        small, small_lse, launches = run(cap)
+        assert launches == 1 and torch.equal(out, small) and torch.equal(lse, small_lse)
+    vis = oracle_visibility(case["parent"], case["n_nodes"], bits_gpu=bits)[:, 0]
+    for l, b, h in ((0, 0, 0), (L - 1, 1, cfg.Hq - 1), (1, 2, G)):
+        want, want_lse = torch_attention_slice(case, l, b, h, h // G, vis, d ** -0.5)
+        n = want.shape[0]
+        assert (out[l][b, :n, h].float() - want).abs().max() <= ATTN_ATOL and not out[l][b, n:, h].any()
+        assert (lse[l][b, h, :n] - want_lse).abs().max() <= 2e-3 and torch.isneginf(lse[l][b, h, n:]).all()
+
+
 @pytest.mark.parametrize("N,d,G", [(65, 64, 4), (65, 128, 4), (129, 128, 4), (160, 64, 4), (44, 128, 8)])
 def test_last_row_tile_beside_the_others_keeps_the_order_of_the_stream(N, d, G):
     """The two launches of an odd last row tile run at the same time.  Inputs written by the kernels directly in front, outputs
