@@ -1785,14 +1785,15 @@ Geometry geometry(int B, int Nmax, int Hq, int Hkv, int d, bool query_device) {
   g.sms = query_device ? tv::sm_count() : 148;
   g.groups = g.sms / g.NP > 0 ? g.sms / g.NP : 1;
   g.grid = g.groups * g.NP;
-  // workspace: (m,l) pairs and partial O, both with 160 slots whatever the device; the flags of the slots in use (one per
-  // CTA) in the (m,l) room of the last ones; then a stretch per layer, none of which is used: how many there are bounds the
-  // layers that share a launch
+  // workspace: (m,l) pairs and partial O, both with 160 slots (one per CTA) whatever the device, the flags of all slots in the O room
+  // of the first one: the pieces of CTA group 0 are all the first of their unit, which leave no partial; then a
+  // stretch per layer, none of which is used: how many there are bounds the layers that share a launch
   constexpr size_t kSlotsMax = 160;
+  static_assert(kSlotsMax * sizeof(unsigned long long) <= 128 * 64 * sizeof(tv_bf16), "the flags fit a slot of one row tile, 64-wide");
   const size_t ml_bytes = (size_t)g.MT * 128 * 2 * sizeof(float);
   g.ml_off = 0;
-  g.flags_off = (kSlotsMax - 2) * ml_bytes;
   g.o_off = (kSlotsMax * ml_bytes + 255) & ~size_t(255);
+  g.flags_off = g.o_off;
   g.layers_off = (g.o_off + kSlotsMax * g.MT * 128 * d * sizeof(tv_bf16) + 255) & ~size_t(255);
   g.per_layer = ((size_t)B * Hkv * g.NP * 2 * sizeof(unsigned long long) + 255) & ~size_t(255);
   g.total = g.layers_off + kWorkspaceLayers * g.per_layer;
@@ -2049,7 +2050,7 @@ int attn_entry(const tv_bf16* q,
   const Geometry g = geometry(B, Nmax, Hq, Hkv, d, true);
   const long long tiles_per_layer = (long long)B * Hkv * ((Scap + kTileN - 1) / kTileN + 2 + kSetupCost);
   TV_REQUIRE(tiles_per_layer < (1ll << 31), "tree_verify_attn: B * Hkv * Scap is too large for the tile scheduler");
-  if (g.sms > 158) return tv::fail(TV_ERR_INVALID_ARG, "tree_verify_attn: device with more than 158 SMs is not supported");
+  if (g.sms > 160) return tv::fail(TV_ERR_INVALID_ARG, "tree_verify_attn: device with more than 160 SMs is not supported");
   if (workspace_bytes < g.layers_off + g.per_layer)
     return tv::fail(TV_ERR_WORKSPACE, "tree_verify_attn: workspace of %zu bytes, need %zu", workspace_bytes,
                     g.layers_off + g.per_layer);
