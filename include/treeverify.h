@@ -163,9 +163,10 @@ TV_API size_t tv_attn_workspace_bytes(int B, int Nmax, int Hq, int Hkv, int d, i
  * all earlier kernels have finished, and nothing is written before that.
  * Using the committed prefix earlier is what tree_verify_attn_layers offers,
  * under a promise by the caller.
- * Launches: one kernel, or two (a short last row tile of long problems runs
- * behind the others; whether it does is decided from the lengths on the
- * device, in caches whose capacity allows such problems).  How the work is
+ * Launches: one kernel, or two (an odd last row tile of long problems runs
+ * beside the others, in wide head groups behind them; whether it does is
+ * decided from the lengths on the device, in caches whose capacity allows
+ * such problems).  How the work is
  * shared between CTAs follows the shape, the capacity and the lengths;
  * results agree to the rounding of the partial sums.
  */

@@ -38,6 +38,9 @@ TV_API int tv_debug_attn_simt(const tv_bf16* q, const tv_bf16* k_cache, const tv
  * there (the other modes take the even cut).
  * mode bit 3: the tile table that is built ahead of the wait for the kernel
  * in front is a wrong one and has to be built again (no result changes).
+ * mode bit 5: the flag by which the second of two launches that run at the
+ * same time knows that it may start is not raised, so that it waits for the
+ * first one (no result changes).
  * With bit 0 or 1 the launch ends by itself: every role leaves its loop, the tensor
  * memory is freed, and TV_ST_TIMEOUT is ORed into status[b] of every
  * sequence (out and lse are unspecified).  Nothing traps or faults; the next

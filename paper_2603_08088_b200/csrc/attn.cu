@@ -17,6 +17,7 @@
 //               two row tiles it serves them in turn, so the softmax of one row
 //               tile runs while the tensor pipe works for the other.
 //   warp 2      raises the flag of the CTA's partials, where another CTA merges them
+//   warp 3      of the first CTA: lets the launch with an odd last row tile start (see beside)
 //   warps 4-7   two softmax warpgroups, one thread per row, online softmax with
 //   warps 8-11  lazy rescale, one for each row tile.  With one row tile and
 //               64-wide heads (KS) one takes the even and one the odd key tiles of
@@ -399,9 +400,10 @@ struct AttnParams {
   int out_al32;                  // out is 32-byte aligned: rows can be written 32 bytes per thread and store
   float scale_log2e;             // scale * log2(e)
   float scale;
-  int beside;                    // launched behind the front launch of the same call, to run beside it: everything in front of
-                                 // that one is complete when this one starts, and it reads nothing that the front launch writes;
-                                 // it waits for the front launch where it ends
+  int beside;                    // launched behind the front launch of the same call, to run beside it: it reads nothing that the
+                                 // front launch writes, and waits for it where it ends, not where it starts (see passed)
+  unsigned long long* passed;    // a pair of launches that runs at the same time: holds passed_tag once the front launch has
+  unsigned long long passed_tag; // seen everything in front of it complete, until the other one ends; else nullptr
   int early;                     // the caller promises that the kernel in front leaves prefix_len, n_nodes, the block
                                  // table and the committed rows alone: they are read before the grid-dependency wait
   unsigned long long wait_limit_ns;   // limit of every bounded wait
@@ -409,6 +411,7 @@ struct AttnParams {
                                  // partials but never announce them (both exercise the expiry of a bounded wait);
                                  // bit 3: the guessed table is built from lengths one tile too long;
                                  // bit 4 (host): the cluster kernel is not left out;
+                                 // bit 5: the flag that lets two launches run at the same time is not raised;
                                  // bit 2: the K/V stream alone - the issuing warp only hands every slot back as
                                  // soon as it is full, no MMA, no softmax, no output (what the memory side can do)
   int L;                         // layers in this launch: their units form one tile space, layer after layer
@@ -497,6 +500,15 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   // Whether an odd last row tile has a launch of its own, from the key tiles of one KV head over all sequences.
   auto splits = [&](int tiles) -> bool { return (unsigned)(prm.Hkv * tiles) * (unsigned)prm.L >= (unsigned)prm.split_tiles; };
+  // The launch beside the others is scheduled when every CTA of the front launch is behind its grid-dependency wait.  What that makes
+  // complete is visible to the front launch; the flag that it released there and every thread here acquires hands it on.  Who does
+  // not find the flag waits for the front launch like any other kernel.
+  const bool beside = MT == 1 && !CL && prm.beside;
+  if (beside && ld_acquire(prm.passed) != prm.passed_tag) gdc_wait();
+  auto end_beside = [&]() {      // who waits for this launch waits for the one in front
+    gdc_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<volatile unsigned long long*>(prm.passed) = 0ull;      // (a graph comes with the tag again)
+  };
   if (MT == 1 && !CL && prm.split_tiles > 0) {      // that launch: nothing to do where the one in front has taken it along
     int tiles = 0;
 #pragma unroll 1
@@ -506,7 +518,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     if (!splits(__reduce_add_sync(0xffffffffu, tiles))) {
       if (threadIdx.x == 0) gdc_launch_dependents();
-      gdc_wait();
+      if (beside) end_beside();
+      else gdc_wait();
       return;
     }
   }
@@ -766,13 +779,14 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // that this kernel leaves prefix_len, n_nodes, the block table and the committed rows alone, the first
       // prefix tiles are requested at once; Q and the tree's K/V - what a preceding kernel may still be
       // producing - wait for that kernel to finish.  Only then may the next kernel be scheduled, so that at
-      // most two launches are in flight.
+      // most two launches are in flight - three behind a pair that runs at the same time, whose second one lets the next
+      // kernel go while the first may still be writing out, lse, status and the workspace.
       // status[] may still be written by the kernel in front (tree_build_mask stores it last), so a flag found
       // before the wait is kept here and raised after it.
       bool synced = false;
       int bad_page_b = -1;
       auto sync_with_predecessor = [&]() {
-        if (!prm.beside) gdc_wait();
+        if (!beside) gdc_wait();
         if (elect_one()) gdc_launch_dependents();
         if (bad_page_b >= 0 && lane == 0) atomicOr(prm.status + bad_page_b, TV_ST_BAD_INDEX);
         bad_page_b = -1;
@@ -797,7 +811,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         __syncwarp();
       };
-      if (!prm.early || prm.beside) sync_with_predecessor();
+      if (!prm.early || beside) sync_with_predecessor();
       bool have_first = !CL && !prm.early && at[0];
       if (have_first) {
         g = at[1];
@@ -875,7 +889,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       if (!synced) sync_with_predecessor();        // a CTA without work still has to let the next kernel go
     } else {
-      if (!prm.beside) gdc_wait();
+      if (!beside) gdc_wait();
       if (elect_one()) gdc_launch_dependents();
     }
     if (CL) {
@@ -1100,8 +1114,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int row = ((warp & 3) << 5) | lane;        // TMEM lane = row inside the tile
     const uint32_t lane_addr = (uint32_t)((warp & 3) << 5) << 16;
     // anc_bits, the workspace and the outputs may belong to the kernel in front until it is done
-    if (prm.beside) __threadfence();      // (nothing does; the fence drops what an earlier launch has left of anc_bits in L1)
-    else gdc_wait();
+    if (!beside) gdc_wait();
     // in-cache layout: a tree that does not fit behind its prefix is reported, not read past the capacity (rows
     // past Scap arrive as zeros and the sequence's output is unspecified).  Raised after the wait: status[] may
     // be written by the kernel in front until then.
@@ -1710,6 +1723,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    // (in front of gdc_launch_dependents in warp 0, where nothing could miss it, the release and its code cost 0.2 to 0.9 us a launch)
+    if (MT == 2 && !CL && threadIdx.x == 96 && prm.passed && blockIdx.x == 0 && !(prm.debug & 32)) {
+      gdc_wait();
+      st_release(prm.passed, prm.passed_tag);
+    }
     // Only the first item of a CTA can be a piece whose partials another CTA merges.  Warp 2 waits for every softmax warp to
     // have stored its part (or to have seen that there is none), and then raises the flag.
     if (!CL && warp == 2 && !*abort_flag && !(prm.debug & 4) && mbar_wait(bar(L::PIECE), 0, abort_flag, wait_limit) && lane == 0 &&
@@ -1722,7 +1740,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   }
 
   // ---- teardown
-  if (prm.beside) gdc_wait();      // who waits for this launch waits for the one in front
+  if (beside) end_beside();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -1789,7 +1807,8 @@ Geometry geometry(int B, int Nmax, int Hq, int Hkv, int d, bool query_device) {
   // of the first one: the pieces of CTA group 0 are all the first of their unit, which leave no partial; then a
   // stretch per layer, none of which is used: how many there are bounds the layers that share a launch
   constexpr size_t kSlotsMax = 160;
-  static_assert(kSlotsMax * sizeof(unsigned long long) <= 128 * 64 * sizeof(tv_bf16), "the flags fit a slot of one row tile, 64-wide");
+  static_assert(kSlotsMax == kMaxGroups && (kSlotsMax + 1) * sizeof(unsigned long long) <= 128 * 64 * sizeof(tv_bf16),
+                "the flags and the one between two launches fit a slot of one row tile, 64-wide");
   const size_t ml_bytes = (size_t)g.MT * 128 * 2 * sizeof(float);
   g.ml_off = 0;
   g.o_off = (kSlotsMax * ml_bytes + 255) & ~size_t(255);
@@ -1916,6 +1935,10 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
       front.split_tiles = odd.tiles_per_sm * g.sms;
       front.front_NP = g.n_row_tiles / 2;
       front.front_groups = odd.front_groups;
+      if (odd.beside) {
+        front.passed = prm.flags + kMaxGroups;
+        front.passed_tag = prm.epoch;
+      }
       const int ctas = front.front_groups * front.front_NP;
       const cudaError_t e = launch_kernel<D, MT, false>((unsigned)(ctas > g.grid ? ctas : g.grid), 1, maps, front, s);
       if (e != cudaSuccess) return e;
@@ -1928,6 +1951,8 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
       prm.epoch = next_epoch();
       if (odd.beside) {
         prm.beside = 1;
+        prm.passed = front.passed;
+        prm.passed_tag = front.passed_tag;
         prm.part_ml += (size_t)ctas * 2 * MT * 128;      // the slots and flags behind those of the front launch
         prm.part_o += (size_t)ctas * MT * 128 * D;
         prm.flags += ctas;

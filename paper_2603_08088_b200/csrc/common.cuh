@@ -33,8 +33,10 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // next kernel be scheduled: the next launch overlaps this kernel's body, and what a kernel reads before its own wait
 // (tree_verify_attn the committed prefix, the accept kernels tokens and tree) is complete unless the kernel directly
 // in front of it writes it.  The scan of tree_accept_behind_attn lets the next one go before its own wait: it is itself
-// only scheduled when everything in front of the attention is complete.  Reads ahead of a wait go past L1 or
-// follow a fence that drops it.
+// only scheduled when everything in front of the attention is complete.  tree_verify_attn may be two launches, of which
+// the second lets the next kernel go while the first still runs (and waits for it where it ends): a kernel behind an
+// attention reads ahead of its wait only what neither of them writes, that is neither out, lse, status nor the workspace.
+// Reads ahead of a wait go past L1 or follow a fence that drops it.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -835,6 +835,30 @@ def test_last_row_tile_beside_the_others_keeps_the_order_of_the_stream(N, d, G):
         assert np.abs(want[0][b:b + 1, :, hk * G:(hk + 1) * G].float().cpu().numpy() - ref_out).max() <= 2e-2
 
 
+@pytest.mark.parametrize("N,d", [(65, 64), (129, 128)])
+@pytest.mark.parametrize("S", [300, 4000])       # the second launch has nothing to do, its share
+def test_last_row_tile_without_leave_to_start_waits_for_the_others(N, d, S):
+    """The second of two launches that run at the same time goes by a flag of the first; where it does not find it (a switch holds it
+    back) it waits, and the results are the same bits, in turn with calls that do find it on one workspace."""
+    B, Hkv, G, cap = 14, 8, 4, 10240
+    cfg = CONFIGS[0].scaled(B=B, L=1, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=S // 2, S_hi=S, Scap=cap, N=N, D=6, V=0, tree="uniform")
+    c = make_case(cfg, seed=N, device="cuda", ragged_nodes=True, with_logits=False)
+    bits = torch.zeros(B, N, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    st = torch.zeros(B, dtype=torch.int32, device="cuda")
+    tv.tree_build_mask(c["parent"], c["n_nodes"], N - 1, 1, bits, st)
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(B, N, cfg.Hq, Hkv, d, cap), dtype=torch.uint8, device="cuda")
+    args = (c["q"][0], c["k_cache"][0], c["v_cache"][0], c["k_tree"][0], c["v_tree"][0], c["prefix_len"], c["n_nodes"], bits, d ** -0.5)
+    want = torch.zeros(B, N, cfg.Hq, d, dtype=torch.bfloat16, device="cuda")
+    tv.tree_verify_attn(*args, want, ws, st)
+    for mode in (32, 0, 32, 32, 0):
+        out = torch.full_like(want, 3.0)
+        n0 = tv.tv_launch_count()
+        tv.tv_debug_attn_expire(*args, out, ws, st, 2_000_000_000, mode)
+        assert tv.tv_launch_count() - n0 == 2
+        torch.cuda.synchronize()
+        assert torch.equal(out, want) and not st.any()
+
+
 @pytest.mark.parametrize("G,N,d", [(2, 40, 64), (4, 40, 64), (2, 40, 128), (4, 40, 128)])
 @pytest.mark.parametrize("S,other", [(300, 300), (1024, 1024), (1025, 1025), (300, 100)])
 def test_equal_units_stay_whole_while_they_are_short(S, other, G, N, d):
