@@ -79,6 +79,7 @@ TV_API int tv_debug_attn_stream_only(const tv_bf16* q, const tv_bf16* k_cache, c
  * Live only in a library built with -DTV_TRACE: while a device buffer of
  * 160 * 4 * 256 uint64 is registered here, every tree_verify_attn launch
  * records a per-CTA, per-role timeline (tag << 48 | globaltimer ns) into it.
+ * The CTAs of a launch that runs beside another follow those of the other.
  * NULL switches it off.
  */
 TV_API void tv_debug_set_attn_trace(unsigned long long* device_buffer);

@@ -1956,6 +1956,7 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
         prm.part_ml += (size_t)ctas * 2 * MT * 128;      // the slots and flags behind those of the front launch
         prm.part_o += (size_t)ctas * MT * 128 * D;
         prm.flags += ctas;
+        if (prm.trace) prm.trace += (size_t)ctas * 4 * kTraceCap;
       }
       return launch_kernel<D, 1, false>((unsigned)prm.groups, 1, maps, prm, s);
     }
