@@ -1,5 +1,5 @@
 """A whole verification step captured into a CUDA graph and replayed: the library launches only on the
-caller's stream, keeps no per-call device state that a replay would find stale (the split-KV counters are
+caller's stream, keeps no per-call device state that a replay would find stale (the split-KV flags are
 cleared by the piece that merges), and so every replay reproduces the eager step bit for bit."""
 import numpy as np
 import pytest
@@ -13,7 +13,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("ci,over", [(4, dict(B=6, L=3, Hq=8, Hkv=2, S_lo=100, S_hi=1500, Scap=1600, V=4096)),
-                                     (1, dict(Hq=8, Hkv=8, S_lo=2048, S_hi=2048, Scap=2304, V=2048, L=2))])
+                                     (1, dict(Hq=8, Hkv=8, S_lo=2048, S_hi=2048, Scap=2304, V=2048, L=2)),
+                                     # an odd last row tile with a launch of its own, beside the others
+                                     (4, dict(B=12, L=8, Hq=16, Hkv=4, N=65, S_lo=1400, S_hi=2800, Scap=3100, V=4096))])
 def test_step_replayed_from_a_cuda_graph_equals_the_eager_step(ci, over):
     cfg = CONFIGS[ci].scaled(**over)
     case = to_device(make_case(cfg, seed=99 + ci))

@@ -85,12 +85,13 @@ def test_status_bits_raised_by_a_one_layer_attention_survive_the_mask_kernel():
 
 
 @pytest.mark.parametrize("in_cache", [False, True])
-@pytest.mark.parametrize("B,L,S", [(1, 1, 1500), (12, 3, 2500)])
-def test_scan_beside_the_attention_changes_nothing(B, L, S, in_cache):
+@pytest.mark.parametrize("B,L,S,N,launches", [(1, 1, 1500, 33, 1), (12, 3, 2500, 33, 1), (12, 8, 2800, 65, 2)])
+def test_scan_beside_the_attention_changes_nothing(B, L, S, N, launches, in_cache):
     """verify_step lets the vocabulary scan overlap the attention in front of it.  Three steps in a row without a
     synchronisation, each on the cache and the lengths the one before has left, give bit for bit what the same calls
-    with the ordered tree_accept give (acceptance and commit wait for the attention in both)."""
-    cfg = CONFIGS[2].scaled(B=B, L=L, Hq=16, Hkv=4, S_lo=S // 2, S_hi=S, Scap=S + 300, V=30001, N=33, D=6)
+    with the ordered tree_accept give (acceptance and commit wait for the attention in both).  One attention launch, and two that
+    run at the same time, of which the second lets the scan go while the first still runs."""
+    cfg = CONFIGS[2].scaled(B=B, L=L, Hq=16, Hkv=4, S_lo=S // 2, S_hi=S, Scap=S + 300, V=30001, N=N, D=6)
     case = to_device(make_case(cfg, seed=B + L))
 
     def steps(ordered):
@@ -104,9 +105,11 @@ def test_scan_beside_the_attention_changes_nothing(B, L, S, in_cache):
             else:
                 tv.tree_build_mask(c["parent"], c["n_nodes"], Dp1 - 1, P, buf.anc_bits, buf.status, depth=buf.depth,
                                    anc_table=buf.anc_table, retrieve_indices=buf.retrieve, n_paths=buf.n_paths)
+                n0 = tv.tv_launch_count()
                 tv.tree_verify_attn_layers(c["q"], c["k_cache"], c["v_cache"], None if in_cache else c["k_tree"],
                                            None if in_cache else c["v_tree"], c["prefix_len"], c["n_nodes"], buf.anc_bits,
                                            cfg.d ** -0.5, buf.out, buf.attn_ws, buf.status, flags=tv.TV_ATTN_STABLE_INPUTS)
+                assert tv.tv_launch_count() - n0 == launches
                 torch.cuda.synchronize()
                 tv.tree_accept(c["logits"], c["tokens"], buf.retrieve, c["n_nodes"], buf.argmax_tok, buf.accept_len,
                                buf.best_path, buf.accepted_nodes, buf.next_token, buf.accept_ws, buf.status)

@@ -102,6 +102,38 @@ def test_waits_that_expire_anywhere_in_the_tile_loop(d, G, N):
     assert expired >= 1
 
 
+@pytest.mark.parametrize("N,d", [(65, 64), (129, 128)])
+def test_waits_that_expire_in_two_launches_at_the_same_time(N, d):
+    """The shapes whose odd last row tile has a launch beside the others, of one row tile per CTA: waits of either launch run out, in
+    the tile loop, for operands that nobody sends and for pieces that are never announced.  Both end, the status says so, and the
+    pair behind them on the same workspace gives its bits."""
+    B, Hkv, G, cap = 14, 8, 4, 10240
+    cfg = CONFIGS[0].scaled(B=B, L=1, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=2600, S_hi=4300, Scap=cap, N=N, D=6, V=0, tree="uniform")
+    c = make_case(cfg, seed=d + N, device="cuda", with_logits=False)
+    bits = torch.zeros(B, N, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    status = torch.zeros(B, dtype=torch.int32, device="cuda")
+    tv.tree_build_mask(c["parent"], c["n_nodes"], N - 1, 1, bits, status)
+    ws = torch.zeros(tv.tv_attn_workspace_bytes(B, N, cfg.Hq, Hkv, d, cap), dtype=torch.uint8, device="cuda")
+    args = (c["q"][0], c["k_cache"][0], c["v_cache"][0], c["k_tree"][0], c["v_tree"][0], c["prefix_len"], c["n_nodes"], bits, d ** -0.5)
+    before, after = (torch.full((B, N, cfg.Hq, d), x, dtype=torch.bfloat16, device="cuda") for x in (3.0, 4.0))
+    n0 = tv.tv_launch_count()
+    tv.tree_verify_attn(*args, before, ws, status)
+    assert tv.tv_launch_count() - n0 == 2
+    torch.cuda.synchronize()
+    assert (i32(status) == 0).all()
+    for limit, mode in [(x, 0) for x in (0, 1000, 2000, 4000, 8000, 16000, 500_000_000)] + [(2_000_000, 1), (2_000_000, 2), (2_000_000, 33)]:
+        got = torch.zeros_like(before)
+        tv.tv_debug_attn_expire(*args, got, ws, status, limit, mode)
+        torch.cuda.synchronize()
+        st = i32(status)
+        assert (st == st[0]).all() and st[0] in ((0, tv.TV_ST_TIMEOUT) if mode == 0 else (tv.TV_ST_TIMEOUT,)), (limit, mode)
+        assert st[0] != 0 or torch.equal(got, before)
+        status.zero_()
+        tv.tree_verify_attn(*args, after, ws, status)
+        torch.cuda.synchronize()
+        assert (i32(status) == 0).all() and torch.equal(before, after), (limit, mode)
+
+
 def test_expired_waits_of_the_cluster_kernel():
     """As above, with a producer that issues nothing: every CTA of a cluster gives up, meets the others at the cluster's barriers
     and leaves."""
