@@ -505,7 +505,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // not find the flag waits for the front launch like any other kernel.
   const bool beside = MT == 1 && !CL && prm.beside;
   if (beside && ld_acquire(prm.passed) != prm.passed_tag) gdc_wait();
-  auto end_beside = [&]() {      // who waits for this launch waits for the one in front
+  // Who waits for this launch waits for the one in front.  All CTAs stay for that: where only the first one did, the next
+  // attention spread over the SMs as they came free (65 nodes, layer after layer: 63.5 -> 79 us, 8 layers a launch 290 -> 349).
+  auto end_beside = [&]() {
     gdc_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<volatile unsigned long long*>(prm.passed) = 0ull;      // (a graph comes with the tag again)
   };
@@ -518,6 +520,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     if (!splits(__reduce_add_sync(0xffffffffu, tiles))) {
       if (threadIdx.x == 0) gdc_launch_dependents();
+      if (blockIdx.x != 0) return;      // one CTA is enough to wait; the others leave their SMs (short calls 44.5 -> 43.4 us)
       if (beside) end_beside();
       else gdc_wait();
       return;
