@@ -166,9 +166,8 @@ TV_API size_t tv_attn_workspace_bytes(int B, int Nmax, int Hq, int Hkv, int d, i
  * Launches: one kernel, or two (an odd last row tile of long problems runs
  * beside the others, in wide head groups behind them; whether it does is
  * decided from the lengths on the device, in caches whose capacity allows
- * such problems).  How the work is
- * shared between CTAs follows the shape, the capacity and the lengths;
- * results agree to the rounding of the partial sums.
+ * such problems).  How the work is shared between CTAs follows the shape, the
+ * capacity and the lengths; results agree to the rounding of the partial sums.
  */
 TV_API int tree_verify_attn(const tv_bf16* q,
                      const tv_bf16* k_cache, const tv_bf16* v_cache,

@@ -76,11 +76,10 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleThreshold = 8.0f;            // in log2 units
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 // Virtual tiles charged per unit by the scheduler: what a CTA pays for one more item (epilogue, masked tiles, refill) is
-// some 5 us, three to four tiles' time.  Eight shapes, one and 32 layers a launch: 4 is 1 to 3 % faster than 2 and 1 to 2 %
-// faster than 1 and 5 on all but the ragged batch (1.8 % slower than 2); 3 is level with 4.  Of 72 shapes 2 is 1 to 4 %
-// faster than 4 on 33 (one row tile above all), and slower on 9, where every unit, or every second, is cut once: us a launch, 2 / 4, 128-wide
-// heads, 8 sequences of 4096 41.7 / 39.8, 32 of 1024 45.2 / 43.9, 4 of 4096 with 128 nodes 41.7 / 40.8, of 4000 ... 4096
-// 58.1 / 56.2, 32 of 650 ... 4550 with one row tile 65.3 / 63.0; 8 of 1024 ... 8192 47.8 / 46.1.
+// some 5 us, three to four tiles' time.  Eight shapes, one and 32 layers a launch: 4 is 1 to 2 % faster than 1 and 5 on most; 3 is
+// level with 4.  Of 72 shapes 2 is 1 to 4 % faster than 4 on 33 (one row tile above all) and slower on 9, where every unit, or every
+// second, is cut once: us a launch, 2 / 4, 128-wide heads, 8 sequences of 4096 41.7 / 39.8, 32 of 1024 45.2 / 43.9, 4 of 4096 with
+// 128 nodes 41.7 / 40.8, of 4000 ... 4096 58.1 / 56.2, 32 of 650 ... 4550 with one row tile 65.3 / 63.0; 8 of 1024 ... 8192 47.8 / 46.1.
 #ifndef TV_SETUP_COST
 #define TV_SETUP_COST 4
 #endif
@@ -104,8 +103,8 @@ constexpr int kMinVirtualTilesPerGroup = TV_MIN_VT;
 // 14.6, 20.4 / 17.8, 26.7 / 29.2; 12 of 40 nodes with 64-wide heads 15.2 / 14.2, 19.2 / 17.1, 23.5 / 21.6, 34.4 / 36.8.
 constexpr int kMaxWholeUnit = 13;
 // An odd last row tile has a launch of its own where the capacity of the cache allows this many key tiles per SM, and the lengths
-// reach those of odd_row_tile.  In a smaller cache the long calls would gain less than the short ones lose to a second
-// launch that finds nothing to do: 65 nodes, 8 sequences, us a call, one launch / two, in a cache of 28 key tiles per SM with lengths of 4
+// reach those of odd_row_tile.  In a smaller cache the short calls would lose what the long ones gain, to a second launch that
+// finds nothing to do: 65 nodes, 8 sequences, us a call, one launch / two, in a cache of 28 key tiles per SM with lengths of 4
 // 31.1 / 33.7, 10 50.7 / 53.2, 14 64.0 / 60.5, in one of 33 with 22 98.6 / 91.1.
 constexpr int kSplitTilesPerSm = 60;
 constexpr int kMaxCluster = 8;     // CTAs that share a unit (16 is not portable; few clusters of 16 fit the GPU at once: 21.7 us
@@ -1930,7 +1929,7 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
   // its group takes.  Where the work is long the last row tile gets a launch of its own, one row tile per CTA, beside the one with
   // the others or behind it (see odd_row_tile).  Only the capacity of the cache is known here: where it allows
   // long work both launches are made, and both go by the lengths on the device (short work: the front launch takes all row tiles,
-  // the other finds nothing to do, some 3 us).
+  // the other finds nothing to do, some 2 us).
   if (MT == 2 && g.n_row_tiles % 2 == 1 && units * tiles >= (long long)kSplitTilesPerSm * g.sms) {
     const tv::OddRowTile odd = tv::odd_row_tile(g.sms, g.n_row_tiles, D);
     if (odd.front_groups > 0) {
