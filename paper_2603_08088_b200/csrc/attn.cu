@@ -387,9 +387,11 @@ struct AttnParams {
   unsigned long long epoch;      // tag of this call
   int B, Nmax, Hq, Hkv, Scap, G, NPT, NP, W, groups;
   int tile0;                     // first row tile of this launch
-  int split_tiles;               // > 0: from this many key tiles on (all units of the launch, by the lengths on the device) the
-                                 // odd last row tile belongs to a launch of its own; below, that launch has no work
-  int front_NP, front_groups;    // NP and groups of the launch in front of it then
+  int split_tiles;               // > 0: one of a pair of launches.  From this many key tiles on (all units of the launch, by the lengths
+                                 // on the device) the odd last row tile belongs to the second one; below, that one has no work
+  int behind_tiles;              // from this many on the second one runs behind the first one, below it runs beside it
+  int split_NP, beside_groups, behind_groups;      // NP of this launch where the last row tile is split off, its groups in either case
+  int slot0;                     // its first slot where it runs beside the other
   int TT;                        // key tiles of the tree's own K/V: ceil(Nmax / 128), 1 or 2
   uint32_t q_box_bytes;          // bytes of one Q box {64, G, NPT}: 16 KB when G divides 128
   unsigned long long* trace;     // optional event trace [cta][role 0..3][kTraceCap] of (tag << 48 | ns), or NULL
@@ -399,10 +401,8 @@ struct AttnParams {
   int out_al32;                  // out is 32-byte aligned: rows can be written 32 bytes per thread and store
   float scale_log2e;             // scale * log2(e)
   float scale;
-  int beside;                    // launched behind the front launch of the same call, to run beside it: it reads nothing that the
-                                 // front launch writes, and waits for it where it ends, not where it starts (see passed)
-  unsigned long long* passed;    // a pair of launches that runs at the same time: holds passed_tag once the front launch has
-  unsigned long long passed_tag; // seen everything in front of it complete, until the other one ends; else nullptr
+  unsigned long long* passed;    // a pair of launches: holds passed_tag once the first one has seen everything in front of the
+  unsigned long long passed_tag; // pair complete, until the second one ends; else nullptr
   int early;                     // the caller promises that the kernel in front leaves prefix_len, n_nodes, the block
                                  // table and the committed rows alone: they are read before the grid-dependency wait
   unsigned long long wait_limit_ns;   // limit of every bounded wait
@@ -497,34 +497,42 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   int* gs = reinterpret_cast<int*>(smem + L::kGs);
   const unsigned long long wait_limit = prm.wait_limit_ns;
 
-  // Whether an odd last row tile has a launch of its own, from the key tiles of one KV head over all sequences.
-  auto splits = [&](int tiles) -> bool { return (unsigned)(prm.Hkv * tiles) * (unsigned)prm.L >= (unsigned)prm.split_tiles; };
-  // The launch beside the others is scheduled when every CTA of the front launch is behind its grid-dependency wait.  What that makes
-  // complete is visible to the front launch; the flag that it released there and every thread here acquires hands it on.  Who does
-  // not find the flag waits for the front launch like any other kernel.
-  const bool beside = MT == 1 && !CL && prm.beside;
-  if (beside && ld_acquire(prm.passed) != prm.passed_tag) gdc_wait();
-  // Who waits for this launch waits for the one in front.  All CTAs stay for that: where only the first one did, the next
+  // What happens to an odd last row tile, from the key tiles of one KV head over all sequences: 0 it stays with the others, 1 it
+  // has a launch beside them, 2 behind them.
+  auto odd_mode = [&](int tiles) -> int {
+    const unsigned all = (unsigned)(prm.Hkv * tiles) * (unsigned)prm.L;
+    return all < (unsigned)prm.split_tiles ? 0 : (all < (unsigned)prm.behind_tiles ? 1 : 2);
+  };
+  // The second launch of a pair.  It is scheduled when every CTA of the first one is behind its grid-dependency wait.  What that makes
+  // complete is visible to the first launch; the flag that it released there and every thread here acquires hands it on.  Who does
+  // not find the flag waits for the first launch like any other kernel.  Beside the first one it reads nothing that one writes, and
+  // waits for it only where it ends; behind it it waits like any other.
+  constexpr bool MAY_BE_SECOND = MT == 1 && !CL;
+  bool beside = false;
+  // Who waits for this launch waits for the first one.  All CTAs with work stay for that: where only one did, the next
   // attention spread over the SMs as they came free (65 nodes, layer after layer: 63.5 -> 79 us, 8 layers a launch 290 -> 349).
-  auto end_beside = [&]() {
+  auto end_pair = [&]() {
     gdc_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<volatile unsigned long long*>(prm.passed) = 0ull;      // (a graph comes with the tag again)
   };
-  if (MT == 1 && !CL && prm.split_tiles > 0) {      // that launch: nothing to do where the one in front has taken it along
+  if (MAY_BE_SECOND && prm.split_tiles > 0) {
+    if (ld_acquire(prm.passed) != prm.passed_tag) gdc_wait();
     int tiles = 0;
 #pragma unroll 1
     for (int b = lane; b < prm.B; b += 32) {
       const int S = __ldcg(prm.prefix_len + b);
       tiles += ((S < 0 ? 0 : (S > prm.Scap ? prm.Scap : S)) + kTileN - 1) / kTileN + prm.TT;
     }
-    if (!splits(__reduce_add_sync(0xffffffffu, tiles))) {
+    const int mode = odd_mode(__reduce_add_sync(0xffffffffu, tiles));
+    beside = mode == 1;
+    if (mode == 0 || (beside && blockIdx.x >= prm.beside_groups)) {      // no work for this CTA
       if (threadIdx.x == 0) gdc_launch_dependents();
-      if (blockIdx.x != 0) return;      // one CTA is enough to wait; the others leave their SMs (short calls 44.5 -> 43.4 us)
-      if (beside) end_beside();
-      else gdc_wait();
+      if (blockIdx.x == 0) end_pair();      // one CTA is enough to wait; the others leave their SMs (short calls 44.5 -> 43.4 us)
       return;
     }
   }
+
+  unsigned long long* const trace = prm.trace && beside ? prm.trace + (size_t)prm.slot0 * 2 * kTraceCap : prm.trace;
 
   // ---- setup: schedule table, barriers, TMEM
   if (threadIdx.x == 64) {     // fetch the five TMA descriptors while the rest of the set-up runs
@@ -605,7 +613,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     return false;
   };
   // one warp: Q and the first prefix tiles of this CTA's first item, a box per lane and turn, in the order of their use
-  // (items[2]: that item; at[0]: it is there; at[1]: where the search goes on; at[2]: CTA groups; at[3]: CTAs of a group)
+  // (items[2]: that item; at[0]: it is there; at[1]: where the search goes on, for the second launch of a pair its first slot; at[2]: CTA
+  // groups; at[3]: CTAs of a group)
   volatile int* at = reinterpret_cast<volatile int*>(items + 3);
   auto prefetch_first = [&]() {
     Item first;
@@ -673,8 +682,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // Small problems use fewer CTA groups, so that a unit is cut into few pieces (each piece costs a partial
         // write and a merge) and every group still gets a worthwhile share of tiles.
         const int units = prm.B * prm.Hkv * prm.L;
-        const bool split = MT == 2 && prm.split_tiles > 0 && splits(run - prm.B * kSetupCost);
-        const int np = split ? prm.front_NP : prm.NP, max_groups = split ? prm.front_groups : prm.groups;
+        const int mode = prm.split_tiles > 0 ? odd_mode(run - prm.B * kSetupCost) : 0;
+        const int np = mode ? prm.split_NP : prm.NP;
+        const int max_groups = mode == 0 ? prm.groups : (mode == 1 ? prm.beside_groups : prm.behind_groups);
         const int want = (int)((unsigned)(prm.Hkv * run) * (unsigned)prm.L / (unsigned)kMinVirtualTilesPerGroup);
         int n = want < 1 ? 1 : (want < max_groups ? want : max_groups);
         // A group count just above a multiple of the unit count is rounded down to it: with units of equal length
@@ -683,6 +693,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // those stay whole, one a group, because a cut and its merge cost more than the idle groups.
         const int over = n % units;
         if (n > units && (over * 16 <= n || (n < 2 * units && same && first_len <= kMaxWholeUnit))) n -= over;
+        if (MAY_BE_SECOND) at[1] = mode == 1 ? prm.slot0 : 0;      // (a launch of a pair builds its table once, the second one)
         at[2] = n;
         at[3] = np;
       }
@@ -773,7 +784,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t item_idx = 0, fill = 0;
       bool ok = true;
       Tracer tr;
-      tr.init(lane == 0 ? prm.trace : nullptr, 0);
+      tr.init(lane == 0 ? trace : nullptr, 0);
       tr.mark(0);
       uint64_t kv_policy;      // the committed prefix is streamed once: first in line for eviction from L2
       asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(kv_policy));
@@ -917,7 +928,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t done[2] = {0, 0};             // KS: key tiles of each warpgroup in earlier items
       bool ok = true;
       Tracer tr;
-      tr.init(lane == 0 ? prm.trace : nullptr, 1);
+      tr.init(lane == 0 ? trace : nullptr, 1);
       tr.mark(0);
       // descriptor words: low = start address >> 4 | LBO field, high = SBO 1024 B | version 1 | 128-byte swizzle
       const uint32_t desc_hi = (uint32_t)(smem_desc(0, 0, 1024) >> 32);
@@ -1134,7 +1145,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t od_phase = 0;                                    // completions of O_DONE so far
       bool ok = true;
       Tracer tr;
-      tr.init((threadIdx.x & 127) == 0 ? prm.trace : nullptr, 2 + wg);
+      tr.init((threadIdx.x & 127) == 0 ? trace : nullptr, 2 + wg);
       tr.mark(0);
       // Rendezvous of the softmax warpgroups through an mbarrier, so that it is bounded like every other wait.
       // All 32 lanes wait together and agree on the outcome, so that the warp-wide TMEM instructions
@@ -1477,6 +1488,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // group is one of them: two short walks over the cut table find both ends.
             const int np = at[3], place = (int)(blockIdx.x / np), groups = at[2];      // (read here: registers are short in the loop)
             const int group = place < groups ? groups - 1 - place : place;
+            const int slot0 = MAY_BE_SECOND && prm.split_tiles > 0 ? at[1] : 0;
             const int real0 = it.layer * (prm.Hkv * cum[prm.B]) + prm.Hkv * cum[it.b] + it.hk * (it.len + kSetupCost) + kSetupCost;
             const int uend = real0 + it.len;
             int k_first = group, k_last = group;
@@ -1485,7 +1497,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const int n_other = k_last - k_first;
             const float inv_own = (row_active && m_used > -INFINITY) ? 1.f / l_sum : 0.f;
             if (group != k_first) {
-              const size_t slot = (size_t)group * np + pair;
+              const size_t slot = (size_t)slot0 + (size_t)group * np + pair;
               uint4* po = reinterpret_cast<uint4*>(prm.part_o) + slot * (D / 8) * kRows;
               float* pml = prm.part_ml + slot * 2 * kRows;
               if (row_active && !(KS && wg)) {
@@ -1511,7 +1523,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 // 8000 59.8 -> 55.9).
 #pragma unroll 1
                 for (int i = 1 + lane; i <= n_other; i += 32) {
-                  unsigned long long* flag = prm.flags + (size_t)(k_first + i) * np + pair;
+                  unsigned long long* flag = prm.flags + slot0 + (size_t)(k_first + i) * np + pair;
                   const unsigned long long t0 = globaltimer_ns();
                   while (ld_acquire(flag) != prm.epoch) {
                     if (*abort_flag || globaltimer_ns() - t0 > wait_limit) {
@@ -1532,7 +1544,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               // bytes and are masked by selects): no thread-divergent branch sits between the warp-wide TMEM ops.
               // (64-wide heads with many pieces a unit: 32-bit slots 48.3 -> 47.8 us a call; the others keep 64 bits, level or 1 %)
               using Slot = std::conditional_t<D == 64, uint32_t, size_t>;
-              auto slot_of = [&](int i) -> Slot { return (Slot)(k_first + i) * (Slot)np + (Slot)pair; };       // i-th other piece, i >= 1
+              auto slot_of = [&](int i) -> Slot { return (Slot)slot0 + (Slot)(k_first + i) * (Slot)np + (Slot)pair; };       // i-th other piece, i >= 1
               auto ml_of = [&](int i) -> const float* { return prm.part_ml + slot_of(i) * 2 * kRows + rr; };
               auto o_of = [&](int i) -> const uint4* { return reinterpret_cast<const uint4*>(prm.part_o) + slot_of(i) * (D / 8) * kRows + rr; };
               // two pieces at a time: (m, l) of the row and the columns of this warpgroup
@@ -1742,7 +1754,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   }
 
   // ---- teardown
-  if (beside) end_beside();
+  if (MAY_BE_SECOND && prm.split_tiles > 0) end_pair();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -1809,8 +1821,8 @@ Geometry geometry(int B, int Nmax, int Hq, int Hkv, int d, bool query_device) {
   // of the first one: the pieces of CTA group 0 are all the first of their unit, which leave no partial; then a
   // stretch per layer, none of which is used: how many there are bounds the layers that share a launch
   constexpr size_t kSlotsMax = 160;
-  static_assert(kSlotsMax == kMaxGroups && (kSlotsMax + 1) * sizeof(unsigned long long) <= 128 * 64 * sizeof(tv_bf16),
-                "the flags and the one between two launches fit a slot of one row tile, 64-wide");
+  static_assert(kSlotsMax == kMaxGroups && (2 * kSlotsMax + 1) * sizeof(unsigned long long) <= 128 * 64 * sizeof(tv_bf16),
+                "the flags, two for a slot of two row tiles, and the one between two launches fit a slot of one row tile, 64-wide");
   const size_t ml_bytes = (size_t)g.MT * 128 * 2 * sizeof(float);
   g.ml_off = 0;
   g.o_off = (kSlotsMax * ml_bytes + 255) & ~size_t(255);
@@ -1932,35 +1944,27 @@ cudaError_t launch(const Geometry& g, const CUtensorMap* maps, AttnParams prm, c
   // the other finds nothing to do, some 2 us).
   if (MT == 2 && g.n_row_tiles % 2 == 1 && units * tiles >= (long long)kSplitTilesPerSm * g.sms) {
     const tv::OddRowTile odd = tv::odd_row_tile(g.sms, g.n_row_tiles, D);
-    if (odd.front_groups > 0) {
+    if (odd.behind_groups > 0) {
+      prm.split_tiles = odd.split_from * g.sms;
+      prm.behind_tiles = odd.behind_from * g.sms;
+      prm.passed = prm.flags + 2 * kMaxGroups;
+      prm.passed_tag = prm.epoch;
       AttnParams front = prm;
-      front.split_tiles = odd.tiles_per_sm * g.sms;
-      front.front_NP = g.n_row_tiles / 2;
-      front.front_groups = odd.front_groups;
-      if (odd.beside) {
-        front.passed = prm.flags + kMaxGroups;
-        front.passed_tag = prm.epoch;
-      }
-      const int ctas = front.front_groups * front.front_NP;
+      front.split_NP = g.n_row_tiles / 2;
+      front.beside_groups = odd.beside_groups;
+      front.behind_groups = odd.behind_groups;
+      const int ctas = front.behind_groups * front.split_NP;      // (never fewer than beside the other launch)
       const cudaError_t e = launch_kernel<D, MT, false>((unsigned)(ctas > g.grid ? ctas : g.grid), 1, maps, front, s);
       if (e != cudaSuccess) return e;
       tv::count_launches(1);
-      prm.split_tiles = front.split_tiles;
       prm.tile0 = g.n_row_tiles - 1;
-      prm.NP = 1;
-      prm.groups = odd.odd_groups;
+      prm.NP = prm.split_NP = 1;
+      prm.beside_groups = odd.odd_groups;
+      prm.behind_groups = g.sms;
+      prm.slot0 = 2 * odd.beside_groups * front.split_NP;         // behind those of the first launch, which are twice as long
       prm.early = 1;          // behind a launch of this very call the inputs are stable
       prm.epoch = next_epoch();
-      if (odd.beside) {
-        prm.beside = 1;
-        prm.passed = front.passed;
-        prm.passed_tag = front.passed_tag;
-        prm.part_ml += (size_t)ctas * 2 * MT * 128;      // the slots and flags behind those of the front launch
-        prm.part_o += (size_t)ctas * MT * 128 * D;
-        prm.flags += ctas;
-        if (prm.trace) prm.trace += (size_t)ctas * 4 * kTraceCap;
-      }
-      return launch_kernel<D, 1, false>((unsigned)prm.groups, 1, maps, prm, s);
+      return launch_kernel<D, 1, false>((unsigned)g.sms, 1, maps, prm, s);
     }
   }
   return launch_kernel<D, MT, false>((unsigned)g.grid, 1, maps, prm, s);

@@ -635,19 +635,21 @@ ODD = [(65, 64, False), (65, 128, True), (129, 64, True), (129, 128, False)]    
 
 
 @pytest.mark.parametrize("N,d,paged", ODD)
-@pytest.mark.parametrize("what", ["short", "below", "at", "long"])
+@pytest.mark.parametrize("what", ["short", "below", "at", "long", "last beside", "first behind"])
 def test_last_row_tile_goes_by_the_lengths_and_not_by_the_capacity(N, d, paged, what):
     """A cache that could hold enough key tiles for two launches.  With short prefixes and one key tile below the bound the call gives
     the bits it gives in a small cache, where it is one launch; at the bound the last row tile is cut elsewhere, and its bits are
-    others; the oracle's values on sampled heads all the same, and far beyond the bound."""
-    B, L, Hkv, G, cap = 10, 4, 8, 4, 4480
+    others; the oracle's values on sampled heads all the same, far beyond the bound, and where the second launch runs behind the first
+    one instead of beside it."""
+    B, L, Hkv, G, cap = 10, 4, 8, 4, 6400
     TT = (N + 127) // 128
     cfg = CONFIGS[0].scaled(B=B, L=L, Hq=G * Hkv, Hkv=Hkv, d=d, S_lo=20, S_hi=400, Scap=cap, N=N, D=6, V=0, tree="uniform")
     case = make_case(cfg, seed=N + d, device="cuda", ragged_nodes=True, with_logits=False)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     if what != "short":
         bound = -(-12 * sms // (L * Hkv))                  # key tiles of the sequences together at which the rule changes
-        total = {"below": bound - 1, "at": bound, "long": bound + 260}[what]
+        behind = -(-(60 if d == 64 else 100) * sms // (L * Hkv))
+        total = {"below": bound - 1, "at": bound, "long": bound + 120, "last beside": behind - 1, "first behind": behind}[what]
         tiles = np.full(B, total // B) + (np.arange(B) < total % B)
         tiles[0] -= 3
         tiles[1] += 3
@@ -679,7 +681,7 @@ def test_last_row_tile_goes_by_the_lengths_and_not_by_the_capacity(N, d, paged, 
 
     out, lse, launches = run(cap)
     assert launches == 2
-    if what != "long":
+    if what in ("short", "below", "at"):
         small, small_lse, launches = run(1024)
         assert launches == 1 and torch.equal(out, small) == (what != "at")
         assert what == "at" or torch.equal(lse, small_lse)
