@@ -164,9 +164,9 @@ TV_API size_t tv_attn_workspace_bytes(int B, int Nmax, int Hq, int Hkv, int d, i
  * Using the committed prefix earlier is what tree_verify_attn_layers offers,
  * under a promise by the caller.
  * Launches: one kernel, or two (an odd last row tile of long problems runs
- * beside the others, in wide head groups behind them; whether it does is
- * decided from the lengths on the device, in caches whose capacity allows
- * such problems).  How the work is shared between CTAs follows the shape, the
+ * beside the others, or behind them; whether it does, and which, is decided
+ * from the lengths on the device, in caches whose capacity allows such
+ * problems).  How the work is shared between CTAs follows the shape, the
  * capacity and the lengths; results agree to the rounding of the partial sums.
  */
 TV_API int tree_verify_attn(const tv_bf16* q,
